@@ -52,12 +52,12 @@ typedef enum {
 
 /* Closure arithmetic. */
 enum {
-    KITRT_FP64 = 0,        /* every sum, factorisation and line search in FP64 */
+    KITRT_FP64 = 0,        /* quadrature sums to FP64 accuracy in 64-bit fixed point (their error is
+                              that of FP64 sums); factorisation and line search in FP64 */
     KITRT_MIXED_TF32 = 1,  /* Hessian-only moment sums on tensor cores (TF32 in, FP32 accumulate);
-                              exponent, gradient, objective and line search in FP64 (the exp to
-                              about 1e-14 relative, its small polynomial term in FP32); the Newton
-                              step's Hessian assembly and Cholesky in FP32, in FP64 for cells
-                              handed over */
+                              exponent, exp and gradient sums as in FP64 mode, objective and line
+                              search in FP64; the Newton step's Hessian assembly and Cholesky in
+                              FP32, in FP64 for cells handed over */
     KITRT_MIXED_BF16 = 2,  /* as MIXED_TF32 with BF16 tensor-core inputs */
     KITRT_LEARNED = 3      /* MLP prediction of alpha, exact mass fix, FP64 residual check, Newton
                               (mixed Hessian) only for cells whose residual exceeds fallback_tol */
@@ -177,10 +177,10 @@ int32_t kitrt_mn_sizes(const kitrt_mn *mn, int32_t *nmom, int32_t *nquad, int32_
  *                      azimuthal sums up to degree L (L = N in the mixed modes, whose higher
  *                      moments run on tensor cores; L = 2N in FP64 mode), per ring the exponent
  *                      coefficients (n FMA) and the moments (nmom(L) FMA);
- *   sweep_fp64_ops     FP64-pipe instructions of the same sweep including the exponentials
- *                      (on the common path of the table-driven method: 8 per exp in FP64
- *                      mode; 2 in the mixed modes, whose exponents are pre-scaled by 2048/ln2
- *                      and whose small polynomial term is formed in FP32);
+ *   sweep_fp64_ops     FP64-pipe instructions that the same sweep takes where it is done in FP64,
+ *                      including the exponentials (8 per exp in FP64 mode, 2 in the mixed modes):
+ *                      a measure of the work; the sweeps themselves run in 64-bit fixed point on
+ *                      the integer pipes;
  *   exps               exponentials per evaluation (Q');
  *   tensor_flops       mixed modes: 3 x 2 (n2 - n) Q' on tensor cores (three split products);
  *   newton_flops       the per-cell Newton step: 2 nnz (Hessian) + n^3/3 + 2n^2 (Cholesky,

@@ -316,65 +316,113 @@ eval_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, Newton
 }
 
 // ---------------------------------------------------------------------------------------------
-// FP64 sweep of the FP64 mode: one thread per listed cell (tiles of 128), every degree-2N moment
-// in the sum-factorised form of sweep.cuh. Work items are (tile, part of the quadrature); each
+// Sweep of the FP64 mode: one thread per listed cell (tiles of 128), every degree-2N moment in the
+// sum-factorised fixed-point form of sweep.cuh. Work items are (tile, part of the quadrature); each
 // stores its partial moments with plain stores into its own column block of Vacc, which the
 // Newton kernel adds in order, so the result does not depend on scheduling.
 // ---------------------------------------------------------------------------------------------
 constexpr int kSweepThreads = 128;
 
+// Dynamic shared memory of sweep64_kernel: the exp table, the moments [n2][thread] and the trial
+// alpha's limbs [n][thread], the azimuthal factors.
+size_t sweep64_smem(int n, int n2, int N, int J)
+{
+    return 2048 * 8 + (size_t)(n2 + n) * kSweepThreads * 8 + (size_t)J * 4 * N * 8;
+}
+
 template <int NN>
 __global__ void __launch_bounds__(kSweepThreads)
-sweep64_kernel(Tables T, NewtonState S, int k, double *__restrict__ Vacc, int vs, int target_items)
+sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, double *__restrict__ Vacc, int vs,
+               int target_items)
 {
-    constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, NA = 2 * NN + 1, NB = 4 * NN + 1;
-    constexpr int TW = 4 * NN + 1;
-    __shared__ double sV[n2 * kSweepThreads];  // [n2][thread]
+    constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, L2 = 2 * NN;
+    extern __shared__ __align__(16) unsigned char sweep_smem[];
+    uint64_t *tab = (uint64_t *)sweep_smem;
+    long long *sV = (long long *)(tab + 2048);
+    int2 *sA = (int2 *)(sV + n2 * kSweepThreads);
+    int2 *trig = sA + n * kSweepThreads;
     const int32_t *list_in = S.list[k & 1];
     const int cnt_in = S.cnt[k % 3];
     if (blockIdx.x == 0 && threadIdx.x == 0) S.cnt[(k + 2) % 3] = 0;
-    const int nunits = T.Qp / 32;
-    const SweepSplit sp = sweep_split(cnt_in, target_items, nunits);
+    const int nunits = T.Qs / 32;
+    const SweepSplit sp = sweep_split(cnt_in, gridDim.x, target_items, nunits);
     const int items = sp.tiles * sp.parts;
-    double *mine = sV + threadIdx.x;
+    if ((int)blockIdx.x >= items) return;
+    for (int j = threadIdx.x; j < 2048; j += kSweepThreads) tab[j] = T.fx_exp[j];
+    for (int j = threadIdx.x; j < T.J * 2 * L2; j += kSweepThreads) trig[j] = T.fx_trig[j];
+    __syncthreads();
+    long long *mine = sV + threadIdx.x;
+    int2 *myA = sA + threadIdx.x;
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
         const int tile = item / sp.parts, part = item % sp.parts;
         const int slot = tile * kSweepThreads + threadIdx.x;
         if (slot >= cnt_in) continue;  // threads are independent: no block barrier below
-        const int p_begin = part * sp.units_per_part * 16;
-        // padding pairs (w = 0) add nothing: stop at the last real pair
-        const int p_end = min(T.npair, min(nunits, (part + 1) * sp.units_per_part) * 16);
+        const int q_begin = part * nunits / sp.parts * 8;
+        // padding quads add nothing: stop at the last real one
+        const int q_end = min(T.nquad, (part + 1) * nunits / sp.parts * 8);
         const int cell = list_in[slot];
-        const size_t off = (size_t)cell * n;
-        const int ph = S.phase[cell];
-        const double lam = ph == PH_NEWTON ? S.lam[cell] : 0.0;
-        double at[n], A[NA], B[NB];
+        const double *al = S.alpha + (size_t)cell * n, *di = S.dir + (size_t)cell * n;
+        const double lam = S.phase[cell] == PH_NEWTON ? S.lam[cell] : 0.0;
+        float bound = 0.0f;
 #pragma unroll
         for (int a = 0; a < n; ++a) {
-            const double al = S.alpha[off + a];
-            at[a] = ph == PH_NEWTON ? fma(lam, S.dir[off + a], al) : al;
+            const double x = lam != 0.0 ? fma(lam, di[a], al[a]) : al[a];
+            const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(x));
+            myA[a * kSweepThreads] = make_int2(w.h, w.l);
+            bound = fmaf(fabsf(d2f_bits(x)), T.fx_mmax[a], bound);
         }
+        // rows outside the fixed-point range (or not finite) take the FP64 exponentials
+        const bool wide = !(bound < kitrt_fx::kFxMaxZ);
+        bool bad = false;
 #pragma unroll
-        for (int c = 0; c < n2; ++c) mine[c * kSweepThreads] = 0.0;
-#pragma unroll
-        for (int j = 0; j < NB; ++j) B[j] = 0.0;
-        auto V = [&](int c) -> double & { return mine[c * kSweepThreads]; };
-        int ring = -1;
-        for (int pr = p_begin; pr < p_end; ++pr) {
-            const int rg = pr < T.npair ? pr / T.P : T.R;
-            if (rg != ring) {
-                if (ring >= 0) ring_flush<2 * NN>(T.ringWP + (size_t)ring * n2, B, V);
-                ring_coeffs<NN>(at, T.ringP + (size_t)rg * n2, A);
-                ring = rg;
+        for (int c = 0; c < n2; ++c) mine[c * kSweepThreads] = 0;
+        long long A0 = 0;
+        Limb A[2 * NN];
+        FxSums<L2> B;
+        B.clear();
+        B.Sx = kitrt_fx::fx_scale_of(u[(size_t)cell * n]);
+        auto trial = [&](int a) {
+            const int2 v = myA[a * kSweepThreads];
+            return Limb{v.x, v.y};
+        };
+        auto moment = [&](int c) -> long long & { return mine[c * kSweepThreads]; };
+        int ring = q_begin / T.J, jq = q_begin - ring * T.J;
+        bool fresh = true;
+#pragma unroll 1
+        for (int qd = q_begin; qd < q_end; ++qd) {
+            if (fresh) {
+                fx_coeffs<NN>(trial, T.fx_ringA + (size_t)ring * n, A0, A);
+                fresh = false;
             }
-            double e1, e2;
-            pair_eval<NN, 2 * NN>(A, T.ptrig + (size_t)pr * TW, pr < T.npair && pr % T.P == 0,
-                                  T.exptab, B, e1, e2);
-        }
-        if (ring >= 0) ring_flush<2 * NN>(T.ringWP + (size_t)ring * n2, B, V);
-        double *col = Vacc + (size_t)part * cnt_in + slot;
+            const int2 *tr = trig + jq * 2 * L2;
+            const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
+            Exp e[4];
+            if (!wide) {
+                long long s[4];
+                fx_exponents<NN>(A0, A, tr, L2, jq == 0, s);
 #pragma unroll
-        for (int c = 0; c < n2; ++c) col[(size_t)c * vs] = mine[c * kSweepThreads];
+                for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_exp(s[t], tab);
+            } else {
+                bad = !fx_slow_quad<NN>(T.Mt, T.Qp, T.exptab, al, di, lam, pa, pb, e) || bad;
+            }
+            if (pb < 0) e[2] = e[3] = Exp{0, -100000};
+            fx_accumulate<L2>(e, tr, L2, jq == 0, pb < 0, qd == q_begin, B, [&](int d) {
+                for (int c = 0; c < n2; ++c) mine[c * kSweepThreads] = kitrt_fx::sar(mine[c * kSweepThreads], d);
+            });
+            if (++jq == T.J) {
+                fx_flush<L2>(T.fx_ringW + (size_t)ring * n2, T.fx_sumshift, B, moment);
+                jq = 0;
+                ++ring;
+                fresh = true;
+            }
+        }
+        if (!fresh) fx_flush<L2>(T.fx_ringW + (size_t)ring * n2, T.fx_sumshift, B, moment);
+        double *col = Vacc + (size_t)part * cnt_in + slot;
+        const int unit = fx_unit(B.Sx, T);
+#pragma unroll 4
+        for (int c = 0; c < n2; ++c)
+            col[(size_t)c * vs] = bad ? __longlong_as_double(0x7ff8000000000000LL)
+                                      : kitrt_fx::fx_to_double(mine[c * kSweepThreads], unit);
     }
 }
 
@@ -559,10 +607,10 @@ int launch_isotropic(const Tables &T, int C, const double *u, double *alpha, cud
 // gradient moments, and every moment of a row handed to the FP64 sweep (its part 0 holds the
 // FP64 sums, its other parts zeros), in FP64.
 __global__ void sum_parts_kernel(NewtonState S, int k, double *__restrict__ Vacc, int vs, int n,
-                                 int n2, int target_items, int nunits, int mixed)
+                                 int n2, int grid, int target_items, int nunits, int mixed)
 {
     const int cnt = S.cnt[k % 3];
-    const int parts = sweep_split(cnt, target_items, nunits).parts;
+    const int parts = sweep_split(cnt, grid, target_items, nunits).parts;
     if (parts <= 1) return;
     const int32_t *list = S.list[k & 1];
     const size_t total = (size_t)n2 * cnt, pstride = (size_t)cnt;
@@ -587,8 +635,8 @@ int launch_sum_parts(kitrt_mn *mn, const NewtonState &S, int k, double *Vacc, cu
     const int mixed = mn->p.mode != KITRT_FP64;
     LaunchScope ls(mn, PK_POST, s, 0);
     sum_parts_kernel<<<mn->nsm * 8, 256, 0, s>>>(S, k, Vacc, mn->vs, mn->n, mn->n2,
-                                                 mixed ? mn->target_mixed : mn->target_fp64,
-                                                 mn->Qp / 32, mixed);
+                                                 mixed ? mn->grid_mixed : mn->grid_fp64,
+                                                 mixed ? mn->target_mixed : mn->target_fp64, mn->Qs / 32, mixed);
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }
 
@@ -600,8 +648,7 @@ int launch_post(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, cons
     int blocks = (C + kPostBlock - 1) / kPostBlock;
     if (blocks > mn->nsm * 32) blocks = mn->nsm * 32;
     const int mixed = mn->p.mode != KITRT_FP64;
-    // sum_parts_kernel has added the sweeps' parts into part 0 (target 0 gives one part)
-    const int target = 0;
+    const int target = 1;
     const size_t smem = post_smem_bytes(mn->n, mn->n2, mn->npairs, mn->gaunt_nnz, mixed != 0,
                                         kUnrolledNewton && mn->N <= 3);
     int rc = KITRT_OK;
@@ -658,15 +705,22 @@ int launch_begin(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
 // Grid of the FP64 sweep: as many CTAs as are resident on all SMs at once.
 int fp64_sweep_grid(const kitrt_mn *mn)
 {
+    const size_t smem = sweep64_smem(mn->n, mn->n2, mn->N, mn->J);
     int resident = 1;
+#define GRID_CASE(NNv)                                                              \
+    case NNv:                                                                       \
+        if (ensure_dyn_smem(sweep64_kernel<NNv>, smem)) return mn->nsm;             \
+        resident = resident_ctas(sweep64_kernel<NNv>, kSweepThreads, smem, 8);      \
+        break;
     switch (mn->N) {
-    case 1: resident = resident_ctas(sweep64_kernel<1>, kSweepThreads, 0, 8); break;
-    case 2: resident = resident_ctas(sweep64_kernel<2>, kSweepThreads, 0, 8); break;
-    case 3: resident = resident_ctas(sweep64_kernel<3>, kSweepThreads, 0, 8); break;
-    case 4: resident = resident_ctas(sweep64_kernel<4>, kSweepThreads, 0, 8); break;
-    case 5: resident = resident_ctas(sweep64_kernel<5>, kSweepThreads, 0, 8); break;
+        GRID_CASE(1)
+        GRID_CASE(2)
+        GRID_CASE(3)
+        GRID_CASE(4)
+        GRID_CASE(5)
     default: break;
     }
+#undef GRID_CASE
     return mn->nsm * resident;
 }
 
@@ -683,7 +737,11 @@ int launch_eval_fp64(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
         // cells handed to the FP64 Hessian: whole sums into part 0 of their list slots
         KITRT_DISPATCH_N(mn->N, (eval_kernel<NN, true, false><<<grid, kWarps * 32, 0, s>>>(T, S, u, k, np, psi32, Vacc, mn->vs)));
     } else {
-        KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN><<<mn->grid_fp64, kSweepThreads, 0, s>>>(T, S, k, Vacc, mn->vs, mn->target_fp64)));
+        const size_t smem = sweep64_smem(mn->n, mn->n2, mn->N, mn->J);
+        int rc = KITRT_OK;
+        KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(sweep64_kernel<NN>, smem));
+        if (rc) return rc;
+        KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN><<<mn->grid_fp64, kSweepThreads, smem, s>>>(T, S, u, k, Vacc, mn->vs, mn->target_fp64)));
     }
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }

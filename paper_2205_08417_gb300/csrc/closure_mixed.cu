@@ -147,10 +147,14 @@ struct MixedSmem {
     static __host__ __device__ constexpr int off_Alo(int b) { return b * buf_bytes + A_bytes; }
     static __host__ __device__ constexpr int off_Bhi(int b) { return b * buf_bytes + 2 * A_bytes; }
     static __host__ __device__ constexpr int off_Blo(int b) { return b * buf_bytes + 2 * A_bytes + B_bytes; }
+    // the trial alpha's limbs during the quadrature, then the second half's moments: [n][128] 8 bytes
     static constexpr int off_V = (2 * buf_bytes + 1023) / 1024 * 1024;
-    static constexpr int V_bytes = kTileM * Dims<NN>::n * 8;      // second half's gradient sums
-    static constexpr int off_bar = off_V + V_bytes;
-    static constexpr int total = off_bar + 64;
+    static constexpr int V_bytes = kTileM * Dims<NN>::n * 8;
+    static constexpr int off_exp = off_V + V_bytes;               // exp table
+    static constexpr int off_sx = off_exp + 2048 * 8;             // [2][128] guard sums, then scales
+    static constexpr int off_bar = off_sx + 2 * kTileM * 4;
+    static constexpr int off_trig = off_bar + 64;                 // [J][2 NN] limbs
+    static int total(int J) { return off_trig + J * 2 * NN * 8; }
     static constexpr int kmma = BF16 ? 16 : 8;                   // MMA K
     // byte offset of element (row r, k) inside an operand chunk
     static __device__ __forceinline__ int elem_off(int r, int k)
@@ -159,22 +163,33 @@ struct MixedSmem {
     }
 };
 
-// E rounded to the tensor-core input format, split into a high and a low part, at (row r, k) of
-// the chunk's operand tiles.
+// Four consecutive E of row r (k = kk .. kk + 3, kk a multiple of 4) rounded to the tensor-core
+// input format, split into a high and a low part, as one 16-byte (TF32) or 8-byte (BF16) piece.
+// TF32 rounding (nearest, ties away) in integer arithmetic.
 template <bool BF16, typename L>
-__device__ __forceinline__ void store_operand(unsigned char *Ahi, unsigned char *Alo, int r, int kk, float e)
+__device__ __forceinline__ void store_operand4(unsigned char *Ahi, unsigned char *Alo, int r, int kk, const float (&e)[4])
 {
     if (BF16) {
-        const __nv_bfloat16 hi = __float2bfloat16_rn(e);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(e - __bfloat162float(hi));
-        *(__nv_bfloat16 *)(Ahi + L::elem_off(r, kk)) = hi;
-        *(__nv_bfloat16 *)(Alo + L::elem_off(r, kk)) = lo;
+        ushort4 hi, lo;
+        unsigned short *h = &hi.x, *l = &lo.x;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const __nv_bfloat16 x = __float2bfloat16_rn(e[i]);
+            h[i] = __bfloat16_as_ushort(x);
+            l[i] = __bfloat16_as_ushort(__float2bfloat16_rn(e[i] - __bfloat162float(x)));
+        }
+        *(ushort4 *)(Ahi + L::elem_off(r, kk)) = hi;
+        *(ushort4 *)(Alo + L::elem_off(r, kk)) = lo;
     } else {
-        uint32_t hi, lo;
-        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hi) : "f"(e));
-        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(e - __uint_as_float(hi)));
-        *(uint32_t *)(Ahi + L::elem_off(r, kk)) = hi;
-        *(uint32_t *)(Alo + L::elem_off(r, kk)) = lo;
+        uint4 hi, lo;
+        uint32_t *h = &hi.x, *l = &lo.x;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            h[i] = (__float_as_uint(e[i]) + 0x1000u) & ~0x1FFFu;
+            l[i] = (__float_as_uint(e[i] - __uint_as_float(h[i])) + 0x1000u) & ~0x1FFFu;
+        }
+        *(uint4 *)(Ahi + L::elem_off(r, kk)) = hi;
+        *(uint4 *)(Alo + L::elem_off(r, kk)) = lo;
     }
 }
 
@@ -187,20 +202,24 @@ __device__ __forceinline__ void store_operand(unsigned char *Ahi, unsigned char 
 template <int NN, bool BF16, bool MOMENTS_ONLY>
 __global__ void __launch_bounds__(kThreads, NN <= 3 ? 2 : 1)
 eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
-                  const double *__restrict__ alpha_in, double *__restrict__ Vacc, int vs_c, int vs_s,
+                  const double *__restrict__ u, const double *__restrict__ alpha_in, double *__restrict__ Vacc, int vs_c, int vs_s,
                   int C, int target_items, float *__restrict__ psi32)
 {
     using D = MixedDims<NN>;
     using L = MixedSmem<NN, BF16>;
-    constexpr int n = D::n, n2 = D::n2, NP = D::NP, NA = 2 * NN + 1;
+    constexpr int n = D::n, n2 = D::n2, NP = D::NP;
     extern __shared__ __align__(1024) unsigned char smem[];
     uint64_t *bar = (uint64_t *)(smem + L::off_bar);
     uint32_t *tmem_slot = (uint32_t *)(smem + L::off_bar + 16);
     int *abort_flag = (int *)(smem + L::off_bar + 24);
-    double *sU = (double *)(smem + L::off_V);  // [n][128]: the second half's gradient moments
+    int2 *sA = (int2 *)(smem + L::off_V);            // [n][128]: limbs of the trial alpha
+    long long *sU = (long long *)(smem + L::off_V);  // [n][128]: the second half's gradient moments
+    float *sB = (float *)(smem + L::off_sx);         // [2][128]
+    int *sX = (int *)(smem + L::off_sx);             // [128]
+    const uint64_t *tab = (const uint64_t *)(smem + L::off_exp);
+    const int2 *trig = (const int2 *)(smem + L::off_trig);
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int Qp = T.Qp, nchunks = Qp / kChunk;
-    constexpr int TW = 4 * NN + 1;  // ptrig row width
+    const int Qp = T.Qp, nchunks = T.Qs / kChunk;
 
     int cnt_in;
     const int32_t *list_in = nullptr;
@@ -211,8 +230,8 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
         cnt_in = S.cnt[k % 3];
         if (blockIdx.x == 0 && tid == 0) S.cnt[(k + 2) % 3] = 0;
     }
-    const SweepSplit sp = sweep_split(cnt_in, target_items, nchunks);
-    const int ks = sp.parts, cpp = sp.units_per_part;
+    const SweepSplit sp = sweep_split(cnt_in, gridDim.x, target_items, nchunks);
+    const int ks = sp.parts;
     const int items = sp.tiles * ks;
     if ((int)blockIdx.x >= items) return;  // no work item for this CTA (uniform per CTA)
 
@@ -223,6 +242,11 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tmem_alloc(tmem_slot, D::tcols);
+    for (int j = tid; j < 2048; j += kThreads) ((uint64_t *)(smem + L::off_exp))[j] = T.fx_exp[j];
+    for (int j = tid; j < T.J * 2 * NN; j += kThreads) {
+        const int p = j / (2 * NN), q = j % (2 * NN);  // cosines 1..NN, then sines 1..NN
+        ((int2 *)(smem + L::off_trig))[j] = T.fx_trig[p * 4 * NN + (q < NN ? q : NN + q)];
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -233,94 +257,130 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
 
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
         const int tile = item / ks, part = item % ks;
-        const int c_begin = part * cpp, c_end = min(nchunks, c_begin + cpp);
+        const int c_begin = part * nchunks / ks, c_end = (part + 1) * nchunks / ks;
         const int base = tile * kTileM;
         const int rows = min(kTileM, cnt_in - base);
         int cell = -1;
         if (r < rows) cell = MOMENTS_ONLY ? base + r : list_in[base + r];
         bool active = cell >= 0;
         if (!MOMENTS_ONLY && active && S.h64[cell]) active = false;  // done by the FP64 sweep
-        double at[n], U[n], A[NA], B[NA];
-#pragma unroll
-        for (int a = 0; a < n; ++a) {
-            U[a] = 0.0;
-            at[a] = 0.0;
-        }
-#pragma unroll
-        for (int j = 0; j < NA; ++j) A[j] = B[j] = 0.0;
+        // trial point: each half forms every other component (inactive rows: 0)
+        const double *al = nullptr, *di = nullptr;
+        double lam = 0.0;
         if (active) {
             if (MOMENTS_ONLY) {
-#pragma unroll
-                for (int a = 0; a < n; ++a) at[a] = alpha_in[(size_t)cell * n + a];
+                al = di = alpha_in + (size_t)cell * n;
             } else {
-                const int ph = S.phase[cell];
-                const double lam = ph == PH_NEWTON ? S.lam[cell] : 0.0;
-#pragma unroll
-                for (int a = 0; a < n; ++a) {
-                    const double al = S.alpha[(size_t)cell * n + a];
-                    at[a] = ph == PH_NEWTON ? fma(lam, S.dir[(size_t)cell * n + a], al) : al;
-                }
+                al = S.alpha + (size_t)cell * n;
+                di = S.dir + (size_t)cell * n;
+                if (S.phase[cell] == PH_NEWTON) lam = S.lam[cell];
             }
-            // the pairs take the exponent in units of ln2/2048 (kexp_scaled)
-#pragma unroll
-            for (int a = 0; a < n; ++a) at[a] *= 2954.639443740597;  // 2048 / ln2
         }
-        int ring = -1;  // ring whose azimuthal sums B holds (uniform within a warp)
+        float bound = 0.0f;
+        for (int a = h; a < n; a += 2) {
+            double x = 0.0;
+            if (active) x = lam != 0.0 ? fma(lam, di[a], al[a]) : al[a];
+            const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(x));
+            sA[a * kTileM + r] = make_int2(w.h, w.l);
+            bound = fmaf(fabsf(d2f_bits(x)), T.fx_mmax[a], bound);
+        }
+        sB[tid] = bound;
+        __syncthreads();
+        // rows outside the fixed-point range (or not finite) take the FP64 exponentials
+        const bool wide = !(sB[r] + sB[kTileM + r] < kitrt_fx::kFxMaxZ);
+        bool bad = false;
+        long long U[n], A0 = 0;
+        Limb A[2 * NN];
+        FxSums<NN> B;
+#pragma unroll
+        for (int a = 0; a < n; ++a) U[a] = 0;
+        B.clear();
+        B.Sx = MOMENTS_ONLY || !active ? 100000 : kitrt_fx::fx_scale_of(u[(size_t)cell * n]);
+        auto trial = [&](int a) {
+            const int2 v = sA[a * kTileM + r];
+            return Limb{v.x, v.y};
+        };
+        auto moment = [&](int a) -> long long & { return U[a]; };
+        // quads of this thread: nch x 4 consecutive ones, starting at q0
+        const int nch = c_end - c_begin;
+        const int q0 = c_begin * (kChunk / 4) + h * nch * (kChunk / 8);
+        int ring = q0 / T.J, jq = q0 - ring * T.J;  // ring and place in it (uniform within a warp)
+        bool fresh = true;                          // the ring's coefficients are not formed yet
+        if (q0 >= T.nquad) B.Sx = -100000;          // only padding: its zero sums follow any scale
         for (int c = c_begin; c < c_end; ++c) {
             const int b = c & 1;
             unsigned char *Ahi = smem + L::off_Ahi(b), *Alo = smem + L::off_Alo(b);
             unsigned char *Bhi = smem + L::off_Bhi(b), *Blo = smem + L::off_Blo(b);
+            bool failed = false;
             if (commits[b] > waited[b]) {
-                // the MMAs that read this buffer must have finished before it is overwritten:
-                // one thread waits on the buffer's mbarrier, the CTA barrier orders the rest
-                if (tid == 0 && !mbar_wait_bounded(&bar[b], waited[b] & 1)) *abort_flag = 1;
+                // the MMAs that read this buffer must have finished before it is overwritten
+                failed = !mbar_wait_bounded(&bar[b], waited[b] & 1);
                 ++waited[b];
-                __syncthreads();
-                if (*abort_flag) break;  // uniform: read after the barrier
             }
             tc_fence_after();
-            // FP64 part: 8 pairs of this row (exponents, exp, gradient sums); E to the operand
-#pragma unroll 2
-            for (int i = 0; i < kChunk / 4; ++i) {
-                const int pr = c * (kChunk / 2) + h * (kChunk / 4) + i;
-                // padding pairs (w = 0, warp-uniform) add nothing: their operand is 0 and their
-                // psi stays at the zeros written at allocation
-                const bool real = pr < T.npair;
-                if (real) {
-                    const int rg = pr / T.P;
-                    if (rg != ring) {
-                        if (ring >= 0)
-                            ring_flush<NN>(T.ringWP + (size_t)ring * n2, B, [&](int cc) -> double & { return U[cc]; });
-                        ring_coeffs<NN>(at, T.ringP + (size_t)rg * n2, A);
-                        ring = rg;
-                    }
-                }
-                float f1 = 0.0f, f2 = 0.0f;
-                if (active && real) {
-                    double e1, e2;
-                    pair_eval<NN, NN, true>(A, T.ptrig + (size_t)pr * TW, pr % T.P == 0, T.exptab, B, e1, e2);
-                    f1 = exp_to_float(e1);
-                    f2 = exp_to_float(e2);
-                    // ansatz of the trial point (the last accepted trial leaves the solution's)
-                    if (psi32) *(float2 *)(psi32 + (size_t)cell * Qp + 2 * pr) = make_float2(f1, f2);
-                }
-                const int kk = h * (kChunk / 2) + 2 * i;
-                store_operand<BF16, L>(Ahi, Alo, r, kk, f1);
-                store_operand<BF16, L>(Ahi, Alo, r, kk + 1, f2);
-            }
-            // stage the chunk of the split table (row-major [2][NP x Qp] in global: high part,
-            // then low part), in 16-byte pieces
+            // stage the chunk of the split table (row-major [2][NP x Qs] in global: high part,
+            // then low part) by asynchronous 16-byte copies, which land during the quads below
             constexpr int per16 = L::T;  // elements per 16 bytes
             constexpr int pieces = NP * (kChunk / per16);
             for (int p = tid; p < 2 * pieces; p += kThreads) {
                 const int hl = p / pieces, pp = p % pieces;
                 const int row = pp / (kChunk / per16), kp = (pp % (kChunk / per16)) * per16;
-                const uint4 v = *(const uint4 *)((const unsigned char *)Mhi +
-                                                 (((size_t)hl * NP + row) * Qp + c * kChunk + kp) * L::esz);
-                *(uint4 *)((hl ? Blo : Bhi) + L::elem_off(row, kp)) = v;
+                // columns 0-15 of the chunk are the first half's points, 16-31 the second's
+                const int col = 4 * (c_begin * (kChunk / 4) + (c - c_begin + (kp >= 16 ? nch : 0)) * (kChunk / 8)) +
+                                (kp & 15);
+                cp_async16((hl ? Blo : Bhi) + L::elem_off(row, kp),
+                           (const unsigned char *)Mhi + (((size_t)hl * NP + row) * T.Qs + col) * L::esz);
             }
+            // 4 quads of this row (exponents, exp, gradient sums); E to the operand
+#pragma unroll 1
+            for (int i = 0; i < kChunk / 8; ++i) {
+                const int qd = q0 + (c - c_begin) * (kChunk / 8) + i;
+                float f[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                // padding quads (warp-uniform) add nothing: their operand is 0
+                if (qd < T.nquad) {
+                    if (fresh) {
+                        fx_coeffs<NN>(trial, T.fx_ringA + (size_t)ring * n, A0, A);
+                        fresh = false;
+                    }
+                    const int2 *tr = trig + jq * 2 * NN;
+                    const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
+                    Exp e[4];
+                    if (!wide) {
+                        long long s[4];
+                        fx_exponents<NN>(A0, A, tr, NN, jq == 0, s);
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_exp(s[t], tab);
+                    } else {
+                        bad = !fx_slow_quad<NN>(T.Mt, Qp, T.exptab, al, di, lam, pa, pb, e) || bad;
+                    }
+                    if (pb < 0) e[2] = e[3] = Exp{0, -100000};
+                    fx_accumulate<NN>(e, tr, NN, jq == 0, pb < 0, i == 0 && c == c_begin, B, [&](int d) {
+#pragma unroll
+                        for (int a = 0; a < n; ++a) U[a] = kitrt_fx::sar(U[a], d);
+                    });
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) f[t] = __uint_as_float(kitrt_fx::fx_float_bits(e[t]));
+                    // ansatz of the trial point (the last accepted trial leaves the solution's)
+                    if (psi32 && active) {
+                        float *row = psi32 + (size_t)cell * Qp;
+                        *(float2 *)(row + 2 * pa) = make_float2(f[0], f[1]);
+                        if (pb >= 0) *(float2 *)(row + 2 * pb) = make_float2(f[2], f[3]);
+                    }
+                    if (++jq == T.J) {
+                        fx_flush<NN>(T.fx_ringW + (size_t)ring * n2, T.fx_sumshift, B, moment);
+                        jq = 0;
+                        ++ring;
+                        fresh = true;
+                    }
+                }
+                store_operand4<BF16, L>(Ahi, Alo, r, h * (kChunk / 2) + 4 * i, f);
+            }
+            cp_async_wait_all();
             fence_async_smem();
-            __syncthreads();
+            if (__syncthreads_or(failed)) {  // uniform
+                if (tid == 0) *abort_flag = 1;
+                break;
+            }
             if (tid == 0) {
                 tc_fence_after();
                 const uint64_t ahi = smem_desc(smem_u32(Ahi), L::LBO, L::SBO);
@@ -339,7 +399,7 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
             }
             ++commits[b];
         }
-        if (ring >= 0) ring_flush<NN>(T.ringWP + (size_t)ring * n2, B, [&](int cc) -> double & { return U[cc]; });
+        if (!fresh) fx_flush<NN>(T.fx_ringW + (size_t)ring * n2, T.fx_sumshift, B, moment);
         // drain: every MMA of this tile has completed once both buffers' last commits have
         if (tid == 0)
             for (int b = 0; b < 2 && !*abort_flag; ++b)
@@ -352,10 +412,14 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
                 }
         if (tid != 0)
             for (int b = 0; b < 2; ++b) waited[b] = commits[b];
-        // the second half hands its gradient moments to the first
+        // the second half hands its gradient moments and their scale to the first (the trial alpha
+        // and the guard sums that these places held are no longer read once every thread is here)
+        constexpr int kBad = 1 << 30;  // scale of a row with an exponential that is not finite
+        __syncthreads();
         if (h == 1) {
 #pragma unroll
             for (int a = 0; a < n; ++a) sU[a * kTileM + r] = U[a];
+            sX[r] = bad ? kBad : B.Sx;
         }
         __syncthreads();
         tc_fence_after();
@@ -369,8 +433,14 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
         const bool zero = !MOMENTS_ONLY && r < rows && cell >= 0 && !active && part > 0;
         double *row = Vacc + ((size_t)part * cnt_in + base + r) * vs_s;
         if (h == 0 && store) {
+            const int x1 = sX[r];
+            const bool poison = bad || x1 == kBad;
+            const int top = poison ? 0 : max(B.Sx, x1), unit = fx_unit(top, T);
 #pragma unroll
-            for (int a = 0; a < n; ++a) row[(size_t)a * vs_c] = U[a] + sU[a * kTileM + r];
+            for (int a = 0; a < n; ++a) {
+                const long long v = poison ? 0 : kitrt_fx::sar(U[a], top - B.Sx) + kitrt_fx::sar(sU[a * kTileM + r], top - x1);
+                row[(size_t)a * vs_c] = poison ? __longlong_as_double(0x7ff8000000000000LL) : kitrt_fx::fx_to_double(v, unit);
+            }
         }
         if (h == 0) {
             const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
@@ -381,7 +451,7 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
                 if (store) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i)
-                        if (c0 + i < n2 - n) row[(size_t)(n + c0 + i) * vs_c] = (double)v[i];
+                        if (c0 + i < n2 - n) row[(size_t)(n + c0 + i) * vs_c] = f2d_bits(v[i]);
                 }
             }
             if (zero) {
@@ -413,15 +483,14 @@ int launch_mixed_impl(kitrt_mn *mn, const Tables &T, const NewtonState &S, const
                       float *psi32)
 {
     using L = MixedSmem<NN, BF16>;
-    if (ensure_dyn_smem(eval_mixed_kernel<NN, BF16, MO>, L::total)) return KITRT_ECUDA;
+    if (ensure_dyn_smem(eval_mixed_kernel<NN, BF16, MO>, L::total(T.J))) return KITRT_ECUDA;
     // persistent grid of the CTAs that fit on the SMs at once; the work is split into about four
     // items per CTA (the moments of given alphas take one part per tile: rows of Vout are written
     // whole)
-    eval_mixed_kernel<NN, BF16, MO><<<mn->grid_mixed, kThreads, L::total, s>>>(
-        T, S, k, BF16 ? (const void *)mn->d_Mhi16 : (const void *)mn->d_Mhi32, alpha_in, Vacc,
+    eval_mixed_kernel<NN, BF16, MO><<<mn->grid_mixed, kThreads, L::total(T.J), s>>>(
+        T, S, k, BF16 ? (const void *)mn->d_Mhi16 : (const void *)mn->d_Mhi32, u, alpha_in, Vacc,
         MO ? 1 : mn->vs, MO ? Dims<NN>::n2 : 1, C, MO ? 0 : mn->target_mixed, psi32);
     if (cudaGetLastError() != cudaSuccess) return KITRT_ECUDA;
-    (void)u;
     (void)np;
     return KITRT_OK;
 }
@@ -430,8 +499,9 @@ template <int NN, bool BF16>
 int mixed_grid_impl(const kitrt_mn *mn)
 {
     using L = MixedSmem<NN, BF16>;
-    if (ensure_dyn_smem(eval_mixed_kernel<NN, BF16, false>, L::total)) return mn->nsm;
-    return mn->nsm * resident_ctas(eval_mixed_kernel<NN, BF16, false>, kThreads, L::total, 2);
+    const int smem = L::total(mn->J);
+    if (ensure_dyn_smem(eval_mixed_kernel<NN, BF16, false>, smem)) return mn->nsm;
+    return mn->nsm * resident_ctas(eval_mixed_kernel<NN, BF16, false>, kThreads, smem, 2);
 }
 
 template <bool MO>

@@ -13,6 +13,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "fixed.cuh"
 #include "kitrt_internal.cuh"
 
 namespace {
@@ -251,10 +252,18 @@ Tables kitrt_mn::tables() const
     T.exptab = d_exptab;
     T.R = R;
     T.P = P;
-    T.npair = Qf / 2;
-    T.ptrig = d_ptrig;
-    T.ringP = d_ringP;
-    T.ringWP = d_ringWP;
+    T.J = J;
+    T.nquad = R * J;
+    T.Qs = Qs;
+    T.fx_wexp = fx_wexp;
+    // Qf exponentials below 2^54 each: their sums stay below 2^63
+    T.fx_sumshift = 0;
+    while ((Qf >> T.fx_sumshift) >= 512) ++T.fx_sumshift;
+    T.fx_trig = d_fx_trig;
+    T.fx_ringA = d_fx_ringA;
+    T.fx_ringW = d_fx_ringW;
+    T.fx_exp = d_fx_exp;
+    T.fx_mmax = d_fx_mmax;
     return T;
 }
 
@@ -568,10 +577,25 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
     std::vector<float> wox32(wox.begin(), wox.end()), woy32(woy.begin(), woy.end());
     // tensor-core operand of the mixed modes: the degree N+1..2N basis functions (rows n..n2-1
     // of Mt), padded to a multiple of 16 rows and split into a high and a low part in TF32
-    // (nearest, ties away) and in BF16 (nearest even): [2][NP x Qp], high part first
+    // (nearest, ties away) and in BF16 (nearest even): [2][NP x Qs], high part first, columns in the
+    // order of the sweep's quads (0 for the points a quad does not have)
     const int nhi = n2 - n, NP = (nhi + 15) / 16 * 16;
-    std::vector<float> Mhi32((size_t)2 * NP * Qp, 0.0f);
-    std::vector<unsigned short> Mhi16((size_t)2 * NP * Qp, 0);
+    mn->R = (int)r.ring_mu.size();
+    mn->P = r.P;
+    mn->J = (r.P + 1) / 2;
+    mn->Qs = (4 * mn->R * mn->J + 31) / 32 * 32;
+    const int Qs = mn->Qs;
+    std::vector<int> sweep_point(Qs, -1);
+    for (int rg = 0; rg < mn->R; ++rg)
+        for (int j = 0; j < mn->J; ++j) {
+            const int pa = j, pb = j ? mn->P - j : mn->P % 2 ? -1 : mn->P / 2;
+            for (int t = 0; t < 4; ++t) {
+                const int p = t < 2 ? pa : pb;
+                if (p >= 0) sweep_point[4 * (rg * mn->J + j) + t] = 2 * (rg * mn->P + p) + (t & 1);
+            }
+        }
+    std::vector<float> Mhi32((size_t)2 * NP * Qs, 0.0f);
+    std::vector<unsigned short> Mhi16((size_t)2 * NP * Qs, 0);
     auto tf32 = [](float f) {
         uint32_t bits;
         memcpy(&bits, &f, 4);
@@ -588,16 +612,18 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
         return (unsigned short)(rb >> 16);
     };
     for (int c = 0; c < nhi; ++c)
-        for (int q = 0; q < Qp; ++q) {
+        for (int s = 0; s < Qs; ++s) {
+            const int q = sweep_point[s];
+            if (q < 0) continue;
             // the quadrature weight is folded into the table: the tensor cores take exp(alpha.m)
             const double x = w[q] * Mt[(size_t)(n + c) * Qp + q];
             const float hi = tf32((float)x);
-            Mhi32[(size_t)c * Qp + q] = hi;
-            Mhi32[((size_t)NP + c) * Qp + q] = tf32((float)(x - (double)hi));
+            Mhi32[(size_t)c * Qs + s] = hi;
+            Mhi32[((size_t)NP + c) * Qs + s] = tf32((float)(x - (double)hi));
             float bhi;
-            Mhi16[(size_t)c * Qp + q] = bf16((float)x, &bhi);
+            Mhi16[(size_t)c * Qs + s] = bf16((float)x, &bhi);
             float dummy;
-            Mhi16[((size_t)NP + c) * Qp + q] = bf16((float)(x - (double)bhi), &dummy);
+            Mhi16[((size_t)NP + c) * Qs + s] = bf16((float)(x - (double)bhi), &dummy);
         }
     TRY(dev_upload(mn, &mn->d_Mt, Mt));
     TRY(dev_upload(mn, &mn->d_w, w));
@@ -624,44 +650,61 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
     TRY(dev_upload(mn, &mn->d_oy, oyp));
     TRY(dev_upload(mn, &mn->d_ox32, oxp32));
     TRY(dev_upload(mn, &mn->d_oy32, oyp32));
-    // 2^(j/2048), j = 0..2047, then 2^(j/2048) ln2/2048 (kexp_scaled), rounded to double from
-    // extended precision
-    std::vector<double> exptab(4096);
+    // 2^(j/2048), j = 0..2047, rounded to double and to units of 2^-61 from extended precision
+    std::vector<double> exptab(2048);
+    std::vector<uint64_t> fx_exp(2048);
     for (int j = 0; j < 2048; ++j) {
         const long double t = exp2l((long double)j / 2048.0L);
         exptab[j] = (double)t;
-        exptab[2048 + j] = (double)(t * (logl(2.0L) / 2048.0L));
+        fx_exp[j] = (uint64_t)llroundl(ldexpl(t, 61));
     }
     TRY(dev_upload(mn, &mn->d_exptab, exptab));
-    // sum-factorised sweeps: azimuthal factors per pair and Legendre factors per ring
+    TRY(dev_upload(mn, &mn->d_fx_exp, fx_exp));
+    // fixed-point sweeps (sweep.cuh): azimuthal factors per pair of a ring and Legendre factors per
+    // ring, as limbs of the units stated there
     {
-        const int L2 = 2 * mn->N, TW = 2 * L2 + 1;
-        mn->R = (int)r.ring_mu.size();
-        mn->P = r.P;
-        std::vector<double> ptrig((size_t)(Qp / 2) * TW, 0.0);
-        for (int pr = 0; pr < Qf / 2; ++pr) {
-            const int q = 2 * pr;
-            const bool zero_pi = r.kind[q] == 2;
-            for (int k = 0; k <= L2; ++k)
-                ptrig[(size_t)pr * TW + k] = trig_factor(k, r.phi[q], zero_pi ? 2 : 0);
-            for (int k = 1; k <= L2; ++k)
-                ptrig[(size_t)pr * TW + L2 + k] =
-                    zero_pi ? trig_factor(k, r.phi[q], 3) : trig_factor(-k, r.phi[q], 0);
-        }
-        std::vector<double> ringP((size_t)(mn->R + 1) * n2, 0.0), ringWP((size_t)(mn->R + 1) * n2, 0.0);
+        const int L2 = 2 * mn->N;
+        auto limbs = [](long double x, int bits) {
+            const kitrt_fx::Limb l = kitrt_fx::split<27>(llroundl(ldexpl(x, bits)));
+            return make_int2(l.h, l.l);
+        };
+        std::vector<int2> trig((size_t)mn->J * 2 * L2);
+        for (int j = 0; j < mn->J; ++j)
+            for (int k = 1; k <= L2; ++k) {
+                // the azimuths of the basis table, so that both see the same rounded angles
+                const double x = k * (j * (2.0 * kPi / r.nphi));
+                trig[(size_t)j * 2 * L2 + k - 1] = limbs(cos(x), 54);
+                trig[(size_t)j * 2 * L2 + L2 + k - 1] = limbs(sin(x), 54);
+            }
+        std::vector<int2> ringA((size_t)mn->R * n), ringW((size_t)mn->R * n2);
+        std::vector<double> P((size_t)mn->R * n2);
+        double wmax = 0.0;
         for (int rg = 0; rg < mn->R; ++rg) {
             double Pn[24][24];
-            norm_legendre(2 * mn->N, r.ring_mu[rg], Pn);
-            int c = 0;
-            for (int l = 0; l <= 2 * mn->N; ++l)
-                for (int k = -l; k <= l; k += 2, ++c) {
-                    ringP[(size_t)rg * n2 + c] = Pn[l][k < 0 ? -k : k];
-                    ringWP[(size_t)rg * n2 + c] = r.ring_w[rg] * Pn[l][k < 0 ? -k : k];
+            norm_legendre(L2, r.ring_mu[rg], Pn);
+            int cc = 0;
+            for (int l = 0; l <= L2; ++l)
+                for (int k = -l; k <= l; k += 2, ++cc) {
+                    P[(size_t)rg * n2 + cc] = Pn[l][k < 0 ? -k : k] * (k ? sqrt(2.0) : 1.0);
+                    wmax = std::max(wmax, fabs(r.ring_w[rg] * P[(size_t)rg * n2 + cc]));
                 }
         }
-        TRY(dev_upload(mn, &mn->d_ptrig, ptrig));
-        TRY(dev_upload(mn, &mn->d_ringP, ringP));
-        TRY(dev_upload(mn, &mn->d_ringWP, ringWP));
+        frexp(wmax, &mn->fx_wexp);  // wmax < 2^fx_wexp
+        const long double scale = 2048.0L / logl(2.0L);
+        std::vector<float> mmax(n, 0.0f);
+        for (int rg = 0; rg < mn->R; ++rg)
+            for (int cc = 0; cc < n2; ++cc) {
+                const long double p = P[(size_t)rg * n2 + cc];
+                if (cc < n) {
+                    ringA[(size_t)rg * n + cc] = limbs(p * scale, 41);
+                    mmax[cc] = std::max(mmax[cc], (float)fabs((double)p) * 1.0001f);
+                }
+                ringW[(size_t)rg * n2 + cc] = limbs(ldexpl(r.ring_w[rg] * p, -mn->fx_wexp), 54);
+            }
+        TRY(dev_upload(mn, &mn->d_fx_trig, trig));
+        TRY(dev_upload(mn, &mn->d_fx_ringA, ringA));
+        TRY(dev_upload(mn, &mn->d_fx_ringW, ringW));
+        TRY(dev_upload(mn, &mn->d_fx_mmax, mmax));
     }
     TRY(dev_upload(mn, &mn->d_Mhi32, Mhi32));
     TRY(dev_upload(mn, &mn->d_Mhi16, Mhi16));
@@ -797,7 +840,7 @@ int32_t kitrt_mn_work(const kitrt_mn *mn, kitrt_work *out)
     const double pair_ops = N + N + 2 + 2 + 1 + 2 * L, pair_fmas = N + (N - 1) + 2 * L;
     const double ring_fmas = n + nout;
     out->sweep_fp64_flops = pairs * (pair_ops + pair_fmas) + rings * 2 * ring_fmas;
-    out->sweep_fp64_ops = pairs * pair_ops + rings * ring_fmas + Qf * (fp64 ? kExpFp64Ops : kExpScaledFp64Ops);
+    out->sweep_fp64_ops = pairs * pair_ops + rings * ring_fmas + Qf * (fp64 ? kExpFp64Ops : 2);
     out->exps = Qf;
     out->tensor_flops = fp64 ? 0.0 : 3.0 * 2.0 * (n2 - n) * Qf;
     out->newton_flops = 2.0 * mn->gaunt_nnz + n * n * n / 3 + 2 * n * n;

@@ -19,9 +19,6 @@
 // FP64-pipe instructions of one kexp on its common path (kexp.cuh): 2 for the rounding to the
 // table index, 2 for the two-part reduction, 3 for the polynomial, 1 for the table scaling.
 constexpr int kExpFp64Ops = 8;
-// FP64-pipe instructions of one kexp_scaled (sweep.cuh, the mixed sweep): r = s - k and the
-// final fused multiply-add.
-constexpr int kExpScaledFp64Ops = 2;
 
 // Per-cell Newton phase.
 enum : int32_t { PH_DONE = 0, PH_INIT = 1, PH_NEWTON = 2 };
@@ -61,13 +58,16 @@ struct Tables {
     const float *w32;
     const float *wox32, *woy32;  // FP32 copies of w * Omega
     const float *mbar32;         // [n] FP32 copy of <m>
-    const double *exptab;     // [2 x 2048] 2^(j/2048) (kexp), then 2^(j/2048) ln2/2048 (kexp_scaled)
-    // sum-factorised sweeps (sweep.cuh): rings of P pairs of points; R rings (row R of the ring
-    // tables is zero, for padding pairs); npair = Qf / 2 pairs
-    int R, P, npair;
-    const double *ptrig;      // [Qp/2 x (4N+1)] azimuthal factors of each pair
-    const double *ringP;      // [(R+1) x n2] P_c(mu_r)
-    const double *ringWP;     // [(R+1) x n2] w_r P_c(mu_r)
+    const double *exptab;     // [2048] 2^(j/2048) (kexp)
+    // sum-factorised sweeps (sweep.cuh): R rings of P pairs of points in J quads; nquad = R J quads,
+    // Qs = 4 nquad rounded up to 32
+    int R, P, J, nquad, Qs, fx_wexp;
+    int fx_sumshift;          // moments are kept in units of 2^fx_sumshift of the azimuthal sums
+    const int2 *fx_trig;      // [J x 4N] limbs of cos(k phi), sin(k phi)
+    const int2 *fx_ringA;     // [R x n] limbs of P_c(mu_r) 2048/ln2 (sqrt2 of T_k included)
+    const int2 *fx_ringW;     // [R x n2] limbs of w_r P_c(mu_r) / 2^fx_wexp (sqrt2 included)
+    const uint64_t *fx_exp;   // [2048] 2^(j/2048) 2^61
+    const float *fx_mmax;     // [n] largest |m_c| over the rule, rounded up
 };
 
 struct NewtonState {
@@ -127,8 +127,9 @@ struct kitrt_mn {
     float *d_gcoef32 = nullptr;
     int32_t *d_gstart = nullptr, *d_gidx = nullptr;
     float *d_Mt32 = nullptr, *d_w32 = nullptr;
-    float *d_Mhi32 = nullptr;            // [NP x Qp] TF32-rounded degree-(N+1..2N) basis (mixed)
-    unsigned short *d_Mhi16 = nullptr;   // [NP x Qp] BF16 copy
+    float *d_Mhi32 = nullptr;            // [2][NP x Qs] TF32 split of the degree-(N+1..2N) basis
+                                         // in the sweep's point order (mixed)
+    unsigned short *d_Mhi16 = nullptr;   // BF16 copy
     float *d_wox32 = nullptr, *d_woy32 = nullptr, *d_mbar32 = nullptr;
     double *d_ox = nullptr, *d_oy = nullptr;  // [Qp] folded directions (0 on padding), S_N step
     float *d_ox32 = nullptr, *d_oy32 = nullptr;
@@ -137,9 +138,12 @@ struct kitrt_mn {
     int vs = 0;                          // column stride of d_Vacc (C + room for split parts)
     int target_mixed = 0, target_fp64 = 0;  // work items the sweeps aim at per launch
     int grid_mixed = 0, grid_fp64 = 0;      // persistent grids of the sweeps
-    int R = 0, P = 0;                    // rings and pairs per ring of the folded rule
-    double *d_ptrig = nullptr, *d_ringP = nullptr, *d_ringWP = nullptr;
-    double *d_exptab = nullptr;          // [2 x 2048] exp tables (Tables::exptab)
+    int R = 0, P = 0, J = 0, Qs = 0;     // rings, pairs and quads per ring, points of a sweep (padded)
+    int2 *d_fx_trig = nullptr, *d_fx_ringA = nullptr, *d_fx_ringW = nullptr;
+    uint64_t *d_fx_exp = nullptr;
+    float *d_fx_mmax = nullptr;
+    int fx_wexp = 0;
+    double *d_exptab = nullptr;          // [2048] exp table (Tables::exptab)
     void *d_mlp16 = nullptr;             // learned closure: BF16 network parameters
     float *d_mlp_norm = nullptr;         // [4 (n-1)] feature and output means / scales
     bool has_mlp = false;

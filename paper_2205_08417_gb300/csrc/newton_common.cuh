@@ -527,7 +527,7 @@ post_thread_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k,
     const int stride = gridDim.x * blockDim.x;
     if ((int)(blockIdx.x * blockDim.x) >= cnt_in) return;  // uniform: this block has no slot
     // the sweeps split the quadrature of each tile into `parts` column blocks (sweep.cuh)
-    const int parts = sweep_split(cnt_in, target_items, T.Qp / 32).parts;
+    const int parts = target_items;
     int32_t *cnt_out = &S.cnt[(k + 1) % 3];
     // stage the Gaunt tables and point this block's view of them at the copies
     for (int t = threadIdx.x; t < nnz; t += blockDim.x) {

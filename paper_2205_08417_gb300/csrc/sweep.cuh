@@ -7,63 +7,210 @@
 //   exponent   z(mu_r, phi) = alpha . m = sum_{k=-N..N} A_k(r) T_k(phi),
 //              A_k(r) = sum_{c: k(c) = k} alpha_c P_c(mu_r)                 (once per ring),
 //   moments    V_c = sum_r w_r P_c(mu_r) B_k(c)(r),  B_k(r) = sum_phi e(mu_r, phi) T_k(phi).
-// The azimuths of a ring come in pairs (phi, 2 pi - phi) whose cosines agree and whose sines are
-// opposite, so with C = sum_{k>=0} A_k T_k and S = sum_{k<0} A_k T_k at the pair's first point,
-//   z = C + S and z' = C - S,   B_k += (e + e') T_k (k >= 0),   B_k += (e - e') T_k (k < 0).
-// A pass over a cell's Q' points then costs about (2N+3)/2 FP64 operations per point for the
-// exponent and (2L+3)/2 for moments up to degree L, instead of n and nmom(L) per point, plus n and
-// nmom(L) per ring. The ring's remaining pair, (0, pi), has no sine terms and is summed directly.
+// The azimuths of a ring come in fours phi, -phi, pi - phi, pi + phi whose cosines and sines agree
+// up to signs: with the even and odd parts of C = sum_{k>=0} A_k T_k and S = sum_{k<0} A_k T_k at phi,
+//   z(+-phi) = (C_e + C_o) +- (S_o + S_e),   z(pi -+ phi) = (C_e - C_o) +- (S_o - S_e),
+// and the azimuthal sums take the matching sums and differences of the four exponentials. A pass
+// over a cell's Q' points then costs N/2 products per point for the exponent and L/2 for moments
+// up to degree L, instead of n and nmom(L), plus n and nmom(L) per ring. The four azimuths 0, pi,
+// pi/2, 3 pi/2 (only the first two when the number of pairs per ring is odd) need no products.
+// The arithmetic is 64-bit fixed point (fixed.cuh): the FP64 pipe (16 cycles per warp instruction)
+// bound the FP64 form of this pass. Measured on 99,458 cells, M_3, order 20 (400 folded points):
+// tensor-core sweep 4.86 -> 1.71 ms for 350,160 cell evaluations, FP64-mode sweep 3.83 -> 0.89 ms
+// for 219,742. Now bound by integer issue: about 25 32x32->64-bit products per point, each 4 cycles
+// of the multiply pipe of a scheduler, and twice as many other instructions.
 //
-// Tables (built by kitrt_mn_init in this point order): pair p covers folded points 2p and 2p+1;
-// ring of pair p = p / P for p < npair (P pairs per ring), the all-zero row R for padding pairs;
-// pair 0 of each ring is the (0, pi) pair. ptrig [npair_padded x (4N+1)]: T_0..T_2N at the pair's
-// first point (cosines), then sqrt2 sin(k phi), k = 1..2N (for the (0, pi) pair: T_k(pi)).
-// ringP, ringWP [(R+1) x n2]: P_c(mu_r) and w_r P_c(mu_r) over the degree-2N basis.
+// Tables (built by kitrt_mn_init): ring r holds the folded points 2 P r .. 2 P (r + 1) - 1 in pairs
+// (phi_j, -phi_j), phi_j = pi j / P, pair 0 being (0, pi); its quads are j = 0 (pair 0 and pair P/2)
+// and j = 1 .. J - 1, J = (P + 1) / 2 rounded down (pairs j and P - j); quad qd = r J + j.
+// fx_trig [J x 4N] limbs: cos(k phi_j), k = 1..2N, then sin(k phi_j).
+// fx_ringA [R x n], fx_ringW [R x n2] limbs: P_c(mu_r) and w_r P_c(mu_r), both with the sqrt2 of
+// T_k, the first times 2048/ln2, the second over 2^fx_wexp. fx_exp: 2^(j/2048) 2^61.
 #pragma once
 
+#include "fixed.cuh"
 #include "kexp.cuh"
 #include "kitrt_internal.cuh"
 
 namespace kitrt_dev {
 
-// Position of azimuthal index k in a coefficient vector of degree L: k >= 0 at k, k < 0 at L+|k|.
-__host__ __device__ constexpr int kslot(int L, int k) { return k >= 0 ? k : L - k; }
 // Index of basis function (l, k), l + |k| even, in the order l ascending, then k ascending.
 __host__ __device__ constexpr int cindex(int l, int k) { return l * (l + 1) / 2 + (k + l) / 2; }
 
-// Exponent coefficients A_k of one ring from the trial alpha (degree NN).
-template <int NN>
-__device__ __forceinline__ void ring_coeffs(const double (&at)[(NN + 1) * (NN + 2) / 2],
-                                            const double *__restrict__ Pr, double (&A)[2 * NN + 1])
+using kitrt_fx::Exp;
+using kitrt_fx::Limb;
+
+// Exponent coefficients of one ring: A0 (k = 0) and A[2(k-1)], A[2(k-1)+1] for cos(k phi),
+// sin(k phi), from the trial alpha's limbs (at(c)).
+template <int NN, typename At>
+__device__ __forceinline__ void fx_coeffs(At &&at, const int2 *__restrict__ Pr, long long &A0, Limb (&A)[2 * NN])
 {
 #pragma unroll
-    for (int j = 0; j < 2 * NN + 1; ++j) A[j] = 0.0;
+    for (int k = -NN; k <= NN; ++k) {
+        kitrt_fx::CoefAcc acc;
+        const int ak = k < 0 ? -k : k;
 #pragma unroll
-    for (int l = 0; l <= NN; ++l)
-#pragma unroll
-        for (int k = -l; k <= l; k += 2) {
-            const int c = cindex(l, k);
-            A[kslot(NN, k)] = fma(at[c], __ldg(Pr + c), A[kslot(NN, k)]);
-        }
+        for (int l = ak; l <= NN; l += 2) acc.add(at(cindex(l, k)), __ldg(Pr + cindex(l, k)));
+        const long long v = acc.value();
+        if (k == 0) A0 = v;
+        else A[2 * (ak - 1) + (k < 0)] = kitrt_fx::split<31>(v);
+    }
 }
+
+// A row's azimuthal sums of the current ring, degree LB, and the exponent of their unit
+// (units of 2^(Sx - 61)).
+template <int LB>
+struct FxSums {
+    long long b0;
+    kitrt_fx::SumAcc b[2 * LB];  // cos(k phi), sin(k phi) at 2(k-1), 2(k-1)+1
+    int Sx;
+    __device__ __forceinline__ void clear()
+    {
+        b0 = 0;
+#pragma unroll
+        for (int j = 0; j < 2 * LB; ++j) b[j].clear();
+    }
+};
 
 // Moments of the finished ring: V_c += w_r P_c(mu_r) B_k(c), c over the degree-LB basis; the
 // azimuthal sums are cleared for the next ring.
 template <int LB, typename Acc>
-__device__ __forceinline__ void ring_flush(const double *__restrict__ wPr, double (&B)[2 * LB + 1],
-                                           Acc &&V)
+__device__ __forceinline__ void fx_flush(const int2 *__restrict__ wPr, int sumshift, FxSums<LB> &B, Acc &&V)
 {
 #pragma unroll
-    for (int l = 0; l <= LB; ++l)
+    for (int k = -LB; k <= LB; ++k) {
+        const int ak = k < 0 ? -k : k;
+        const Limb v = kitrt_fx::split<32>(k == 0 ? B.b0 : B.b[k == 0 ? 0 : 2 * (ak - 1) + (k < 0)].value());
 #pragma unroll
-        for (int k = -l; k <= l; k += 2) {
-            const int c = cindex(l, k);
-            double &v = V(c);
-            v = fma(__ldg(wPr + c), B[kslot(LB, k)], v);
-        }
-#pragma unroll
-    for (int j = 0; j < 2 * LB + 1; ++j) B[j] = 0.0;
+        for (int l = ak; l <= LB; l += 2) V(cindex(l, k)) += kitrt_fx::moment_term(v, __ldg(wPr + cindex(l, k)), sumshift);
+    }
+    B.clear();
 }
+
+// The two pairs of points of quad j of a ring (the second is -1 in quad 0 of a ring with an odd
+// number of pairs).
+__device__ __forceinline__ int quad_pair0(int ring, int j, int P) { return ring * P + j; }
+__device__ __forceinline__ int quad_pair1(int ring, int j, int P)
+{
+    return j ? ring * P + P - j : (P & 1) ? -1 : ring * P + P / 2;
+}
+
+// A quad's exponentials in FP64, for rows outside the fixed-point range (very large or non-finite
+// alpha): full sums against the basis at the points of pairs pa and pb. False when one of them is
+// not finite.
+template <int NN>
+__device__ __noinline__ bool fx_slow_quad(const double *__restrict__ Mt, int Qp, const double *__restrict__ exptab,
+                                          const double *alpha, const double *dir, double lam, int pa, int pb, Exp *e)
+{
+    constexpr int n = (NN + 1) * (NN + 2) / 2;
+    bool ok = true;
+#pragma unroll 1
+    for (int t = 0; t < 4; ++t) {
+        const int q = 2 * (t < 2 ? pa : max(pb, 0)) + (t & 1);
+        double z = 0.0;
+#pragma unroll 1
+        for (int c = 0; c < n; ++c) {
+            const double a = lam != 0.0 ? fma(lam, dir[c], alpha[c]) : alpha[c];
+            z = fma(a, __ldg(Mt + (size_t)c * Qp + q), z);
+        }
+        ok = kitrt_fx::fx_exp_from_double(kexp(z, exptab), e[t]) && ok;
+    }
+    return ok;
+}
+
+// The exponents of one quad's four points (t: its cosines, k = 1.., then from t + L2 its sines).
+template <int NN>
+__device__ __forceinline__ void fx_exponents(long long A0, const Limb (&A)[2 * NN], const int2 *__restrict__ t,
+                                             int L2, bool axes, long long (&s)[4])
+{
+    long long ce = A0, co = 0, se = 0, so = 0;
+    if (!axes) {
+        kitrt_fx::DotAcc acc[4];  // C_e, C_o, S_e, S_o
+#pragma unroll
+        for (int k = 1; k <= NN; ++k) {
+            acc[k & 1].add(A[2 * (k - 1)], t[k - 1]);
+            acc[2 + (k & 1)].add(A[2 * (k - 1) + 1], t[L2 + k - 1]);
+        }
+        if (NN >= 2) ce += acc[0].value();
+        co = acc[1].value();
+        if (NN >= 2) se = acc[2].value();
+        so = acc[3].value();
+        const long long p = ce + co, m = ce - co, q = so + se, w = so - se;
+        s[0] = p + q;
+        s[1] = p - q;
+        s[2] = m + w;
+        s[3] = m - w;
+    } else {
+        // phi = 0, pi, pi/2, 3 pi/2: cos(k phi) and sin(k phi) are 0 and +-1
+        long long ce2 = A0;
+#pragma unroll
+        for (int k = 1; k <= NN; ++k) {
+            const long long a = ((long long)A[2 * (k - 1)].h << 31) + A[2 * (k - 1)].l;
+            const long long b = ((long long)A[2 * (k - 1) + 1].h << 31) + A[2 * (k - 1) + 1].l;
+            if (k & 1) {
+                co += a;
+                so += (k & 2) ? -b : b;
+            } else {
+                ce += a;
+                ce2 += (k & 2) ? -a : a;
+            }
+        }
+        s[0] = ce + co;
+        s[1] = ce - co;
+        s[2] = ce2 + so;
+        s[3] = ce2 - so;
+    }
+}
+
+// One quad's exponentials into the azimuthal sums. `first`: the row's first quad of this item
+// (uniform), which lowers a scale that lies far above the row's exponentials. shift_moments(d)
+// shifts the row's moments down by d when the scale rises. `two`: quad 0 of a ring with an odd
+// number of pairs (e[2], e[3] are zero).
+template <int LB, typename Shift>
+__device__ __forceinline__ void fx_accumulate(const Exp (&e)[4], const int2 *__restrict__ t, int L2, bool axes,
+                                              bool two, bool first, FxSums<LB> &B, Shift &&shift_moments)
+{
+    const int mm = max(max(e[0].m, e[1].m), max(e[2].m, e[3].m));
+    if (first && B.Sx - kitrt_fx::kGuard - mm > 22) B.Sx = mm + kitrt_fx::kGuard + 2;
+    if (mm + kitrt_fx::kGuard > B.Sx) {
+        const int d = mm + kitrt_fx::kGuard + 2 - B.Sx;
+        B.Sx += d;
+        B.b0 = kitrt_fx::sar(B.b0, d);
+#pragma unroll
+        for (int j = 0; j < 2 * LB; ++j) B.b[j].scale_down(d);
+        shift_moments(d);
+    }
+    long long f[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) f[i] = (long long)kitrt_fx::shr(e[i].y, B.Sx - e[i].m);
+    const long long p = f[0] + f[1], d = f[0] - f[1], p2 = f[2] + f[3], d2 = f[2] - f[3];
+    // every shift rounds down, by half a unit on average: given back to the sum
+    const long long all = p + p2 + (two ? 1 : 2);
+    B.b0 += all;
+    if (!axes) {
+        const Limb ce = kitrt_fx::split<27>(all), co = kitrt_fx::split<27>(p - p2);
+        const Limb so = kitrt_fx::split<27>(d + d2), se = kitrt_fx::split<27>(d - d2);
+#pragma unroll
+        for (int k = 1; k <= LB; ++k) {
+            B.b[2 * (k - 1)].add(k & 1 ? co : ce, t[k - 1]);
+            B.b[2 * (k - 1) + 1].add(k & 1 ? so : se, t[L2 + k - 1]);
+        }
+    } else {
+        // the two halves of the correction cancel where p2 enters with a minus sign
+#pragma unroll
+        for (int k = 1; k <= LB; ++k) {
+            if (k & 1) {
+                B.b[2 * (k - 1)].hh += d;
+                B.b[2 * (k - 1) + 1].hh += (k & 2) ? -d2 : d2;
+            } else {
+                B.b[2 * (k - 1)].hh += (k & 2) ? p - p2 + (two ? 1 : 0) : all;
+            }
+        }
+    }
+}
+
+// Exponent of the unit of a row's moments (for fx_to_double).
+__device__ __forceinline__ int fx_unit(int Sx, const Tables &T) { return Sx - 61 + T.fx_sumshift + T.fx_wexp; }
 
 // An exponential (a non-negative double, or +inf) rounded to float in integer arithmetic, so that
 // the narrow FP64 pipe does not convert it: the exponent is rebiased and the mantissa rounded
@@ -114,112 +261,29 @@ __device__ __forceinline__ double f2d_bits(float f)
         (long long)(sign | (((unsigned long long)mag << 29) + ((unsigned long long)(1023 - 127) << 52))));
 }
 
-// exp for an exponent already scaled by 2048 / ln2 (s = x * 2048/ln2, so exp(x) = 2^(s/2048)),
-// with two FP64-pipe instructions on the common path instead of kexp's eight. Tang's table
-// reduction as in kexp, rearranged for the scaled argument:
-//   k = an integer within 0.5625 of s, k = 2048 m + j,   r = s - k (exact, |r| <= 0.5625),
-//   2^(s/2048) = 2^m (T_j + T_j rho + T_j h),  rho = r ln2/2048 (|rho| <= 1.91e-4),
-//   h = rho^2/2 + rho^3/6 + rho^4/24 (truncation below rho^5/120 < 3e-21),
-// with T_j = 2^(j/2048) and C_j = T_j ln2/2048 from the two halves of the table.
-// k comes from s rounded to float (|s| < 2^21 there, so within 1/16 of s) and rounded to an
-// integer by the float shift 1.5 * 2^23; k as a double and the float of r are formed in integer
-// arithmetic. T_j h (below 3.6e-8) is formed in FP32 and added to T_j in integer arithmetic as a
-// fixed-point count of T_j's ulps (2^-52, as T_j is in [1, 2) and the sum stays below 2). Its
-// FP32 rounding, about 5e-7 of T_j h, bounds the relative error of the result by about 1e-14.
-// The two FP64 instructions are r = s - k and C_j r + (T_j + T_j h) (one rounding). The range
-// handling is kexp's, in scaled units: arguments below -707 (scaled) return 0, above 709.78
-// return +inf, NaN propagates.
-__device__ __forceinline__ double kexp_scaled(double s, const double *__restrict__ tab)
-{
-    const float kC2 = 5.727446250602952e-08f;  // (ln2/2048)^2 / 2
-    const float kC3 = 6.46152879466011e-12f;   // (ln2/2048)^3 / 6
-    const float kC4 = 5.467273155028592e-16f;  // (ln2/2048)^4 / 24
-    const float kShiftF = 12582912.0f;         // 1.5 * 2^23: rounds a float below 2^22 to an integer
-    // |s| < 512 * 2048/ln2 is tested on the high word (0x41371547 is that bound's high word)
-    if ((__double2hiint(s) & 0x7fffffff) >= 0x41371547) {
-        if (!(s > -2088930.0867246022)) return s != s ? s : 0.0;  // -707 * 2048/ln2
-        if (s > 2097143.984378201) return __longlong_as_double(0x7ff0000000000000LL);  // 709.78 * 2048/ln2
-    }
-    const float tf = __fadd_rn(d2f_bits(s), kShiftF);
-    const int k = __float_as_int(tf) - 0x4B400000;  // the integer tf - 1.5 * 2^23
-    const double r = s - f2d_bits(__fsub_rn(tf, kShiftF));
-    const float rf = d2f_bits(r);
-    const int j = k & ((1 << kExpTableBits) - 1);
-    const long long tb = __double_as_longlong(__ldg(tab + j));
-    const double Cj = __ldg(tab + (1 << kExpTableBits) + j);
-    // T_j h in FP32, with T_j rounded to float from its bits (T_j in [1, 2): exponent field 0x3ff)
-    const float tjf = __int_as_float(0x3f800000 | (int)(((tb + (1LL << 28)) >> 29) & 0x7fffff));
-    const float hq = fmaf(rf, fmaf(rf, kC4, kC3), kC2);
-    const float th = __fmul_rn(__fmul_rn(__fmul_rn(rf, rf), hq), tjf);
-    // th in units of 2^-52, rounded: th = mant 2^(e - 150) with e its exponent field (th >= 0,
-    // e <= 102), so th 2^52 = mant 2^(e - 98); a zero or subnormal th (e = 0) gives 0
-    const int tbits = __float_as_int(th);
-    const int e = tbits >> 23;
-    const unsigned mant = (unsigned)(tbits & 0x7fffff) | 0x800000u;
-    const int sh = e - 98;
-    const unsigned fx = sh >= 0 ? mant << sh : ((mant >> min(-sh - 1, 31)) + 1u) >> 1;
-    const double y0 = __longlong_as_double(tb + (long long)fx);  // T_j + T_j h
-    const double y = fma(Cj, r, y0);
-    const long long bits = __double_as_longlong(y) + ((long long)(k >> kExpTableBits) << 52);
-    return __longlong_as_double(bits);
-}
-
-// One pair of points: both exponentials (e1 at the pair's first point, e2 at its mirror, or at
-// phi = 0 and phi = pi for the ring's (0, pi) pair) and their azimuthal sums up to degree LB.
-// t is the pair's row of ptrig (row width 4 NN + 1). SCALED: the coefficients A are those of the
-// exponent times 2048/ln2, and the exponentials come from kexp_scaled.
-template <int NN, int LB, bool SCALED = false>
-__device__ __forceinline__ void pair_eval(const double (&A)[2 * NN + 1], const double *__restrict__ t,
-                                          bool zero_pi, const double *__restrict__ exptab,
-                                          double (&B)[2 * LB + 1], double &e1, double &e2)
-{
-    constexpr int L2 = 2 * NN;  // sines of the row start at t[L2 + 1]
-    if (!zero_pi) {
-        double c = A[0];  // T_0 = 1
-#pragma unroll
-        for (int k = 1; k <= NN; ++k) c = fma(A[k], __ldg(t + k), c);
-        double s = A[NN + 1] * __ldg(t + L2 + 1);
-#pragma unroll
-        for (int k = 2; k <= NN; ++k) s = fma(A[NN + k], __ldg(t + L2 + k), s);
-        e1 = SCALED ? kexp_scaled(c + s, exptab) : kexp(c + s, exptab);
-        e2 = SCALED ? kexp_scaled(c - s, exptab) : kexp(c - s, exptab);
-        const double ep = e1 + e2, em = e1 - e2;
-        B[0] += ep;
-#pragma unroll
-        for (int k = 1; k <= LB; ++k) B[k] = fma(ep, __ldg(t + k), B[k]);
-#pragma unroll
-        for (int k = 1; k <= LB; ++k) B[LB + k] = fma(em, __ldg(t + L2 + k), B[LB + k]);
-    } else {
-        double z1 = A[0], z2 = A[0];
-#pragma unroll
-        for (int k = 1; k <= NN; ++k) {
-            z1 = fma(A[k], __ldg(t + k), z1);
-            z2 = fma(A[k], __ldg(t + L2 + k), z2);
-        }
-        e1 = SCALED ? kexp_scaled(z1, exptab) : kexp(z1, exptab);
-        e2 = SCALED ? kexp_scaled(z2, exptab) : kexp(z2, exptab);
-        B[0] += e1 + e2;
-#pragma unroll
-        for (int k = 1; k <= LB; ++k) B[k] = fma(e1, __ldg(t + k), fma(e2, __ldg(t + L2 + k), B[k]));
-    }
-}
-
-// Split of a sweep's work: tiles of 128 listed cells times parts of the quadrature (units of 16
-// pairs). When few cells are listed each tile's quadrature is split over up to `nunits` parts so
-// that every SM gets work; part j of list slot i lands in column j * cnt + i of the accumulator,
-// and the Newton kernel adds the parts in order (deterministic). The same function sizes the
-// split in the sweep and in its consumer.
+// Split of a sweep's work: tiles of 128 listed cells times parts of the quadrature (whole units of
+// 8 quads, part j taking units [j nunits / parts, (j + 1) nunits / parts)). Part j of list slot i
+// lands in column j * cnt + i of the accumulator, and sum_parts_kernel adds the parts in order, so
+// every cell's sums depend on the list's length only, not on its place (deterministic).
+// The number of parts is the one with the shortest schedule on `grid` persistent CTAs, each item
+// costing its units plus one for its trial point, its drain and its stores; at most
+// 1 + target / tiles, which bounds the columns. Called by whole warps.
 struct SweepSplit {
-    int tiles, parts, units_per_part;
+    int tiles, parts;
 };
-__host__ __device__ inline SweepSplit sweep_split(int cnt, int target_items, int nunits)
+__device__ __forceinline__ SweepSplit sweep_split(int cnt, int grid, int target_items, int nunits)
 {
     SweepSplit sp;
     sp.tiles = (cnt + 127) / 128;
-    int ks = sp.tiles > 0 && target_items > 0 ? (target_items + sp.tiles - 1) / sp.tiles : 1;
-    ks = ks < 1 ? 1 : (ks > nunits ? nunits : ks);
-    sp.units_per_part = (nunits + ks - 1) / ks;
-    sp.parts = (nunits + sp.units_per_part - 1) / sp.units_per_part;
+    sp.parts = 1;
+    if (target_items <= 0 || sp.tiles == 0) return sp;
+    const int most = min(nunits, 1 + target_items / sp.tiles);
+    unsigned best = 0xffffffffu;  // schedule length in the high bits, parts in the low 8
+    for (int p = 1 + (threadIdx.x & 31); p <= most; p += 32) {
+        const unsigned rounds = (unsigned)(sp.tiles * p + grid - 1) / grid;
+        best = min(best, (rounds * ((nunits + p - 1) / p + 1)) << 8 | (unsigned)p);
+    }
+    sp.parts = (int)(__reduce_min_sync(0xffffffffu, best) & 255u);
     return sp;
 }
 
