@@ -112,53 +112,19 @@ begin_test_kernel(NewtonState S, const double *__restrict__ u, const double *__r
     }
 }
 
+// One thread per listed cell: every FP64 instruction of the triangular solves keeps all 32 lanes
+// busy, and one warp per scheduler already fills the FP64 pipe (64 cycles per instruction). For
+// N <= 3 the factor is read into registers; for N >= 4 (120 or 231 entries) its rows are read in
+// order, once for the forward and once for the backward substitution (which works row by row too),
+// the vector in shared memory. There it took the place of a warp per cell: M_5, 996,872 cells,
+// 8.2 -> 7.0 ms a step (bound by the rows' strided reads).
 template <int NN>
-__global__ void __launch_bounds__(kWarps * 32)
-predict_kernel(NewtonState S, const double *__restrict__ u, NewtonParams np)
-{
-    constexpr int n = Dims<NN>::n, npairs = Dims<NN>::npairs;
-    __shared__ double sH[kWarps][n * n];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    double *H = sH[wib];
-    const int cnt = S.cnt[8];
-    for (int it = blockIdx.x * kWarps + wib; it < cnt; it += gridDim.x * kWarps) {
-        const int cell = S.list[1][it];
-        const size_t off = (size_t)cell * n;
-        const double ua = lane < n ? u[off + lane] : 0.0;
-        const double al = lane < n ? S.alpha[off + lane] : 0.0;
-        const double g = lane < n ? fma(lane >= np.reg0 ? np.gamma : 0.0, al, S.U[off + lane] - ua) : 0.0;
-        const double ar2 = warp_sum(lane < n && lane >= np.reg0 ? al * al : 0.0);
-        for (int a = lane; a < n; a += 32)
-            for (int b = 0; b <= a; ++b) H[a * n + b] = S.L[(size_t)cell * npairs + tri_idx(a, b)];
-        __syncwarp();
-        const double d = warp_chol_solve<n>(H, -g, lane);
-        __syncwarp();
-        const double gn2 = warp_sum(g * g), un2 = warp_sum(ua * ua);
-        if (lane < n) S.dir[off + lane] = d;
-        if (sqrt(gn2) <= np.tau * sqrt(un2)) {
-            if (lane == 0) S.phase[cell] = PH_DONE;  // converged; d is the polish step
-            continue;
-        }
-        const double au = warp_sum(al * ua), gd = warp_sum(g * d);
-        if (lane == 0) {
-            if (S.gnorm) S.gnorm[cell] = sqrt(gn2);
-            const double fs = S.fsum[cell];
-            S.f0[cell] = fma(0.5 * np.gamma, ar2, fs - au);
-            S.gd[cell] = gd;
-            S.lam[cell] = 1.0;
-            S.phase[cell] = PH_NEWTON;
-        }
-        push(S.list[0], &S.cnt[0], cell, lane);
-    }
-}
-
-// Thread-per-cell version of predict_kernel for N <= 3 (the packed factor fits in registers):
-// every FP64 instruction of the triangular solves keeps all 32 lanes busy.
-template <int NN>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kThreadBlock)
 predict_thread_kernel(NewtonState S, const double *__restrict__ u, NewtonParams np)
 {
     constexpr int n = Dims<NN>::n, npairs = Dims<NN>::npairs;
+    constexpr bool in_regs = NN <= 3;
+    __shared__ double sy[in_regs ? 1 : n][kThreadBlock];
     const int cnt = S.cnt[8];
     const int stride = gridDim.x * blockDim.x;
     const int rounds = (cnt + stride - 1) / stride;
@@ -169,43 +135,70 @@ predict_thread_kernel(NewtonState S, const double *__restrict__ u, NewtonParams 
         if (it < cnt) {
             cell = S.list[1][it];
             const size_t off = (size_t)cell * n;
-            double Lp[npairs], y[n], g[n];
-            double gn2 = 0.0, un2 = 0.0, au = 0.0, ar2 = 0.0;
-#pragma unroll
-            for (int p = 0; p < npairs; ++p) Lp[p] = S.L[(size_t)cell * npairs + p];
-#pragma unroll
-            for (int a = 0; a < n; ++a) {
+            const double *L = S.L + (size_t)cell * npairs;
+            double gn2 = 0.0, un2 = 0.0, au = 0.0, ar2 = 0.0, gd = 0.0;
+            auto gradient = [&](int a) {
                 const double ua = u[off + a], al = S.alpha[off + a];
-                g[a] = S.U[off + a] - ua;
+                double g = S.U[off + a] - ua;
                 if (a >= np.reg0) {
-                    g[a] = fma(np.gamma, al, g[a]);
+                    g = fma(np.gamma, al, g);
                     ar2 = fma(al, al, ar2);
                 }
-                gn2 = fma(g[a], g[a], gn2);
+                gn2 = fma(g, g, gn2);
                 un2 = fma(ua, ua, un2);
                 au = fma(al, ua, au);
-                y[a] = -g[a];
-            }
+                return g;
+            };
             // d = -H^-1 g with the stored factor (1/L_jj on its diagonal)
+            if constexpr (in_regs) {
+                double Lp[npairs], y[n], g[n];
 #pragma unroll
-            for (int i = 0; i < n; ++i) {
-                double t = y[i];
+                for (int p = 0; p < npairs; ++p) Lp[p] = L[p];
 #pragma unroll
-                for (int k = 0; k < i; ++k) t = fma(-Lp[tri_idx(i, k)], y[k], t);
-                y[i] = t * Lp[tri_idx(i, i)];
-            }
+                for (int a = 0; a < n; ++a) {
+                    g[a] = gradient(a);
+                    y[a] = -g[a];
+                }
 #pragma unroll
-            for (int i = n - 1; i >= 0; --i) {
-                double t = y[i];
+                for (int i = 0; i < n; ++i) {
+                    double t = y[i];
 #pragma unroll
-                for (int k = i + 1; k < n; ++k) t = fma(-Lp[tri_idx(k, i)], y[k], t);
-                y[i] = t * Lp[tri_idx(i, i)];
-            }
-            double gd = 0.0;
+                    for (int k = 0; k < i; ++k) t = fma(-Lp[tri_idx(i, k)], y[k], t);
+                    y[i] = t * Lp[tri_idx(i, i)];
+                }
 #pragma unroll
-            for (int a = 0; a < n; ++a) {
-                S.dir[off + a] = y[a];
-                gd = fma(g[a], y[a], gd);
+                for (int i = n - 1; i >= 0; --i) {
+                    double t = y[i];
+#pragma unroll
+                    for (int k = i + 1; k < n; ++k) t = fma(-Lp[tri_idx(k, i)], y[k], t);
+                    y[i] = t * Lp[tri_idx(i, i)];
+                }
+#pragma unroll
+                for (int a = 0; a < n; ++a) {
+                    S.dir[off + a] = y[a];
+                    gd = fma(g[a], y[a], gd);
+                }
+            } else {
+                double *y = &sy[0][threadIdx.x];
+#pragma unroll 1
+                for (int i = 0; i < n; ++i) {
+                    const double *row = L + tri_idx(i, 0);
+                    double t = -gradient(i);
+#pragma unroll 4
+                    for (int k = 0; k < i; ++k) t = fma(-row[k], y[k * kThreadBlock], t);
+                    y[i * kThreadBlock] = t * row[i];
+                }
+                // g . d = -|L^-1 g|^2
+#pragma unroll 1
+                for (int i = 0; i < n; ++i) gd = fma(-y[i * kThreadBlock], y[i * kThreadBlock], gd);
+#pragma unroll 1
+                for (int i = n - 1; i >= 0; --i) {
+                    const double *row = L + tri_idx(i, 0);
+                    const double x = y[i * kThreadBlock] * row[i];
+                    S.dir[off + i] = x;
+#pragma unroll 4
+                    for (int k = 0; k < i; ++k) y[k * kThreadBlock] = fma(-row[k], x, y[k * kThreadBlock]);
+                }
             }
             if (sqrt(gn2) <= np.tau * sqrt(un2)) {
                 S.phase[cell] = PH_DONE;  // converged; d is the polish step
@@ -566,19 +559,13 @@ int grid_for(const kitrt_mn *mn, int C, int per_sm)
     return need < cap ? (need > 0 ? need : 1) : cap;
 }
 
-// The predictor: thread per cell while the packed factor fits in registers (N <= 3), else warp
-// per cell with the factor in shared memory.
 template <int NN>
 void predict_launch(kitrt_mn *mn, const NewtonState &S, int C, const double *u, NewtonParams np,
                     cudaStream_t s)
 {
-    if constexpr (NN <= 3) {
-        int tb = (C + kThreadBlock - 1) / kThreadBlock;
-        if (tb > mn->nsm * 32) tb = mn->nsm * 32;
-        predict_thread_kernel<NN><<<tb > 0 ? tb : 1, kThreadBlock, 0, s>>>(S, u, np);
-    } else {
-        predict_kernel<NN><<<grid_for(mn, C, 8), kWarps * 32, 0, s>>>(S, u, np);
-    }
+    int tb = (C + kThreadBlock - 1) / kThreadBlock;
+    if (tb > mn->nsm * 32) tb = mn->nsm * 32;
+    predict_thread_kernel<NN><<<tb > 0 ? tb : 1, kThreadBlock, 0, s>>>(S, u, np);
 }
 
 }  // namespace
@@ -600,62 +587,84 @@ int launch_isotropic(const Tables &T, int C, const double *u, double *alpha, cud
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }
 
-// Sum of each listed slot's quadrature parts (written by the sweeps, sweep.cuh) into its part-0
-// column, in order, element-wise over the [n2 x cnt] moments with every SM taking part, so that
-// the Newton kernel's serial per-cell chain reads one column instead of `parts`. Tensor-core
-// rows' Hessian-only moments (degree > N) are FP32 accumulator values and are added in FP32; the
-// gradient moments, and every moment of a row handed to the FP64 sweep (its part 0 holds the
-// FP64 sums, its other parts zeros), in FP64.
-__global__ void sum_parts_kernel(NewtonState S, int k, double *__restrict__ Vacc, int vs, int n,
-                                 int n2, int grid, int target_items, int nunits, int mixed)
+// FP64 mode, rounds of more than `above` cells: the sum of each listed slot's quadrature parts
+// (sweep.cuh) into its part-0 column, in order, element-wise over the [n2 x cnt] moments with every
+// SM taking part, so that the thread-per-cell Newton kernel reads one column.
+__global__ void sum_parts_kernel(NewtonState S, int k, double *__restrict__ Vacc, int vs, int n2, int grid,
+                                 int target_items, int nunits, int above)
 {
     const int cnt = S.cnt[k % 3];
+    if (cnt <= above) return;
     const int parts = sweep_split(cnt, grid, target_items, nunits).parts;
     if (parts <= 1) return;
-    const int32_t *list = S.list[k & 1];
     const size_t total = (size_t)n2 * cnt, pstride = (size_t)cnt;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
          e += (size_t)gridDim.x * blockDim.x) {
         const int c = (int)(e / cnt), j = (int)(e - (size_t)c * cnt);
         double *col = Vacc + (size_t)c * vs + j;
-        if (mixed && c >= n && !S.h64[list[j]]) {
-            float v = d2f_bits(col[0]);
-            for (int p = 1; p < parts; ++p) v += d2f_bits(col[(size_t)p * pstride]);
-            col[0] = f2d_bits(v);
-        } else {
-            double v = col[0];
-            for (int p = 1; p < parts; ++p) v += col[(size_t)p * pstride];
-            col[0] = v;
-        }
+        double v = col[0];
+        for (int p = 1; p < parts; ++p) v += col[(size_t)p * pstride];
+        col[0] = v;
     }
 }
 
-int launch_sum_parts(kitrt_mn *mn, const NewtonState &S, int k, double *Vacc, cudaStream_t s)
-{
-    const int mixed = mn->p.mode != KITRT_FP64;
-    LaunchScope ls(mn, PK_POST, s, 0);
-    sum_parts_kernel<<<mn->nsm * 8, 256, 0, s>>>(S, k, Vacc, mn->vs, mn->n, mn->n2,
-                                                 mixed ? mn->grid_mixed : mn->grid_fp64,
-                                                 mixed ? mn->target_mixed : mn->target_fp64, mn->Qs / 32, mixed);
-    return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
-}
+// Cells up to which a round of the FP64 mode goes to the 8-lane kernel (N <= 3): there a warp's FP64
+// instructions serve 4 cells instead of 32, which is slower once the thread-per-cell kernel fills
+// the SMs. M_3: 8 lanes take about 8 us per 2,500 cells, a thread per cell 45 us up to 39,000.
+constexpr int kGroupUpTo = 8192;
 
+// Newton step of the listed cells.
 int launch_post(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, const double *u, int k,
                 NewtonParams np, double *Vacc, cudaStream_t s)
 {
-    // 64-thread blocks: the listed cells (often a few thousand) fill the low block indices, and
-    // small blocks spread them over every SM instead of a few
-    int blocks = (C + kPostBlock - 1) / kPostBlock;
-    if (blocks > mn->nsm * 32) blocks = mn->nsm * 32;
-    const int mixed = mn->p.mode != KITRT_FP64;
-    const int target = 1;
-    const size_t smem = post_smem_bytes(mn->n, mn->n2, mn->npairs, mn->gaunt_nnz, mixed != 0,
-                                        kUnrolledNewton && mn->N <= 3);
-    int rc = KITRT_OK;
-    KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(post_thread_kernel<NN>, smem));
-    if (rc) return rc;
+    const bool mixed = mn->p.mode != KITRT_FP64;
+    const int upto = mixed || mn->N > 3 ? 0x7fffffff : kGroupUpTo;
+    const int sweep_grid = mixed ? mn->grid_mixed : mn->grid_fp64, target = mixed ? mn->target_mixed : mn->target_fp64;
+    if (C > upto) {
+        LaunchScope ls(mn, PK_POST, s, 0);
+        sum_parts_kernel<<<mn->nsm * 8, 256, 0, s>>>(S, k, Vacc, mn->vs, mn->n2, sweep_grid, target, mn->Qs / 32, upto);
+        if (cudaGetLastError() != cudaSuccess) return KITRT_ECUDA;
+    }
+    if (C > upto) {
+        // 64-thread blocks: small blocks spread the listed cells over every SM
+        int blocks = (C + kPostBlock - 1) / kPostBlock;
+        if (blocks > mn->nsm * 32) blocks = mn->nsm * 32;
+        const size_t smem = post_smem_bytes(mn->n, mn->n2, mn->npairs, mn->gaunt_nnz);
+        LaunchScope ls(mn, PK_POST, s, 0);
+        int rc = KITRT_OK;
+#define THREAD_CASE(NNv)                                                                                       \
+    case NNv:                                                                                                  \
+        rc = ensure_dyn_smem(post_thread_kernel<NNv>, smem);                                                   \
+        if (!rc)                                                                                               \
+            post_thread_kernel<NNv><<<blocks, kPostBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs,             \
+                                                                     mn->gaunt_nnz, upto);                     \
+        break;
+        switch (mn->N) {
+            THREAD_CASE(1)
+            THREAD_CASE(2)
+            THREAD_CASE(3)
+        default: return KITRT_EINVAL;
+        }
+#undef THREAD_CASE
+        if (rc) return rc;
+        if (cudaGetLastError() != cudaSuccess) return KITRT_ECUDA;
+    }
+    const size_t smem = group_smem_bytes(mn->n2, mn->npairs, mn->gaunt_nnz, mixed);
+    int blocks = (C + kGroupCells - 1) / kGroupCells;
+    const int most = mn->nsm * (mn->N > 3 ? 2 : 4);
+    if (blocks > most) blocks = most;
+    if (blocks < 1) blocks = 1;
     LaunchScope ls(mn, PK_POST, s, 0);
-    KITRT_DISPATCH_N(mn->N, post_thread_kernel<NN><<<blocks > 0 ? blocks : 1, kPostBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mixed, target, mn->gaunt_nnz));
+    int rc = KITRT_OK;
+    if (mixed) {
+        KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(post_group_kernel<NN, true>, smem));
+        if (rc) return rc;
+        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, true><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, upto)));
+    } else {
+        KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(post_group_kernel<NN, false>, smem));
+        if (rc) return rc;
+        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, false><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, upto)));
+    }
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }
 

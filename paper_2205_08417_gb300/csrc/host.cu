@@ -907,8 +907,8 @@ static int run_closure(kitrt_mn *mn, int C, const double *u, const double *alpha
     int k = 0;
     for (int batch = mn->pass_hint;; batch = 4) {
         for (int b = 0; b < batch; ++b, ++k) {
-            // quadrature sweeps write each listed cell's moment row; the thread-per-cell Newton
-            // step then takes every listed cell
+            // quadrature sweeps write each listed cell's moment columns; the Newton step then takes
+            // every listed cell
             if (mn->p.mode == KITRT_FP64) {
                 rc = launch_eval_fp64(mn, T, mn->st, C, u, k, np, s, false, nullptr, mn->d_Vacc);
             } else {
@@ -919,7 +919,6 @@ static int run_closure(kitrt_mn *mn, int C, const double *u, const double *alpha
                 if (k > 0) rc = launch_eval_fp64(mn, T, mn->st, C, u, k, np, s, true, psi32, mn->d_Vacc);
                 if (!rc) rc = launch_eval_mixed(mn, T, mn->st, C, u, k, np, s, psi32);
             }
-            if (!rc) rc = launch_sum_parts(mn, mn->st, k, mn->d_Vacc, s);
             if (!rc) rc = launch_post(mn, T, mn->st, C, u, k, np, mn->d_Vacc, s);
             if (rc) return rc;
         }

@@ -251,7 +251,6 @@ int mixed_sweep_grid(const kitrt_mn *mn);
 int launch_eval_fp64(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
                      const double *u, int k, NewtonParams np, cudaStream_t s,
                      bool filter = false, float *psi32 = nullptr, double *Vacc = nullptr);
-int launch_sum_parts(kitrt_mn *mn, const NewtonState &S, int k, double *Vacc, cudaStream_t s);
 int launch_post(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, const double *u, int k,
                 NewtonParams np, double *Vacc, cudaStream_t s);
 int launch_finish(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,

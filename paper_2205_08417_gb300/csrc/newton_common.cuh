@@ -242,70 +242,52 @@ __device__ __forceinline__ void push_agg(int32_t *list, int32_t *cnt, int cell, 
     if (pred) list[base + __popc(m & ((1u << lane) - 1u))] = cell;
 }
 
-#define KITRT_PT_NAME newton_post_thread_rolled
-#define KITRT_PT_UNROLL _Pragma("unroll 1")
-#include "newton_post_thread_body.cuh"
-#undef KITRT_PT_NAME
-#undef KITRT_PT_UNROLL
-
-// Compact thread-per-cell Newton step (N <= 3), the same logic as newton_post_thread with a
-// small instruction footprint: the Hessian assembly, the Cholesky factorisation and the two
-// triangular solves run as rolled loops over per-thread slices of shared memory (entry e of a
-// thread at e * B + thread), instead of fully unrolled code over registers. With about one warp
-// per SM in a typical round, the unrolled body (several thousand instructions, run once) waited
-// mostly on instruction fetch (ncu: stalls on no_instruction ~3x those on memory); rolled loops
-// run from the instruction cache. R is float (mixed modes, tensor-core cells) or double (FP64
-// mode, and mixed-mode cells handed to the FP64 Hessian); dual, gradient, tests and iterate are
-// FP64 either way (see the thread body's precision note).
-__device__ __forceinline__ float r_fma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double r_fma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float r_rsqrt(float a) { return rsqrtf(a); }
-__device__ __forceinline__ double r_rsqrt(double a) { return rsqrt(a); }
-__device__ __forceinline__ bool r_pos(float d) { return d > 0.0f && d < 3.0e38f; }
-__device__ __forceinline__ bool r_pos(double d) { return d > 0.0; }
+// Newton step of one listed cell after a round of sweeps, in the FP64 mode for N <= 3 when many
+// cells are listed (launch_post): one thread per cell, so that every FP64 instruction works for 32
+// cells. The Hessian assembly, the Cholesky factorisation and the two triangular solves run as
+// rolled loops over per-thread slices of shared memory (entry e of a thread at e * B + thread):
+// fully unrolled code (several thousand instructions, run once) waited mostly on instruction fetch
+// (ncu: stalls on no_instruction ~3x those on memory).
 
 // H (packed lower, + gamma on the regularized diagonal) from the Gaunt terms, its Cholesky factor
-// (1/L_jj on the diagonal) in place, then y <- -H^-1 y in place. Vr: the moments in precision R,
-// entry c at Vr[c BV]; entry e of L and y at e B.
-// Returns false when the factorisation breaks down.
-template <int NN, typename R>
-__device__ bool hess_factor_solve(const Tables &T, const R *__restrict__ coef, const NewtonParams &np,
-                                  const R *Vr, int BV, R *L, R *y, int B)
+// (1/L_jj on the diagonal) in place, then y <- -H^-1 y in place. V: the moments, entry c at V[c B];
+// entry e of L and y at e B. Returns false when the factorisation breaks down.
+template <int NN>
+__device__ bool hess_factor_solve(const Tables &T, const NewtonParams &np, const double *V, double *L, double *y, int B)
 {
     constexpr int n = Dims<NN>::n, npairs = Dims<NN>::npairs;
 #pragma unroll 1
     for (int p = 0; p < npairs; ++p) {
-        R h = R(0);
+        double h = 0.0;
         const int t1 = T.gstart[p + 1];
 #pragma unroll 1
-        for (int t = T.gstart[p]; t < t1; ++t) h = r_fma(coef[t], Vr[(size_t)T.gidx[t] * BV], h);
+        for (int t = T.gstart[p]; t < t1; ++t) h = fma(T.gcoef[t], V[(size_t)T.gidx[t] * B], h);
         L[(size_t)p * B] = h;
     }
     if (np.gamma != 0.0) {
-        const R gam = (R)np.gamma;
 #pragma unroll 1
-        for (int j = np.reg0; j < n; ++j) L[(size_t)tri_idx(j, j) * B] += gam;
+        for (int j = np.reg0; j < n; ++j) L[(size_t)tri_idx(j, j) * B] += np.gamma;
     }
     bool spd = true;
 #pragma unroll 1
     for (int j = 0; j < n; ++j) {
         const int jj = j * (j + 1) / 2;
-        R d = L[(size_t)(jj + j) * B];
+        double d = L[(size_t)(jj + j) * B];
 #pragma unroll 1
         for (int k = 0; k < j; ++k) {
-            const R l = L[(size_t)(jj + k) * B];
-            d = r_fma(-l, l, d);
+            const double l = L[(size_t)(jj + k) * B];
+            d = fma(-l, l, d);
         }
-        spd = spd && r_pos(d);
-        const R rinv = r_rsqrt(d > R(0) ? d : R(1));
+        spd = spd && d > 0.0;
+        const double rinv = rsqrt(d > 0.0 ? d : 1.0);
         L[(size_t)(jj + j) * B] = rinv;
 #pragma unroll 1
         for (int i = j + 1; i < n; ++i) {
             const int ii = i * (i + 1) / 2;
-            R sacc = L[(size_t)(ii + j) * B];
+            double sacc = L[(size_t)(ii + j) * B];
 #pragma unroll 1
             for (int k = 0; k < j; ++k)
-                sacc = r_fma(-L[(size_t)(ii + k) * B], L[(size_t)(jj + k) * B], sacc);
+                sacc = fma(-L[(size_t)(ii + k) * B], L[(size_t)(jj + k) * B], sacc);
             L[(size_t)(ii + j) * B] = sacc * rinv;
         }
     }
@@ -313,39 +295,33 @@ __device__ bool hess_factor_solve(const Tables &T, const R *__restrict__ coef, c
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
         const int ii = i * (i + 1) / 2;
-        R sacc = y[(size_t)i * B];
+        double sacc = y[(size_t)i * B];
 #pragma unroll 1
-        for (int k = 0; k < i; ++k) sacc = r_fma(-L[(size_t)(ii + k) * B], y[(size_t)k * B], sacc);
+        for (int k = 0; k < i; ++k) sacc = fma(-L[(size_t)(ii + k) * B], y[(size_t)k * B], sacc);
         y[(size_t)i * B] = sacc * L[(size_t)(ii + i) * B];
     }
 #pragma unroll 1
     for (int i = n - 1; i >= 0; --i) {
-        R sacc = y[(size_t)i * B];
+        double sacc = y[(size_t)i * B];
 #pragma unroll 1
-        for (int k = i + 1; k < n; ++k)
-            sacc = r_fma(-L[(size_t)tri_idx(k, i) * B], y[(size_t)k * B], sacc);
+        for (int k = i + 1; k < n; ++k) sacc = fma(-L[(size_t)tri_idx(k, i) * B], y[(size_t)k * B], sacc);
         y[(size_t)i * B] = sacc * L[(size_t)tri_idx(i, i) * B];
     }
     return true;
 }
 
-// V, Vf: the cell's moments as in newton_post_thread (Vf: FP32 Hessian-only moments of a
-// tensor-core cell); Lbase, ybase: shared-memory regions of [npairs x B] and [n x B] doubles, of
-// which this thread (tid) owns column tid. The FP32 path keeps its floats in the low half of the
-// same 8-byte slots (float stride 2B), so that threads of one block on different paths never
-// touch each other's slots.
+// V: the cell's moments; Lsm, ysm: this thread's columns of [npairs x B] and [n x B] doubles.
+// Returns true when the cell continues (must be appended to the next list).
 template <int NN>
 __device__ bool newton_cell(const Tables &T, const NewtonState &S, const NewtonParams &np, int cell,
-                            const double *__restrict__ V, float *__restrict__ Vf, double *Lbase,
-                            double *ybase, int tid, int B, const double *__restrict__ u, bool mixed,
-                            int &evals_out)
+                            const double *__restrict__ V, double *Lsm, double *ysm, int B,
+                            const double *__restrict__ u, int &evals_out)
 {
     constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, npairs = Dims<NN>::npairs;
     const size_t off = (size_t)cell * n;
     const int ph = S.phase[cell];
     const double lam = ph == PH_NEWTON ? S.lam[cell] : 0.0;
     const bool reg = np.gamma != 0.0;
-    const bool h32 = mixed && !S.h64[cell];
     double at[n], ua[n];
     double au = 0.0, ar2 = 0.0;
 #pragma unroll
@@ -358,9 +334,7 @@ __device__ bool newton_cell(const Tables &T, const NewtonState &S, const NewtonP
     }
     bool finite = true;
 #pragma unroll
-    for (int c = 0; c < n2; ++c)
-        finite = finite && (c < n || !h32 ? finite_bits(V[(size_t)c * B])
-                                          : (__float_as_uint(Vf[(size_t)c * B]) & 0x7f800000u) != 0x7f800000u);
+    for (int c = 0; c < n2; ++c) finite = finite && finite_bits(V[(size_t)c * B]);
     const double fs = V[0] * T.rm0;
     const double ft = reg ? fma(0.5 * np.gamma, ar2, fs - au) : fs - au;
     const int ev = S.evals[cell] + 1;
@@ -386,14 +360,6 @@ __device__ bool newton_cell(const Tables &T, const NewtonState &S, const NewtonP
     if (!accept) {
         const int h = S.halv[cell] + 1;
         if (h > np.max_halvings) {
-            if (h32) {
-                // the line search could not follow the direction from the tensor-core Hessian:
-                // restart from the accepted point with the FP64 Hessian
-                hand_over(S, cell);
-                S.halv[cell] = 0;
-                S.phase[cell] = PH_INIT;
-                return true;
-            }
             fail_t(KITRT_ELINESEARCH);
             return false;
         }
@@ -401,42 +367,21 @@ __device__ bool newton_cell(const Tables &T, const NewtonState &S, const NewtonP
         S.lam[cell] = 0.5 * lam;
         return true;
     }
-    double g[n];
+    double g[n], y[n];
 #pragma unroll
     for (int a = 0; a < n; ++a) {
         g[a] = V[(size_t)a * B] - ua[a];
         if (reg && a >= np.reg0) g[a] = fma(np.gamma, at[a], g[a]);
+        ysm[(size_t)a * B] = -g[a];
     }
-    double y[n];
-    if (h32) {
-        float *Lf = reinterpret_cast<float *>(Lbase + tid), *yf = reinterpret_cast<float *>(ybase + tid);
-        const int B2 = 2 * B;
-#pragma unroll
-        for (int c = 0; c < n; ++c) Vf[(size_t)c * B] = d2f_bits(V[(size_t)c * B]);
-#pragma unroll
-        for (int a = 0; a < n; ++a) yf[(size_t)a * B2] = -d2f_bits(g[a]);
-        if (!hess_factor_solve<NN, float>(T, T.gcoef32, np, Vf, B, Lf, yf, B2)) {
-            hand_over(S, cell);  // rounding broke positive definiteness: redo this point in FP64
-            return true;
-        }
-#pragma unroll
-        for (int a = 0; a < n; ++a) y[a] = f2d_bits(yf[(size_t)a * B2]);
-#pragma unroll 1
-        for (int p = 0; p < npairs; ++p) S.L[(size_t)cell * npairs + p] = f2d_bits(Lf[(size_t)p * B2]);
-    } else {
-        double *Lsm = Lbase + tid, *ysm = ybase + tid;
-#pragma unroll
-        for (int a = 0; a < n; ++a) ysm[(size_t)a * B] = -g[a];
-        if (!hess_factor_solve<NN, double>(T, T.gcoef, np, V, B, Lsm, ysm, B)) {
-            // FP64 mode, or the FP64 Hessian of a handed-over cell: no further fallback
-            fail_t(KITRT_ECHOL);
-            return false;
-        }
-#pragma unroll
-        for (int a = 0; a < n; ++a) y[a] = ysm[(size_t)a * B];
-#pragma unroll 1
-        for (int p = 0; p < npairs; ++p) S.L[(size_t)cell * npairs + p] = Lsm[(size_t)p * B];
+    if (!hess_factor_solve<NN>(T, np, V, Lsm, ysm, B)) {
+        fail_t(KITRT_ECHOL);
+        return false;
     }
+#pragma unroll
+    for (int a = 0; a < n; ++a) y[a] = ysm[(size_t)a * B];
+#pragma unroll 1
+    for (int p = 0; p < npairs; ++p) S.L[(size_t)cell * npairs + p] = Lsm[(size_t)p * B];
 #pragma unroll
     for (int a = 0; a < n; ++a) {
         S.alpha[off + a] = at[a];
@@ -444,7 +389,6 @@ __device__ bool newton_cell(const Tables &T, const NewtonState &S, const NewtonP
     }
     S.fsum[cell] = fs;
     S.f0[cell] = ft;
-    if (S.lfac) S.lfac[cell] = 1;
     double gn2 = 0.0, un2 = 0.0, gd = 0.0;
 #pragma unroll
     for (int a = 0; a < n; ++a) {
@@ -465,8 +409,6 @@ __device__ bool newton_cell(const Tables &T, const NewtonState &S, const NewtonP
         fail_t(KITRT_ENOCONVERGE);
         return false;
     }
-    if (mixed && ph == PH_NEWTON && gn > kStallRatio * S.gnorm[cell]) hand_over(S, cell);
-    if (S.gnorm) S.gnorm[cell] = gn;
     S.gd[cell] = gd;
     S.lam[cell] = 1.0;
     S.halv[cell] = 0;
@@ -474,74 +416,49 @@ __device__ bool newton_cell(const Tables &T, const NewtonState &S, const NewtonP
     return true;
 }
 
-// Newton logic of every listed cell after a round of sweeps: thread per list slot, reading the
-// slot's moment row. Counters (evaluations, largest count) are warp-aggregated.
-// A round's list is often a few thousand cells, about one warp per SM, so the kernel is bound by
-// the latency of each thread's serial chain, not by throughput. Two things keep that chain short:
-//  - the slot's n2 moments are summed over the sweep's parts into shared memory one part at a
-//    time (the n2 loads of a part in flight together: `parts` round trips to memory, not n2 x
-//    parts);
-//  - the Gaunt tables (term ranges, moment indices, coefficients) are staged in shared memory
-//    once per block, so the table-driven Hessian assembly waits on shared memory, not on L2.
-// In the mixed modes the parts of a tensor-core cell's Hessian-only moments (degree > N) are FP32
-// numbers (tensor-core accumulators) and are added in FP32 into the FP32 copy; the degree <= N
-// moments (gradient and dual) are always added in FP64.
 constexpr int kPostBlock = 64;
-// N <= 3: the compact body (newton_cell: rolled loops over a shared-memory factor); N >= 4: the
-// thread body with its loops rolled over a factor in local memory (the shared-memory slices of
-// 120 or 231 doubles per thread would leave room for too few blocks on the large passes).
-constexpr bool kUnrolledNewton = true;
 
-// Dynamic shared memory of post_thread_kernel: [n2 x kPostBlock] doubles (moments), for N <= 3
-// the compact body's [npairs x kPostBlock] and [n x kPostBlock] doubles (factor, solve vector),
-// the Gaunt coefficients of the mode (FP64, or FP32 in the mixed modes), [n2 x kPostBlock] floats
-// (mixed modes), the moment indices and the npairs + 1 term starts.
-__host__ __device__ inline size_t post_smem_bytes(int n, int n2, int npairs, int nnz, bool mixed,
-                                                  bool compact)
+// Dynamic shared memory of post_thread_kernel: [n2 x kPostBlock], [npairs x kPostBlock] and
+// [n x kPostBlock] doubles (moments, factor, solve vector), the Gaunt coefficients, the moment
+// indices and the npairs + 1 term starts.
+__host__ __device__ inline size_t post_smem_bytes(int n, int n2, int npairs, int nnz)
 {
-    return (size_t)n2 * kPostBlock * 8 + (compact ? (size_t)(npairs + n) * kPostBlock * 8 : 0) +
-           (size_t)nnz * (mixed ? 4 : 8) + (mixed ? (size_t)n2 * kPostBlock * 4 : 0) +
-           (size_t)nnz * 4 + (size_t)(npairs + 1) * 4;
+    return (size_t)(n2 + npairs + n) * kPostBlock * 8 + (size_t)nnz * 12 + (size_t)(npairs + 1) * 4;
 }
 
+// The listed cells, when more than `above` of them, one thread each (their parts already summed by
+// sum_parts_kernel); otherwise post_group_kernel takes the round.
 template <int NN>
 __global__ void __launch_bounds__(kPostBlock)
 post_thread_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, NewtonParams np,
-                   const double *__restrict__ Vacc, int vs, int mixed, int target_items, int nnz)
+                   const double *__restrict__ Vacc, int vs, int nnz, int above)
 {
     constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, npairs = Dims<NN>::npairs;
-    constexpr bool compact = kUnrolledNewton && NN <= 3;
     extern __shared__ __align__(16) unsigned char post_smem[];
     double *sV = reinterpret_cast<double *>(post_smem);                     // [n2][thread]
     double *sL = sV + (size_t)n2 * kPostBlock;                              // [npairs][thread]
     double *sy = sL + (size_t)npairs * kPostBlock;                          // [n][thread]
-    // byte layout of post_smem_bytes: sV | sL, sy (compact) | coef | sVf (mixed) | gidx | gstart
-    unsigned char *coef = post_smem + (size_t)(n2 + (compact ? npairs + n : 0)) * kPostBlock * 8;
-    float *sVf = reinterpret_cast<float *>(coef + (size_t)nnz * (mixed ? 4 : 8));  // [n2][thread]
-    int32_t *gidx = reinterpret_cast<int32_t *>(reinterpret_cast<unsigned char *>(sVf) +
-                                                (mixed ? (size_t)n2 * kPostBlock * 4 : 0));
+    double *coef = sy + (size_t)n * kPostBlock;
+    int32_t *gidx = reinterpret_cast<int32_t *>(coef + nnz);
     int32_t *gstart = gidx + nnz;
     const int32_t *list_in = S.list[k & 1];
     int32_t *list_out = S.list[(k + 1) & 1];
     const int cnt_in = S.cnt[k % 3];
     const int stride = gridDim.x * blockDim.x;
-    if ((int)(blockIdx.x * blockDim.x) >= cnt_in) return;  // uniform: this block has no slot
-    // the sweeps split the quadrature of each tile into `parts` column blocks (sweep.cuh)
-    const int parts = target_items;
+    // uniform: not this kernel's round, or this block has no slot
+    if (cnt_in <= above || (int)(blockIdx.x * blockDim.x) >= cnt_in) return;
     int32_t *cnt_out = &S.cnt[(k + 1) % 3];
     // stage the Gaunt tables and point this block's view of them at the copies
     for (int t = threadIdx.x; t < nnz; t += blockDim.x) {
         gidx[t] = T.gidx[t];
-        if (mixed) reinterpret_cast<float *>(coef)[t] = T.gcoef32[t];
-        else reinterpret_cast<double *>(coef)[t] = T.gcoef[t];
+        coef[t] = T.gcoef[t];
     }
     for (int t = threadIdx.x; t <= npairs; t += blockDim.x) gstart[t] = T.gstart[t];
     __syncthreads();
     Tables Ts = T;
     Ts.gidx = gidx;
     Ts.gstart = gstart;
-    if (mixed) Ts.gcoef32 = reinterpret_cast<const float *>(coef);
-    else Ts.gcoef = reinterpret_cast<const double *>(coef);
+    Ts.gcoef = coef;
     const int rounds = (cnt_in + stride - 1) / stride;
     for (int rd = 0; rd < rounds; ++rd) {
         const int it = rd * stride + blockIdx.x * blockDim.x + threadIdx.x;
@@ -549,37 +466,397 @@ post_thread_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k,
         int cell = -1, ev = 0;
         if (it < cnt_in) {
             cell = list_in[it];
-            const bool h32 = mixed && !S.h64[cell];
-            // the slot's moments are column `it` of each part's block of the [n2 x vs]
-            // accumulator (every one written by this round's sweeps): consecutive slots (threads)
-            // read consecutive addresses; the parts are added in order
             double *mine = sV + threadIdx.x;
-            float *minef = sVf + threadIdx.x;
 #pragma unroll
-            for (int c = 0; c < n2; ++c) {
-                if (c < n || !h32) mine[c * kPostBlock] = 0.0;
-                else minef[c * kPostBlock] = 0.0f;
-            }
-            for (int p = 0; p < parts; ++p) {
-                const double *row = Vacc + (size_t)p * cnt_in + it;
-#pragma unroll
-                for (int c = 0; c < n2; ++c) {
-                    const double x = row[(size_t)c * vs];
-                    if (c < n || !h32) mine[c * kPostBlock] += x;
-                    else minef[c * kPostBlock] += d2f_bits(x);
-                }
-            }
-            if constexpr (compact)
-                cont = newton_cell<NN>(Ts, S, np, cell, mine, minef, sL, sy, threadIdx.x, kPostBlock,
-                                       u, mixed != 0, ev);
-            else
-                cont = newton_post_thread_rolled<NN>(Ts, S, np, cell, mine, minef, kPostBlock, u, mixed != 0, ev);
+            for (int c = 0; c < n2; ++c) mine[c * kPostBlock] = Vacc[(size_t)c * vs + it];
+            cont = newton_cell<NN>(Ts, S, np, cell, mine, sL + threadIdx.x, sy + threadIdx.x, kPostBlock, u, ev);
         }
         // every slot taken in this round is one evaluation
         const unsigned act = __activemask();
         const unsigned live = __ballot_sync(act, it < cnt_in);
         const int evmax = __reduce_max_sync(act, ev);
         if ((threadIdx.x & 31) == __ffs(act) - 1 && live) {
+            atomicAdd(&S.cnt[6], __popc(live));
+            atomicMax(&S.cnt[4], evmax);
+        }
+        push_agg(list_out, cnt_out, cell, cont);
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Newton step with 8 lanes per cell (every mixed-mode round; FP64 mode for N >= 4 or few cells).
+//
+// A round lists anything from a few hundred to all cells. One thread per cell leaves a serial chain
+// of a few thousand dependent instructions, and its factor does not fit a thread's registers for
+// N >= 4 (120 or 231 entries). Here 8 lanes share a cell: lane g owns the rows g, g + 8, g + 16 of
+// the Hessian and its factor in registers, pivots and columns travel by shuffles, and the packed
+// matrix passes through shared memory only to be assembled (entries dealt to the lanes) and to be
+// written out in whole rows. Measured against the thread-per-cell kernels with their separate
+// summation of the sweeps' parts (part of the load here), Newton time of a run: M_5, 996,872 cells,
+// two steps 70.3 -> 15.2 ms; M_4, 20,000 cells 1.09 -> 0.23 ms; M_3, 99,458 cells, four steps
+// 0.94 -> 0.82 ms; M_2 in FP64 mode, 3,872 cells 0.25 -> 0.17 ms.
+// ---------------------------------------------------------------------------------------------
+constexpr int kGroupBlock = 256;
+constexpr int kGroupCells = kGroupBlock / 8;  // cells per block and pass
+constexpr int kGroupPitch = kGroupCells + 1;  // row pitch of the moments in shared memory
+
+__device__ __forceinline__ float r_fma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double r_fma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ bool r_pos(float d) { return d > 0.0f && d < 3.0e38f; }
+__device__ __forceinline__ bool r_pos(double d) { return d > 0.0; }
+__device__ __forceinline__ float r_rsqrt(float a) { return rsqrtf(a); }
+// 1/sqrt(a): the FP32 value improved by one third-order step y (1 + e/2 + 3 e^2 / 8), e = 1 - a y^2
+// (the binomial series of (1 - e)^(-1/2); e is about 1e-7, the dropped term 1e-22), five FP64
+// instructions; outside the float range the library function.
+static __device__ __noinline__ double r_rsqrt_any(double a) { return rsqrt(a); }
+__device__ __forceinline__ double r_rsqrt(double a)
+{
+    if (!(a > 1e-37 && a < 1e37)) return r_rsqrt_any(a);
+    const double y = f2d_bits(rsqrtf(d2f_bits(a)));
+    const double e = fma(-a * y, y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+__device__ __forceinline__ double group_sum(double v)
+{
+    v += __shfl_xor_sync(kFull, v, 4);
+    v += __shfl_xor_sync(kFull, v, 2);
+    v += __shfl_xor_sync(kFull, v, 1);
+    return v;
+}
+
+// f(Int<B>) ... f(Int<E - 1>): a loop whose index is a compile-time constant
+template <int I>
+struct Int {
+    __host__ __device__ constexpr operator int() const { return I; }
+};
+template <int B, int E, typename F>
+__device__ __forceinline__ void static_for(F &&f)
+{
+    if constexpr (B < E) {
+        f(Int<B>{});
+        static_for<B + 1, E>(f);
+    }
+}
+
+// Assembly, factorisation and solve of one cell per group, in precision R: H from the Gaunt terms
+// (coef, idx; Vr: the block's moments in R, entry c of this cell at Vr[c kGroupPitch]) into Hs
+// [npairs], its factor (1/L_jj on the diagonal) back into Hs, and y <- H^-1 y (row g + 8 s in y[s]).
+// Whole warps; cells that do not take part compute along. Returns whether H was positive definite.
+template <int NN, typename R, typename Coef, typename Idx>
+__device__ __forceinline__ bool group_factor_solve(const Coef *__restrict__ coef, const Idx *__restrict__ idx,
+                                                   const int32_t *__restrict__ gstart, const R *Vr, R *Hs,
+                                                   R gamma, int reg0, int g, R (&y)[(Dims<NN>::n + 7) / 8])
+{
+    constexpr int n = Dims<NN>::n, npairs = Dims<NN>::npairs, SL = (n + 7) / 8;
+    for (int p = g; p < npairs; p += 8) {
+        R h = R(0);
+        const int t1 = gstart[p + 1];
+        for (int t = gstart[p]; t < t1; ++t) h = r_fma((R)coef[t], Vr[(int)idx[t] * kGroupPitch], h);
+        Hs[p] = h;
+    }
+    __syncwarp();
+    // row g + 8 s in r[s n ..] (columns beyond the row are not used); every index below is a
+    // compile-time constant, so that the rows stay in registers
+    R r[SL * n];
+    static_for<0, SL>([&](auto S) {
+        static_for<0, (8 * S + 8 < n ? 8 * S + 8 : n)>([&](auto K) {
+            const int row = g + 8 * S;
+            r[S * n + K] = row < n && K <= row ? Hs[row * (row + 1) / 2 + K] : R(0);
+            if (K == row && row >= reg0) r[S * n + K] += gamma;
+        });
+    });
+    bool spd = true;
+    static_for<0, n>([&](auto J) {
+        constexpr int j = J, sj = J / 8, own = sj * n + j;
+        const R d = __shfl_sync(kFull, r[own], j & 7, 8);
+        spd = spd && r_pos(d);
+        const R rinv = r_rsqrt(d > R(0) ? d : R(1));
+        static_for<sj, SL>([&](auto S) {
+            const R scaled = r[S * n + j] * rinv;
+            r[S * n + j] = g + 8 * S == j ? rinv : scaled;
+        });
+        static_for<j + 1, n>([&](auto K) {
+            const R l = __shfl_sync(kFull, r[(K / 8) * n + j], K & 7, 8);
+            static_for<K / 8, SL>([&](auto S) { r[S * n + K] = r_fma(-r[S * n + j], l, r[S * n + K]); });
+        });
+        // forward substitution with the finished column
+        const R yj = __shfl_sync(kFull, y[sj] * r[own], j & 7, 8);
+        static_for<sj, SL>([&](auto S) {
+            const R next = r_fma(-r[S * n + j], yj, y[S]);
+            y[S] = g + 8 * S == j ? yj : g + 8 * S > j ? next : y[S];
+        });
+    });
+    __syncwarp();
+    static_for<0, SL>([&](auto S) {
+        static_for<0, (8 * S + 8 < n ? 8 * S + 8 : n)>([&](auto K) {
+            const int row = g + 8 * S;
+            if (row < n && K <= row) Hs[row * (row + 1) / 2 + K] = r[S * n + K];
+        });
+    });
+    __syncwarp();
+    // backward substitution: row j of the factor from shared memory
+    static_for<0, n>([&](auto I) {
+        constexpr int j = n - 1 - I, sj = j / 8;
+        const R xj = __shfl_sync(kFull, y[sj] * r[sj * n + j], j & 7, 8);
+        static_for<0, sj + 1>([&](auto S) {
+            const int row = g + 8 * S;
+            if (row < j) y[S] = r_fma(-Hs[j * (j + 1) / 2 + row], xj, y[S]);
+            if (row == j) y[S] = xj;
+        });
+    });
+    return spd;
+}
+
+// Dynamic shared memory of post_group_kernel: moments [n2][pitch] (FP64, and FP32 in the mixed
+// modes), one packed matrix per cell, the Gaunt coefficients of the mode, indices and starts, and
+// the pass's cells.
+__host__ __device__ inline size_t group_smem_bytes(int n2, int npairs, int nnz, bool mixed)
+{
+    return (size_t)n2 * kGroupPitch * (mixed ? 12 : 8) + (size_t)kGroupCells * npairs * 8 + (size_t)nnz * (mixed ? 4 : 8) +
+           (size_t)((nnz + 3) / 4 * 4) + (size_t)(npairs + 1) * 4 + 2 * kGroupCells * 4;
+}
+
+template <int NN, bool MIXED>
+__global__ void __launch_bounds__(kGroupBlock, 2)
+post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, NewtonParams np,
+                  const double *__restrict__ Vacc, int vs, int nnz, int sweep_grid, int target_items, int upto)
+{
+    constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, npairs = Dims<NN>::npairs, SL = (n + 7) / 8;
+    extern __shared__ __align__(16) unsigned char group_smem[];
+    double *sV = reinterpret_cast<double *>(group_smem);                           // [n2][pitch]
+    double *sH = sV + n2 * kGroupPitch;                                            // [cell][npairs]
+    unsigned char *coef = reinterpret_cast<unsigned char *>(sH + kGroupCells * npairs);
+    float *sVf = reinterpret_cast<float *>(coef + (size_t)nnz * (MIXED ? 4 : 8));  // [n2][pitch]
+    int32_t *gstart = reinterpret_cast<int32_t *>(sVf + (MIXED ? n2 * kGroupPitch : 0));
+    int32_t *scell = gstart + npairs + 1, *sh64 = scell + kGroupCells;
+    unsigned char *gidx = reinterpret_cast<unsigned char *>(sh64 + kGroupCells);
+    const int32_t *list_in = S.list[k & 1];
+    int32_t *list_out = S.list[(k + 1) & 1];
+    const int cnt_in = S.cnt[k % 3];
+    // uniform: not this kernel's round, or no slot for this block
+    if (cnt_in > upto || (int)blockIdx.x * kGroupCells >= cnt_in) return;
+    const int parts = sweep_split(cnt_in, sweep_grid, target_items, T.Qs / 32).parts;
+    int32_t *cnt_out = &S.cnt[(k + 1) % 3];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane & 7, slot = tid >> 3;
+    for (int t = tid; t < nnz; t += kGroupBlock) {
+        gidx[t] = (unsigned char)T.gidx[t];
+        if (MIXED) reinterpret_cast<float *>(coef)[t] = T.gcoef32[t];
+        else reinterpret_cast<double *>(coef)[t] = T.gcoef[t];
+    }
+    for (int t = tid; t <= npairs; t += kGroupBlock) gstart[t] = T.gstart[t];
+    const bool reg = np.gamma != 0.0;
+    for (int base = blockIdx.x * kGroupCells; base < cnt_in; base += gridDim.x * kGroupCells) {
+        __syncthreads();  // the previous pass has read its shared memory
+        if (tid < kGroupCells) {
+            const int c = base + tid < cnt_in ? list_in[base + tid] : -1;
+            scell[tid] = c;
+            sh64[tid] = MIXED && c >= 0 ? S.h64[c] : 0;
+        }
+        __syncthreads();
+        // the moments of the pass's cells, the sweeps' parts added in order: in FP32 for the
+        // Hessian-only moments of tensor-core cells (accumulator values), else in FP64
+        for (int e = tid; e < n2 * kGroupCells; e += kGroupBlock) {
+            const int c = e / kGroupCells, j = e % kGroupCells;
+            const double *col = Vacc + (size_t)c * vs + min(base + j, cnt_in - 1);
+            if (MIXED && c >= n && !sh64[j]) {
+                float v = d2f_bits(col[0]);
+#pragma unroll 4
+                for (int p = 1; p < parts; ++p) v += d2f_bits(col[(size_t)p * cnt_in]);
+                sVf[c * kGroupPitch + j] = v;
+            } else {
+                double v = col[0];
+#pragma unroll 4
+                for (int p = 1; p < parts; ++p) v += col[(size_t)p * cnt_in];
+                sV[c * kGroupPitch + j] = v;
+                if (MIXED) sVf[c * kGroupPitch + j] = d2f_bits(v);
+            }
+        }
+        __syncthreads();
+        const int cell = scell[slot];
+        const bool valid = cell >= 0, h32 = MIXED && !sh64[slot];
+        const size_t off = (size_t)(valid ? cell : 0) * n;
+        const double *V = sV + slot;
+        const float *Vf = sVf + slot;
+        const int ph = valid ? S.phase[cell] : PH_DONE;
+        const double lam = ph == PH_NEWTON ? S.lam[cell] : 0.0;
+        double at[SL], ua[SL], gr[SL];
+        double au = 0.0, ar2 = 0.0;
+#pragma unroll
+        for (int s = 0; s < SL; ++s) {
+            const int c = g + 8 * s;
+            const bool in = valid && c < n;
+            const double al = in ? S.alpha[off + c] : 0.0;
+            at[s] = in && ph == PH_NEWTON ? fma(lam, S.dir[off + c], al) : al;
+            ua[s] = in ? u[off + c] : 0.0;
+            au = fma(at[s], ua[s], au);
+            if (reg && c >= np.reg0) ar2 = fma(at[s], at[s], ar2);
+        }
+        bool fin = true;
+        for (int c = g; c < n2; c += 8)
+            fin = fin && (c < n || !h32 ? finite_bits(V[c * kGroupPitch])
+                                        : (__float_as_uint(Vf[c * kGroupPitch]) & 0x7f800000u) != 0x7f800000u);
+        const bool finite = ((~__ballot_sync(kFull, fin) >> (lane & 24)) & 0xffu) == 0;
+        au = group_sum(au);
+        if (reg) ar2 = group_sum(ar2);
+        const double fs = V[0] * T.rm0;
+        const double ft = reg ? fma(0.5 * np.gamma, ar2, fs - au) : fs - au;
+        bool accept = valid && finite;
+        int ev = 0;
+        double gnorm0 = 0.0;
+        if (valid) {
+            if (ph == PH_NEWTON) {
+                const double fs0 = S.fsum[cell], f0 = S.f0[cell];
+                const double slack = 64.0 * 2.220446049250313e-16 * (fs0 + fabs(fs0 - f0));
+                accept = finite && ft <= f0 + np.c1 * lam * S.gd[cell] + slack;
+                if (MIXED) gnorm0 = S.gnorm[cell];
+            }
+            ev = S.evals[cell] + 1;
+        }
+        // the Newton direction -H^-1 (<m e> - u + gamma alpha^r) of the accepted cells
+        double y[SL];
+#pragma unroll
+        for (int s = 0; s < SL; ++s) {
+            const int c = g + 8 * s;
+            gr[s] = c < n ? V[c * kGroupPitch] - ua[s] : 0.0;
+            if (reg && c < n && c >= np.reg0) gr[s] = fma(np.gamma, at[s], gr[s]);
+            y[s] = 0.0;
+        }
+        const int reg0 = reg ? np.reg0 : n;
+        bool spd = false;
+        if (MIXED && __any_sync(kFull, accept && h32)) {
+            float yf[SL];
+#pragma unroll
+            for (int s = 0; s < SL; ++s) yf[s] = -d2f_bits(gr[s]);
+            float *Hs = reinterpret_cast<float *>(sH + warp * 4 * npairs) + (lane >> 3) * npairs;
+            const bool ok = group_factor_solve<NN, float>(reinterpret_cast<const float *>(coef), gidx, gstart, Vf, Hs,
+                                                          (float)np.gamma, reg0, g, yf);
+            if (h32) {
+                spd = ok;
+#pragma unroll
+                for (int s = 0; s < SL; ++s) y[s] = f2d_bits(yf[s]);
+            }
+            const unsigned keep = __ballot_sync(kFull, accept && h32 && ok);
+            const float *W = reinterpret_cast<const float *>(sH + warp * 4 * npairs);
+            for (int e = lane; e < 4 * npairs; e += 32) {
+                const int q = e / npairs;
+                if ((keep >> (8 * q)) & 1)
+                    S.L[(size_t)scell[warp * 4 + q] * npairs + (e - q * npairs)] = f2d_bits(W[e]);
+            }
+            __syncwarp();
+        }
+        if (!MIXED || __any_sync(kFull, accept && !h32)) {
+            double yd[SL];
+#pragma unroll
+            for (int s = 0; s < SL; ++s) yd[s] = -gr[s];
+            double *Hs = sH + slot * npairs;
+            bool ok;
+            if (MIXED)
+                ok = group_factor_solve<NN, double>(T.gcoef, T.gidx, T.gstart, V, Hs, np.gamma, reg0, g, yd);
+            else
+                ok = group_factor_solve<NN, double>(reinterpret_cast<const double *>(coef), gidx, gstart, V, Hs,
+                                                    np.gamma, reg0, g, yd);
+            if (!h32) {
+                spd = ok;
+#pragma unroll
+                for (int s = 0; s < SL; ++s) y[s] = yd[s];
+            }
+            const unsigned keep = __ballot_sync(kFull, accept && !h32 && ok);
+            const double *W = sH + warp * 4 * npairs;
+            for (int e = lane; e < 4 * npairs; e += 32) {
+                const int q = e / npairs;
+                if ((keep >> (8 * q)) & 1) S.L[(size_t)scell[warp * 4 + q] * npairs + (e - q * npairs)] = W[e];
+            }
+            __syncwarp();
+        }
+        double gn2 = 0.0, un2 = 0.0, gd = 0.0;
+#pragma unroll
+        for (int s = 0; s < SL; ++s) {
+            gn2 = fma(gr[s], gr[s], gn2);
+            un2 = fma(ua[s], ua[s], un2);
+            gd = fma(gr[s], y[s], gd);
+        }
+        gn2 = group_sum(gn2);
+        un2 = group_sum(un2);
+        gd = group_sum(gd);
+        const bool step = accept && spd;
+        if (step) {
+#pragma unroll
+            for (int s = 0; s < SL; ++s) {
+                const int c = g + 8 * s;
+                if (c < n) {
+                    S.alpha[off + c] = at[s];
+                    S.U[off + c] = V[c * kGroupPitch];
+                    S.dir[off + c] = y[s];
+                }
+            }
+        }
+        bool cont = false;
+        if (g == 0 && valid) {
+            S.evals[cell] = ev;
+            int code = 0;  // status of a cell that fails here
+            if (step) {
+                S.fsum[cell] = fs;
+                S.f0[cell] = ft;
+                if (S.lfac) S.lfac[cell] = 1;
+                int iters = S.iters[cell];
+                if (ph == PH_NEWTON) ++iters;
+                S.iters[cell] = iters;
+                const double gn = sqrt(gn2);
+                if (gn <= np.tau * sqrt(un2)) {
+                    S.phase[cell] = PH_DONE;
+                } else if (iters >= np.max_iter) {
+                    code = KITRT_ENOCONVERGE;
+                } else {
+                    // a Newton step on the tensor-core Hessian that does not halve the residual
+                    // sends the cell to the FP64 Hessian
+                    if (MIXED && ph == PH_NEWTON && gn > kStallRatio * gnorm0) hand_over(S, cell);
+                    if (MIXED) S.gnorm[cell] = gn;
+                    S.gd[cell] = gd;
+                    S.lam[cell] = 1.0;
+                    S.halv[cell] = 0;
+                    S.phase[cell] = PH_NEWTON;
+                    cont = true;
+                }
+            } else if (accept) {
+                // FP32 rounding broke positive definiteness: redo this point with the FP64 Hessian;
+                // no further fallback there
+                if (h32) {
+                    hand_over(S, cell);
+                    cont = true;
+                } else {
+                    code = KITRT_ECHOL;
+                }
+            } else if (ph == PH_INIT) {
+                code = KITRT_ENOTREALIZABLE;
+            } else {
+                const int h = S.halv[cell] + 1;
+                if (h <= np.max_halvings) {
+                    S.halv[cell] = h;
+                    S.lam[cell] = 0.5 * lam;
+                    cont = true;
+                } else if (h32) {
+                    // the line search could not follow the direction from the tensor-core Hessian:
+                    // restart from the accepted point with the FP64 Hessian
+                    hand_over(S, cell);
+                    S.halv[cell] = 0;
+                    S.phase[cell] = PH_INIT;
+                    cont = true;
+                } else {
+                    code = KITRT_ELINESEARCH;
+                }
+            }
+            if (code) {
+                S.status[cell] = code;
+                S.phase[cell] = PH_DONE;
+                atomicAdd(&S.cnt[3], 1);
+            }
+        }
+        __syncwarp();
+        // every listed cell of this pass is one evaluation
+        const unsigned live = __ballot_sync(kFull, valid && g == 0);
+        const int evmax = __reduce_max_sync(kFull, ev);
+        if (lane == 0 && live) {
             atomicAdd(&S.cnt[6], __popc(live));
             atomicMax(&S.cnt[4], evmax);
         }
