@@ -420,47 +420,110 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
 }
 
 // ---------------------------------------------------------------------------------------------
-// finish: final alpha (alpha_k plus the polish step if enabled) to the caller, and optionally the
-// ansatz psi at every folded point (FP64 and/or FP32).
+// finish: final alpha (alpha_k plus the polish step if enabled) to the caller and the FP64 ansatz psi
+// at every folded point. Lanes are cells; the block's 4 warps take a quarter of the quads each of the
+// same 32 cells, in the fixed-point form of the sweeps (exponents of four azimuths from one set of
+// products). FP64 exponents and exponentials (18 FP64 instructions a point for M_3) bound the former
+// kernel (a warp per cell): 1.23 -> 0.33 ms a step on 99,458 cells, M_3, order 20, where 318 MB are
+// written.
 // ---------------------------------------------------------------------------------------------
+constexpr int kFinishWarps = 4;
+
 template <int NN>
-__global__ void __launch_bounds__(kWarps * 32)
-finish_kernel(Tables T, NewtonState S, double *__restrict__ alpha_out, double *__restrict__ psi,
-              float *__restrict__ psi32, int polish, int compare_prev, int C)
+__device__ __noinline__ void psi_row_fp64(const Tables &T, const double *alpha, double *row, int q0, int q1)
 {
     constexpr int n = Dims<NN>::n;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int Qp = T.Qp;
-    for (int cell = blockIdx.x * kWarps + wib; cell < C; cell += gridDim.x * kWarps) {
+    for (int q = q0; q < q1; ++q) {
+        double z = 0.0;
+        for (int b = 0; b < n; ++b) z = fma(alpha[b], T.Mt[(size_t)b * T.Qp + q], z);
+        row[q] = kexp(z, T.exptab);
+    }
+}
+
+template <int NN>
+__global__ void __launch_bounds__(kFinishWarps * 32)
+finish_kernel(Tables T, NewtonState S, double *__restrict__ alpha_out, double *__restrict__ psi, int polish,
+              int compare_prev, int C)
+{
+    constexpr int n = Dims<NN>::n;
+    extern __shared__ __align__(16) unsigned char finish_smem[];
+    uint64_t *tab = (uint64_t *)finish_smem;
+    int2 *trig = (int2 *)(tab + 2048);                 // [J][2 NN]
+    int2 *sA = trig + T.J * 2 * NN;                    // [n][32]
+    float *sB = (float *)(sA + n * 32);                // [warp][32]
+    int *sDiff = (int *)(sB + kFinishWarps * 32);      // [warp][32]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if ((int)blockIdx.x * 32 >= C) return;
+    for (int e = tid; e < 2048; e += blockDim.x) tab[e] = T.fx_exp[e];
+    for (int e = tid; e < T.J * 2 * NN; e += blockDim.x) {
+        const int p = e / (2 * NN), q = e % (2 * NN);
+        trig[e] = T.fx_trig[p * 4 * NN + (q < NN ? q : NN + q)];
+    }
+    for (int base = blockIdx.x * 32; base < C; base += gridDim.x * 32) {
+        const int cell = min(base + lane, C - 1);
         const size_t off = (size_t)cell * n;
-        const bool ok = S.status[cell] == 0;
-        double a = lane < n ? S.alpha[off + lane] : 0.0;
-        if (ok && polish && lane < n) a += S.dir[off + lane];
-        // alpha_out still holds the previous step's alpha (and psi its ansatz) when compare_prev
-        // is set: a bitwise-unchanged alpha leaves psi as it is
-        if (compare_prev) {
-            const double prev = lane < n ? alpha_out[off + lane] : 0.0;
-            if (__all_sync(kFull, prev == a)) continue;
+        const bool add = polish && S.status[cell] == 0;
+        __syncthreads();  // the tables, and the previous pass's reads of sA
+        // every warp forms its share of the components; alpha_out still holds the previous step's
+        // alpha (and psi its ansatz) when compare_prev is set: a bitwise-unchanged alpha leaves psi
+        // as it is
+        float bound = 0.0f;
+        int differs = compare_prev ? 0 : 1;
+        for (int c = warp; c < n; c += kFinishWarps) {
+            double a = S.alpha[off + c];
+            if (add) a += S.dir[off + c];
+            if (compare_prev && !(alpha_out[off + c] == a)) differs = 1;
+            const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(a));
+            sA[c * 32 + lane] = make_int2(w.h, w.l);
+            bound = fmaf(fabsf(d2f_bits(a)), T.fx_mmax[c], bound);
+            if (base + lane < C) alpha_out[off + c] = a;  // this thread alone reads and writes it
         }
-        if (lane < n) alpha_out[off + lane] = a;
-        if (!psi && !psi32) continue;
-        double av[n];
+        sB[tid] = bound;
+        sDiff[tid] = differs;
+        __syncthreads();
+        differs = 0;
+        bound = 0.0f;
 #pragma unroll
-        for (int b = 0; b < n; ++b) av[b] = __shfl_sync(kFull, a, b);
-        for (int q = lane; q < T.Qf; q += 32) {
-            double z = 0.0;
+        for (int w = 0; w < kFinishWarps; ++w) {
+            differs |= sDiff[w * 32 + lane];
+            bound += sB[w * 32 + lane];
+        }
+        const bool store = differs && base + lane < C;
+        if (!__any_sync(kFull, store)) continue;
+        const int qd0 = warp * T.nquad / kFinishWarps, qd1 = (warp + 1) * T.nquad / kFinishWarps;
+        double *row = psi + (size_t)cell * T.Qp;
+        const bool wide = !(bound < kitrt_fx::kFxMaxZ);  // outside the fixed-point range
+        if (store && wide)
+            psi_row_fp64<NN>(T, alpha_out + off, row, warp * T.Qf / kFinishWarps, (warp + 1) * T.Qf / kFinishWarps);
+        int ring = qd0 / T.J, jq = qd0 - ring * T.J;
+        bool fresh = true;
+        long long A0 = 0;
+        Limb A[2 * NN];
+#pragma unroll 1
+        for (int qd = qd0; qd < qd1; ++qd) {
+            if (fresh) {
+                fx_coeffs<NN>(
+                    [&](int c) {
+                        const int2 v = sA[c * 32 + lane];
+                        return Limb{v.x, v.y};
+                    },
+                    T.fx_ringA + (size_t)ring * n, A0, A);
+                fresh = false;
+            }
+            const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
+            long long s[4];
+            fx_exponents<NN>(A0, A, trig + jq * 2 * NN, NN, jq == 0, s);
+            double e[4];
 #pragma unroll
-            for (int b = 0; b < n; ++b) z = fma(av[b], T.Mt[b * Qp + q], z);
-            if (psi) {
-                const double e = kexp(z, T.exptab);
-                psi[(size_t)cell * Qp + q] = e;
-                if (psi32) psi32[(size_t)cell * Qp + q] = (float)e;
-            } else {
-                // FP32 ansatz for the mixed modes: exact FP64 exponent split into z_hi + z_lo,
-                // exp(z) = expf(z_hi) (1 + z_lo) to FP32 accuracy without an FP64 exp
-                const float zh = (float)z;
-                const float zl = (float)(z - (double)zh);
-                psi32[(size_t)cell * Qp + q] = expf(zh) * (1.0f + zl);
+            for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_double(kitrt_fx::fx_exp(s[t], tab));
+            if (store && !wide) {
+                *(double2 *)(row + 2 * pa) = make_double2(e[0], e[1]);
+                if (pb >= 0) *(double2 *)(row + 2 * pb) = make_double2(e[2], e[3]);
+            }
+            if (++jq == T.J) {
+                jq = 0;
+                ++ring;
+                fresh = true;
             }
         }
     }
@@ -756,18 +819,19 @@ int launch_eval_fp64(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
 }
 
 int launch_finish(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
-                  double *alpha_out, double *psi, float *psi32, int polish, int compare_prev,
-                  cudaStream_t s)
+                  double *alpha_out, double *psi, int polish, int compare_prev, cudaStream_t s)
 {
-    const int grid = grid_for(mn, C, 8);
     LaunchScope ls(mn, PK_FINISH, s, C);
-    if (!psi && !psi32) {
+    if (!psi) {
         const size_t total = (size_t)C * T.n;
         int blocks = (int)((total + 255) / 256);
         if (blocks > mn->nsm * 8) blocks = mn->nsm * 8;
         finish_alpha_kernel<<<blocks > 0 ? blocks : 1, 256, 0, s>>>(S, alpha_out, polish, T.n, C);
         return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
     }
-    KITRT_DISPATCH_N(mn->N, finish_kernel<NN><<<grid, kWarps * 32, 0, s>>>(T, S, alpha_out, psi, psi32, polish, compare_prev, C));
+    const size_t smem = 2048 * 8 + (size_t)T.J * 2 * mn->N * 8 + (size_t)T.n * 32 * 8 + kFinishWarps * 32 * 8;
+    int blocks = (C + 31) / 32;
+    if (blocks > mn->nsm * 16) blocks = mn->nsm * 16;
+    KITRT_DISPATCH_N(mn->N, finish_kernel<NN><<<blocks > 0 ? blocks : 1, kFinishWarps * 32, smem, s>>>(T, S, alpha_out, psi, polish, compare_prev, C));
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }

@@ -701,6 +701,26 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
                 }
                 ringW[(size_t)rg * n2 + cc] = limbs(ldexpl(r.ring_w[rg] * p, -mn->fx_wexp), 54);
             }
+        // the quads' tables of the FP64 flux: the axes' quad (j = 0: 0, pi, pi/2, 3 pi/2) takes
+        // cos = 1 and the sign of sin(k pi/2) for odd k, 0 for even k
+        std::vector<double> fr((size_t)mn->R * n), fa((size_t)mn->J * n), fsc((size_t)mn->J * 2);
+        for (int rg = 0; rg < mn->R; ++rg)
+            for (int cc = 0; cc < n; ++cc)
+                fr[(size_t)rg * n + cc] = r.ring_w[rg] * sqrt(1.0 - r.ring_mu[rg] * r.ring_mu[rg]) * P[(size_t)rg * n2 + cc];
+        for (int j = 0; j < mn->J; ++j) {
+            const double phi = j * (2.0 * kPi / r.nphi);
+            fsc[2 * j] = j ? sin(phi) : 0.0;
+            fsc[2 * j + 1] = j ? cos(phi) : 1.0;
+            int cc = 0;
+            for (int l = 0; l <= mn->N; ++l)
+                for (int k = -l; k <= l; k += 2, ++cc)
+                    fa[(size_t)j * n + cc] = j ? (k >= 0 ? cos(k * phi) : sin(-k * phi))
+                                               : (k >= 0 ? 1.0 : k & 1 ? ((-k) & 2 ? -1.0 : 1.0) : 0.0);
+        }
+        TRY(dev_upload(mn, &mn->d_flux_ring, fr));
+        TRY(dev_upload(mn, &mn->d_flux_az, fa));
+        TRY(dev_upload(mn, &mn->d_flux_sc, fsc));
+        TRY(dev_upload(mn, &mn->d_zero64, std::vector<double>(Qp, 0.0)));
         TRY(dev_upload(mn, &mn->d_fx_trig, trig));
         TRY(dev_upload(mn, &mn->d_fx_ringA, ringA));
         TRY(dev_upload(mn, &mn->d_fx_ringW, ringW));
@@ -966,7 +986,7 @@ int kitrt_internal_step(kitrt_mn *mn, double *u, double *alpha, const double *sa
     const int C = mn->mesh->C;
     int rc = run_closure(mn, C, u, alpha, first, s, nullptr);
     if (rc) return rc;
-    rc = launch_finish(mn, mn->tables(), mn->st, C, alpha, mn->d_psi, nullptr, polish_of(mn), !first, s);
+    rc = launch_finish(mn, mn->tables(), mn->st, C, alpha, mn->d_psi, polish_of(mn), !first, s);
     if (rc) return rc;
     return launch_flux_update(mn, mn->tables(), C, mn->d_psi, nullptr, u, sa, ss, q, dt, mn->p.bc, s);
 }
@@ -982,7 +1002,7 @@ int32_t kitrt_closure_batch(kitrt_mn *mn, const double *u, double *alpha, int32_
     if (stats) memset(stats, 0, sizeof(*stats));
     const int64_t launches0 = mn->launch_count;
     int rc = run_closure(mn, ncells, u, alpha, 1, s, stats);
-    int rc2 = launch_finish(mn, mn->tables(), mn->st, ncells, alpha, nullptr, nullptr,
+    int rc2 = launch_finish(mn, mn->tables(), mn->st, ncells, alpha, nullptr,
                             polish_of(mn), 0, s);
     if (status)
         CUDA_OK(cudaMemcpyAsync(status, mn->st.status, sizeof(int32_t) * ncells,
@@ -1046,7 +1066,7 @@ int32_t kitrt_step(kitrt_mn *mn, double *u, double *alpha, const double *sigma_a
                              fp64 ? nullptr : mn->d_psi32);
             if (!rc && it == 0 && stage == 0) rc = stability_verdict(mn);
             if (!rc)
-                rc = launch_finish(mn, T, mn->st, C, alpha, fp64 ? mn->d_psi : nullptr, nullptr,
+                rc = launch_finish(mn, T, mn->st, C, alpha, fp64 ? mn->d_psi : nullptr,
                                    polish_of(mn), it > 0 || stage > 0, s);
             if (!rc) rc = launch_recon(mn, T, psi, mn->d_psif, !fp64, mn->p.bc, s);
             if (!rc)
@@ -1067,7 +1087,7 @@ int32_t kitrt_step(kitrt_mn *mn, double *u, double *alpha, const double *sigma_a
         // compare_prev (skip psi when alpha is bitwise unchanged) only once alpha holds the
         // previous step's output, which is always the case after the first step of a call and for
         // a first step that continued every cell; a cold first step recomputes psi everywhere
-        rc = launch_finish(mn, T, mn->st, C, alpha, fp64 ? mn->d_psi : nullptr, nullptr,
+        rc = launch_finish(mn, T, mn->st, C, alpha, fp64 ? mn->d_psi : nullptr,
                            polish_of(mn), it > 0, s);
         if (rc) break;
         rc = launch_flux_update(mn, T, C, fp64 ? mn->d_psi : nullptr, fp64 ? nullptr : mn->d_psi32,
