@@ -26,10 +26,12 @@
 #include "kexp.cuh"
 #include "kitrt_internal.cuh"
 #include "newton_common.cuh"
+#include "quad_lane.cuh"
 
 namespace {
 
 using namespace kitrt_dev;
+using namespace kitrt_quad;
 constexpr int kWarps = 8;
 
 __global__ void objective_kernel(const double *__restrict__ u, int n, const double *__restrict__ sa,
@@ -43,134 +45,210 @@ __global__ void objective_kernel(const double *__restrict__ u, int n, const doub
     if ((threadIdx.x & 31) == 0 && part != 0.0) atomicAdd(J, part);
 }
 
-// L_cq = lambda_c . m_q at every folded point.
-__global__ void lambda_dot_m_kernel(Tables T, const double *__restrict__ lam, double *__restrict__ Lq, int C)
+// The reverse step of one cell splits into four kernels, each in the layout that its work asks for:
+//   moments and ansatz at the closed alpha   fixed-point sweep, a thread per cell (closure_fp64.cu)
+//   L_cq = lambda_c . m_q / A_c              quads: the basis factorises into azimuth and ring
+//   r_i = sum_q mu_iq psi_iq m_q             quads, as the FP64 flux (each face is outflow for exactly
+//                                            one of a direction and its opposite)
+//   H_i^-1 r_i, lambda, block gradients      8 lanes per cell, as the Newton step
+// One kernel with a warp per cell did all of it in FP64 (70 FP64 instructions a point, 38 sums
+// reduced over the warp, the factorisation with a row per lane): 59,168 cells, M_3, order 10:
+// 3.05 -> 0.66 ms per reverse step.
+
+template <int NN>
+__global__ void __launch_bounds__(kWarps * 32)
+lambda_dot_m_kernel(int Qp, QuadTab X, const double *__restrict__ lam, const double *__restrict__ area,
+                    double *__restrict__ Lq, int C)
 {
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int n = T.n, Qp = T.Qp;
-    for (int c = blockIdx.x * kWarps + wib; c < C; c += gridDim.x * kWarps) {
-        double l[KITRT_MAX_NMOM];
-        for (int a = 0; a < n; ++a) l[a] = lam[(size_t)c * n + a];
-        for (int q = lane; q < Qp; q += 32) {
-            double s = 0.0;
-            for (int a = 0; a < n; ++a) s = fma(l[a], T.Mt[a * Qp + q], s);
-            Lq[(size_t)c * Qp + q] = s;
+    constexpr int n = Dims<NN>::n;
+    extern __shared__ __align__(16) double lambda_smem[];  // [R x n] Legendre factors
+    for (int e = threadIdx.x; e < X.R * n; e += blockDim.x) lambda_smem[e] = X.ringP[e];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, cpw = 32 / X.J;
+    const QuadLane Q(X, lane);
+    for (int base = (blockIdx.x * kWarps + wib) * cpw; base < C; base += gridDim.x * kWarps * cpw) {
+        const int i = min(base + Q.ci, C - 1);
+        const bool store = Q.live && base + Q.ci < C;
+        const double inv = 1.0 / area[i];
+        double b[n];
+#pragma unroll
+        for (int a = 0; a < n; ++a) b[a] = lam[(size_t)i * n + a] * inv * X.az[Q.j * n + a];
+        double *row = Lq + (size_t)i * Qp;
+#pragma unroll 1
+        for (int r = 0; r < X.R; ++r, row += 2 * X.P) {
+            double v[4];
+            quad_evaluate<NN>(Q.axes, lambda_smem + r * n, b, v);
+            if (store) {
+                row[Q.oA1] = v[0];
+                row[Q.oA2] = v[1];
+                if (Q.hasB) {
+                    row[Q.oB1] = v[2];
+                    row[Q.oB2] = v[3];
+                }
+            }
         }
     }
 }
 
 template <int NN>
-__global__ void __launch_bounds__(kWarps * 32)
-adjoint_cell_kernel(Tables T, const int4 *__restrict__ nbr, const double *__restrict__ nrm,
-                    const double *__restrict__ area, const double *__restrict__ u,
-                    const double *__restrict__ alpha, const double *__restrict__ lam_next,
-                    const double *__restrict__ Lq, const double *__restrict__ sa,
-                    const double *__restrict__ ss, const uint8_t *__restrict__ target,
-                    const int32_t *__restrict__ block, double dt, int bc, int C,
-                    double *__restrict__ lam, double *__restrict__ gsa, double *__restrict__ gss,
-                    int32_t *__restrict__ fail)
+__global__ void __launch_bounds__(kWarps * 32, 2)
+adjoint_flux_kernel(int Qp, QuadTab X, const int4 *__restrict__ nbr, const double *__restrict__ nrm,
+                    const double *__restrict__ psi, const double *__restrict__ Lq, double dt, int bc, int C,
+                    double *__restrict__ rout)
 {
-    constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, npairs = Dims<NN>::npairs;
-    __shared__ double sH[kWarps][n * n];
-    __shared__ double sV[kWarps][n2];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int Qp = T.Qp;
-    double *H = sH[wib], *Vs = sV[wib];
-    for (int i = blockIdx.x * kWarps + wib; i < C; i += gridDim.x * kWarps) {
-        const size_t off = (size_t)i * n;
+    constexpr int n = Dims<NN>::n;
+    extern __shared__ __align__(16) double adj_smem[];
+    double *sR = adj_smem, *sT = sR + X.R * n, *sRed = sT + X.J * n;  // sRed [warp][n][32]
+    for (int e = threadIdx.x; e < X.R * n; e += blockDim.x) sR[e] = X.ring[e];
+    for (int e = threadIdx.x; e < X.J * n; e += blockDim.x) sT[e] = X.az[e];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, J = X.J, cpw = 32 / J;
+    double *red = sRed + wib * n * 32;
+    const QuadLane Q(X, lane);
+    for (int base = (blockIdx.x * kWarps + wib) * cpw; base < C; base += gridDim.x * kWarps * cpw) {
+        const int i = min(base + Q.ci, C - 1);
         const int4 nb = nbr[i];
-        const int js[3] = {nb.x, nb.y, nb.z};
-        double nx[3], ny[3];
+        const int nbf[3] = {nb.x, nb.y, nb.z};
+        const double *ps = psi + (size_t)i * Qp, *own = Lq + (size_t)i * Qp;
+        const double *outA[3], *outB[3];
+        double xA[3], xB[3];
+        unsigned firstA = 0, firstB = 0;  // bit f: the face is outflow for the pair's first direction
+        unsigned wall = 0;                // bit f: Neumann wall, whose ghost returns the cell's own psi
 #pragma unroll
         for (int f = 0; f < 3; ++f) {
-            nx[f] = nrm[6 * (size_t)i + 2 * f];
-            ny[f] = nrm[6 * (size_t)i + 2 * f + 1];
+            const double nx = nrm[6 * (size_t)i + 2 * f], ny = nrm[6 * (size_t)i + 2 * f + 1];
+            const double *row = nbf[f] >= 0 ? Lq + (size_t)nbf[f] * Qp : X.zrow;
+            if (nbf[f] < 0 && bc == 0) wall |= 1u << f;
+            const double dA = fma(nx, Q.sA, ny * Q.cA), dB = fma(nx, Q.sB, ny * Q.cB);
+            const bool fA = dA > 0.0, fB = dB > 0.0;
+            firstA |= (unsigned)fA << f;
+            firstB |= (unsigned)fB << f;
+            outA[f] = row + (fA ? Q.oA1 : Q.oA2);
+            outB[f] = row + (fB ? Q.oB1 : Q.oB2);
+            xA[f] = Q.live ? fabs(dA) : 0.0;
+            xB[f] = Q.live && Q.hasB ? fabs(dB) : 0.0;
         }
-        const double inv_Ai = 1.0 / area[i];
-        double inv_Aj[3];
+        double G[n];
 #pragma unroll
-        for (int f = 0; f < 3; ++f) inv_Aj[f] = js[f] >= 0 ? 1.0 / area[js[f]] : 0.0;
-        const double al = lane < n ? alpha[off + lane] : 0.0;
-        double av[n];
-#pragma unroll
-        for (int a = 0; a < n; ++a) av[a] = __shfl_sync(kFull, al, a);
-        double V[n2], r[n];
-#pragma unroll
-        for (int c = 0; c < n2; ++c) V[c] = 0.0;
-#pragma unroll
-        for (int a = 0; a < n; ++a) r[a] = 0.0;
-        for (int q = lane; q < Qp; q += 32) {
-            double z = 0.0;
-#pragma unroll
-            for (int a = 0; a < n; ++a) z = fma(av[a], T.Mt[a * Qp + q], z);
-            const double psi = kexp(z, T.exptab);
-            const double e = T.w[q] * psi;
-#pragma unroll
-            for (int c = 0; c < n2; ++c) V[c] = fma(e, T.Mt[c * Qp + q], V[c]);
-            const double Li = Lq[(size_t)i * Qp + q];
-            double acc = 0.0;
+        for (int a = 0; a < n; ++a) G[a] = 0.0;
+#pragma unroll 1
+        for (int r = 0; r < X.R; ++r) {
+            const int at = r * 2 * X.P;
+            const double a1 = own[at + Q.oA1], a2 = own[at + Q.oA2], b1 = own[at + Q.oB1], b2 = own[at + Q.oB2];
+            const double pa1 = ps[at + Q.oA1], pa2 = ps[at + Q.oA2], pb1 = ps[at + Q.oB1], pb2 = ps[at + Q.oB2];
+            double ap = 0.0, am = 0.0, bp = 0.0, bm = 0.0;
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
-                const double d = fma(T.wox[q], nx[f], T.woy[q] * ny[f]);  // w_q Omega_q . n_if
-                if (d > 0.0) {
-                    acc = fma(Li * inv_Ai, d, acc);
-                    if (js[f] >= 0) acc = fma(-Lq[(size_t)js[f] * Qp + q] * inv_Aj[f], d, acc);
-                } else if (js[f] < 0 && bc == 0) {
-                    acc = fma(Li * inv_Ai, d, acc);
+                const bool fA = (firstA >> f) & 1, fB = (firstB >> f) & 1;
+                const double da = (fA ? a1 : a2) - outA[f][at], db = (fB ? b1 : b2) - outB[f][at];
+                const double ca = xA[f] * (fA ? pa1 : pa2), cb = xB[f] * (fB ? pb1 : pb2);
+                ap = fma(ca, da, ap);
+                am = fma(fA ? ca : -ca, da, am);
+                bp = fma(cb, db, bp);
+                bm = fma(fB ? cb : -cb, db, bm);
+            }
+            if (wall) {
+                // the wall's inflow: the other direction of each pair
+#pragma unroll
+                for (int f = 0; f < 3; ++f) {
+                    if (!((wall >> f) & 1)) continue;
+                    const bool fA = (firstA >> f) & 1, fB = (firstB >> f) & 1;
+                    const double ta = xA[f] * (fA ? pa2 * a2 : pa1 * a1), tb = xB[f] * (fB ? pb2 * b2 : pb1 * b1);
+                    ap -= ta;
+                    am += fA ? ta : -ta;
+                    bp -= tb;
+                    bm += fB ? tb : -tb;
                 }
             }
-            const double t = -dt * acc * psi;  // mu_iq psi_iq
-#pragma unroll
-            for (int a = 0; a < n; ++a) r[a] = fma(t, T.Mt[a * Qp + q], r[a]);
-        }
-#pragma unroll
-        for (int c = 0; c < n2; ++c) V[c] = warp_sum(V[c]);
-        double ra = 0.0;
-#pragma unroll
-        for (int a = 0; a < n; ++a) {
-            const double v = warp_sum(r[a]);
-            if (lane == a) ra = v;
+            quad_project<NN>(Q.axes, ap, am, bp, bm, sR + r * n, G);
         }
         __syncwarp();
 #pragma unroll
-        for (int c = 0; c < n2; ++c)
-            if (lane == (c & 31)) Vs[c] = V[c];
+        for (int a = 0; a < n; ++a) red[a * 32 + lane] = G[a] * sT[Q.j * n + a];
         __syncwarp();
-        for (int p = lane; p < npairs; p += 32) {
-            int a = 0;
-            while ((a + 1) * (a + 2) / 2 <= p) ++a;
-            const int b = p - a * (a + 1) / 2;
-            double h = 0.0;
-            for (int t = T.gstart[p]; t < T.gstart[p + 1]; ++t) h = fma(T.gcoef[t], Vs[T.gidx[t]], h);
-            H[a * n + b] = h;
-            H[b * n + a] = h;
+        for (int e = lane; e < cpw * n; e += 32) {
+            const int cc = e / n, a = e - cc * n, ic = base + cc;
+            if (ic >= C) continue;
+            double v = 0.0;
+            for (int t = 0; t < J; ++t) v += red[a * 32 + cc * J + t];
+            rout[(size_t)ic * n + a] = -dt * v;
         }
-        __syncwarp();
-        double x = 0.0;
-        if (warp_cholesky<n>(H, lane)) {
-            x = warp_chol_solve<n>(H, ra, lane);
-        } else if (lane == 0) {
-            atomicAdd(fail, 1);
+    }
+}
+
+// lambda^s from lambda^{s+1}, and the block gradients: 8 lanes per cell, 32 cells per block and pass.
+template <int NN>
+__global__ void __launch_bounds__(kGroupBlock, 2)
+adjoint_solve_kernel(Tables T, const double *__restrict__ V, int vs, const double *__restrict__ rin,
+                     const double *__restrict__ u, const double *__restrict__ lam_next, const double *__restrict__ area,
+                     const double *__restrict__ sa, const double *__restrict__ ss, const uint8_t *__restrict__ target,
+                     const int32_t *__restrict__ block, double dt, int C, int nnz, double *__restrict__ lam,
+                     double *__restrict__ gsa, double *__restrict__ gss, int32_t *__restrict__ fail)
+{
+    constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, npairs = Dims<NN>::npairs, SL = (n + 7) / 8;
+    extern __shared__ __align__(16) double solve_smem[];
+    double *sV = solve_smem, *sH = sV + n2 * kGroupPitch, *coef = sH + kGroupCells * npairs;
+    int32_t *gstart = reinterpret_cast<int32_t *>(coef + nnz);
+    unsigned char *gidx = reinterpret_cast<unsigned char *>(gstart + npairs + 1);
+    const int tid = threadIdx.x, lane = tid & 31, g = lane & 7, slot = tid >> 3;
+    for (int t = tid; t < nnz; t += kGroupBlock) {
+        gidx[t] = (unsigned char)T.gidx[t];
+        coef[t] = T.gcoef[t];
+    }
+    for (int t = tid; t <= npairs; t += kGroupBlock) gstart[t] = T.gstart[t];
+    for (int base = blockIdx.x * kGroupCells; base < C; base += gridDim.x * kGroupCells) {
+        __syncthreads();
+        for (int e = tid; e < n2 * kGroupCells; e += kGroupBlock) {
+            const int c = e / kGroupCells, j = e % kGroupCells;
+            sV[c * kGroupPitch + j] = V[(size_t)c * vs + min(base + j, C - 1)];
         }
-        __syncwarp();
-        const double li = lane < n ? lam_next[off + lane] : 0.0;
-        const double l0 = __shfl_sync(kFull, li, 0);
-        const double ua = lane < n ? u[off + lane] : 0.0;
-        const double u0 = __shfl_sync(kFull, ua, 0);
+        __syncthreads();
+        const bool valid = base + slot < C;
+        const int i = min(base + slot, C - 1);
+        const size_t off = (size_t)i * n;
+        double x[SL], li[SL], ua[SL];
+#pragma unroll
+        for (int s = 0; s < SL; ++s) {
+            const int c = g + 8 * s;
+            x[s] = c < n ? rin[off + c] : 0.0;
+            li[s] = c < n ? lam_next[off + c] : 0.0;
+            ua[s] = c < n ? u[off + c] : 0.0;
+        }
+        const bool spd = group_factor_solve<NN, double>(coef, gidx, gstart, sV + slot, sH + slot * npairs, 0.0, n, g, x);
+        const double l0 = __shfl_sync(kFull, li[0], 0, 8), u0 = __shfl_sync(kFull, ua[0], 0, 8);
         const double sai = sa[i], ssi = ss[i];
         const bool tgt = target[i] != 0;
-        if (lane < n) {
-            double v = li + dt * (-(sai + ssi) * li + (lane == 0 ? ssi * l0 : 0.0)) + x;
-            if (lane == 0 && tgt) v += dt * area[i] * sai / T.m0;
-            lam[off + lane] = v;
+        double lu = 0.0, lus = 0.0;
+#pragma unroll
+        for (int s = 0; s < SL; ++s) {
+            const int c = g + 8 * s;
+            lu = fma(li[s], ua[s], lu);
+            if (c > 0) lus = fma(li[s], ua[s], lus);
+            if (valid && c < n) {
+                double v = li[s] + dt * (-(sai + ssi) * li[s] + (c == 0 ? ssi * l0 : 0.0)) + (spd ? x[s] : 0.0);
+                if (c == 0 && tgt) v += dt * area[i] * sai / T.m0;
+                lam[off + c] = v;
+            }
         }
-        const double lu = warp_sum(li * ua);
-        const double lus = warp_sum(li * (ua - (lane == 0 ? u0 : 0.0)));
-        if (lane == 0) {
-            const int b = block[i];
-            atomicAdd(&gsa[b], -dt * lu + (tgt ? dt * area[i] * u0 / T.m0 : 0.0));
-            atomicAdd(&gss[b], -dt * lus);
+        lu = group_sum(lu);
+        lus = group_sum(lus);
+        double da = -dt * lu + (tgt ? dt * area[i] * u0 / T.m0 : 0.0), ds = -dt * lus;
+        if (!valid) da = ds = 0.0;
+        if (g == 0 && valid && !spd) atomicAdd(fail, 1);
+        // the warp's four cells mostly lie in one block: one atomic then
+        const int blk = block[i];
+        const bool one = __all_sync(kFull, blk == __shfl_sync(kFull, blk, 0));
+        if (one) {
+            da += __shfl_xor_sync(kFull, da, 8);
+            ds += __shfl_xor_sync(kFull, ds, 8);
+            da += __shfl_xor_sync(kFull, da, 16);
+            ds += __shfl_xor_sync(kFull, ds, 16);
         }
+        if (one ? lane == 0 : g == 0) {
+            atomicAdd(&gsa[blk], da);
+            atomicAdd(&gss[blk], ds);
+        }
+        __syncwarp();
     }
 }
 
@@ -208,6 +286,7 @@ extern "C" int32_t kitrt_adjoint(kitrt_mn *mn, const double *u0, const double *a
                             sizeof(double) * Cn, sizeof(double) * Cn,   // u, a
                             sizeof(double) * Cn, sizeof(double) * Cn,   // lam, lam2
                             sizeof(double) * (size_t)C * Qp,            // Lq
+                            sizeof(double) * Cn,                        // r
                             sizeof(double) * (1 + 2 * (size_t)nblocks), // J, dJ_dsa, dJ_dss
                             sizeof(int32_t)};                           // fail
     constexpr int kBufs = sizeof(sizes) / sizeof(sizes[0]);
@@ -236,9 +315,10 @@ extern "C" int32_t kitrt_adjoint(kitrt_mn *mn, const double *u0, const double *a
     double *lam = (double *)(base + offs[6]);
     double *lam2 = (double *)(base + offs[7]);
     double *Lq = (double *)(base + offs[8]);
-    double *dJ = (double *)(base + offs[9]);  // J, then dJ/dsigma_a, then dJ/dsigma_s
+    double *r = (double *)(base + offs[9]);
+    double *dJ = (double *)(base + offs[10]);  // J, then dJ/dsigma_a, then dJ/dsigma_s
     double *dJ_sa = dJ + 1, *dJ_ss = dJ + 1 + nblocks;
-    int32_t *fail = (int32_t *)(base + offs[10]);
+    int32_t *fail = (int32_t *)(base + offs[11]);
     auto cleanup = [](int rc) { return rc; };
     int rc0 = check_stability(mn, sigma_a, sigma_s, dt, s, true);
     if (rc0) return rc0;
@@ -246,7 +326,12 @@ extern "C" int32_t kitrt_adjoint(kitrt_mn *mn, const double *u0, const double *a
     const kitrt_mesh *m = mn->mesh;
     const double inv_m0 = 1.0 / T.m0;
     const int tb = (C + 255) / 256 < mn->nsm * 8 ? (C + 255) / 256 : mn->nsm * 8;
-    const int wb = (C + kWarps - 1) / kWarps < mn->nsm * 8 ? (C + kWarps - 1) / kWarps : mn->nsm * 8;
+    const QuadTab X = quad_tab(mn);
+    const int per_block = kWarps * (32 / mn->J), qb = std::min((C + per_block - 1) / per_block, mn->nsm * 2);
+    const int lb = std::min((C + per_block - 1) / per_block, mn->nsm * 8);
+    const int sb = std::min((C + kGroupCells - 1) / kGroupCells, mn->nsm * 2);
+    const size_t smem_l = sizeof(double) * mn->R * n, smem_f = sizeof(double) * n * ((size_t)mn->R + mn->J + kWarps * 32);
+    const size_t smem_s = group_smem_bytes(mn->n2, mn->npairs, mn->gaunt_nnz, false);
 #define CK(x)                                          \
     do {                                               \
         if ((x) != cudaSuccess) return cleanup(KITRT_ECUDA); \
@@ -282,15 +367,21 @@ extern "C" int32_t kitrt_adjoint(kitrt_mn *mn, const double *u0, const double *a
             CK(cudaMemcpyAsync(seg_a + Cn * (st - s0), a, sizeof(double) * Cn, cudaMemcpyDeviceToDevice, s));
         }
         for (int st = s1 - 1; st >= s0; --st) {
+            const double *us = seg_u + Cn * (st - s0), *as = seg_a + Cn * (st - s0);
+            const int rc = launch_adjoint_closure(mn, T, C, us, as, mn->d_Vacc, mn->vs, mn->d_psi, s);
+            if (rc) return cleanup(rc);
             LaunchScope ls(mn, PK_ADJOINT, s, C);
-            lambda_dot_m_kernel<<<wb, kWarps * 32, 0, s>>>(T, lam, Lq, C);
-#define ADJ_CASE(NNv)                                                                                       \
-    case NNv:                                                                                               \
-        adjoint_cell_kernel<NNv><<<wb, kWarps * 32, 0, s>>>(T, m->d_nbr, m->d_nrm, m->d_area,               \
-                                                            seg_u + Cn * (st - s0), seg_a + Cn * (st - s0), \
-                                                            lam, Lq, sigma_a, sigma_s, target,              \
-                                                            block_of_cell, dt, mn->p.bc, C, lam2, dJ_sa,    \
-                                                            dJ_ss, fail);                                   \
+            mn->launch_count += 2;  // three kernels in this scope
+#define ADJ_CASE(NNv)                                                                                          \
+    case NNv:                                                                                                  \
+        if (ensure_dyn_smem(adjoint_flux_kernel<NNv>, smem_f) || ensure_dyn_smem(adjoint_solve_kernel<NNv>, smem_s)) \
+            return cleanup(KITRT_ECUDA);                                                                       \
+        lambda_dot_m_kernel<NNv><<<lb, kWarps * 32, smem_l, s>>>(Qp, X, lam, m->d_area, Lq, C);                \
+        adjoint_flux_kernel<NNv><<<qb, kWarps * 32, smem_f, s>>>(Qp, X, m->d_nbr, m->d_nrm, mn->d_psi, Lq, dt, \
+                                                                 mn->p.bc, C, r);                              \
+        adjoint_solve_kernel<NNv><<<sb, kGroupBlock, smem_s, s>>>(T, mn->d_Vacc, mn->vs, r, us, lam, m->d_area, \
+                                                                  sigma_a, sigma_s, target, block_of_cell, dt, \
+                                                                  C, mn->gaunt_nnz, lam2, dJ_sa, dJ_ss, fail); \
         break;
             switch (mn->N) {
                 ADJ_CASE(1)

@@ -316,6 +316,13 @@ eval_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, Newton
 // ---------------------------------------------------------------------------------------------
 constexpr int kSweepThreads = 128;
 
+// An exponential of the sweeps as a double: the range test that fx_double leaves out (rows of the
+// FP64 exponentials reach 0 and, when not finite, y = 2^61 with a large m).
+__device__ __forceinline__ double fx_psi(const Exp &e) 
+{
+    return e.m < -1022 ? 0.0 : e.m > 1023 ? __longlong_as_double(0x7ff0000000000000LL) : kitrt_fx::fx_double(e);
+}
+
 // Dynamic shared memory of sweep64_kernel: the exp table, the moments [n2][thread] and the trial
 // alpha's limbs [n][thread], the azimuthal factors.
 size_t sweep64_smem(int n, int n2, int N, int J)
@@ -323,10 +330,12 @@ size_t sweep64_smem(int n, int n2, int N, int J)
     return 2048 * 8 + (size_t)(n2 + n) * kSweepThreads * 8 + (size_t)J * 4 * N * 8;
 }
 
-template <int NN>
+// GIVEN: every cell at the given alpha instead of the listed cells at their trial points (one part),
+// and the FP64 ansatz of every point into psi (the adjoint's reverse step).
+template <int NN, bool GIVEN>
 __global__ void __launch_bounds__(kSweepThreads)
 sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, double *__restrict__ Vacc, int vs,
-               int target_items)
+               int target_items, const double *__restrict__ alpha, double *__restrict__ psi, int C)
 {
     constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, L2 = 2 * NN;
     extern __shared__ __align__(16) unsigned char sweep_smem[];
@@ -334,11 +343,11 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
     long long *sV = (long long *)(tab + 2048);
     int2 *sA = (int2 *)(sV + n2 * kSweepThreads);
     int2 *trig = sA + n * kSweepThreads;
-    const int32_t *list_in = S.list[k & 1];
-    const int cnt_in = S.cnt[k % 3];
-    if (blockIdx.x == 0 && threadIdx.x == 0) S.cnt[(k + 2) % 3] = 0;
+    const int32_t *list_in = GIVEN ? nullptr : S.list[k & 1];
+    const int cnt_in = GIVEN ? C : S.cnt[k % 3];
+    if (!GIVEN && blockIdx.x == 0 && threadIdx.x == 0) S.cnt[(k + 2) % 3] = 0;
     const int nunits = T.Qs / 32;
-    const SweepSplit sp = sweep_split(cnt_in, gridDim.x, target_items, nunits);
+    const SweepSplit sp = sweep_split(cnt_in, gridDim.x, GIVEN ? 0 : target_items, nunits);
     const int items = sp.tiles * sp.parts;
     if ((int)blockIdx.x >= items) return;
     for (int j = threadIdx.x; j < 2048; j += kSweepThreads) tab[j] = T.fx_exp[j];
@@ -353,9 +362,9 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
         const int q_begin = part * nunits / sp.parts * 8;
         // padding quads add nothing: stop at the last real one
         const int q_end = min(T.nquad, (part + 1) * nunits / sp.parts * 8);
-        const int cell = list_in[slot];
-        const double *al = S.alpha + (size_t)cell * n, *di = S.dir + (size_t)cell * n;
-        const double lam = S.phase[cell] == PH_NEWTON ? S.lam[cell] : 0.0;
+        const int cell = GIVEN ? slot : list_in[slot];
+        const double *al = (GIVEN ? alpha : S.alpha) + (size_t)cell * n, *di = GIVEN ? al : S.dir + (size_t)cell * n;
+        const double lam = !GIVEN && S.phase[cell] == PH_NEWTON ? S.lam[cell] : 0.0;
         float bound = 0.0f;
 #pragma unroll
         for (int a = 0; a < n; ++a) {
@@ -397,6 +406,11 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
                 for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_exp(s[t], tab);
             } else {
                 bad = !fx_slow_quad<NN>(T.Mt, T.Qp, T.exptab, al, di, lam, pa, pb, e) || bad;
+            }
+            if (GIVEN) {
+                double *row = psi + (size_t)cell * T.Qp;
+                *(double2 *)(row + 2 * pa) = make_double2(fx_psi(e[0]), fx_psi(e[1]));
+                if (pb >= 0) *(double2 *)(row + 2 * pb) = make_double2(fx_psi(e[2]), fx_psi(e[3]));
             }
             if (pb < 0) e[2] = e[3] = Exp{0, -100000};
             fx_accumulate<L2>(e, tr, L2, jq == 0, pb < 0, qd == q_begin, B, [&](int d) {
@@ -781,8 +795,8 @@ int fp64_sweep_grid(const kitrt_mn *mn)
     int resident = 1;
 #define GRID_CASE(NNv)                                                              \
     case NNv:                                                                       \
-        if (ensure_dyn_smem(sweep64_kernel<NNv>, smem)) return mn->nsm;             \
-        resident = resident_ctas(sweep64_kernel<NNv>, kSweepThreads, smem, 8);      \
+        if (ensure_dyn_smem(sweep64_kernel<NNv, false>, smem)) return mn->nsm;             \
+        resident = resident_ctas(sweep64_kernel<NNv, false>, kSweepThreads, smem, 8);      \
         break;
     switch (mn->N) {
         GRID_CASE(1)
@@ -811,10 +825,26 @@ int launch_eval_fp64(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
     } else {
         const size_t smem = sweep64_smem(mn->n, mn->n2, mn->N, mn->J);
         int rc = KITRT_OK;
-        KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(sweep64_kernel<NN>, smem));
+        KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(sweep64_kernel<NN, false>, smem));
         if (rc) return rc;
-        KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN><<<mn->grid_fp64, kSweepThreads, smem, s>>>(T, S, u, k, Vacc, mn->vs, mn->target_fp64)));
+        KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN, false><<<mn->grid_fp64, kSweepThreads, smem, s>>>(T, S, u, k, Vacc, mn->vs, mn->target_fp64, nullptr, nullptr, 0)));
     }
+    return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
+}
+
+// Degree-2N moments (columns of V, stride vs) and FP64 ansatz of every cell at the given alphas, whose
+// zeroth moments are about u's.
+int launch_adjoint_closure(kitrt_mn *mn, const Tables &T, int C, const double *u, const double *alpha, double *V,
+                           int vs, double *psi, cudaStream_t s)
+{
+    const size_t smem = sweep64_smem(mn->n, mn->n2, mn->N, mn->J);
+    const int tiles = (C + kSweepThreads - 1) / kSweepThreads;
+    const NewtonState S{};
+    int rc = KITRT_OK;
+    KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(sweep64_kernel<NN, true>, smem));
+    if (rc) return rc;
+    LaunchScope ls(mn, PK_ADJOINT, s, C);
+    KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN, true><<<std::min(tiles, mn->grid_fp64), kSweepThreads, smem, s>>>(T, S, u, 0, V, vs, 0, alpha, psi, C)));
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }
 

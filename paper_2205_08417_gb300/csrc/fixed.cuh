@@ -10,7 +10,7 @@
 //   exponent s = (alpha . m) 2048 / ln2 in units of 2^-42 (2^-53.5 of alpha . m), |s| < 2^61.5: rows
 //   with sum_c |alpha_c| max|m_c| >= kFxMaxZ take their exponentials from the FP64 kexp instead;
 //   azimuthal factors cos(k phi), sin(k phi) in units of 2^-54, the weighted Legendre factors of
-//   the moments in units of 2^-54 of a power of two, the exponent's in units of 2^-41;
+//   the moments in units of 2^-57 of a power of two, the exponent's in units of 2^-45;
 //   exponential e = y 2^(m - 61), y in [2^61, 2^62]: T_j (1 + p) with the 2048-entry table and
 //   p = exp(r ln2/2048) - 1 on r in [0, 1) by a cubic whose quartic term is folded in (error below
 //   2^-57); |error| of y below 2^-51 relative;
@@ -94,12 +94,12 @@ struct SumAcc {
     KITRT_FX void scale_down(int n) { hh = sar(hh, n), m = sar(m, n); }
 };
 
-// One term B w P of a moment: B an azimuthal sum (below 2^61), wP in units of 2^-54 (27-bit limbs),
+// One term B w P of a moment: B an azimuthal sum (below 2^61, split<32>), wP in units of 2^-57 (split<27>),
 // in units of 2^sh of B (0 <= sh <= 4).
 KITRT_FX long long moment_term(Limb b, int2 wp, int sh)
 {
-    return (wide(b.h, wp.x) << (5 - sh)) + ((wide(b.h, wp.y) + (1LL << (21 + sh))) >> (22 + sh)) +
-           ((wide(b.l, wp.x) + (wide(b.l, wp.y) >> 27) + (1LL << (26 + sh))) >> (27 + sh));
+    return ((wide(b.h, wp.x) << 2) >> sh) + ((wide(b.h, wp.y) + (1LL << (24 + sh))) >> (25 + sh)) +
+           ((wide(b.l, wp.x) + (wide(b.l, wp.y) >> 27) + (1LL << (29 + sh))) >> (30 + sh));
 }
 
 // A double as an integer in units of 2^-52, rounded (|x| < 2048).
@@ -143,9 +143,9 @@ KITRT_FX double fx_to_double(long long v, int e)
 }
 
 // Sums of products alpha_c P_c of one exponent coefficient A_k: alpha_c in units of 2^-52 (split<32>),
-// P_c in units of 2^-41 (27-bit limbs).
+// P_c in units of 2^-45 (split<27>).
 struct CoefAcc {
-    long long hh = 0, hl = 1LL << 18, lh = 1LL << 23, ll = 0;
+    long long hh = 0, hl = 1LL << 22, lh = 1LL << 27, ll = 0;
     KITRT_FX void add(Limb a, int2 p)
     {
         hh += wide(a.h, p.x);
@@ -154,7 +154,7 @@ struct CoefAcc {
         ll += wide(a.l, p.y);
     }
     // in units of 2^-42
-    KITRT_FX long long value() const { return (hh << 8) + (hl >> 19) + (lh >> 24) + (ll >> 51); }
+    KITRT_FX long long value() const { return (hh << 4) + (hl >> 23) + (lh >> 28) + (ll >> 55); }
 };
 
 // An exponential as (y, m): e = y 2^(m - 61).

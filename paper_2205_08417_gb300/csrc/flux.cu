@@ -14,10 +14,12 @@
 
 #include "flux_group.cuh"
 #include "kitrt_internal.cuh"
+#include "quad_lane.cuh"
 
 namespace {
 
 using namespace kitrt_flux;
+using namespace kitrt_quad;
 constexpr int kWarps = 8;
 
 // FP64 flux (FP64 mode). The FP64 pipe is the bound (a warp-wide FP64 instruction holds it for 16
@@ -35,17 +37,9 @@ constexpr int kWarps = 8;
 // at 16 cycles for each of the 347 warp instructions of three cells.
 // RHO: the transformed CSD equation's density (Sec. 2, Eq. BoltzmannCSDTrafo): the transported
 // value is psi / rho, so each row is scaled by its cell's 1/rho (invrho) before differencing.
-struct Flux64Tab {
-    const double *ring;  // [R x n] w_r sin(theta_r) P_c(mu_r)
-    const double *az;    // [J x n] azimuthal factors T_c of each quad, with the signs of the axes' quad
-    const double *sc;    // [J x 2] sin, cos of phi_j
-    const double *zrow;  // [Qp] zeros: the vacuum ghost's row
-    int R, P, J;
-};
-
 template <int NN, bool RHO>
 __global__ void __launch_bounds__(kWarps * 32, 2)
-flux64_kernel(Tables T, Flux64Tab X, const int4 *__restrict__ nbr, const double *__restrict__ nrm,
+flux64_kernel(Tables T, QuadTab X, const int4 *__restrict__ nbr, const double *__restrict__ nrm,
               const double *__restrict__ area, const double *__restrict__ psi,
               const double *__restrict__ invrho, double *__restrict__ u,
               const double *__restrict__ sa, const double *__restrict__ ss,
@@ -61,18 +55,9 @@ flux64_kernel(Tables T, Flux64Tab X, const int4 *__restrict__ nbr, const double 
     const int J = X.J, P = X.P, cpw = 32 / J;  // cells per warp
     const int Qp = T.Qp;
     double *red = sRed + wib * n * 32;
-    const bool live = lane < cpw * J;
-    const int ci = live ? lane / J : cpw - 1, j = live ? lane - ci * J : 0;
-    const bool axes = j == 0;
-    // the pairs A = (phi, pi + phi) and B = (-phi, pi - phi) of the lane's quad, or (0, pi) and
-    // (pi/2, 3 pi/2): places in the ring, and sin, cos of each pair's first direction
-    const int oA1 = axes ? 0 : 2 * j, oA2 = axes ? 1 : 2 * (P - j) + 1;
-    const bool hasB = !axes || (P & 1) == 0;
-    const int oB1 = axes ? (hasB ? P : 0) : 2 * j + 1, oB2 = axes ? (hasB ? P + 1 : 0) : 2 * (P - j);
-    const double sphi = X.sc[2 * j], cphi = X.sc[2 * j + 1];
-    const double sB = axes ? 1.0 : -sphi, cB = axes ? 0.0 : cphi;
+    const QuadLane Q(X, lane);
     for (int base = (blockIdx.x * kWarps + wib) * cpw; base < C; base += gridDim.x * kWarps * cpw) {
-        const int i = min(base + ci, C - 1);
+        const int i = min(base + Q.ci, C - 1);
         const int4 nb = nbr[i];
         const int nbf[3] = {nb.x, nb.y, nb.z};
         const double *own = psi + (size_t)i * Qp;
@@ -87,14 +72,14 @@ flux64_kernel(Tables T, Flux64Tab X, const int4 *__restrict__ nbr, const double 
             // fluctuation exactly 0) or zeros (vacuum: fluctuation -psi_i)
             const double *row = nbf[f] >= 0 ? psi + (size_t)nbf[f] * Qp : bc == 0 ? own : X.zrow;
             g[f] = RHO && nbf[f] >= 0 ? invrho[nbf[f]] : ri;
-            const double dA = fma(nx, sphi, ny * cphi), dB = fma(nx, sB, ny * cB);
+            const double dA = fma(nx, Q.sA, ny * Q.cA), dB = fma(nx, Q.sB, ny * Q.cB);
             const bool fA = __double2hiint(dA) < 0, fB = __double2hiint(dB) < 0;
             firstA |= (unsigned)fA << f;
             firstB |= (unsigned)fB << f;
-            upA[f] = row + (fA ? oA1 : oA2);
-            upB[f] = row + (fB ? oB1 : oB2);
-            cA[f] = live ? -fabs(dA) : 0.0;
-            cB3[f] = live && hasB ? -fabs(dB) : 0.0;
+            upA[f] = row + (fA ? Q.oA1 : Q.oA2);
+            upB[f] = row + (fB ? Q.oB1 : Q.oB2);
+            cA[f] = Q.live ? -fabs(dA) : 0.0;
+            cB3[f] = Q.live && Q.hasB ? -fabs(dB) : 0.0;
         }
         double G[n];
 #pragma unroll
@@ -102,7 +87,7 @@ flux64_kernel(Tables T, Flux64Tab X, const int4 *__restrict__ nbr, const double 
 #pragma unroll 1
         for (int r = 0; r < X.R; ++r) {
             const int at = r * 2 * P;
-            double a1 = own[at + oA1], a2 = own[at + oA2], b1 = own[at + oB1], b2 = own[at + oB2];
+            double a1 = own[at + Q.oA1], a2 = own[at + Q.oA2], b1 = own[at + Q.oB1], b2 = own[at + Q.oB2];
             double wA[3], wB[3];
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
@@ -128,23 +113,11 @@ flux64_kernel(Tables T, Flux64Tab X, const int4 *__restrict__ nbr, const double 
                 bp = f ? fma(cB3[f], db, bp) : cB3[f] * db;
                 bm = f ? fma(fB ? cB3[f] : -cB3[f], db, bm) : (fB ? bp : -bp);
             }
-            // the combinations that the cosines and sines of even and odd k take
-            const double all = ap + bp, even2 = ap - bp;
-            const double v2 = axes ? even2 : all;  // cos, k = 2 mod 4
-            const double oc = axes ? am : am + bm, os = axes ? bm : am - bm;
-            const double *w = sR + r * n;
-#pragma unroll
-            for (int l = 0; l <= NN; ++l)
-#pragma unroll
-                for (int k = -l; k <= l; k += 2) {
-                    const int a = l * (l + 1) / 2 + (k + l) / 2;
-                    const double v = k >= 0 ? (k & 1 ? oc : k & 2 ? v2 : all) : (k & 1 ? os : even2);
-                    G[a] = fma(w[a], v, G[a]);
-                }
+            quad_project<NN>(Q.axes, ap, am, bp, bm, sR + r * n, G);
         }
         __syncwarp();
 #pragma unroll
-        for (int a = 0; a < n; ++a) red[a * 32 + lane] = G[a] * sT[j * n + a];
+        for (int a = 0; a < n; ++a) red[a * 32 + lane] = G[a] * sT[Q.j * n + a];
         __syncwarp();
         for (int e = lane; e < cpw * n; e += 32) {
             const int cc = e / n, a = e - cc * n, ic = base + cc;
@@ -287,7 +260,7 @@ int launch_flux_update(kitrt_mn *mn, const Tables &T, int C, const double *psi,
                        const double *q, double dt, int bc, cudaStream_t s)
 {
     const kitrt_mesh *m = mn->mesh;
-    const Flux64Tab X{mn->d_flux_ring, mn->d_flux_az, mn->d_flux_sc, mn->d_zero64, mn->R, mn->P, mn->J};
+    const QuadTab X = quad_tab(mn);
     const int per_block = kWarps * (32 / mn->J), need = (C + per_block - 1) / per_block;
     const int grid = need < mn->nsm * 2 ? (need > 0 ? need : 1) : mn->nsm * 2;
     const size_t smem64 = sizeof(double) * mn->n * ((size_t)mn->R + mn->J + kWarps * 32);

@@ -696,17 +696,19 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
             for (int cc = 0; cc < n2; ++cc) {
                 const long double p = P[(size_t)rg * n2 + cc];
                 if (cc < n) {
-                    ringA[(size_t)rg * n + cc] = limbs(p * scale, 41);
+                    ringA[(size_t)rg * n + cc] = limbs(p * scale, 45);
                     mmax[cc] = std::max(mmax[cc], (float)fabs((double)p) * 1.0001f);
                 }
-                ringW[(size_t)rg * n2 + cc] = limbs(ldexpl(r.ring_w[rg] * p, -mn->fx_wexp), 54);
+                ringW[(size_t)rg * n2 + cc] = limbs(ldexpl(r.ring_w[rg] * p, -mn->fx_wexp), 57);
             }
         // the quads' tables of the FP64 flux: the axes' quad (j = 0: 0, pi, pi/2, 3 pi/2) takes
         // cos = 1 and the sign of sin(k pi/2) for odd k, 0 for even k
-        std::vector<double> fr((size_t)mn->R * n), fa((size_t)mn->J * n), fsc((size_t)mn->J * 2);
+        std::vector<double> fr((size_t)mn->R * n), frP((size_t)mn->R * n), fa((size_t)mn->J * n), fsc((size_t)mn->J * 2);
         for (int rg = 0; rg < mn->R; ++rg)
-            for (int cc = 0; cc < n; ++cc)
+            for (int cc = 0; cc < n; ++cc) {
+                frP[(size_t)rg * n + cc] = P[(size_t)rg * n2 + cc];
                 fr[(size_t)rg * n + cc] = r.ring_w[rg] * sqrt(1.0 - r.ring_mu[rg] * r.ring_mu[rg]) * P[(size_t)rg * n2 + cc];
+            }
         for (int j = 0; j < mn->J; ++j) {
             const double phi = j * (2.0 * kPi / r.nphi);
             fsc[2 * j] = j ? sin(phi) : 0.0;
@@ -718,6 +720,7 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
                                                : (k >= 0 ? 1.0 : k & 1 ? ((-k) & 2 ? -1.0 : 1.0) : 0.0);
         }
         TRY(dev_upload(mn, &mn->d_flux_ring, fr));
+        TRY(dev_upload(mn, &mn->d_flux_ringP, frP));
         TRY(dev_upload(mn, &mn->d_flux_az, fa));
         TRY(dev_upload(mn, &mn->d_flux_sc, fsc));
         TRY(dev_upload(mn, &mn->d_zero64, std::vector<double>(Qp, 0.0)));

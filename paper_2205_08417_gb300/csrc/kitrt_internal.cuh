@@ -144,8 +144,8 @@ struct kitrt_mn {
     float *d_fx_mmax = nullptr;
     int fx_wexp = 0;
     double *d_exptab = nullptr;          // [2048] exp table (Tables::exptab)
-    // FP64 flux and adjoint: ring, azimuth and direction tables of the quads (flux.cu), a zero row
-    double *d_flux_ring = nullptr, *d_flux_az = nullptr, *d_flux_sc = nullptr, *d_zero64 = nullptr;
+    // FP64 flux and adjoint: ring, azimuth and direction tables of the quads (quad_lane.cuh), a zero row
+    double *d_flux_ring = nullptr, *d_flux_ringP = nullptr, *d_flux_az = nullptr, *d_flux_sc = nullptr, *d_zero64 = nullptr;
     void *d_mlp16 = nullptr;             // learned closure: BF16 network parameters
     float *d_mlp_norm = nullptr;         // [4 (n-1)] feature and output means / scales
     bool has_mlp = false;
@@ -260,6 +260,8 @@ int launch_finish(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
 int launch_ansatz(const Tables &T, int C, const double *alpha, double *psi, cudaStream_t s);
 int launch_moments_fp64(kitrt_mn *mn, const Tables &T, int C, const double *alpha, double *V,
                         cudaStream_t s);
+int launch_adjoint_closure(kitrt_mn *mn, const Tables &T, int C, const double *u, const double *alpha,
+                           double *V, int vs, double *psi, cudaStream_t s);
 int launch_gaunt(kitrt_mn *mn, const Tables &T, int C, const double *V, double *H, cudaStream_t s);
 int launch_eval_mixed(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, const double *u,
                       int k, NewtonParams np, cudaStream_t s, float *psi32);
