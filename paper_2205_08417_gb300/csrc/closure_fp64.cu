@@ -13,6 +13,7 @@
 // fills.
 #include <math.h>
 
+#include "async_copy.cuh"
 #include "kitrt_internal.cuh"
 #include "kexp.cuh"
 #include "newton_common.cuh"
@@ -114,28 +115,45 @@ begin_test_kernel(NewtonState S, const double *__restrict__ u, const double *__r
 
 // One thread per listed cell: every FP64 instruction of the triangular solves keeps all 32 lanes
 // busy, and one warp per scheduler already fills the FP64 pipe (64 cycles per instruction). For
-// N <= 3 the factor is read into registers; for N >= 4 (120 or 231 entries) its rows are read in
-// order, once for the forward and once for the backward substitution (which works row by row too),
-// the vector in shared memory. There it took the place of a warp per cell: M_5, 996,872 cells,
-// 8.2 -> 7.0 ms a step (bound by the rows' strided reads).
+// N <= 3 the factor is read into registers. For N >= 4 (120 or 231 entries) a block of one warp
+// copies its 32 cells' factors into shared memory (asynchronously, whole rows at a time: read by the
+// threads themselves each load touches 32 lines) and works from there, the vector in shared memory
+// too. M_5, 996,872 cells: a warp per cell took 8.2 ms a step, strided reads 7.0, this 3.4 (with the test that precedes it).
 template <int NN>
-__global__ void __launch_bounds__(kThreadBlock)
-predict_thread_kernel(NewtonState S, const double *__restrict__ u, NewtonParams np)
+struct PredictDims {
+    static constexpr bool in_regs = NN <= 3;
+    static constexpr int threads = in_regs ? kThreadBlock : 32;
+    static constexpr int pitch = Dims<NN>::npairs | 1;  // odd: a column of 32 rows is free of conflicts
+    static constexpr size_t smem = in_regs ? 0 : sizeof(double) * 32 * (pitch + Dims<NN>::n);
+};
+
+template <int NN>
+__global__ void __launch_bounds__(PredictDims<NN>::threads)
+predict_kernel(NewtonState S, const double *__restrict__ u, NewtonParams np)
 {
+    using D = PredictDims<NN>;
     constexpr int n = Dims<NN>::n, npairs = Dims<NN>::npairs;
-    constexpr bool in_regs = NN <= 3;
-    __shared__ double sy[in_regs ? 1 : n][kThreadBlock];
+    extern __shared__ __align__(16) double predict_smem[];  // [32][pitch] factors, [n][32] vectors
     const int cnt = S.cnt[8];
     const int stride = gridDim.x * blockDim.x;
     const int rounds = (cnt + stride - 1) / stride;
     for (int rd = 0; rd < rounds; ++rd) {
         const int it = rd * stride + blockIdx.x * blockDim.x + threadIdx.x;
         bool cont = false;
-        int cell = -1;
+        int cell = it < cnt ? S.list[1][it] : -1;
+        if constexpr (!D::in_regs) {
+            __syncwarp();
+            for (int r = 0; r < 32; ++r) {
+                const int c = __shfl_sync(kFull, cell, r);
+                if (c < 0) break;
+                const double *row = S.L + (size_t)c * npairs;
+                for (int p = threadIdx.x; p < npairs; p += 32) kitrt_async::cp_async8(predict_smem + r * D::pitch + p, row + p);
+            }
+            kitrt_async::cp_async_wait_all();
+            __syncwarp();
+        }
         if (it < cnt) {
-            cell = S.list[1][it];
             const size_t off = (size_t)cell * n;
-            const double *L = S.L + (size_t)cell * npairs;
             double gn2 = 0.0, un2 = 0.0, au = 0.0, ar2 = 0.0, gd = 0.0;
             auto gradient = [&](int a) {
                 const double ua = u[off + a], al = S.alpha[off + a];
@@ -150,7 +168,8 @@ predict_thread_kernel(NewtonState S, const double *__restrict__ u, NewtonParams 
                 return g;
             };
             // d = -H^-1 g with the stored factor (1/L_jj on its diagonal)
-            if constexpr (in_regs) {
+            if constexpr (D::in_regs) {
+                const double *L = S.L + (size_t)cell * npairs;
                 double Lp[npairs], y[n], g[n];
 #pragma unroll
                 for (int p = 0; p < npairs; ++p) Lp[p] = L[p];
@@ -179,25 +198,25 @@ predict_thread_kernel(NewtonState S, const double *__restrict__ u, NewtonParams 
                     gd = fma(g[a], y[a], gd);
                 }
             } else {
-                double *y = &sy[0][threadIdx.x];
+                const double *L = predict_smem + threadIdx.x * D::pitch;
+                double *y = predict_smem + 32 * D::pitch + threadIdx.x;
 #pragma unroll 1
                 for (int i = 0; i < n; ++i) {
                     const double *row = L + tri_idx(i, 0);
                     double t = -gradient(i);
 #pragma unroll 4
-                    for (int k = 0; k < i; ++k) t = fma(-row[k], y[k * kThreadBlock], t);
-                    y[i * kThreadBlock] = t * row[i];
+                    for (int k = 0; k < i; ++k) t = fma(-row[k], y[k * 32], t);
+                    t *= row[i];
+                    y[i * 32] = t;
+                    gd = fma(-t, t, gd);  // g . d = -|L^-1 g|^2
                 }
-                // g . d = -|L^-1 g|^2
-#pragma unroll 1
-                for (int i = 0; i < n; ++i) gd = fma(-y[i * kThreadBlock], y[i * kThreadBlock], gd);
 #pragma unroll 1
                 for (int i = n - 1; i >= 0; --i) {
                     const double *row = L + tri_idx(i, 0);
-                    const double x = y[i * kThreadBlock] * row[i];
+                    const double x = y[i * 32] * row[i];
                     S.dir[off + i] = x;
 #pragma unroll 4
-                    for (int k = 0; k < i; ++k) y[k * kThreadBlock] = fma(-row[k], x, y[k * kThreadBlock]);
+                    for (int k = 0; k < i; ++k) y[k * 32] = fma(-row[k], x, y[k * 32]);
                 }
             }
             if (sqrt(gn2) <= np.tau * sqrt(un2)) {
@@ -220,13 +239,11 @@ predict_thread_kernel(NewtonState S, const double *__restrict__ u, NewtonParams 
 // Armijo decision, and on acceptance the Hessian, its Cholesky factor, the convergence test and
 // the next Newton direction.
 // ---------------------------------------------------------------------------------------------
-// FUSED: the warp also runs the per-cell Newton logic (used by the allocation-free closure);
-// otherwise the sweep writes the cell's moments to column `list slot` of Vacc [n2 x C] for the
-// post kernel.
-template <int NN, bool FILTER, bool FUSED>
+// One warp per listed cell, sums and Newton logic in one kernel without an accumulator: the
+// allocation-free closure.
+template <int NN>
 __global__ void __launch_bounds__(kWarps * 32)
-eval_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, NewtonParams np,
-            float *__restrict__ psi32, double *__restrict__ Vacc, int vs)
+eval_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, NewtonParams np)
 {
     constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2;
     __shared__ double sH[kWarps][n * n];
@@ -236,18 +253,13 @@ eval_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, Newton
     int32_t *list_out = S.list[(k + 1) & 1];
     const int cnt_in = S.cnt[k % 3];
     int32_t *cnt_out = &S.cnt[(k + 1) % 3];
-    // FILTER: the FP64 companion of the mixed sweep; it only takes cells flagged for an FP64
-    // Hessian and leaves the counter bookkeeping to the mixed kernel
-    if (!FILTER && blockIdx.x == 0 && threadIdx.x == 0) S.cnt[(k + 2) % 3] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) S.cnt[(k + 2) % 3] = 0;
     double *H = sH[wib];
     double *Vs = sV[wib];
     const int Qp = T.Qp;
     const double *__restrict__ Mt = T.Mt;
     const double *__restrict__ wq = T.w;
-
-    // one listed cell: its trial point, the quadrature sums, then (FUSED) the Newton logic or
-    // (otherwise) its moments into column `it` of Vacc
-    auto cell_pass = [&](int it) {
+    for (int it = blockIdx.x * kWarps + wib; it < cnt_in; it += gridDim.x * kWarps) {
         const int cell = list_in[it];
         const size_t off = (size_t)cell * n;
         const int ph = S.phase[cell];
@@ -267,22 +279,12 @@ eval_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, Newton
             double z = 0.0;
 #pragma unroll
             for (int a = 0; a < n; ++a) z = fma(atv[a], Mt[a * Qp + q], z);
-            const double ez = kexp(z, T.exptab);
-            // the ansatz of the trial point: the last accepted trial of a closure leaves the
-            // ansatz of its solution behind, so no separate pass is needed
-            if (psi32) psi32[(size_t)cell * Qp + q] = exp_to_float(ez);
-            const double e = wq[q] * ez;
+            const double e = wq[q] * kexp(z, T.exptab);
 #pragma unroll
             for (int c = 0; c < n2; ++c) V[c] = fma(e, Mt[c * Qp + q], V[c]);
         }
 #pragma unroll
         for (int c = 0; c < n2; ++c) V[c] = warp_sum(V[c]);
-        if (!FUSED) {
-#pragma unroll
-            for (int c = 0; c < n2; ++c)
-                if (lane == (c & 31)) Vacc[(size_t)c * vs + it] = V[c];
-            return;
-        }
         __syncwarp();
 #pragma unroll
         for (int c = 0; c < n2; ++c)
@@ -290,21 +292,6 @@ eval_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, Newton
         __syncwarp();
         newton_post<NN>(T, S, np, cell, ph, lam, at, ua, Vs, H, list_out, cnt_out, lane, false);
         __syncwarp();
-    };
-    if (FILTER) {
-        // the FP64 companion of the mixed sweep takes only the (rare) cells flagged for an FP64
-        // Hessian: each warp tests 32 list entries at once and evaluates the flagged ones
-        for (int b0 = (blockIdx.x * kWarps + wib) * 32; b0 < cnt_in; b0 += gridDim.x * kWarps * 32) {
-            const int e = b0 + lane;
-            unsigned m = __ballot_sync(kFull, e < cnt_in && S.h64[list_in[e]] != 0);
-            while (m) {
-                const int b = __ffs(m) - 1;
-                m &= m - 1;
-                cell_pass(b0 + b);
-            }
-        }
-    } else {
-        for (int it = blockIdx.x * kWarps + wib; it < cnt_in; it += gridDim.x * kWarps) cell_pass(it);
     }
 }
 
@@ -330,13 +317,20 @@ size_t sweep64_smem(int n, int n2, int N, int J)
     return 2048 * 8 + (size_t)(n2 + n) * kSweepThreads * 8 + (size_t)J * 4 * N * 8;
 }
 
-// GIVEN: every cell at the given alpha instead of the listed cells at their trial points (one part),
-// and the FP64 ansatz of every point into psi (the adjoint's reverse step).
-template <int NN, bool GIVEN>
+// Which cells a sweep takes, and what it writes besides the moments.
+enum class Cells {
+    kListed,   // FP64 mode: the listed cells at their trial points
+    kHanded,   // mixed modes: the cells handed over to the FP64 Hessian (positions in the list), their
+               // trial points' FP32 ansatz into psi
+    kGiven     // every cell at the given alpha (one part), its FP64 ansatz into psi (the adjoint)
+};
+
+template <int NN, Cells CELLS>
 __global__ void __launch_bounds__(kSweepThreads)
 sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, double *__restrict__ Vacc, int vs,
-               int target_items, const double *__restrict__ alpha, double *__restrict__ psi, int C)
+               int target_items, const double *__restrict__ alpha, void *__restrict__ psi, int C)
 {
+    constexpr bool GIVEN = CELLS == Cells::kGiven, HANDED = CELLS == Cells::kHanded;
     constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, L2 = 2 * NN;
     extern __shared__ __align__(16) unsigned char sweep_smem[];
     uint64_t *tab = (uint64_t *)sweep_smem;
@@ -344,8 +338,10 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
     int2 *sA = (int2 *)(sV + n2 * kSweepThreads);
     int2 *trig = sA + n * kSweepThreads;
     const int32_t *list_in = GIVEN ? nullptr : S.list[k & 1];
-    const int cnt_in = GIVEN ? C : S.cnt[k % 3];
-    if (!GIVEN && blockIdx.x == 0 && threadIdx.x == 0) S.cnt[(k + 2) % 3] = 0;
+    const int32_t *pos_in = HANDED ? S.handed[k & 1] : nullptr;
+    const int cnt_in = GIVEN ? C : HANDED ? S.cnt[12 + k % 3] : S.cnt[k % 3];
+    if (HANDED && cnt_in == 0) return;
+    if (CELLS == Cells::kListed && blockIdx.x == 0 && threadIdx.x == 0) S.cnt[(k + 2) % 3] = 0;
     const int nunits = T.Qs / 32;
     const SweepSplit sp = sweep_split(cnt_in, gridDim.x, GIVEN ? 0 : target_items, nunits);
     const int items = sp.tiles * sp.parts;
@@ -362,7 +358,7 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
         const int q_begin = part * nunits / sp.parts * 8;
         // padding quads add nothing: stop at the last real one
         const int q_end = min(T.nquad, (part + 1) * nunits / sp.parts * 8);
-        const int cell = GIVEN ? slot : list_in[slot];
+        const int cell = GIVEN ? slot : list_in[HANDED ? pos_in[slot] : slot];
         const double *al = (GIVEN ? alpha : S.alpha) + (size_t)cell * n, *di = GIVEN ? al : S.dir + (size_t)cell * n;
         const double lam = !GIVEN && S.phase[cell] == PH_NEWTON ? S.lam[cell] : 0.0;
         float bound = 0.0f;
@@ -407,8 +403,19 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
             } else {
                 bad = !fx_slow_quad<NN>(T.Mt, T.Qp, T.exptab, al, di, lam, pa, pb, e) || bad;
             }
+            if (HANDED) {
+                // ansatz of the trial point (the last accepted trial leaves the solution's)
+                if (psi) {
+                    float *row = (float *)psi + (size_t)cell * T.Qp;
+                    float f[4];
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) f[t] = __uint_as_float(kitrt_fx::fx_float_bits(e[t]));
+                    *(float2 *)(row + 2 * pa) = make_float2(f[0], f[1]);
+                    if (pb >= 0) *(float2 *)(row + 2 * pb) = make_float2(f[2], f[3]);
+                }
+            }
             if (GIVEN) {
-                double *row = psi + (size_t)cell * T.Qp;
+                double *row = (double *)psi + (size_t)cell * T.Qp;
                 *(double2 *)(row + 2 * pa) = make_double2(fx_psi(e[0]), fx_psi(e[1]));
                 if (pb >= 0) *(double2 *)(row + 2 * pb) = make_double2(fx_psi(e[2]), fx_psi(e[3]));
             }
@@ -637,12 +644,15 @@ int grid_for(const kitrt_mn *mn, int C, int per_sm)
 }
 
 template <int NN>
-void predict_launch(kitrt_mn *mn, const NewtonState &S, int C, const double *u, NewtonParams np,
-                    cudaStream_t s)
+int predict_launch(kitrt_mn *mn, const NewtonState &S, int C, const double *u, NewtonParams np,
+                   cudaStream_t s)
 {
-    int tb = (C + kThreadBlock - 1) / kThreadBlock;
+    using D = PredictDims<NN>;
+    if (ensure_dyn_smem(predict_kernel<NN>, D::smem)) return KITRT_ECUDA;
+    int tb = (C + D::threads - 1) / D::threads;
     if (tb > mn->nsm * 32) tb = mn->nsm * 32;
-    predict_thread_kernel<NN><<<tb > 0 ? tb : 1, kThreadBlock, 0, s>>>(S, u, np);
+    predict_kernel<NN><<<tb > 0 ? tb : 1, D::threads, D::smem, s>>>(S, u, np);
+    return KITRT_OK;
 }
 
 }  // namespace
@@ -736,11 +746,11 @@ int launch_post(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, cons
     if (mixed) {
         KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(post_group_kernel<NN, true>, smem));
         if (rc) return rc;
-        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, true><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, upto)));
+        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, true><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, mn->grid_fp64, mn->target_fp64, upto)));
     } else {
         KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(post_group_kernel<NN, false>, smem));
         if (rc) return rc;
-        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, false><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, upto)));
+        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, false><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, mn->grid_fp64, mn->target_fp64, upto)));
     }
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }
@@ -784,7 +794,9 @@ int launch_begin(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
     }
     if (first == 1 || learned) return KITRT_OK;
     LaunchScope ls(mn, PK_BEGIN, s, 0);
-    KITRT_DISPATCH_N(mn->N, predict_launch<NN>(mn, S, C, u, np, s));
+    int rc = KITRT_OK;
+    KITRT_DISPATCH_N(mn->N, rc = predict_launch<NN>(mn, S, C, u, np, s));
+    if (rc) return rc;
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }
 
@@ -795,8 +807,8 @@ int fp64_sweep_grid(const kitrt_mn *mn)
     int resident = 1;
 #define GRID_CASE(NNv)                                                              \
     case NNv:                                                                       \
-        if (ensure_dyn_smem(sweep64_kernel<NNv, false>, smem)) return mn->nsm;             \
-        resident = resident_ctas(sweep64_kernel<NNv, false>, kSweepThreads, smem, 8);      \
+        if (ensure_dyn_smem(sweep64_kernel<NNv, Cells::kListed>, smem)) return mn->nsm;             \
+        resident = resident_ctas(sweep64_kernel<NNv, Cells::kListed>, kSweepThreads, smem, 8);      \
         break;
     switch (mn->N) {
         GRID_CASE(1)
@@ -810,25 +822,40 @@ int fp64_sweep_grid(const kitrt_mn *mn)
     return mn->nsm * resident;
 }
 
-int launch_eval_fp64(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
-                     const double *u, int k, NewtonParams np, cudaStream_t s, bool filter,
-                     float *psi32, double *Vacc)
+int launch_eval_fp64(kitrt_mn *mn, const Tables &T, const NewtonState &S, const double *u, int k, cudaStream_t s)
+{
+    LaunchScope ls(mn, PK_EVAL, s, 0);
+    const size_t smem = sweep64_smem(mn->n, mn->n2, mn->N, mn->J);
+    int rc = KITRT_OK;
+    KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(sweep64_kernel<NN, Cells::kListed>, smem));
+    if (rc) return rc;
+    KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN, Cells::kListed><<<mn->grid_fp64, kSweepThreads, smem, s>>>(T, S, u, k, mn->d_Vacc, mn->vs, mn->target_fp64, nullptr, nullptr, 0)));
+    return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
+}
+
+// Mixed modes: the cells handed over to the FP64 Hessian in earlier rounds. They are few (often none)
+// and lie side by side in the list, so they are swept from a list of their own, split over as many
+// parts as fill the SMs, into columns of their own (a warp per flagged entry of the list took 0.3 to
+// 0.8 ms a round for a handful of M_5 cells, and 1.19 of 2.8 ms of a checkerboard step).
+int launch_eval_handed(kitrt_mn *mn, const Tables &T, const NewtonState &S, const double *u, int k, float *psi32,
+                       cudaStream_t s)
+{
+    LaunchScope ls(mn, PK_EVAL, s, 0);
+    const size_t smem = sweep64_smem(mn->n, mn->n2, mn->N, mn->J);
+    int rc = KITRT_OK;
+    KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(sweep64_kernel<NN, Cells::kHanded>, smem));
+    if (rc) return rc;
+    KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN, Cells::kHanded><<<mn->grid_fp64, kSweepThreads, smem, s>>>(T, S, u, k, mn->d_Vacc + mn->vs / 2, mn->vs, mn->target_fp64, nullptr, psi32, 0)));
+    return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
+}
+
+// The allocation-free closure's round (the caller passes a launch-only view without a mesh).
+int launch_eval_fused(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, const double *u, int k,
+                      NewtonParams np, cudaStream_t s)
 {
     const int grid = grid_for(mn, C, 4);
     LaunchScope ls(mn, PK_EVAL, s, 0);
-    if (!Vacc) {
-        // fused sweep: no accumulator (the caller may pass a launch-only view without a mesh)
-        KITRT_DISPATCH_N(mn->N, (eval_kernel<NN, false, true><<<grid, kWarps * 32, 0, s>>>(T, S, u, k, np, psi32, Vacc, 0)));
-    } else if (filter) {
-        // cells handed to the FP64 Hessian: whole sums into part 0 of their list slots
-        KITRT_DISPATCH_N(mn->N, (eval_kernel<NN, true, false><<<grid, kWarps * 32, 0, s>>>(T, S, u, k, np, psi32, Vacc, mn->vs)));
-    } else {
-        const size_t smem = sweep64_smem(mn->n, mn->n2, mn->N, mn->J);
-        int rc = KITRT_OK;
-        KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(sweep64_kernel<NN, false>, smem));
-        if (rc) return rc;
-        KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN, false><<<mn->grid_fp64, kSweepThreads, smem, s>>>(T, S, u, k, Vacc, mn->vs, mn->target_fp64, nullptr, nullptr, 0)));
-    }
+    KITRT_DISPATCH_N(mn->N, (eval_kernel<NN><<<grid, kWarps * 32, 0, s>>>(T, S, u, k, np)));
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }
 
@@ -841,10 +868,10 @@ int launch_adjoint_closure(kitrt_mn *mn, const Tables &T, int C, const double *u
     const int tiles = (C + kSweepThreads - 1) / kSweepThreads;
     const NewtonState S{};
     int rc = KITRT_OK;
-    KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(sweep64_kernel<NN, true>, smem));
+    KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(sweep64_kernel<NN, Cells::kGiven>, smem));
     if (rc) return rc;
     LaunchScope ls(mn, PK_ADJOINT, s, C);
-    KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN, true><<<std::min(tiles, mn->grid_fp64), kSweepThreads, smem, s>>>(T, S, u, 0, V, vs, 0, alpha, psi, C)));
+    KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN, Cells::kGiven><<<std::min(tiles, mn->grid_fp64), kSweepThreads, smem, s>>>(T, S, u, 0, V, vs, 0, alpha, psi, C)));
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }
 

@@ -228,7 +228,7 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
     } else {
         list_in = S.list[k & 1];
         cnt_in = S.cnt[k % 3];
-        if (blockIdx.x == 0 && tid == 0) S.cnt[(k + 2) % 3] = 0;
+        if (blockIdx.x == 0 && tid == 0) S.cnt[(k + 2) % 3] = S.cnt[12 + (k + 2) % 3] = 0;
     }
     const SweepSplit sp = sweep_split(cnt_in, gridDim.x, target_items, nchunks);
     const int ks = sp.parts;
@@ -426,11 +426,8 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
         if (*abort_flag) break;
         // partial moments of this work item into its column of the accumulator: the FP64
         // gradient moments of both halves, the tensor-core moments from TMEM (warps 0-3)
-        // A row handed to the FP64 Hessian gets its whole sums in part 0 from the FP64 sweep; its
-        // other parts are stored as zeros, so that every column the Newton kernel reads was
-        // written in this round.
+        // A row handed to the FP64 Hessian has its sums in columns of its own.
         const bool store = r < rows && (MOMENTS_ONLY || active);
-        const bool zero = !MOMENTS_ONLY && r < rows && cell >= 0 && !active && part > 0;
         double *row = Vacc + ((size_t)part * cnt_in + base + r) * vs_s;
         if (h == 0 && store) {
             const int x1 = sX[r];
@@ -453,10 +450,6 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
                     for (int i = 0; i < 16; ++i)
                         if (c0 + i < n2 - n) row[(size_t)(n + c0 + i) * vs_c] = f2d_bits(v[i]);
                 }
-            }
-            if (zero) {
-#pragma unroll
-                for (int c = 0; c < n2; ++c) row[(size_t)c * vs_c] = 0.0;
             }
         }
         tc_fence_before();

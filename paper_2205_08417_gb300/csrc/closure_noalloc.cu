@@ -142,7 +142,7 @@ extern "C" int32_t kitrt_closure_noalloc(const kitrt_mn *mn, const double *u, do
     int k = 0;
     for (;;) {
         for (int b = 0; b < batch; ++b, ++k) {
-            rc = launch_eval_fp64(&view, T, S, C, u, k, np, s);
+            rc = launch_eval_fused(&view, T, S, C, u, k, np, s);
             if (rc) return rc;
         }
         if (cudaMemcpyAsync(cnt, S.cnt, sizeof(cnt), cudaMemcpyDeviceToHost, s) != cudaSuccess)

@@ -774,6 +774,7 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
     mn->grid_fp64 = fp64_sweep_grid(mn);
     mn->target_fp64 = 2 * mn->grid_fp64;
     mn->vs = (int)C + 128 * std::max(mn->target_mixed, mn->target_fp64) + 128;
+    if (p.mode != KITRT_FP64) mn->vs *= 2;
     TRY(dev_alloc(mn, &mn->d_Vacc, (size_t)mn->vs * n2));
     if (cudaMemset(mn->d_Vacc, 0, sizeof(double) * (size_t)mn->vs * n2) != cudaSuccess) {
         kitrt_mn_destroy(mn);
@@ -792,6 +793,8 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
         }
         if (p.mode == KITRT_LEARNED) TRY(dev_alloc(mn, &mn->d_alpha_nn, C * (size_t)n));
         TRY(dev_alloc(mn, &S.h64, C));
+        TRY(dev_alloc(mn, &S.handed[0], C));
+        TRY(dev_alloc(mn, &S.handed[1], C));
         TRY(dev_alloc(mn, &S.gnorm, C));
         if (p.mode == KITRT_LEARNED) {
             TRY(dev_alloc(mn, &S.lfac, C));
@@ -933,13 +936,13 @@ static int run_closure(kitrt_mn *mn, int C, const double *u, const double *alpha
             // quadrature sweeps write each listed cell's moment columns; the Newton step then takes
             // every listed cell
             if (mn->p.mode == KITRT_FP64) {
-                rc = launch_eval_fp64(mn, T, mn->st, C, u, k, np, s, false, nullptr, mn->d_Vacc);
+                rc = launch_eval_fp64(mn, T, mn->st, u, k, s);
             } else {
                 // FP64 sweep of the cells handed over in earlier rounds (none in the first: the
                 // closure starts with every hand-over cleared), then the tensor-core sweep of the
                 // others (cells handed over now wait for the next round, so no cell is evaluated
                 // twice in one round)
-                if (k > 0) rc = launch_eval_fp64(mn, T, mn->st, C, u, k, np, s, true, psi32, mn->d_Vacc);
+                if (k > 0) rc = launch_eval_handed(mn, T, mn->st, u, k, psi32, s);
                 if (!rc) rc = launch_eval_mixed(mn, T, mn->st, C, u, k, np, s, psi32);
             }
             if (!rc) rc = launch_post(mn, T, mn->st, C, u, k, np, mn->d_Vacc, s);

@@ -84,7 +84,9 @@ struct NewtonState {
     int32_t *halv;     // [C] halvings in the current iteration
     int32_t *evals;    // [C] evaluations in this closure
     int32_t *status;   // [C]
-    int32_t *h64;      // [C] mixed modes: 1 = this cell evaluates its Hessian in FP64 (else NULL)
+    int32_t *h64;      // [C] mixed modes: non-zero = this cell evaluates its Hessian in FP64, from its
+                       //   second round on 1 + its place in handed (else NULL)
+    int32_t *handed[2];  // [C] mixed modes: list positions of those cells (ping-pong)
     double *gnorm;     // [C] mixed modes: ||g|| at the last accepted point (else NULL)
     int32_t *lfac;     // [C] learned mode: 1 once S.L holds a factor of this cell (else NULL)
     int32_t *list[2];  // active cell lists (ping-pong)
@@ -92,7 +94,8 @@ struct NewtonState {
                        //   evals, cnt[5] fallbacks, cnt[6] evaluations, cnt[7] timeout status,
                        //   cnt[8] predictor list length, cnt[9] learned-mode steps taken
                        //   from a stored factor, cnt[10] learned-mode residual passes of the
-                       //   network's proposals, cnt[11] mixed-mode hand-overs to the FP64 Hessian
+                       //   network's proposals, cnt[11] mixed-mode hand-overs to the FP64 Hessian,
+                       //   cnt[12..14] rotating counters of handed
 };
 
 struct NewtonParams {
@@ -134,8 +137,9 @@ struct kitrt_mn {
     double *d_ox = nullptr, *d_oy = nullptr;  // [Qp] folded directions (0 on padding), S_N step
     float *d_ox32 = nullptr, *d_oy32 = nullptr;
     double *d_V = nullptr;               // [C x n2] moments scratch (kitrt_hessian)
-    double *d_Vacc = nullptr;            // [n2 x vs] sweeps: partial moments per list slot and part
-    int vs = 0;                          // column stride of d_Vacc (C + room for split parts)
+    double *d_Vacc = nullptr;            // [n2 x vs] sweeps: partial moments per list slot and part; in the
+                                         // mixed modes the second half of the columns is for handed cells
+    int vs = 0;                          // column stride of d_Vacc
     int target_mixed = 0, target_fp64 = 0;  // work items the sweeps aim at per launch
     int grid_mixed = 0, grid_fp64 = 0;      // persistent grids of the sweeps
     int R = 0, P = 0, J = 0, Qs = 0;     // rings, pairs and quads per ring, points of a sweep (padded)
@@ -250,9 +254,11 @@ int launch_learned_pass(kitrt_mn *mn, const Tables &T, const NewtonState &S, int
                         float *psi32, int first, cudaStream_t s);
 int fp64_sweep_grid(const kitrt_mn *mn);
 int mixed_sweep_grid(const kitrt_mn *mn);
-int launch_eval_fp64(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
-                     const double *u, int k, NewtonParams np, cudaStream_t s,
-                     bool filter = false, float *psi32 = nullptr, double *Vacc = nullptr);
+int launch_eval_fp64(kitrt_mn *mn, const Tables &T, const NewtonState &S, const double *u, int k, cudaStream_t s);
+int launch_eval_handed(kitrt_mn *mn, const Tables &T, const NewtonState &S, const double *u, int k, float *psi32,
+                       cudaStream_t s);
+int launch_eval_fused(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, const double *u, int k,
+                      NewtonParams np, cudaStream_t s);
 int launch_post(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, const double *u, int k,
                 NewtonParams np, double *Vacc, cudaStream_t s);
 int launch_finish(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,

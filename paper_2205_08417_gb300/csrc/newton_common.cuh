@@ -229,17 +229,20 @@ __device__ void newton_post(const Tables &T, const NewtonState &S, const NewtonP
 namespace kitrt_dev {
 
 // Warp-aggregated append of `cell` to a list when pred holds (all active lanes must call it).
-__device__ __forceinline__ void push_agg(int32_t *list, int32_t *cnt, int cell, bool pred)
+// Returns the cell's position in the list.
+__device__ __forceinline__ int push_agg(int32_t *list, int32_t *cnt, int cell, bool pred)
 {
     const unsigned act = __activemask();
     const unsigned m = __ballot_sync(act, pred);
-    if (!m) return;
+    if (!m) return 0;
     const int lane = threadIdx.x & 31;
     const int leader = __ffs(m) - 1;
     int base = 0;
     if (lane == leader) base = atomicAdd(cnt, __popc(m));
     base = __shfl_sync(act, base, leader);
-    if (pred) list[base + __popc(m & ((1u << lane) - 1u))] = cell;
+    const int at = base + __popc(m & ((1u << lane) - 1u));
+    if (pred) list[at] = cell;
+    return at;
 }
 
 // Newton step of one listed cell after a round of sweeps, in the FP64 mode for N <= 3 when many
@@ -620,7 +623,8 @@ __host__ __device__ inline size_t group_smem_bytes(int n2, int npairs, int nnz, 
 template <int NN, bool MIXED>
 __global__ void __launch_bounds__(kGroupBlock, 2)
 post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, NewtonParams np,
-                  const double *__restrict__ Vacc, int vs, int nnz, int sweep_grid, int target_items, int upto)
+                  const double *__restrict__ Vacc, int vs, int nnz, int sweep_grid, int target_items, int grid64, int target64,
+                  int upto)
 {
     constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, npairs = Dims<NN>::npairs, SL = (n + 7) / 8;
     extern __shared__ __align__(16) unsigned char group_smem[];
@@ -637,6 +641,9 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
     // uniform: not this kernel's round, or no slot for this block
     if (cnt_in > upto || (int)blockIdx.x * kGroupCells >= cnt_in) return;
     const int parts = sweep_split(cnt_in, sweep_grid, target_items, T.Qs / 32).parts;
+    // handed cells: columns from vs / 2 on, split on their own
+    const int handed = MIXED ? S.cnt[12 + k % 3] : 0;
+    const int parts64 = MIXED ? sweep_split(handed, grid64, target64, T.Qs / 32).parts : 1;
     int32_t *cnt_out = &S.cnt[(k + 1) % 3];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane & 7, slot = tid >> 3;
     for (int t = tid; t < nnz; t += kGroupBlock) {
@@ -658,16 +665,18 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
         // Hessian-only moments of tensor-core cells (accumulator values), else in FP64
         for (int e = tid; e < n2 * kGroupCells; e += kGroupBlock) {
             const int c = e / kGroupCells, j = e % kGroupCells;
-            const double *col = Vacc + (size_t)c * vs + min(base + j, cnt_in - 1);
+            const int f = MIXED ? sh64[j] : 0;  // 1 + place among the handed cells
+            const double *col = Vacc + (size_t)c * vs + (f ? vs / 2 + f - 1 : min(base + j, cnt_in - 1));
             if (MIXED && c >= n && !sh64[j]) {
                 float v = d2f_bits(col[0]);
 #pragma unroll 4
                 for (int p = 1; p < parts; ++p) v += d2f_bits(col[(size_t)p * cnt_in]);
                 sVf[c * kGroupPitch + j] = v;
             } else {
+                const int np_ = f ? parts64 : parts, step = f ? handed : cnt_in;
                 double v = col[0];
 #pragma unroll 4
-                for (int p = 1; p < parts; ++p) v += col[(size_t)p * cnt_in];
+                for (int p = 1; p < np_; ++p) v += col[(size_t)p * step];
                 sV[c * kGroupPitch + j] = v;
                 if (MIXED) sVf[c * kGroupPitch + j] = d2f_bits(v);
             }
@@ -860,7 +869,12 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
             atomicAdd(&S.cnt[6], __popc(live));
             atomicMax(&S.cnt[4], evmax);
         }
-        push_agg(list_out, cnt_out, cell, cont);
+        const int at_out = push_agg(list_out, cnt_out, cell, cont);
+        if (MIXED && cont && S.h64[cell]) {
+            const int f = atomicAdd(&S.cnt[12 + (k + 1) % 3], 1);
+            S.handed[(k + 1) & 1][f] = at_out;
+            S.h64[cell] = 1 + f;
+        }
     }
 }
 
