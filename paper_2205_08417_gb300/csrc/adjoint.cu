@@ -57,7 +57,7 @@ __global__ void objective_kernel(const double *__restrict__ u, int n, const doub
 
 template <int NN>
 __global__ void __launch_bounds__(kWarps * 32)
-lambda_dot_m_kernel(int Qp, QuadTab X, const double *__restrict__ lam, const double *__restrict__ area,
+lambda_dot_m_kernel(int Qp, QuadTab<double> X, const double *__restrict__ lam, const double *__restrict__ area,
                     double *__restrict__ Lq, int C)
 {
     constexpr int n = Dims<NN>::n;
@@ -65,7 +65,7 @@ lambda_dot_m_kernel(int Qp, QuadTab X, const double *__restrict__ lam, const dou
     for (int e = threadIdx.x; e < X.R * n; e += blockDim.x) lambda_smem[e] = X.ringP[e];
     __syncthreads();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, cpw = 32 / X.J;
-    const QuadLane Q(X, lane);
+    const QuadLane<double> Q(X, lane);
     for (int base = (blockIdx.x * kWarps + wib) * cpw; base < C; base += gridDim.x * kWarps * cpw) {
         const int i = min(base + Q.ci, C - 1);
         const bool store = Q.live && base + Q.ci < C;
@@ -92,7 +92,7 @@ lambda_dot_m_kernel(int Qp, QuadTab X, const double *__restrict__ lam, const dou
 
 template <int NN>
 __global__ void __launch_bounds__(kWarps * 32, 2)
-adjoint_flux_kernel(int Qp, QuadTab X, const int4 *__restrict__ nbr, const double *__restrict__ nrm,
+adjoint_flux_kernel(int Qp, QuadTab<double> X, const int4 *__restrict__ nbr, const double *__restrict__ nrm,
                     const double *__restrict__ psi, const double *__restrict__ Lq, double dt, int bc, int C,
                     double *__restrict__ rout)
 {
@@ -104,7 +104,7 @@ adjoint_flux_kernel(int Qp, QuadTab X, const int4 *__restrict__ nbr, const doubl
     __syncthreads();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, J = X.J, cpw = 32 / J;
     double *red = sRed + wib * n * 32;
-    const QuadLane Q(X, lane);
+    const QuadLane<double> Q(X, lane);
     for (int base = (blockIdx.x * kWarps + wib) * cpw; base < C; base += gridDim.x * kWarps * cpw) {
         const int i = min(base + Q.ci, C - 1);
         const int4 nb = nbr[i];
@@ -326,7 +326,7 @@ extern "C" int32_t kitrt_adjoint(kitrt_mn *mn, const double *u0, const double *a
     const kitrt_mesh *m = mn->mesh;
     const double inv_m0 = 1.0 / T.m0;
     const int tb = (C + 255) / 256 < mn->nsm * 8 ? (C + 255) / 256 : mn->nsm * 8;
-    const QuadTab X = quad_tab(mn);
+    const QuadTab<double> X = quad_tab64(mn);
     const int per_block = kWarps * (32 / mn->J), qb = std::min((C + per_block - 1) / per_block, mn->nsm * 2);
     const int lb = std::min((C + per_block - 1) / per_block, mn->nsm * 8);
     const int sb = std::min((C + kGroupCells - 1) / kGroupCells, mn->nsm * 2);

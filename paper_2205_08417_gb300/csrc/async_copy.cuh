@@ -1,6 +1,5 @@
-// mbarrier and bulk-copy (TMA) helpers shared by the kernels that stage data in shared memory:
-// the tensor-core sweep (mbarrier completion of tcgen05 MMAs), the S_N step and the FP32 flux
-// (tiles of consecutive cells' rows copied with cp.async.bulk). Every wait is bounded.
+// mbarrier and asynchronous-copy helpers of the kernels that stage data in shared memory: the
+// tensor-core sweep (mbarrier completion of tcgen05 MMAs, bounded waits) and the predictor.
 #pragma once
 
 #include <stdint.h>
@@ -17,12 +16,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p)
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
@@ -48,17 +41,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return false;
 }
 
-// Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) from global to shared
-// memory, completing on `bar`.
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
-
 // Asynchronous 16-byte and 8-byte copies of this thread from global to shared memory, and the wait for all of
 // this thread's copies.
 __device__ __forceinline__ void cp_async16(void *dst, const void *src)
@@ -70,12 +52,5 @@ __device__ __forceinline__ void cp_async8(void *dst, const void *src)
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Orders this thread's earlier generic-proxy accesses of shared memory before later async-proxy
-// (bulk copy) writes to it.
-__device__ __forceinline__ void fence_proxy_async_smem()
-{
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 
 }  // namespace kitrt_async

@@ -39,7 +39,7 @@ constexpr int kWarps = 8;
 // value is psi / rho, so each row is scaled by its cell's 1/rho (invrho) before differencing.
 template <int NN, bool RHO>
 __global__ void __launch_bounds__(kWarps * 32, 2)
-flux64_kernel(Tables T, QuadTab X, const int4 *__restrict__ nbr, const double *__restrict__ nrm,
+flux64_kernel(Tables T, QuadTab<double> X, const int4 *__restrict__ nbr, const double *__restrict__ nrm,
               const double *__restrict__ area, const double *__restrict__ psi,
               const double *__restrict__ invrho, double *__restrict__ u,
               const double *__restrict__ sa, const double *__restrict__ ss,
@@ -55,7 +55,7 @@ flux64_kernel(Tables T, QuadTab X, const int4 *__restrict__ nbr, const double *_
     const int J = X.J, P = X.P, cpw = 32 / J;  // cells per warp
     const int Qp = T.Qp;
     double *red = sRed + wib * n * 32;
-    const QuadLane Q(X, lane);
+    const QuadLane<double> Q(X, lane);
     for (int base = (blockIdx.x * kWarps + wib) * cpw; base < C; base += gridDim.x * kWarps * cpw) {
         const int i = min(base + Q.ci, C - 1);
         const int4 nb = nbr[i];
@@ -260,7 +260,7 @@ int launch_flux_update(kitrt_mn *mn, const Tables &T, int C, const double *psi,
                        const double *q, double dt, int bc, cudaStream_t s)
 {
     const kitrt_mesh *m = mn->mesh;
-    const QuadTab X = quad_tab(mn);
+    const QuadTab<double> X = quad_tab64(mn);
     const int per_block = kWarps * (32 / mn->J), need = (C + per_block - 1) / per_block;
     const int grid = need < mn->nsm * 2 ? (need > 0 ? need : 1) : mn->nsm * 2;
     const size_t smem64 = sizeof(double) * mn->n * ((size_t)mn->R + mn->J + kWarps * 32);

@@ -470,7 +470,6 @@ int32_t kitrt_mn_destroy(kitrt_mn *mn)
     }
     for (void *p : mn->allocs) cudaFree(p);
     if (mn->h_cnt) cudaFreeHost(mn->h_cnt);
-    if (mn->h_sn_flag) cudaFreeHost(mn->h_sn_flag);
     if (mn->h_check) cudaFreeHost(mn->h_check);
     if (mn->d_adj) cudaFree(mn->d_adj);
     delete mn;
@@ -639,17 +638,6 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
     TRY(dev_upload(mn, &mn->d_w32, w32));
     TRY(dev_upload(mn, &mn->d_wox32, wox32));
     TRY(dev_upload(mn, &mn->d_woy32, woy32));
-    // unweighted folded directions for the S_N step (0 on padding)
-    std::vector<double> oxp(Qp, 0.0), oyp(Qp, 0.0);
-    for (int q = 0; q < Qf; ++q) {
-        oxp[q] = mn->h_ox[q];
-        oyp[q] = mn->h_oy[q];
-    }
-    std::vector<float> oxp32(oxp.begin(), oxp.end()), oyp32(oyp.begin(), oyp.end());
-    TRY(dev_upload(mn, &mn->d_ox, oxp));
-    TRY(dev_upload(mn, &mn->d_oy, oyp));
-    TRY(dev_upload(mn, &mn->d_ox32, oxp32));
-    TRY(dev_upload(mn, &mn->d_oy32, oyp32));
     // 2^(j/2048), j = 0..2047, rounded to double and to units of 2^-61 from extended precision
     std::vector<double> exptab(2048);
     std::vector<uint64_t> fx_exp(2048);
@@ -701,14 +689,21 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
                 }
                 ringW[(size_t)rg * n2 + cc] = limbs(ldexpl(r.ring_w[rg] * p, -mn->fx_wexp), 57);
             }
-        // the quads' tables of the FP64 flux: the axes' quad (j = 0: 0, pi, pi/2, 3 pi/2) takes
-        // cos = 1 and the sign of sin(k pi/2) for odd k, 0 for even k
-        std::vector<double> fr((size_t)mn->R * n), frP((size_t)mn->R * n), fa((size_t)mn->J * n), fsc((size_t)mn->J * 2);
-        for (int rg = 0; rg < mn->R; ++rg)
+        // tables of the quads (quad_lane.cuh): w sin(theta) P, w P, P and sin(theta) per ring, the
+        // azimuthal factors (the axes' quad j = 0 (0, pi, pi/2, 3 pi/2) takes cos = 1 and the sign of
+        // sin(k pi/2) for odd k, 0 for even k), sin and cos of phi_j, a zero row
+        const size_t Rn = (size_t)mn->R * n, Jn = (size_t)mn->J * n;
+        std::vector<double> qt(3 * Rn + mn->R + Jn + 2 * mn->J + Qp, 0.0);
+        double *fS = qt.data() + 3 * Rn, *fa = fS + mn->R, *fsc = fa + Jn;
+        for (int rg = 0; rg < mn->R; ++rg) {
+            fS[rg] = sqrt(1.0 - r.ring_mu[rg] * r.ring_mu[rg]);
             for (int cc = 0; cc < n; ++cc) {
-                frP[(size_t)rg * n + cc] = P[(size_t)rg * n2 + cc];
-                fr[(size_t)rg * n + cc] = r.ring_w[rg] * sqrt(1.0 - r.ring_mu[rg] * r.ring_mu[rg]) * P[(size_t)rg * n2 + cc];
+                const double p = P[(size_t)rg * n2 + cc];
+                qt[(size_t)rg * n + cc] = r.ring_w[rg] * fS[rg] * p;
+                qt[Rn + (size_t)rg * n + cc] = r.ring_w[rg] * p;
+                qt[2 * Rn + (size_t)rg * n + cc] = p;
             }
+        }
         for (int j = 0; j < mn->J; ++j) {
             const double phi = j * (2.0 * kPi / r.nphi);
             fsc[2 * j] = j ? sin(phi) : 0.0;
@@ -719,11 +714,8 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
                     fa[(size_t)j * n + cc] = j ? (k >= 0 ? cos(k * phi) : sin(-k * phi))
                                                : (k >= 0 ? 1.0 : k & 1 ? ((-k) & 2 ? -1.0 : 1.0) : 0.0);
         }
-        TRY(dev_upload(mn, &mn->d_flux_ring, fr));
-        TRY(dev_upload(mn, &mn->d_flux_ringP, frP));
-        TRY(dev_upload(mn, &mn->d_flux_az, fa));
-        TRY(dev_upload(mn, &mn->d_flux_sc, fsc));
-        TRY(dev_upload(mn, &mn->d_zero64, std::vector<double>(Qp, 0.0)));
+        TRY(dev_upload(mn, &mn->d_quad64, qt));
+        TRY(dev_upload(mn, &mn->d_quad32, std::vector<float>(qt.begin(), qt.end())));
         TRY(dev_upload(mn, &mn->d_fx_trig, trig));
         TRY(dev_upload(mn, &mn->d_fx_ringA, ringA));
         TRY(dev_upload(mn, &mn->d_fx_ringW, ringW));
@@ -808,7 +800,6 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
         kitrt_mn_destroy(mn);
         return KITRT_ENOMEM;
     }
-    TRY(dev_alloc(mn, &mn->d_sn_flag, 1));
     {
         double *cellc = nullptr;
         TRY(dev_alloc(mn, &cellc, C * 12));
@@ -828,10 +819,6 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
     }
     TRY(dev_alloc(mn, &mn->d_check, 2));
     if (cudaMallocHost(&mn->h_check, 2 * sizeof(unsigned long long)) != cudaSuccess) {
-        kitrt_mn_destroy(mn);
-        return KITRT_ENOMEM;
-    }
-    if (cudaMallocHost(&mn->h_sn_flag, sizeof(int32_t)) != cudaSuccess) {
         kitrt_mn_destroy(mn);
         return KITRT_ENOMEM;
     }

@@ -134,8 +134,6 @@ struct kitrt_mn {
                                          // in the sweep's point order (mixed)
     unsigned short *d_Mhi16 = nullptr;   // BF16 copy
     float *d_wox32 = nullptr, *d_woy32 = nullptr, *d_mbar32 = nullptr;
-    double *d_ox = nullptr, *d_oy = nullptr;  // [Qp] folded directions (0 on padding), S_N step
-    float *d_ox32 = nullptr, *d_oy32 = nullptr;
     double *d_V = nullptr;               // [C x n2] moments scratch (kitrt_hessian)
     double *d_Vacc = nullptr;            // [n2 x vs] sweeps: partial moments per list slot and part; in the
                                          // mixed modes the second half of the columns is for handed cells
@@ -148,8 +146,8 @@ struct kitrt_mn {
     float *d_fx_mmax = nullptr;
     int fx_wexp = 0;
     double *d_exptab = nullptr;          // [2048] exp table (Tables::exptab)
-    // FP64 flux and adjoint: ring, azimuth and direction tables of the quads (quad_lane.cuh), a zero row
-    double *d_flux_ring = nullptr, *d_flux_ringP = nullptr, *d_flux_az = nullptr, *d_flux_sc = nullptr, *d_zero64 = nullptr;
+    double *d_quad64 = nullptr;          // tables of the quads (quad_lane.cuh), FP64 and FP32
+    float *d_quad32 = nullptr;
     void *d_mlp16 = nullptr;             // learned closure: BF16 network parameters
     float *d_mlp_norm = nullptr;         // [4 (n-1)] feature and output means / scales
     bool has_mlp = false;
@@ -176,8 +174,6 @@ struct kitrt_mn {
     unsigned long long *d_check = nullptr, *h_check = nullptr;
     void *d_adj = nullptr;     // kitrt_adjoint workspace (grown on demand)
     size_t adj_bytes = 0;
-    int32_t *d_sn_flag = nullptr;  // S_N step: device status (KITRT_ETIMEOUT on an expired wait)
-    int32_t *h_sn_flag = nullptr;  // pinned copy
     void *d_sn_cell = nullptr;     // [C x 12] per-cell coefficients of the S_N step (FP32 or FP64)
     std::vector<void *> allocs;
     // tracing
