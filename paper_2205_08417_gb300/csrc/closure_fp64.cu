@@ -129,18 +129,19 @@ struct PredictDims {
 
 template <int NN>
 __global__ void __launch_bounds__(PredictDims<NN>::threads)
-predict_kernel(NewtonState S, const double *__restrict__ u, NewtonParams np)
+predict_kernel(NewtonState S, const double *__restrict__ u, NewtonParams np, const int32_t *__restrict__ list,
+               const int32_t *__restrict__ count)
 {
     using D = PredictDims<NN>;
     constexpr int n = Dims<NN>::n, npairs = Dims<NN>::npairs;
     extern __shared__ __align__(16) double predict_smem[];  // [32][pitch] factors, [n][32] vectors
-    const int cnt = S.cnt[8];
+    const int cnt = *count;
     const int stride = gridDim.x * blockDim.x;
     const int rounds = (cnt + stride - 1) / stride;
     for (int rd = 0; rd < rounds; ++rd) {
         const int it = rd * stride + blockIdx.x * blockDim.x + threadIdx.x;
         bool cont = false;
-        int cell = it < cnt ? S.list[1][it] : -1;
+        int cell = it < cnt ? list[it] : -1;
         if constexpr (!D::in_regs) {
             __syncwarp();
             for (int r = 0; r < 32; ++r) {
@@ -645,13 +646,13 @@ int grid_for(const kitrt_mn *mn, int C, int per_sm)
 
 template <int NN>
 int predict_launch(kitrt_mn *mn, const NewtonState &S, int C, const double *u, NewtonParams np,
-                   cudaStream_t s)
+                   const int32_t *list, const int32_t *count, cudaStream_t s)
 {
     using D = PredictDims<NN>;
     if (ensure_dyn_smem(predict_kernel<NN>, D::smem)) return KITRT_ECUDA;
     int tb = (C + D::threads - 1) / D::threads;
     if (tb > mn->nsm * 32) tb = mn->nsm * 32;
-    predict_kernel<NN><<<tb > 0 ? tb : 1, D::threads, D::smem, s>>>(S, u, np);
+    predict_kernel<NN><<<tb > 0 ? tb : 1, D::threads, D::smem, s>>>(S, u, np, list, count);
     return KITRT_OK;
 }
 
@@ -793,9 +794,17 @@ int launch_begin(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
         if (cudaGetLastError() != cudaSuccess) return KITRT_ECUDA;
     }
     if (first == 1 || learned) return KITRT_OK;
+    return launch_predict(mn, S, C, u, np, S.list[1], S.cnt + 8, s);
+}
+
+// The first Newton step of the cells in `list` (device, *count of them, at most C) from their stored
+// moments and factors.
+int launch_predict(kitrt_mn *mn, const NewtonState &S, int C, const double *u, NewtonParams np, const int32_t *list,
+                   const int32_t *count, cudaStream_t s)
+{
     LaunchScope ls(mn, PK_BEGIN, s, 0);
     int rc = KITRT_OK;
-    KITRT_DISPATCH_N(mn->N, rc = predict_launch<NN>(mn, S, C, u, np, s));
+    KITRT_DISPATCH_N(mn->N, rc = predict_launch<NN>(mn, S, C, u, np, list, count, s));
     if (rc) return rc;
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }

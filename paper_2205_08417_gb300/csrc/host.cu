@@ -783,7 +783,14 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
             kitrt_mn_destroy(mn);
             return KITRT_ECUDA;
         }
-        if (p.mode == KITRT_LEARNED) TRY(dev_alloc(mn, &mn->d_alpha_nn, C * (size_t)n));
+        if (p.mode == KITRT_LEARNED) {
+            // component 0 stays 0: the network gives the others
+            TRY(dev_alloc(mn, &mn->d_alpha_nn, C * (size_t)n));
+            if (cudaMemset(mn->d_alpha_nn, 0, sizeof(double) * C * n) != cudaSuccess) {
+                kitrt_mn_destroy(mn);
+                return KITRT_ECUDA;
+            }
+        }
         TRY(dev_alloc(mn, &S.h64, C));
         TRY(dev_alloc(mn, &S.handed[0], C));
         TRY(dev_alloc(mn, &S.handed[1], C));
@@ -910,7 +917,7 @@ static int run_closure(kitrt_mn *mn, int C, const double *u, const double *alpha
     if (rc) return rc;
     if (learned) {
         rc = launch_mlp_infer(mn, u, mn->st.list[1], mn->st.cnt + 8, C, mn->d_alpha_nn, s);
-        if (!rc) rc = launch_learned_pass(mn, T, mn->st, C, u, psi32, first == 1, s);
+        if (!rc) rc = launch_learned_pass(mn, T, mn->st, C, u, np, psi32, first, s);
         if (rc) return rc;
     }
     // rounds are launched in batches between two reads of the counters; the first batch is as long

@@ -95,7 +95,8 @@ struct NewtonState {
                        //   cnt[8] predictor list length, cnt[9] learned-mode steps taken
                        //   from a stored factor, cnt[10] learned-mode residual passes of the
                        //   network's proposals, cnt[11] mixed-mode hand-overs to the FP64 Hessian,
-                       //   cnt[12..14] rotating counters of handed
+                       //   cnt[12..14] rotating counters of handed, cnt[15] learned-mode cells for
+                       //   the predictor (in handed[0])
 };
 
 struct NewtonParams {
@@ -247,7 +248,9 @@ int launch_begin(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
 int launch_mlp_infer(kitrt_mn *mn, const double *u, const int32_t *list, const int32_t *cnt, int C,
                      double *alpha, cudaStream_t s);
 int launch_learned_pass(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, const double *u,
-                        float *psi32, int first, cudaStream_t s);
+                        NewtonParams np, float *psi32, int first, cudaStream_t s);
+int launch_predict(kitrt_mn *mn, const NewtonState &S, int C, const double *u, NewtonParams np, const int32_t *list,
+                   const int32_t *count, cudaStream_t s);
 int fp64_sweep_grid(const kitrt_mn *mn);
 int mixed_sweep_grid(const kitrt_mn *mn);
 int launch_eval_fp64(kitrt_mn *mn, const Tables &T, const NewtonState &S, const double *u, int k, cudaStream_t s);

@@ -19,111 +19,202 @@
 namespace {
 
 using namespace kitrt_dev;
-constexpr int kWarps = 8;
+constexpr int kWarps = 8;  // of the moment generator
+
+// The network's points of the listed cells (S.list[1]): U'_a and the ansatz exp(z') of every point, in
+// the fixed-point form of the sweeps (sweep.cuh). One thread per listed cell, work items (tile of 128
+// cells, part of the quadrature) as in the FP64-mode sweep. A warp per cell in FP64 (28 FP64
+// instructions a point for M_3) took, with the decision below and the network, 1.06 ms for 76,564
+// M_3 closures of 400 points; now 0.30 ms.
+constexpr int kSweepThreads = 128;
+
+size_t learned_smem(int n, int N, int J) { return 2048 * 8 + (size_t)n * kSweepThreads * 8 + (size_t)J * 2 * N * 8; }
 
 template <int NN>
-__global__ void __launch_bounds__(kWarps * 32)
-learned_pass_kernel(Tables T, NewtonState S, const double *__restrict__ u,
-                    const double *__restrict__ alpha_nn, double tol, float *__restrict__ psi32,
-                    int first)
+__global__ void __launch_bounds__(kSweepThreads)
+learned_sweep_kernel(Tables T, NewtonState S, const double *__restrict__ alpha_nn, double *__restrict__ Vacc, int vs,
+                     int target_items, float *__restrict__ psi32)
 {
-    constexpr int n = Dims<NN>::n, npairs = Dims<NN>::npairs;
-    __shared__ double sH[kWarps][n * n];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int Qp = T.Qp;
-    const int count = S.cnt[8];
-    for (int it = blockIdx.x * kWarps + wib; it < count; it += gridDim.x * kWarps) {
-        const int cell = S.list[1][it];
-        const size_t off = (size_t)cell * n;
-        const double ua = lane < n ? u[off + lane] : 0.0;
-        const double al = (lane >= 1 && lane < n) ? alpha_nn[off + lane] : 0.0;
-        double atv[n];
-#pragma unroll
-        for (int a = 0; a < n; ++a) atv[a] = __shfl_sync(kFull, al, a);
-        double Up[n];
-#pragma unroll
-        for (int a = 0; a < n; ++a) Up[a] = 0.0;
-        for (int q = lane; q < Qp; q += 32) {
-            double z = 0.0;
-#pragma unroll
-            for (int a = 1; a < n; ++a) z = fma(atv[a], T.Mt[a * Qp + q], z);
-            const double ez = kexp(z, T.exptab);
-            if (psi32) psi32[(size_t)cell * Qp + q] = exp_to_float(ez);
-            const double e = T.w[q] * ez;
-#pragma unroll
-            for (int a = 0; a < n; ++a) Up[a] = fma(e, T.Mt[a * Qp + q], Up[a]);
-        }
-        double Ua = 0.0;
+    constexpr int n = Dims<NN>::n;
+    extern __shared__ __align__(16) unsigned char learned_smem_raw[];
+    uint64_t *tab = (uint64_t *)learned_smem_raw;
+    int2 *sA = (int2 *)(tab + 2048);
+    int2 *trig = sA + n * kSweepThreads;
+    const int cnt = S.cnt[8], nunits = T.Qs / 32;
+    const SweepSplit sp = sweep_split(cnt, gridDim.x, target_items, nunits);
+    const int items = sp.tiles * sp.parts;
+    if ((int)blockIdx.x >= items) return;
+    for (int j = threadIdx.x; j < 2048; j += kSweepThreads) tab[j] = T.fx_exp[j];
+    for (int j = threadIdx.x; j < T.J * 2 * NN; j += kSweepThreads) {
+        const int p = j / (2 * NN), q = j % (2 * NN);
+        trig[j] = T.fx_trig[p * 4 * NN + (q < NN ? q : NN + q)];
+    }
+    __syncthreads();
+    int2 *myA = sA + threadIdx.x;
+    for (int item = blockIdx.x; item < items; item += gridDim.x) {
+        const int tile = item / sp.parts, part = item % sp.parts;
+        const int slot = tile * kSweepThreads + threadIdx.x;
+        if (slot >= cnt) continue;  // threads are independent: no block barrier below
+        const int q_begin = part * nunits / sp.parts * 8;
+        const int q_end = min(T.nquad, (part + 1) * nunits / sp.parts * 8);
+        const int cell = S.list[1][slot];
+        const double *al = alpha_nn + (size_t)cell * n;  // al[0] = 0: alpha_0 follows from the mass
+        float bound = 0.0f;
 #pragma unroll
         for (int a = 0; a < n; ++a) {
-            const double v = warp_sum(Up[a]);
-            if (lane == a) Ua = v;
+            const double x = a ? al[a] : 0.0;
+            const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(x));
+            myA[a * kSweepThreads] = make_int2(w.h, w.l);
+            bound = fmaf(fabsf(d2f_bits(x)), T.fx_mmax[a], bound);
         }
-        const double u0 = __shfl_sync(kFull, ua, 0), U0p = __shfl_sync(kFull, Ua, 0);
-        const double c = u0 / U0p;                // exp(alpha_0 m_0)
-        const double alpha0 = log(c) / T.m0;
-        const double U = c * Ua;                  // moments of the mass-corrected ansatz
-        const double r = (lane >= 1 && lane < n) ? U - ua : 0.0;
-        const double r2 = warp_sum(r * r), un2 = warp_sum(ua * ua);
-        // dual objective of the network's point: <exp(alpha.m)> = u_0 / m_0 after the mass fix
-        const double f_nn = u0 / T.m0 - (alpha0 * u0 + warp_sum(al * ua));
-        if (lane == 0) atomicAdd(&S.cnt[10], 1);  // a quadrature pass of this cell (the network's)
-        const bool finite = isfinite(alpha0) && isfinite(r2) && isfinite(f_nn) && u0 > 0.0;
-        const bool ok = finite && r2 <= tol * tol * un2;
-        if (ok) {
-            if (lane == 0) S.alpha[off] = alpha0;
-            if (lane >= 1 && lane < n) S.alpha[off + lane] = al;
-            if (lane < n) S.U[off + lane] = lane == 0 ? u0 : U;
-            if (lane == 0) {
-                S.fsum[cell] = u0 / T.m0;
-                S.phase[cell] = PH_DONE;
+        const bool wide = !(bound < kitrt_fx::kFxMaxZ);
+        bool bad = false;
+        long long U[n], A0 = 0;
+#pragma unroll
+        for (int c = 0; c < n; ++c) U[c] = 0;
+        Limb A[2 * NN];
+        FxSums<NN> B;
+        B.clear();
+        B.Sx = 100000;  // the first quad decides
+        auto trial = [&](int a) {
+            const int2 v = myA[a * kSweepThreads];
+            return Limb{v.x, v.y};
+        };
+        auto moment = [&](int c) -> long long & { return U[c]; };
+        int ring = q_begin / T.J, jq = q_begin - ring * T.J;
+        bool fresh = true;
+#pragma unroll 1
+        for (int qd = q_begin; qd < q_end; ++qd) {
+            if (fresh) {
+                fx_coeffs<NN>(trial, T.fx_ringA + (size_t)ring * n, A0, A);
+                fresh = false;
+            }
+            const int2 *tr = trig + jq * 2 * NN;
+            const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
+            Exp e[4];
+            if (!wide) {
+                long long s[4];
+                fx_exponents<NN>(A0, A, tr, NN, jq == 0, s);
+#pragma unroll
+                for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_exp(s[t], tab);
+            } else {
+                bad = !fx_slow_quad<NN>(T.Mt, T.Qp, T.exptab, al, al, 0.0, pa, pb, e) || bad;
             }
             if (psi32) {
-                const float cf = (float)c;
-                for (int q = lane; q < Qp; q += 32) psi32[(size_t)cell * Qp + q] *= cf;
+                float *row = psi32 + (size_t)cell * T.Qp;
+                float f[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) f[t] = __uint_as_float(kitrt_fx::fx_float_bits(e[t]));
+                *(float2 *)(row + 2 * pa) = make_float2(f[0], f[1]);
+                if (pb >= 0) *(float2 *)(row + 2 * pb) = make_float2(f[2], f[3]);
             }
-        } else {
-            // Newton starts from the better of the network's point and the cell's previous alpha
-            // (its objective needs no quadrature: <exp> of the previous point is stored)
+            if (pb < 0) e[2] = e[3] = Exp{0, -100000};
+            fx_accumulate<NN>(e, tr, NN, jq == 0, pb < 0, qd == q_begin, B, [&](int d) {
+#pragma unroll
+                for (int c = 0; c < n; ++c) U[c] = kitrt_fx::sar(U[c], d);
+            });
+            if (++jq == T.J) {
+                fx_flush<NN>(T.fx_ringW + (size_t)ring * Dims<NN>::n2, T.fx_sumshift, B, moment);
+                jq = 0;
+                ++ring;
+                fresh = true;
+            }
+        }
+        if (!fresh) fx_flush<NN>(T.fx_ringW + (size_t)ring * Dims<NN>::n2, T.fx_sumshift, B, moment);
+        double *col = Vacc + (size_t)part * cnt + slot;
+        const int unit = fx_unit(B.Sx, T);
+#pragma unroll
+        for (int c = 0; c < n; ++c)
+            col[(size_t)c * vs] = bad ? __longlong_as_double(0x7ff8000000000000LL) : kitrt_fx::fx_to_double(U[c], unit);
+    }
+}
+
+// The decision per listed cell, one thread each: the network's point is kept, or Newton starts from it
+// (an evaluation), or from the previous closure's point: with an evaluation, or, when its moments and
+// a factor of the cell are stored, with the predictor's step (list S.handed[0], counter cnt[15]).
+template <int NN>
+__global__ void __launch_bounds__(64)
+learned_decide_kernel(Tables T, NewtonState S, const double *__restrict__ u, const double *__restrict__ alpha_nn,
+                      const double *__restrict__ Vacc, int vs, int sweep_grid, int target_items, double tol,
+                      float *__restrict__ psi32, int first)
+{
+    constexpr int n = Dims<NN>::n;
+    const int cnt = S.cnt[8], lane = threadIdx.x & 31;
+    const int parts = sweep_split(cnt, sweep_grid, target_items, T.Qs / 32).parts;
+    const int rounds = (cnt + gridDim.x * blockDim.x - 1) / (gridDim.x * blockDim.x);
+    for (int rd = 0; rd < rounds; ++rd) {
+        const int it = (rd * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
+        const bool live = it < cnt;
+        bool ok = false, to_eval = false, to_predict = false;
+        int cell = 0;
+        double c = 1.0;
+        if (live) {
+            cell = S.list[1][it];
+            const size_t off = (size_t)cell * n;
+            auto moment = [&](int a) {
+                const double *col = Vacc + (size_t)a * vs + it;
+                double v = col[0];
+                for (int p = 1; p < parts; ++p) v += col[(size_t)p * cnt];
+                return v;
+            };
+            const double u0 = u[off];
+            c = u0 / moment(0);                       // exp(alpha_0 m_0)
+            const double alpha0 = log(c) / T.m0;
+            // residual and dual objective of the mass-corrected ansatz (<exp(alpha.m)> = u_0 / m_0)
+            double r2 = 0.0, un2 = u0 * u0, au = alpha0 * u0, au_prev = first != 1 ? S.alpha[off] * u0 : 0.0;
+#pragma unroll 1
+            for (int a = 1; a < n; ++a) {
+                const double ua = u[off + a], U = c * moment(a), r = U - ua;
+                r2 = fma(r, r, r2);
+                un2 = fma(ua, ua, un2);
+                au = fma(alpha_nn[off + a], ua, au);
+                if (first != 1) au_prev = fma(S.alpha[off + a], ua, au_prev);
+            }
+            const double f_nn = u0 / T.m0 - au;
+            const bool finite = isfinite(alpha0) && isfinite(r2) && isfinite(f_nn) && u0 > 0.0;
+            ok = finite && r2 <= tol * tol * un2;
             bool use_nn = finite;
-            if (first != 1 && finite) {
-                const double ap = lane < n ? S.alpha[off + lane] : 0.0;
-                const double f_prev = S.fsum[cell] - warp_sum(ap * ua);
+            if (!ok && first != 1 && finite) {
+                // the better start by dual objective (<exp> of the previous point is stored)
+                const double f_prev = S.fsum[cell] - au_prev;
                 use_nn = !(isfinite(f_prev) && f_prev <= f_nn);
             }
-            if (use_nn) {
-                if (lane == 0) S.alpha[off] = alpha0;
-                if (lane >= 1 && lane < n) S.alpha[off + lane] = al;
+            if (ok || use_nn) {
+                S.alpha[off] = alpha0;
+#pragma unroll 1
+                for (int a = 1; a < n; ++a) S.alpha[off + a] = alpha_nn[off + a];
             }
-            if (!use_nn && first != 1 && S.lfac && S.lfac[cell]) {
-                // the previous closure's point is the better start, and its moments and a
-                // factor of this cell are stored: take the Newton step from them at once, as the
-                // predictor of the other modes does, instead of evaluating that point again
-                double *H = sH[wib];
-                const double ap = lane < n ? S.alpha[off + lane] : 0.0;
-                const double g = lane < n ? S.U[off + lane] - ua : 0.0;
-                for (int a = lane; a < n; a += 32)
-                    for (int b = 0; b <= a; ++b) H[a * n + b] = S.L[(size_t)cell * npairs + tri_idx(a, b)];
-                __syncwarp();
-                const double d = warp_chol_solve<n>(H, -g, lane);
-                __syncwarp();
-                const double gn2 = warp_sum(g * g), au = warp_sum(ap * ua), gd = warp_sum(g * d);
-                if (lane < n) S.dir[off + lane] = d;
-                if (lane == 0) {
-                    if (S.gnorm) S.gnorm[cell] = sqrt(gn2);
-                    S.f0[cell] = S.fsum[cell] - au;
-                    S.gd[cell] = gd;
-                    S.lam[cell] = 1.0;
-                    S.phase[cell] = PH_NEWTON;
-                    atomicAdd(&S.cnt[5], 1);
-                    atomicAdd(&S.cnt[9], 1);  // a step from the stored factor
-                }
-            } else if (lane == 0) {
+            if (ok) {
+                S.U[off] = u0;
+#pragma unroll 1
+                for (int a = 1; a < n; ++a) S.U[off + a] = c * moment(a);
+                S.fsum[cell] = u0 / T.m0;
+                S.phase[cell] = PH_DONE;
+            } else if (!use_nn && first != 1 && S.lfac && S.lfac[cell]) {
+                to_predict = true;
+            } else {
                 S.phase[cell] = PH_INIT;
-                atomicAdd(&S.cnt[5], 1);
+                to_eval = true;
             }
-            push(S.list[0], &S.cnt[0], cell, lane);
         }
+        // accepted cells: the ansatz takes the mass correction (a row at a time by the whole warp)
+        unsigned rows = __ballot_sync(kFull, ok && psi32);
+        while (rows) {
+            const int src = __ffs(rows) - 1;
+            rows &= rows - 1;
+            const int rc = __shfl_sync(kFull, cell, src);
+            const float cf = (float)__shfl_sync(kFull, c, src);
+            for (int q = lane; q < T.Qp; q += 32) psi32[(size_t)rc * T.Qp + q] *= cf;
+        }
+        const unsigned nlive = __popc(__ballot_sync(kFull, live)), nfall = __popc(__ballot_sync(kFull, to_eval || to_predict)),
+                       npred = __popc(__ballot_sync(kFull, to_predict));
+        if (lane == 0) {
+            if (nlive) atomicAdd(&S.cnt[10], (int)nlive);  // quadrature passes of the network's points
+            if (nfall) atomicAdd(&S.cnt[5], (int)nfall);
+            if (npred) atomicAdd(&S.cnt[9], (int)npred);   // steps from the stored factor
+        }
+        push_agg(S.list[0], &S.cnt[0], cell, to_eval);
+        push_agg(S.handed[0], &S.cnt[15], cell, to_predict);
     }
 }
 
@@ -171,27 +262,36 @@ __global__ void to_bf16_kernel(const float *__restrict__ x, __nv_bfloat16 *__res
 }  // namespace
 
 int launch_learned_pass(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, const double *u,
-                        float *psi32, int first, cudaStream_t s)
+                        NewtonParams np, float *psi32, int first, cudaStream_t s)
 {
-    int need = (C + kWarps - 1) / kWarps;
-    const int cap = mn->nsm * 8;
-    const int grid = need < cap ? (need > 0 ? need : 1) : cap;
-    LaunchScope ls(mn, PK_MLP, s, 0);
-#define LP_CASE(NNv)                                                                               \
-    case NNv:                                                                                      \
-        learned_pass_kernel<NNv><<<grid, kWarps * 32, 0, s>>>(T, S, u, mn->d_alpha_nn, mn->p.fallback_tol, \
-                                                              psi32, first);                           \
+    const size_t smem = learned_smem(mn->n, mn->N, mn->J);
+    int blocks = (C + 63) / 64;
+    if (blocks > mn->nsm * 16) blocks = mn->nsm * 16;
+    if (blocks < 1) blocks = 1;
+    {
+        LaunchScope ls(mn, PK_MLP, s, 0);
+        mn->launch_count += 1;  // two kernels in this scope
+#define LP_CASE(NNv)                                                                                       \
+    case NNv:                                                                                              \
+        if (ensure_dyn_smem(learned_sweep_kernel<NNv>, smem)) return KITRT_ECUDA;                          \
+        learned_sweep_kernel<NNv><<<mn->grid_fp64, kSweepThreads, smem, s>>>(T, S, mn->d_alpha_nn, mn->d_Vacc, mn->vs, \
+                                                                             mn->target_fp64, psi32);      \
+        learned_decide_kernel<NNv><<<blocks, 64, 0, s>>>(T, S, u, mn->d_alpha_nn, mn->d_Vacc, mn->vs, mn->grid_fp64,   \
+                                                         mn->target_fp64, mn->p.fallback_tol, psi32, first); \
         break;
-    switch (mn->N) {
-        LP_CASE(1)
-        LP_CASE(2)
-        LP_CASE(3)
-        LP_CASE(4)
-        LP_CASE(5)
-    default: return KITRT_EINVAL;
-    }
+        switch (mn->N) {
+            LP_CASE(1)
+            LP_CASE(2)
+            LP_CASE(3)
+            LP_CASE(4)
+            LP_CASE(5)
+        default: return KITRT_EINVAL;
+        }
 #undef LP_CASE
-    return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
+        if (cudaGetLastError() != cudaSuccess) return KITRT_ECUDA;
+    }
+    if (first == 1) return KITRT_OK;
+    return launch_predict(mn, S, C, u, np, S.handed[0], S.cnt + 15, s);
 }
 
 extern "C" {
