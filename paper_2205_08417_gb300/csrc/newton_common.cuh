@@ -611,6 +611,72 @@ __device__ __forceinline__ bool group_factor_solve(const Coef *__restrict__ coef
     return spd;
 }
 
+// The same in FP64 with the matrix in shared memory throughout: the few cells of the mixed modes that
+// were handed over to the FP64 Hessian. The register version would set the register count of the
+// whole kernel (and with it how many blocks an SM holds) for cells that are mostly not there.
+template <int NN>
+__device__ __forceinline__ bool group_factor_solve_shared(const Tables &T, const double *V, double *Hs, double gamma,
+                                                          int reg0, int g, double (&y)[(Dims<NN>::n + 7) / 8])
+{
+    constexpr int n = Dims<NN>::n, npairs = Dims<NN>::npairs, SL = (n + 7) / 8;
+#pragma unroll 1
+    for (int p = g; p < npairs; p += 8) {
+        double h = 0.0;
+        const int t1 = T.gstart[p + 1];
+#pragma unroll 1
+        for (int t = T.gstart[p]; t < t1; ++t) h = fma(T.gcoef[t], V[T.gidx[t] * kGroupPitch], h);
+        Hs[p] = h;
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int j = reg0 + g; j < n; j += 8) Hs[tri_idx(j, j)] += gamma;
+    __syncwarp();
+    bool spd = true;
+#pragma unroll 1
+    for (int j = 0; j < n; ++j) {
+        const double d = Hs[tri_idx(j, j)];
+        spd = spd && r_pos(d);
+        const double rinv = r_rsqrt(d > 0.0 ? d : 1.0);
+        __syncwarp();
+        if (g == 0) Hs[tri_idx(j, j)] = rinv;
+#pragma unroll 1
+        for (int i = j + 1 + g; i < n; i += 8) Hs[tri_idx(i, j)] *= rinv;
+        __syncwarp();
+#pragma unroll 1
+        for (int i = j + 1 + g; i < n; i += 8) {
+            const double l = Hs[tri_idx(i, j)];
+#pragma unroll 1
+            for (int k = j + 1; k <= i; ++k) Hs[tri_idx(i, k)] = fma(-l, Hs[tri_idx(k, j)], Hs[tri_idx(i, k)]);
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int sj = 0; sj < SL; ++sj)
+#pragma unroll 1
+        for (int j = 8 * sj; j < (8 * sj + 8 < n ? 8 * sj + 8 : n); ++j) {
+            const double yj = __shfl_sync(kFull, y[sj] * Hs[tri_idx(j, j)], j & 7, 8);
+#pragma unroll
+            for (int s = sj; s < SL; ++s) {
+                const int row = g + 8 * s;
+                if (row == j) y[s] = yj;
+                else if (row > j && row < n) y[s] = fma(-Hs[tri_idx(row, j)], yj, y[s]);
+            }
+        }
+#pragma unroll
+    for (int sj = SL - 1; sj >= 0; --sj)
+#pragma unroll 1
+        for (int j = (8 * sj + 8 < n ? 8 * sj + 8 : n) - 1; j >= 8 * sj; --j) {
+            const double xj = __shfl_sync(kFull, y[sj] * Hs[tri_idx(j, j)], j & 7, 8);
+#pragma unroll
+            for (int s = 0; s <= sj; ++s) {
+                const int row = g + 8 * s;
+                if (row == j) y[s] = xj;
+                else if (row < j) y[s] = fma(-Hs[tri_idx(j, row)], xj, y[s]);
+            }
+        }
+    return spd;
+}
+
 // Dynamic shared memory of post_group_kernel: moments [n2][pitch] (FP64, and FP32 in the mixed
 // modes), one packed matrix per cell, the Gaunt coefficients of the mode, indices and starts, and
 // the pass's cells.
@@ -621,7 +687,7 @@ __host__ __device__ inline size_t group_smem_bytes(int n2, int npairs, int nnz, 
 }
 
 template <int NN, bool MIXED>
-__global__ void __launch_bounds__(kGroupBlock, 2)
+__global__ void __launch_bounds__(kGroupBlock, MIXED && NN <= 3 ? 3 : 2)
 post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, NewtonParams np,
                   const double *__restrict__ Vacc, int vs, int nnz, int sweep_grid, int target_items, int grid64, int target64,
                   int upto)
@@ -760,8 +826,8 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
             for (int s = 0; s < SL; ++s) yd[s] = -gr[s];
             double *Hs = sH + slot * npairs;
             bool ok;
-            if (MIXED)
-                ok = group_factor_solve<NN, double>(T.gcoef, T.gidx, T.gstart, V, Hs, np.gamma, reg0, g, yd);
+            if constexpr (MIXED)
+                ok = group_factor_solve_shared<NN>(T, V, Hs, np.gamma, reg0, g, yd);
             else
                 ok = group_factor_solve<NN, double>(reinterpret_cast<const double *>(coef), gidx, gstart, V, Hs,
                                                     np.gamma, reg0, g, yd);
