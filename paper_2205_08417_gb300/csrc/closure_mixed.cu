@@ -153,8 +153,12 @@ struct MixedSmem {
     static constexpr int off_exp = off_V + V_bytes;               // exp table
     static constexpr int off_sx = off_exp + 2048 * 8;             // [2][128] guard sums, then scales
     static constexpr int off_bar = off_sx + 2 * kTileM * 4;
-    static constexpr int off_trig = off_bar + 64;                 // [J][2 NN] limbs
-    static int total(int J) { return off_trig + J * 2 * NN * 8; }
+    static constexpr int off_trig = off_bar + 64;                 // [J][2 NN] limbs, then the rings'
+    // Legendre factors [R][n], [R][n] (exponent, moments) when there is room for them: two CTAs per SM
+    // for N <= 3, one above
+    static constexpr int limit = NN <= 3 ? 115000 : 230000;
+    static __host__ __device__ bool rings(int J, int R) { return off_trig + (J * 2 * NN + R * 2 * Dims<NN>::n) * 8 <= limit; }
+    static int total(int J, int R) { return off_trig + (J * 2 * NN + (rings(J, R) ? R * 2 * Dims<NN>::n : 0)) * 8; }
     static constexpr int kmma = BF16 ? 16 : 8;                   // MMA K
     // byte offset of element (row r, k) inside an operand chunk
     static __device__ __forceinline__ int elem_off(int r, int k)
@@ -246,6 +250,19 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
     for (int j = tid; j < T.J * 2 * NN; j += kThreads) {
         const int p = j / (2 * NN), q = j % (2 * NN);  // cosines 1..NN, then sines 1..NN
         ((int2 *)(smem + L::off_trig))[j] = T.fx_trig[p * 4 * NN + (q < NN ? q : NN + q)];
+    }
+    // the rings' Legendre factors: exponent coefficients, and the moments' (first n of each ring)
+    const int2 *ringA = T.fx_ringA, *ringW = T.fx_ringW;
+    int ringW_pitch = n2;
+    if (L::rings(T.J, T.R)) {
+        int2 *sr = (int2 *)(smem + L::off_trig) + T.J * 2 * NN;
+        for (int j = tid; j < T.R * n; j += kThreads) {
+            sr[j] = T.fx_ringA[j];
+            sr[T.R * n + j] = T.fx_ringW[j / n * n2 + j % n];
+        }
+        ringA = sr;
+        ringW = sr + T.R * n;
+        ringW_pitch = n;
     }
     tc_fence_before();
     __syncthreads();
@@ -339,7 +356,7 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
                 // padding quads (warp-uniform) add nothing: their operand is 0
                 if (qd < T.nquad) {
                     if (fresh) {
-                        fx_coeffs<NN>(trial, T.fx_ringA + (size_t)ring * n, A0, A);
+                        fx_coeffs<NN>(trial, ringA + ring * n, A0, A);
                         fresh = false;
                     }
                     const int2 *tr = trig + jq * 2 * NN;
@@ -367,7 +384,7 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
                         if (pb >= 0) *(float2 *)(row + 2 * pb) = make_float2(f[2], f[3]);
                     }
                     if (++jq == T.J) {
-                        fx_flush<NN>(T.fx_ringW + (size_t)ring * n2, T.fx_sumshift, B, moment);
+                        fx_flush<NN>(ringW + ring * ringW_pitch, T.fx_sumshift, B, moment);
                         jq = 0;
                         ++ring;
                         fresh = true;
@@ -399,7 +416,7 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
             }
             ++commits[b];
         }
-        if (!fresh) fx_flush<NN>(T.fx_ringW + (size_t)ring * n2, T.fx_sumshift, B, moment);
+        if (!fresh) fx_flush<NN>(ringW + ring * ringW_pitch, T.fx_sumshift, B, moment);
         // drain: every MMA of this tile has completed once both buffers' last commits have
         if (tid == 0)
             for (int b = 0; b < 2 && !*abort_flag; ++b)
@@ -476,11 +493,11 @@ int launch_mixed_impl(kitrt_mn *mn, const Tables &T, const NewtonState &S, const
                       float *psi32)
 {
     using L = MixedSmem<NN, BF16>;
-    if (ensure_dyn_smem(eval_mixed_kernel<NN, BF16, MO>, L::total(T.J))) return KITRT_ECUDA;
+    if (ensure_dyn_smem(eval_mixed_kernel<NN, BF16, MO>, L::total(T.J, T.R))) return KITRT_ECUDA;
     // persistent grid of the CTAs that fit on the SMs at once; the work is split into about four
     // items per CTA (the moments of given alphas take one part per tile: rows of Vout are written
     // whole)
-    eval_mixed_kernel<NN, BF16, MO><<<mn->grid_mixed, kThreads, L::total(T.J), s>>>(
+    eval_mixed_kernel<NN, BF16, MO><<<mn->grid_mixed, kThreads, L::total(T.J, T.R), s>>>(
         T, S, k, BF16 ? (const void *)mn->d_Mhi16 : (const void *)mn->d_Mhi32, u, alpha_in, Vacc,
         MO ? 1 : mn->vs, MO ? Dims<NN>::n2 : 1, C, MO ? 0 : mn->target_mixed, psi32);
     if (cudaGetLastError() != cudaSuccess) return KITRT_ECUDA;
@@ -492,7 +509,7 @@ template <int NN, bool BF16>
 int mixed_grid_impl(const kitrt_mn *mn)
 {
     using L = MixedSmem<NN, BF16>;
-    const int smem = L::total(mn->J);
+    const int smem = L::total(mn->J, mn->R);
     if (ensure_dyn_smem(eval_mixed_kernel<NN, BF16, false>, smem)) return mn->nsm;
     return mn->nsm * resident_ctas(eval_mixed_kernel<NN, BF16, false>, kThreads, smem, 2);
 }

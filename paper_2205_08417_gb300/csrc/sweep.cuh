@@ -43,14 +43,14 @@ using kitrt_fx::Limb;
 // Exponent coefficients of one ring: A0 (k = 0) and A[2(k-1)], A[2(k-1)+1] for cos(k phi),
 // sin(k phi), from the trial alpha's limbs (at(c)).
 template <int NN, typename At>
-__device__ __forceinline__ void fx_coeffs(At &&at, const int2 *__restrict__ Pr, long long &A0, Limb (&A)[2 * NN])
+__device__ __forceinline__ void fx_coeffs(At &&at, const int2 *Pr, long long &A0, Limb (&A)[2 * NN])
 {
 #pragma unroll
     for (int k = -NN; k <= NN; ++k) {
         kitrt_fx::CoefAcc acc;
         const int ak = k < 0 ? -k : k;
 #pragma unroll
-        for (int l = ak; l <= NN; l += 2) acc.add(at(cindex(l, k)), __ldg(Pr + cindex(l, k)));
+        for (int l = ak; l <= NN; l += 2) acc.add(at(cindex(l, k)), Pr[cindex(l, k)]);
         const long long v = acc.value();
         if (k == 0) A0 = v;
         else A[2 * (ak - 1) + (k < 0)] = kitrt_fx::split<31>(v);
@@ -75,14 +75,14 @@ struct FxSums {
 // Moments of the finished ring: V_c += w_r P_c(mu_r) B_k(c), c over the degree-LB basis; the
 // azimuthal sums are cleared for the next ring.
 template <int LB, typename Acc>
-__device__ __forceinline__ void fx_flush(const int2 *__restrict__ wPr, int sumshift, FxSums<LB> &B, Acc &&V)
+__device__ __forceinline__ void fx_flush(const int2 *wPr, int sumshift, FxSums<LB> &B, Acc &&V)
 {
 #pragma unroll
     for (int k = -LB; k <= LB; ++k) {
         const int ak = k < 0 ? -k : k;
         const Limb v = kitrt_fx::split<32>(k == 0 ? B.b0 : B.b[k == 0 ? 0 : 2 * (ak - 1) + (k < 0)].value());
 #pragma unroll
-        for (int l = ak; l <= LB; l += 2) V(cindex(l, k)) += kitrt_fx::moment_term(v, __ldg(wPr + cindex(l, k)), sumshift);
+        for (int l = ak; l <= LB; l += 2) V(cindex(l, k)) += kitrt_fx::moment_term(v, wPr[cindex(l, k)], sumshift);
     }
     B.clear();
 }
