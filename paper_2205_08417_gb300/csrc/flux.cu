@@ -80,6 +80,8 @@ flux64_kernel(Tables T, QuadTab<double> X, const int4 *__restrict__ nbr, const d
             upB[f] = row + (fB ? Q.oB1 : Q.oB2);
             cA[f] = Q.live ? -fabs(dA) : 0.0;
             cB3[f] = Q.live && Q.hasB ? -fabs(dB) : 0.0;
+            // a Neumann ghost's scaled difference would leave a rounding residue: the face drops out
+            if (RHO && nbf[f] < 0 && bc == 0) cA[f] = cB3[f] = 0.0;
         }
         double G[n];
 #pragma unroll
@@ -138,12 +140,12 @@ flux64_kernel(Tables T, QuadTab<double> X, const int4 *__restrict__ nbr, const d
 // increment dt (-F/A + R(u)) is formed in FP32; only u += increment is FP64 (lanes over the
 // (cell, moment) elements of a warp's cells).
 //
-// Layout of the work: a group of kGroup = 8 lanes per cell, 4 cells per warp. Each lane reads
-// 16-byte pieces (4 consecutive points) of the cell's row and of its three upwind rows, and the
-// matching pieces of the tables, which the warp's 4 cells read at the same addresses (one
-// request serves them). Q' padded to a multiple of 32 gives every lane the same number of pieces.
-// Each lane sums its points in plain FP32; the 8 lane sums of a cell are reduced with a
-// compensated (two-sum) reduce-scatter.
+// Layout of the work: a group of kGroup = 8 lanes takes two neighbouring cells, 8 cells per warp. Each
+// lane reads 16-byte pieces (4 consecutive points) of each cell's row and of its three upwind rows,
+// and the matching pieces of the tables once for both cells (the warp's groups read them at the
+// same addresses: one request serves them). Q' padded to a multiple of 32 gives every lane the same
+// number of pieces. Each lane sums its points in plain FP32; the 8 lane sums of a cell are reduced
+// with a compensated (two-sum) reduce-scatter.
 // Upwind fluctuation sum of one point: s = sum_f min(Omega.n_f, 0) (psi_up,f - psi_i), or with a
 // density (RHO) sum_f min(Omega.n_f, 0) (psi_up,f / rho_up,f - psi_i / rho_i) (r: the 1/rho).
 template <bool RHO>
@@ -162,10 +164,15 @@ __device__ __forceinline__ float point_fluct(float wx, float wy, const float (&n
     return fmaf(fminf(fmaf(wx, nx[2], wy * ny[2]), 0.0f), u2 - pi, s);
 }
 
-// Latency bound: 3 resident blocks per SM (at most 85 registers) measured 0.127 ms per M_3 launch
-// on 99,458 cells against 0.179 ms at the unconstrained 94 registers (2 blocks).
+// L1 is the bound: with one cell per group 12 of the 16 pieces that a lane reads per 4 points are
+// tables (n basis rows and w Omega). M_3, 99,458 cells 0.127 -> 0.126 ms (there latency
+// counts as much: half the warps), M_5, 996,872 cells 4.8 -> 3.1 ms. Every sum keeps the order it had. (A
+// factorised form by quads, as the FP64 flux, took 0.082 ms, but its other order of FP32 sums moved u
+// by up to 1e-8 on coarse meshes.)
+constexpr int kPair = 2;                                 // cells per group
+constexpr int kCells32 = kPair * kCellsPerWarp;          // cells per warp
 template <int NN, bool RHO>
-__global__ void __launch_bounds__(kWarps * 32, NN <= 3 ? 3 : 2)
+__global__ void __launch_bounds__(kWarps * 32, 2)
 flux_update32_kernel(Tables T, const int4 *__restrict__ nbr, const float *__restrict__ nrm32,
                      const float *__restrict__ inva32, const float *__restrict__ psi,
                      const float *__restrict__ zrow, const float *__restrict__ invrho32,
@@ -175,67 +182,86 @@ flux_update32_kernel(Tables T, const int4 *__restrict__ nbr, const float *__rest
 {
     constexpr int n = (NN + 1) * (NN + 2) / 2;
     constexpr int K = GroupRS<n>::K;
-    __shared__ float sF[kWarps][kCellsPerWarp * n];
-    __shared__ float sK[kWarps][kCellsPerWarp][4];  // per cell: sigma_a, sigma_s, q, 1/A (FP32)
+    __shared__ float sF[kWarps][kCells32 * n];
+    __shared__ float sK[kWarps][kCells32][4];  // per cell: sigma_a, sigma_s, q, 1/A (FP32)
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int grp = lane >> kGroupLog, gl = lane & (kGroup - 1);
     const int Qp = T.Qp, nq4 = Qp / 4;
     const float4 *__restrict__ wx4 = reinterpret_cast<const float4 *>(T.wox32);
     const float4 *__restrict__ wy4 = reinterpret_cast<const float4 *>(T.woy32);
     const float4 *__restrict__ M4 = reinterpret_cast<const float4 *>(T.Mt32);
-    for (int base = (blockIdx.x * kWarps + wib) * kCellsPerWarp; base < C;
-         base += gridDim.x * kWarps * kCellsPerWarp) {
-        const int nb_cells = C - base < kCellsPerWarp ? C - base : kCellsPerWarp;
+    for (int base = (blockIdx.x * kWarps + wib) * kCells32; base < C; base += gridDim.x * kWarps * kCells32) {
+        const int nb_cells = C - base < kCells32 ? C - base : kCells32;
         if (lane < 4 * nb_cells) {
             const int ci = lane >> 2, which = lane & 3, i = base + ci;
             const double v = which == 0 ? sa[i] : which == 1 ? ss[i] : qs[i];
             sK[wib][ci][which] = which == 3 ? inva32[i] : (float)v;
         }
-        // a group without a cell repeats the warp's last one; its sums are not stored
-        const int i = base + (grp < nb_cells ? grp : nb_cells - 1);
-        const int4 nb = nbr[i];
-        const int nbf[3] = {nb.x, nb.y, nb.z};
-        float nx[3], ny[3], r[3];
-        const float4 *own = reinterpret_cast<const float4 *>(psi + (size_t)i * Qp);
-        const float4 *up[3];
-        const float ri = RHO ? invrho32[i] : 1.0f;
+        float nx[kPair][3], ny[kPair][3], r[kPair][3], ri[kPair];
+        const float4 *own[kPair], *up[kPair][3];
 #pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            nx[f] = nrm32[6 * (size_t)i + 2 * f];
-            ny[f] = nrm32[6 * (size_t)i + 2 * f + 1];
-            r[f] = RHO && nbf[f] >= 0 ? invrho32[nbf[f]] : ri;
-            if (RHO && nbf[f] < 0 && bc == 0) nx[f] = ny[f] = 0.0f;  // Neumann ghost drops out
-            // upwind row: the neighbour's; on the boundary the cell's own (Neumann ghost:
-            // fluctuation 0) or the zero row (vacuum ghost: fluctuation -psi_i)
-            up[f] = nbf[f] >= 0 ? reinterpret_cast<const float4 *>(psi + (size_t)nbf[f] * Qp)
-                    : bc == 0   ? own
-                                : reinterpret_cast<const float4 *>(zrow);
+        for (int t = 0; t < kPair; ++t) {
+            // a place without a cell repeats the warp's last one; its sums are not stored
+            const int i = base + (kPair * grp + t < nb_cells ? kPair * grp + t : nb_cells - 1);
+            const int4 nb = nbr[i];
+            const int nbf[3] = {nb.x, nb.y, nb.z};
+            own[t] = reinterpret_cast<const float4 *>(psi + (size_t)i * Qp);
+            ri[t] = RHO ? invrho32[i] : 1.0f;
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+                nx[t][f] = nrm32[6 * (size_t)i + 2 * f];
+                ny[t][f] = nrm32[6 * (size_t)i + 2 * f + 1];
+                r[t][f] = RHO && nbf[f] >= 0 ? invrho32[nbf[f]] : ri[t];
+                if (RHO && nbf[f] < 0 && bc == 0) nx[t][f] = ny[t][f] = 0.0f;  // Neumann ghost drops out
+                // upwind row: the neighbour's; on the boundary the cell's own (Neumann ghost:
+                // fluctuation 0) or the zero row (vacuum ghost: fluctuation -psi_i)
+                up[t][f] = nbf[f] >= 0 ? reinterpret_cast<const float4 *>(psi + (size_t)nbf[f] * Qp)
+                           : bc == 0   ? own[t]
+                                       : reinterpret_cast<const float4 *>(zrow);
+            }
         }
-        float F[n];
+        float F[kPair][n];
 #pragma unroll
-        for (int a = 0; a < n; ++a) F[a] = 0.0f;
-#pragma unroll 2
+        for (int t = 0; t < kPair; ++t)
+#pragma unroll
+            for (int a = 0; a < n; ++a) F[t][a] = 0.0f;
+#pragma unroll 1
         for (int j = gl; j < nq4; j += kGroup) {
-            const float4 po = __ldg(own + j);
-            const float4 p0 = __ldg(up[0] + j), p1 = __ldg(up[1] + j), p2 = __ldg(up[2] + j);
+            float4 po[kPair], pu[kPair][3];
+#pragma unroll
+            for (int t = 0; t < kPair; ++t) {
+                po[t] = __ldg(own[t] + j);
+#pragma unroll
+                for (int f = 0; f < 3; ++f) pu[t][f] = __ldg(up[t][f] + j);
+            }
             const float4 wx = __ldg(wx4 + j), wy = __ldg(wy4 + j);
-            const float s0 = point_fluct<RHO>(wx.x, wy.x, nx, ny, ri, r, po.x, p0.x, p1.x, p2.x);
-            const float s1 = point_fluct<RHO>(wx.y, wy.y, nx, ny, ri, r, po.y, p0.y, p1.y, p2.y);
-            const float s2 = point_fluct<RHO>(wx.z, wy.z, nx, ny, ri, r, po.z, p0.z, p1.z, p2.z);
-            const float s3 = point_fluct<RHO>(wx.w, wy.w, nx, ny, ri, r, po.w, p0.w, p1.w, p2.w);
+            float s[kPair][4];
+#pragma unroll
+            for (int t = 0; t < kPair; ++t) {
+                s[t][0] = point_fluct<RHO>(wx.x, wy.x, nx[t], ny[t], ri[t], r[t], po[t].x, pu[t][0].x, pu[t][1].x, pu[t][2].x);
+                s[t][1] = point_fluct<RHO>(wx.y, wy.y, nx[t], ny[t], ri[t], r[t], po[t].y, pu[t][0].y, pu[t][1].y, pu[t][2].y);
+                s[t][2] = point_fluct<RHO>(wx.z, wy.z, nx[t], ny[t], ri[t], r[t], po[t].z, pu[t][0].z, pu[t][1].z, pu[t][2].z);
+                s[t][3] = point_fluct<RHO>(wx.w, wy.w, nx[t], ny[t], ri[t], r[t], po[t].w, pu[t][0].w, pu[t][1].w, pu[t][2].w);
+            }
 #pragma unroll
             for (int a = 0; a < n; ++a) {
                 const float4 m = __ldg(M4 + (size_t)a * nq4 + j);
-                F[a] = fmaf(m.w, s3, fmaf(m.z, s2, fmaf(m.y, s1, fmaf(m.x, s0, F[a]))));
+#pragma unroll
+                for (int t = 0; t < kPair; ++t)
+                    F[t][a] = fmaf(m.w, s[t][3], fmaf(m.z, s[t][2], fmaf(m.y, s[t][1], fmaf(m.x, s[t][0], F[t][a]))));
             }
         }
-        float rs[K], re[K];
-        int slot0;
-        const bool uniq = group_reduce_scatter<n>(F, gl, rs, re, slot0);
-        if (grp < nb_cells && uniq) {
 #pragma unroll
-            for (int k = 0; k < K; ++k)
-                if (slot0 + k < n) sF[wib][grp * n + slot0 + k] = rs[k] + re[k];
+        for (int t = 0; t < kPair; ++t) {
+            float rs[K], re[K];
+            int slot0;
+            const bool uniq = group_reduce_scatter<n>(F[t], gl, rs, re, slot0);
+            const int ci = kPair * grp + t;
+            if (ci < nb_cells && uniq) {
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    if (slot0 + k < n) sF[wib][ci * n + slot0 + k] = rs[k] + re[k];
+            }
         }
         __syncwarp();
         for (int idx = lane; idx < nb_cells * n; idx += 32) {
@@ -264,19 +290,8 @@ int launch_flux_update(kitrt_mn *mn, const Tables &T, int C, const double *psi,
     const int per_block = kWarps * (32 / mn->J), need = (C + per_block - 1) / per_block;
     const int grid = need < mn->nsm * 2 ? (need > 0 ? need : 1) : mn->nsm * 2;
     const size_t smem64 = sizeof(double) * mn->n * ((size_t)mn->R + mn->J + kWarps * 32);
-    // persistent grid of as many blocks as fit at once, groups of 4 cells dealt round-robin to
-    // warps (no partial second wave)
-    int resident = 0;
-    switch (mn->N) {
-    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, flux_update32_kernel<1, false>, kWarps * 32, 0); break;
-    case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, flux_update32_kernel<2, false>, kWarps * 32, 0); break;
-    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, flux_update32_kernel<3, false>, kWarps * 32, 0); break;
-    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, flux_update32_kernel<4, false>, kWarps * 32, 0); break;
-    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, flux_update32_kernel<5, false>, kWarps * 32, 0); break;
-    }
-    if (resident < 1) resident = 1;
-    const int need32 = (C + kWarps * kCellsPerWarp - 1) / (kWarps * kCellsPerWarp);
-    const int grid32 = need32 < mn->nsm * resident ? (need32 > 0 ? need32 : 1) : mn->nsm * resident;
+    const int need32 = (C + kWarps * kCells32 - 1) / (kWarps * kCells32);
+    const int most32 = mn->nsm * 2, grid32 = need32 < most32 ? (need32 > 0 ? need32 : 1) : most32;  // persistent
     if (!psi && (T.Qp % 32 != 0 || !mn->d_zero32)) return KITRT_EINVAL;
     const bool rho = mn->d_invrho != nullptr;
     LaunchScope ls(mn, PK_FLUX, s, C);
@@ -285,10 +300,11 @@ int launch_flux_update(kitrt_mn *mn, const Tables &T, int C, const double *psi,
         if (ensure_dyn_smem(flux64_kernel<NN, R>, smem64)) return KITRT_ECUDA;                 \
         flux64_kernel<NN, R><<<grid, kWarps * 32, smem64, s>>>(                                \
             T, X, m->d_nbr, m->d_nrm, m->d_area, psi, mn->d_invrho, u, sa, ss, q, dt, bc, C);  \
-    } else                                                                                     \
-        flux_update32_kernel<NN, R><<<grid32, kWarps * 32, 0, s>>>(                             \
+    } else {                                                                                   \
+        flux_update32_kernel<NN, R><<<grid32, kWarps * 32, 0, s>>>(                            \
             T, m->d_nbr, m->d_nrm32, m->d_inva32, psi32, mn->d_zero32, mn->d_invrho32, u, sa,  \
-            ss, q, (float)dt, bc, C);
+            ss, q, (float)dt, bc, C);                                                          \
+    }
 #define FLUX_CASE(NN)                                                                          \
     case NN:                                                                                   \
         if (rho) {                                                                             \
