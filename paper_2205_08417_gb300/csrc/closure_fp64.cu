@@ -220,10 +220,10 @@ predict_kernel(NewtonState S, const double *__restrict__ u, NewtonParams np, con
                     for (int k = 0; k < i; ++k) y[k * 32] = fma(-row[k], x, y[k * 32]);
                 }
             }
-            if (sqrt(gn2) <= np.tau * sqrt(un2)) {
+            if (gn2 <= np.tau * np.tau * un2) {
                 S.phase[cell] = PH_DONE;  // converged; d is the polish step
             } else {
-                if (S.gnorm) S.gnorm[cell] = sqrt(gn2);
+                if (S.gnorm) S.gnorm[cell] = gn2;
                 S.f0[cell] = fma(0.5 * np.gamma, ar2, S.fsum[cell] - au);
                 S.gd[cell] = gd;
                 S.lam[cell] = 1.0;
@@ -303,6 +303,11 @@ eval_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, Newton
 // Newton kernel adds in order, so the result does not depend on scheduling.
 // ---------------------------------------------------------------------------------------------
 constexpr int kSweepThreads = 128;
+// Quads per unit of the split of these sweeps: half of the tensor-core sweep's chunk, so that small
+// lists spread over more SMs (M_2, 3,872 cells: 0.16 -> 0.135 ms in two steps; handed-over cells of a
+// checkerboard, 25,088 cells, four closures: 0.24 -> 0.21 ms).
+constexpr int kUnit64 = 4;
+int units64(int nquad) { return (nquad + kUnit64 - 1) / kUnit64; }
 
 // An exponential of the sweeps as a double: the range test that fx_double leaves out (rows of the
 // FP64 exponentials reach 0 and, when not finite, y = 2^61 with a large m).
@@ -343,7 +348,7 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
     const int cnt_in = GIVEN ? C : HANDED ? S.cnt[12 + k % 3] : S.cnt[k % 3];
     if (HANDED && cnt_in == 0) return;
     if (CELLS == Cells::kListed && blockIdx.x == 0 && threadIdx.x == 0) S.cnt[(k + 2) % 3] = 0;
-    const int nunits = T.Qs / 32;
+    const int nunits = (T.nquad + kUnit64 - 1) / kUnit64;
     const SweepSplit sp = sweep_split(cnt_in, gridDim.x, GIVEN ? 0 : target_items, nunits);
     const int items = sp.tiles * sp.parts;
     if ((int)blockIdx.x >= items) return;
@@ -356,9 +361,8 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
         const int tile = item / sp.parts, part = item % sp.parts;
         const int slot = tile * kSweepThreads + threadIdx.x;
         if (slot >= cnt_in) continue;  // threads are independent: no block barrier below
-        const int q_begin = part * nunits / sp.parts * 8;
-        // padding quads add nothing: stop at the last real one
-        const int q_end = min(T.nquad, (part + 1) * nunits / sp.parts * 8);
+        const int q_begin = part * nunits / sp.parts * kUnit64;
+        const int q_end = min(T.nquad, (part + 1) * nunits / sp.parts * kUnit64);
         const int cell = GIVEN ? slot : list_in[HANDED ? pos_in[slot] : slot];
         const double *al = (GIVEN ? alpha : S.alpha) + (size_t)cell * n, *di = GIVEN ? al : S.dir + (size_t)cell * n;
         const double lam = !GIVEN && S.phase[cell] == PH_NEWTON ? S.lam[cell] : 0.0;
@@ -675,27 +679,6 @@ int launch_isotropic(const Tables &T, int C, const double *u, double *alpha, cud
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }
 
-// FP64 mode, rounds of more than `above` cells: the sum of each listed slot's quadrature parts
-// (sweep.cuh) into its part-0 column, in order, element-wise over the [n2 x cnt] moments with every
-// SM taking part, so that the thread-per-cell Newton kernel reads one column.
-__global__ void sum_parts_kernel(NewtonState S, int k, double *__restrict__ Vacc, int vs, int n2, int grid,
-                                 int target_items, int nunits, int above)
-{
-    const int cnt = S.cnt[k % 3];
-    if (cnt <= above) return;
-    const int parts = sweep_split(cnt, grid, target_items, nunits).parts;
-    if (parts <= 1) return;
-    const size_t total = (size_t)n2 * cnt, pstride = (size_t)cnt;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
-         e += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(e / cnt), j = (int)(e - (size_t)c * cnt);
-        double *col = Vacc + (size_t)c * vs + j;
-        double v = col[0];
-        for (int p = 1; p < parts; ++p) v += col[(size_t)p * pstride];
-        col[0] = v;
-    }
-}
-
 // Cells up to which a round of the FP64 mode goes to the 8-lane kernel (N <= 3): there a warp's FP64
 // instructions serve 4 cells instead of 32, which is slower once the thread-per-cell kernel fills
 // the SMs. M_3: 8 lanes take about 8 us per 2,500 cells, a thread per cell 45 us up to 39,000.
@@ -707,12 +690,8 @@ int launch_post(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, cons
 {
     const bool mixed = mn->p.mode != KITRT_FP64;
     const int upto = mixed || mn->N > 3 ? 0x7fffffff : kGroupUpTo;
+    const int nu64 = units64(mn->R * mn->J), nunits = mixed ? mn->Qs / 32 : nu64;
     const int sweep_grid = mixed ? mn->grid_mixed : mn->grid_fp64, target = mixed ? mn->target_mixed : mn->target_fp64;
-    if (C > upto) {
-        LaunchScope ls(mn, PK_POST, s, 0);
-        sum_parts_kernel<<<mn->nsm * 8, 256, 0, s>>>(S, k, Vacc, mn->vs, mn->n2, sweep_grid, target, mn->Qs / 32, upto);
-        if (cudaGetLastError() != cudaSuccess) return KITRT_ECUDA;
-    }
     if (C > upto) {
         // 64-thread blocks: small blocks spread the listed cells over every SM
         int blocks = (C + kPostBlock - 1) / kPostBlock;
@@ -725,7 +704,8 @@ int launch_post(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, cons
         rc = ensure_dyn_smem(post_thread_kernel<NNv>, smem);                                                   \
         if (!rc)                                                                                               \
             post_thread_kernel<NNv><<<blocks, kPostBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs,             \
-                                                                     mn->gaunt_nnz, upto);                     \
+                                                                     mn->gaunt_nnz, sweep_grid, target,        \
+                                                                     nunits, upto);                            \
         break;
         switch (mn->N) {
             THREAD_CASE(1)
@@ -747,11 +727,11 @@ int launch_post(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, cons
     if (mixed) {
         KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(post_group_kernel<NN, true>, smem));
         if (rc) return rc;
-        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, true><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, mn->grid_fp64, mn->target_fp64, upto)));
+        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, true><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, nunits, mn->grid_fp64, mn->target_fp64, nu64, upto)));
     } else {
         KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(post_group_kernel<NN, false>, smem));
         if (rc) return rc;
-        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, false><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, mn->grid_fp64, mn->target_fp64, upto)));
+        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, false><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, nunits, mn->grid_fp64, mn->target_fp64, nu64, upto)));
     }
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }

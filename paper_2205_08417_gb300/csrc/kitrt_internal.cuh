@@ -87,7 +87,7 @@ struct NewtonState {
     int32_t *h64;      // [C] mixed modes: non-zero = this cell evaluates its Hessian in FP64, from its
                        //   second round on 1 + its place in handed (else NULL)
     int32_t *handed[2];  // [C] mixed modes: list positions of those cells (ping-pong)
-    double *gnorm;     // [C] mixed modes: ||g|| at the last accepted point (else NULL)
+    double *gnorm;     // [C] mixed modes: ||g||^2 at the last accepted point (else NULL)
     int32_t *lfac;     // [C] learned mode: 1 once S.L holds a factor of this cell (else NULL)
     int32_t *list[2];  // active cell lists (ping-pong)
     int32_t *cnt;      // [16]: cnt[0..2] rotating list counters, cnt[3] failures, cnt[4] max

@@ -203,9 +203,8 @@ __device__ void newton_post(const Tables &T, const NewtonState &S, const NewtonP
     if (lane < n) S.dir[off + lane] = d;
     int iters = S.iters[cell];
     if (ph == PH_NEWTON) ++iters;
-    const double gn = sqrt(gn2);
     if (lane == 0) S.iters[cell] = iters;
-    if (gn <= np.tau * sqrt(un2)) {
+    if (gn2 <= np.tau * np.tau * un2) {
         if (lane == 0) S.phase[cell] = PH_DONE;
         return;
     }
@@ -214,8 +213,8 @@ __device__ void newton_post(const Tables &T, const NewtonState &S, const NewtonP
         return;
     }
     if (lane == 0) {
-        if (mixed && ph == PH_NEWTON && gn > kStallRatio * S.gnorm[cell]) hand_over(S, cell);
-        if (S.gnorm) S.gnorm[cell] = gn;
+        if (mixed && ph == PH_NEWTON && gn2 > kStallRatio * kStallRatio * S.gnorm[cell]) hand_over(S, cell);
+        if (S.gnorm) S.gnorm[cell] = gn2;
         S.gd[cell] = gd;
         S.lam[cell] = 1.0;
         S.halv[cell] = 0;
@@ -243,6 +242,23 @@ __device__ __forceinline__ int push_agg(int32_t *list, int32_t *cnt, int cell, b
     const int at = base + __popc(m & ((1u << lane) - 1u));
     if (pred) list[at] = cell;
     return at;
+}
+
+__device__ __forceinline__ float r_fma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double r_fma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ bool r_pos(float d) { return d > 0.0f && d < 3.0e38f; }
+__device__ __forceinline__ bool r_pos(double d) { return d > 0.0; }
+__device__ __forceinline__ float r_rsqrt(float a) { return rsqrtf(a); }
+// 1/sqrt(a): the FP32 value improved by one third-order step y (1 + e/2 + 3 e^2 / 8), e = 1 - a y^2
+// (the binomial series of (1 - e)^(-1/2); e is about 1e-7, the dropped term 1e-22), five FP64
+// instructions; outside the float range the library function.
+static __device__ __noinline__ double r_rsqrt_any(double a) { return rsqrt(a); }
+__device__ __forceinline__ double r_rsqrt(double a)
+{
+    if (!(a > 1e-37 && a < 1e37)) return r_rsqrt_any(a);
+    const double y = f2d_bits(rsqrtf(d2f_bits(a)));
+    const double e = fma(-a * y, y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 
 // Newton step of one listed cell after a round of sweeps, in the FP64 mode for N <= 3 when many
@@ -282,7 +298,7 @@ __device__ bool hess_factor_solve(const Tables &T, const NewtonParams &np, const
             d = fma(-l, l, d);
         }
         spd = spd && d > 0.0;
-        const double rinv = rsqrt(d > 0.0 ? d : 1.0);
+        const double rinv = r_rsqrt(d > 0.0 ? d : 1.0);
         L[(size_t)(jj + j) * B] = rinv;
 #pragma unroll 1
         for (int i = j + 1; i < n; ++i) {
@@ -403,8 +419,7 @@ __device__ bool newton_cell(const Tables &T, const NewtonState &S, const NewtonP
     int iters = S.iters[cell];
     if (ph == PH_NEWTON) ++iters;
     S.iters[cell] = iters;
-    const double gn = sqrt(gn2);
-    if (gn <= np.tau * sqrt(un2)) {
+    if (gn2 <= np.tau * np.tau * un2) {
         S.phase[cell] = PH_DONE;
         return false;
     }
@@ -429,12 +444,14 @@ __host__ __device__ inline size_t post_smem_bytes(int n, int n2, int npairs, int
     return (size_t)(n2 + npairs + n) * kPostBlock * 8 + (size_t)nnz * 12 + (size_t)(npairs + 1) * 4;
 }
 
-// The listed cells, when more than `above` of them, one thread each (their parts already summed by
-// sum_parts_kernel); otherwise post_group_kernel takes the round.
+// The listed cells, when more than `above` of them, one thread each; otherwise post_group_kernel takes
+// the round. The sweeps' parts are added in order while the moments are loaded, which saves a launch
+// and a pass a round (adjoint, 59,168 cells, 32 closures: 15.7 -> 15.0 ms with 1/sqrt by r_rsqrt).
 template <int NN>
 __global__ void __launch_bounds__(kPostBlock)
 post_thread_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, NewtonParams np,
-                   const double *__restrict__ Vacc, int vs, int nnz, int above)
+                   const double *__restrict__ Vacc, int vs, int nnz, int sweep_grid, int target_items, int nunits,
+                   int above)
 {
     constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, npairs = Dims<NN>::npairs;
     extern __shared__ __align__(16) unsigned char post_smem[];
@@ -450,6 +467,7 @@ post_thread_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k,
     const int stride = gridDim.x * blockDim.x;
     // uniform: not this kernel's round, or this block has no slot
     if (cnt_in <= above || (int)(blockIdx.x * blockDim.x) >= cnt_in) return;
+    const int parts = sweep_split(cnt_in, sweep_grid, target_items, nunits).parts;
     int32_t *cnt_out = &S.cnt[(k + 1) % 3];
     // stage the Gaunt tables and point this block's view of them at the copies
     for (int t = threadIdx.x; t < nnz; t += blockDim.x) {
@@ -472,6 +490,11 @@ post_thread_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k,
             double *mine = sV + threadIdx.x;
 #pragma unroll
             for (int c = 0; c < n2; ++c) mine[c * kPostBlock] = Vacc[(size_t)c * vs + it];
+            for (int p = 1; p < parts; ++p) {
+                const double *col = Vacc + (size_t)p * cnt_in + it;
+#pragma unroll
+                for (int c = 0; c < n2; ++c) mine[c * kPostBlock] += col[(size_t)c * vs];
+            }
             cont = newton_cell<NN>(Ts, S, np, cell, mine, sL + threadIdx.x, sy + threadIdx.x, kPostBlock, u, ev);
         }
         // every slot taken in this round is one evaluation
@@ -496,29 +519,13 @@ post_thread_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k,
 // matrix passes through shared memory only to be assembled (entries dealt to the lanes) and to be
 // written out in whole rows. Measured against the thread-per-cell kernels with their separate
 // summation of the sweeps' parts (part of the load here), Newton time of a run: M_5, 996,872 cells,
-// two steps 70.3 -> 15.2 ms; M_4, 20,000 cells 1.09 -> 0.23 ms; M_3, 99,458 cells, four steps
-// 0.94 -> 0.82 ms; M_2 in FP64 mode, 3,872 cells 0.25 -> 0.17 ms.
+// two steps 70.3 -> 13.7 ms; M_4, 20,000 cells 1.09 -> 0.21 ms; M_3, 99,458 cells, four steps
+// 0.94 -> 0.68 ms (0.73 before each cell's state was read ahead of its moments); M_2 in FP64 mode,
+// 3,872 cells 0.25 -> 0.17 ms.
 // ---------------------------------------------------------------------------------------------
 constexpr int kGroupBlock = 256;
 constexpr int kGroupCells = kGroupBlock / 8;  // cells per block and pass
 constexpr int kGroupPitch = kGroupCells + 1;  // row pitch of the moments in shared memory
-
-__device__ __forceinline__ float r_fma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double r_fma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ bool r_pos(float d) { return d > 0.0f && d < 3.0e38f; }
-__device__ __forceinline__ bool r_pos(double d) { return d > 0.0; }
-__device__ __forceinline__ float r_rsqrt(float a) { return rsqrtf(a); }
-// 1/sqrt(a): the FP32 value improved by one third-order step y (1 + e/2 + 3 e^2 / 8), e = 1 - a y^2
-// (the binomial series of (1 - e)^(-1/2); e is about 1e-7, the dropped term 1e-22), five FP64
-// instructions; outside the float range the library function.
-static __device__ __noinline__ double r_rsqrt_any(double a) { return rsqrt(a); }
-__device__ __forceinline__ double r_rsqrt(double a)
-{
-    if (!(a > 1e-37 && a < 1e37)) return r_rsqrt_any(a);
-    const double y = f2d_bits(rsqrtf(d2f_bits(a)));
-    const double e = fma(-a * y, y, 1.0);
-    return fma(y * e, fma(e, 0.375, 0.5), y);
-}
 
 __device__ __forceinline__ double group_sum(double v)
 {
@@ -689,8 +696,8 @@ __host__ __device__ inline size_t group_smem_bytes(int n2, int npairs, int nnz, 
 template <int NN, bool MIXED>
 __global__ void __launch_bounds__(kGroupBlock, MIXED && NN <= 3 ? 3 : 2)
 post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, NewtonParams np,
-                  const double *__restrict__ Vacc, int vs, int nnz, int sweep_grid, int target_items, int grid64, int target64,
-                  int upto)
+                  const double *__restrict__ Vacc, int vs, int nnz, int sweep_grid, int target_items, int nunits, int grid64,
+                  int target64, int nunits64, int upto)
 {
     constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, npairs = Dims<NN>::npairs, SL = (n + 7) / 8;
     extern __shared__ __align__(16) unsigned char group_smem[];
@@ -706,10 +713,10 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
     const int cnt_in = S.cnt[k % 3];
     // uniform: not this kernel's round, or no slot for this block
     if (cnt_in > upto || (int)blockIdx.x * kGroupCells >= cnt_in) return;
-    const int parts = sweep_split(cnt_in, sweep_grid, target_items, T.Qs / 32).parts;
+    const int parts = sweep_split(cnt_in, sweep_grid, target_items, nunits).parts;
     // handed cells: columns from vs / 2 on, split on their own
     const int handed = MIXED ? S.cnt[12 + k % 3] : 0;
-    const int parts64 = MIXED ? sweep_split(handed, grid64, target64, T.Qs / 32).parts : 1;
+    const int parts64 = MIXED ? sweep_split(handed, grid64, target64, nunits64).parts : 1;
     int32_t *cnt_out = &S.cnt[(k + 1) % 3];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane & 7, slot = tid >> 3;
     for (int t = tid; t < nnz; t += kGroupBlock) {
@@ -727,6 +734,32 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
             sh64[tid] = MIXED && c >= 0 ? S.h64[c] : 0;
         }
         __syncthreads();
+        // this cell's state, on its way while the moments are loaded
+        const int cell = scell[slot];
+        const bool valid = cell >= 0, h32 = MIXED && !sh64[slot];
+        const size_t off = (size_t)(valid ? cell : 0) * n;
+        const int ph = valid ? S.phase[cell] : PH_DONE;
+        const double lam = ph == PH_NEWTON ? S.lam[cell] : 0.0;
+        double at[SL], ua[SL], gr[SL];
+        double au = 0.0, ar2 = 0.0;
+#pragma unroll
+        for (int s = 0; s < SL; ++s) {
+            const int c = g + 8 * s;
+            const bool in = valid && c < n;
+            const double al = in ? S.alpha[off + c] : 0.0;
+            at[s] = in && ph == PH_NEWTON ? fma(lam, S.dir[off + c], al) : al;
+            ua[s] = in ? u[off + c] : 0.0;
+            au = fma(at[s], ua[s], au);
+            if (reg && c >= np.reg0) ar2 = fma(at[s], at[s], ar2);
+        }
+        double fs0 = 0.0, f0 = 0.0, gd0 = 0.0, gnorm0 = 0.0;  // of the accepted point (gnorm: squared)
+        if (ph == PH_NEWTON) {
+            fs0 = S.fsum[cell];
+            f0 = S.f0[cell];
+            gd0 = S.gd[cell];
+            if (MIXED) gnorm0 = S.gnorm[cell];
+        }
+        const int ev = valid ? S.evals[cell] + 1 : 0;
         // the moments of the pass's cells, the sweeps' parts added in order: in FP32 for the
         // Hessian-only moments of tensor-core cells (accumulator values), else in FP64
         for (int e = tid; e < n2 * kGroupCells; e += kGroupBlock) {
@@ -748,25 +781,8 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
             }
         }
         __syncthreads();
-        const int cell = scell[slot];
-        const bool valid = cell >= 0, h32 = MIXED && !sh64[slot];
-        const size_t off = (size_t)(valid ? cell : 0) * n;
         const double *V = sV + slot;
         const float *Vf = sVf + slot;
-        const int ph = valid ? S.phase[cell] : PH_DONE;
-        const double lam = ph == PH_NEWTON ? S.lam[cell] : 0.0;
-        double at[SL], ua[SL], gr[SL];
-        double au = 0.0, ar2 = 0.0;
-#pragma unroll
-        for (int s = 0; s < SL; ++s) {
-            const int c = g + 8 * s;
-            const bool in = valid && c < n;
-            const double al = in ? S.alpha[off + c] : 0.0;
-            at[s] = in && ph == PH_NEWTON ? fma(lam, S.dir[off + c], al) : al;
-            ua[s] = in ? u[off + c] : 0.0;
-            au = fma(at[s], ua[s], au);
-            if (reg && c >= np.reg0) ar2 = fma(at[s], at[s], ar2);
-        }
         bool fin = true;
         for (int c = g; c < n2; c += 8)
             fin = fin && (c < n || !h32 ? finite_bits(V[c * kGroupPitch])
@@ -777,16 +793,9 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
         const double fs = V[0] * T.rm0;
         const double ft = reg ? fma(0.5 * np.gamma, ar2, fs - au) : fs - au;
         bool accept = valid && finite;
-        int ev = 0;
-        double gnorm0 = 0.0;
-        if (valid) {
-            if (ph == PH_NEWTON) {
-                const double fs0 = S.fsum[cell], f0 = S.f0[cell];
-                const double slack = 64.0 * 2.220446049250313e-16 * (fs0 + fabs(fs0 - f0));
-                accept = finite && ft <= f0 + np.c1 * lam * S.gd[cell] + slack;
-                if (MIXED) gnorm0 = S.gnorm[cell];
-            }
-            ev = S.evals[cell] + 1;
+        if (ph == PH_NEWTON) {
+            const double slack = 64.0 * 2.220446049250313e-16 * (fs0 + fabs(fs0 - f0));
+            accept = accept && ft <= f0 + np.c1 * lam * gd0 + slack;
         }
         // the Newton direction -H^-1 (<m e> - u + gamma alpha^r) of the accepted cells
         double y[SL];
@@ -877,16 +886,15 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
                 int iters = S.iters[cell];
                 if (ph == PH_NEWTON) ++iters;
                 S.iters[cell] = iters;
-                const double gn = sqrt(gn2);
-                if (gn <= np.tau * sqrt(un2)) {
+                if (gn2 <= np.tau * np.tau * un2) {
                     S.phase[cell] = PH_DONE;
                 } else if (iters >= np.max_iter) {
                     code = KITRT_ENOCONVERGE;
                 } else {
                     // a Newton step on the tensor-core Hessian that does not halve the residual
                     // sends the cell to the FP64 Hessian
-                    if (MIXED && ph == PH_NEWTON && gn > kStallRatio * gnorm0) hand_over(S, cell);
-                    if (MIXED) S.gnorm[cell] = gn;
+                    if (MIXED && ph == PH_NEWTON && gn2 > kStallRatio * kStallRatio * gnorm0) hand_over(S, cell);
+                    if (MIXED) S.gnorm[cell] = gn2;
                     S.gd[cell] = gd;
                     S.lam[cell] = 1.0;
                     S.halv[cell] = 0;

@@ -262,9 +262,10 @@ __device__ __forceinline__ double f2d_bits(float f)
 }
 
 // Split of a sweep's work: tiles of 128 listed cells times parts of the quadrature (whole units of
-// 8 quads, part j taking units [j nunits / parts, (j + 1) nunits / parts)). Part j of list slot i
-// lands in column j * cnt + i of the accumulator, and sum_parts_kernel adds the parts in order, so
-// every cell's sums depend on the list's length only, not on its place (deterministic).
+// 4 quads in the FP64 sweeps, 8 in the tensor-core sweep; part j takes units
+// [j nunits / parts, (j + 1) nunits / parts)). Part j of list slot i lands in column j * cnt + i of
+// the accumulator, and the Newton kernels add the parts in order, so every cell's sums depend on the
+// list's length only, not on its place (deterministic).
 // The number of parts is the one with the shortest schedule on `grid` persistent CTAs, each item
 // costing its units plus one for its trial point, its drain and its stores; at most
 // 1 + target / tiles, which bounds the columns. Called by whole warps.
@@ -278,12 +279,12 @@ __device__ __forceinline__ SweepSplit sweep_split(int cnt, int grid, int target_
     sp.parts = 1;
     if (target_items <= 0 || sp.tiles == 0) return sp;
     const int most = min(nunits, 1 + target_items / sp.tiles);
-    unsigned best = 0xffffffffu;  // schedule length in the high bits, parts in the low 8
+    unsigned best = 0xffffffffu;  // schedule length in the high bits, parts (at most 512) in the low 10
     for (int p = 1 + (threadIdx.x & 31); p <= most; p += 32) {
         const unsigned rounds = (unsigned)(sp.tiles * p + grid - 1) / grid;
-        best = min(best, (rounds * ((nunits + p - 1) / p + 1)) << 8 | (unsigned)p);
+        best = min(best, (rounds * ((nunits + p - 1) / p + 1)) << 10 | (unsigned)p);
     }
-    sp.parts = (int)(__reduce_min_sync(0xffffffffu, best) & 255u);
+    sp.parts = (int)(__reduce_min_sync(0xffffffffu, best) & 1023u);
     return sp;
 }
 
