@@ -185,22 +185,23 @@ def oracle_timing(W, steps: int, warmup: int, sample_cells: int):
 # ------------------------------------------------------------------------------------------------
 # GPU leg
 # ------------------------------------------------------------------------------------------------
-def fp64_peak_tflops(torch):
-    """Measured FP64 throughput of cuBLAS DGEMM (4096^3, best of 5) on this GPU."""
-    n = 4096
-    a = torch.randn(n, n, dtype=torch.float64, device="cuda")
-    b = torch.randn(n, n, dtype=torch.float64, device="cuda")
-    torch.matmul(a, b)
-    torch.cuda.synchronize()
-    best = 1e9
-    for _ in range(5):
-        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        e0.record()
-        torch.matmul(a, b)
-        e1.record()
-        e1.synchronize()
-        best = min(best, e0.elapsed_time(e1) / 1e3)
-    return 2.0 * n ** 3 / best / 1e12
+def multiplier_peak(torch, sm_mhz):
+    """32 x 32 -> 64-bit integer multiplications per second (in 1e12) that the SMs can issue: four
+    schedulers of an SM, each one warp instruction (32 lanes) every 4 cycles, at the given clock."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return sms * 4 * 32 / 4 * sm_mhz * 1e6 / 1e12
+
+
+def sweep_multiplies(W, fp64):
+    """32 x 32-bit multiplications of one cell evaluation in the 64-bit fixed-point sweep. A quad of
+    azimuths (J of them in each of the R rings) takes 3 per product of its 2N exponent terms and its
+    2L moment sums (two limbs each way, without the low product), and 7 per exponential; a ring
+    takes 3 per exponent coefficient and 4 per moment. L = N in the mixed modes, 2N in FP64 mode."""
+    N, R = W["N"], (W["order"] + 1) // 2
+    J = (W["order"] + 1) // 2
+    L = 2 * N if fp64 else N
+    nout = (L + 1) * (L + 2) // 2
+    return R * J * (3 * 2 * N + 4 * 7 + 3 * 2 * L) + R * (3 * W["n"] + 4 * nout)
 
 
 def train_network(K, torch, W, samples, seed=4):
@@ -282,9 +283,9 @@ def run_mode(K, torch, W, mode, steps, warmup, t_start, tau, e2e=True, net=None,
     return out
 
 
-# DRAM bytes (read + write) per launch of the S_N step from one ncu capture of the bench's own
-# launches (profiles/sn_tile_kernel_m3_line_source_100k.md); other workloads have no capture.
-SN_TRAFFIC = {("m3_line_source_100k", True): 286.9e6}
+# DRAM bytes (read + write) per launch of the S_N step from one ncu capture on the same mesh and
+# rule (profiles/sn_quad_kernel_m3_line_source_100k.md); other workloads have no capture.
+SN_TRAFFIC = {("m3_line_source_100k", True): 284.1e6}
 
 
 def run_sn(K, torch, W, steps, warmup, fp32, hbm_peak, workload):
@@ -365,14 +366,15 @@ def mode_line(W, r, steps):
     return line
 
 
-def sweep_roofline(r, work, peak):
+def sweep_roofline(W, r, work, peak):
     key = "closure_eval_fp64" if r["mode"] == "fp64" else "closure_eval_mixed"
     pe = r["prof"].get(key)
     if not pe or pe["total_ms"] <= 0:
         return None
     t = pe["total_ms"] / 1e3
-    out = {"kernel": key, "fp64_ops_per_cell_eval": work["sweep_fp64_ops"],
-           "fp64_pipe_frac": pe["units"] * work["sweep_fp64_ops"] / t / 1e12 / (peak / 2.0),
+    ops = sweep_multiplies(W, r["mode"] == "fp64")
+    out = {"kernel": key, "multiplies_per_cell_eval": ops,
+           "multiplier_frac": pe["units"] * ops / t / 1e12 / peak,
            "cell_evals": pe["units"]}
     if work["tensor_flops"]:
         out["tensor_tflops"] = pe["units"] * work["tensor_flops"] / t / 1e12
@@ -486,7 +488,7 @@ def run_extras(K, torch, args, peak, hbm_peak, head_results):
                      net=net5 if mode == "learned" else None)
         res5[mode] = r
         line = mode_line(W5, r, 5)
-        line["sweep"] = sweep_roofline(r, r["solver"].work(), peak)
+        line["sweep"] = sweep_roofline(W5, r, r["solver"].work(), peak)
         line["flux"] = flux_roofline(W5, W5["n"], W5["order"] ** 2, r["prof"], hbm_peak,
                                      fp32=mode != "fp64")
         d5["modes"][mode] = line
@@ -550,7 +552,6 @@ def main():
     W = make_workload(args.workload)
 
     modes = [args.mode] + [m for m in args.compare.split(",") if m and m not in (args.mode, "none")]
-    peak = fp64_peak_tflops(torch)
     results = {}
     clocks = None
     log(f"workload {args.workload}: {W['C']} cells, modes {modes}")
@@ -579,6 +580,8 @@ def main():
         hp = hbm_peak_gbs()
         sn = {"sn_fp32": run_sn(K, torch, W, args.steps, args.warmup, True, hp, args.workload),
               "sn_fp64": run_sn(K, torch, W, args.steps, args.warmup, False, hp, args.workload)}
+    # the maximum clock: 2070 MHz where nvidia-smi did not answer
+    peak = multiplier_peak(torch, (clocks or {}).get("sm_max_mhz") or 2070.0)
     extras = None
     if not args.no_extras and world == 1:
         extras = run_extras(K, torch, args, peak, hbm_peak_gbs(), results)
@@ -594,15 +597,13 @@ def main():
     n, Qf = W["n"], W["order"] ** 2  # folded points Q' = Q/2 = order^2
     work = head["solver"].work()
     fl = work["sweep_fp64_flops"]
-    ops = work["sweep_fp64_ops"]
+    ops = sweep_multiplies(W, args.mode == "fp64")
     ekey = "closure_eval_fp64" if args.mode == "fp64" else "closure_eval_mixed"
     pe = head["prof"][ekey]
     sweep_s = pe["total_ms"] / 1e3
-    # the sweep is bound by the FP64 pipe: every FP64 instruction (FMA, add, multiply, and the
-    # eight of each table-driven exp) takes one issue slot of it; the pipe's sustained rate is the
-    # measured DGEMM rate over 2 flops per FMA
+    # the sweep runs in 64-bit fixed point on the integer pipes: its 32 x 32 -> 64-bit
+    # multiplications against the rate at which the multipliers take them
     achieved = pe["units"] * ops / sweep_s / 1e12
-    peak_ops = peak / 2.0
     closure_ms = sum(head["prof"][k]["total_ms"] for k in head["prof"] if k.startswith("closure"))
     closures_per_s = C * args.steps / (closure_ms / 1e3)
 
@@ -641,16 +642,15 @@ def main():
         "closures_per_s": closures_per_s,
         "evaluations_per_cell_step": head["stats"]["evaluations"] / (C * args.steps),
         "roofline": {"kernel": ekey,
-                     "bound": "alu", "achieved": achieved, "peak": peak_ops,
-                     "unit": "T FP64 instructions/s",
-                     "frac": achieved / peak_ops, "traffic": None,
-                     "peak_source": "FP64 pipe: measured cuBLAS DGEMM 4096^3 in this run "
-                                    f"({peak:.3f} TFLOP/s) / 2 flops per FMA instruction; achieved "
-                                    "counts the sweep's FP64 instructions per cell evaluation "
-                                    "(sum-factorised exponent and moments; 2 per exp in the mixed "
-                                    "modes, 8 in FP64 mode) x evaluations "
+                     "bound": "alu", "achieved": achieved, "peak": peak,
+                     "unit": "T 32x32->64-bit multiplications/s",
+                     "frac": achieved / peak, "traffic": None,
+                     "peak_source": "SMs x 4 schedulers x 32 lanes / 4 cycles per wide multiply-add "
+                                    "x the maximum SM clock; achieved counts the fixed-point sweep's "
+                                    "wide multiplications per cell evaluation (exponents, "
+                                    "exponentials, moment sums, per-ring factors) x evaluations "
                                     "/ the sweep's CUDA-event time",
-                     "fp64_ops_per_cell_eval": ops,
+                     "multiplies_per_cell_eval": ops,
                      "fp64_flops_per_cell_eval": fl,
                      "fp64_tflops_achieved": pe["units"] * fl / sweep_s / 1e12,
                      "exps_per_cell_eval": work["exps"],
