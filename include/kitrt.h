@@ -368,7 +368,7 @@ int32_t kitrt_sn_step(kitrt_mn *mn, void *psi, void *work, int32_t fp32, const d
  *                    checkpoint segment (states are recomputed forward inside a segment).
  *   J                host [1]; dJ_dsa, dJ_dss host [nblocks] (overwritten).
  * The first call (or one needing more than the last) allocates the checkpoint and segment buffers
- * in the solver's workspace (about (nsteps/ckpt_every + 2 ckpt_every + 4) C n doubles + C Q'
+ * in the solver's workspace (about (nsteps/ckpt_every + 2 ckpt_every + 5) C n doubles + C Q'
  * doubles); later calls reuse them and allocate nothing; kitrt_mn_destroy frees them. Checks the
  * stability condition of kitrt_step (KITRT_EINVAL) and synchronises with `stream` before
  * returning. */

@@ -2,24 +2,32 @@
 //
 // The Hessian <m m^T e> of the dual needs the moments V_c = sum_q w_q e_q m~_c(q) of the ansatz
 // against the degree-2N basis (H_ab = sum_c G_abc V_c, Gaunt coefficients G). Its first n
-// moments are the gradient's <m e> and stay in FP64; the remaining n2 - n moments enter only the
+// moments are the gradient's <m e> and keep 64 bits; the remaining n2 - n moments enter only the
 // Hessian and are a batched dense contraction
 //     V_hi[cells x (n2-n)] = E[cells x Q'] . (w M_hi)[Q' x (n2-n)],   E = exp(alpha.m)
 // that runs on the 5th-generation tensor cores: tcgen05.mma with TF32 (kind::tf32) or BF16
 // (kind::f16) operands and FP32 accumulation in tensor memory (the quadrature weights are folded
-// into the basis table). Exponents, exp and the gradient moments run in FP64 in the
-// sum-factorised form of sweep.cuh (pairs of mirrored azimuths, coefficients per ring); the
-// objective, the Cholesky factorisation and the line search stay in FP64 (newton_post).
+// into the basis table). Exponents, exponentials and the gradient moments run in the 64-bit fixed
+// point of fixed.cuh, in the sum-factorised form of sweep.cuh (quads of azimuths, coefficients per
+// ring): the FP64 pipe, one warp instruction per 16 cycles of an SM, held the former FP64 form at
+// 4.86 ms (M_3, 99,458 cells, 12 rounds) where this takes 1.53, and at 142 ms (M_5, 996,872 cells,
+// 8 rounds) where it takes 39.9. The objective, the gradient's tests and the line search stay in
+// FP64 (post_group_kernel).
 //
-// One CTA (256 threads) owns a tile of 128 listed cells (the MMA's M = 128 rows, row = cell).
-// The quadrature runs in chunks of 16 pairs (32 points): every thread evaluates 8 pairs of one
-// row in FP64, accumulates its FP64 gradient moments, and stores E rounded to TF32/BF16 into
-// shared memory in the canonical K-major core-matrix layout (8 rows x 16 bytes per core matrix,
-// no swizzle); the threads also stage the matching 32 columns of the weighted M_hi. One elected
-// thread issues the MMAs of the chunk and commits them to an mbarrier; chunks alternate between
-// two buffers so that the next chunk's FP64 work overlaps the tensor-core work of the previous
-// one. Every wait is bounded: on expiry the kernel records KITRT_ETIMEOUT, drains what it issued
-// (bounded) and frees its tensor memory.
+// What bounds it (M_3, a round of 99,458 cells): issue 56% of active cycles, the multipliers' pipe
+// 51% of elapsed, the ALU 50%; the rest is fixed latency with 16 warps on an SM (8 for N >= 4, where
+// a row's state takes 216 registers; 16 warps there, with the moments in shared memory, took 42.4 ms
+// against 39.9 for M_5: more instructions and barrier waits than the latency it hid).
+//
+// One CTA (256 threads) owns a tile of 128 listed cells (the MMA's M = 128 rows, row = cell). The
+// quadrature runs in chunks of 8 quads (32 points): each of a row's two threads takes 4 quads of its
+// own half of the item's range, accumulates their gradient moments, and stores E split into two
+// TF32/BF16 parts in shared memory in the canonical K-major core-matrix layout (8 rows x 16 bytes
+// per core matrix, no swizzle); the matching 32 columns of the weighted M_hi arrive by asynchronous
+// copies meanwhile. One elected thread issues the MMAs of the chunk and commits them to an
+// mbarrier; chunks alternate between two buffers so that the next chunk's arithmetic overlaps the
+// tensor-core work of the previous one. Every wait is bounded: on expiry the kernel records
+// KITRT_ETIMEOUT, drains what it issued (bounded) and frees its tensor memory.
 #include <cuda_bf16.h>
 #include <math.h>
 #include <stdint.h>

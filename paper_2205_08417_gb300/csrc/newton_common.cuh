@@ -142,7 +142,7 @@ __device__ void newton_post(const Tables &T, const NewtonState &S, const NewtonP
     if (!accept) {
         const int h = S.halv[cell] + 1;
         if (h > np.max_halvings && mixed && !S.h64[cell]) {
-            // as in newton_post_thread: restart from the accepted point with the FP64 Hessian
+            // as in post_group_kernel: restart from the accepted point with the FP64 Hessian
             if (lane == 0) {
                 hand_over(S, cell);
                 S.halv[cell] = 0;

@@ -227,19 +227,6 @@ __device__ __forceinline__ void fx_accumulate(const Exp (&e)[4], const int2 *__r
 // Exponent of the unit of a row's moments (for fx_to_double).
 __device__ __forceinline__ int fx_unit(int Sx, const Tables &T) { return Sx - 61 + T.fx_sumshift + T.fx_wexp; }
 
-// An exponential (a non-negative double, or +inf) rounded to float in integer arithmetic, so that
-// the narrow FP64 pipe does not convert it: the exponent is rebiased and the mantissa rounded
-// half away from zero at bit 29 (a carry into the exponent is the correct result); values below
-// the smallest normal float give 0, values beyond the float range give +inf.
-__device__ __forceinline__ float exp_to_float(double e)
-{
-    const long long b = __double_as_longlong(e);
-    const int ex = (int)(b >> 52);  // sign is 0
-    if (ex < 1023 - 126) return 0.0f;
-    const long long f = ((b + (1LL << 28)) >> 29) - ((long long)(1023 - 127) << 23);
-    return f >= (255LL << 23) ? __int_as_float(0x7f800000) : __int_as_float((int)f);
-}
-
 // Conversions done in integer arithmetic, so that the narrow FP64 pipe does not execute them.
 // Whether a double is finite (exponent field not all ones).
 __device__ __forceinline__ bool finite_bits(double x)
