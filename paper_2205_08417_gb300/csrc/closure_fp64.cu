@@ -118,21 +118,34 @@ begin_test_kernel(NewtonState S, const double *__restrict__ u, const double *__r
 // N <= 3 the factor is read into registers. For N >= 4 (120 or 231 entries) a block of one warp
 // copies its 32 cells' factors into shared memory (asynchronously, whole rows at a time: read by the
 // threads themselves each load touches 32 lines) and works from there, the vector in shared memory
-// too. M_5, 996,872 cells: a warp per cell took 8.2 ms a step, strided reads 7.0, this 3.4 (with the test that precedes it).
-template <int NN>
+// too. M_5, 996,872 cells: a warp per cell took 8.2 ms a step, strided reads 7.0, whole factors in
+// shared memory (3 warps on an SM) 3.4, with the test that precedes it. SEG (M_5, more cells than those 3
+// warps on every SM take at once) stages the rows in segments of at most kSegPairs entries, each but
+// the last once more for the backward solve, so that 8 warps fit: 2.2 ms. With one wave the segments'
+// round trips only add latency: M_4, 20,000 cells, 6 warps on an SM, two steps 0.094 ms whole, 0.114 in
+// segments.
+template <int NN, bool SEG>
 struct PredictDims {
     static constexpr bool in_regs = NN <= 3;
     static constexpr int threads = in_regs ? kThreadBlock : 32;
-    static constexpr int pitch = Dims<NN>::npairs | 1;  // odd: a column of 32 rows is free of conflicts
+    static constexpr int kSegPairs = SEG ? 79 : Dims<NN>::npairs;
+    static constexpr int pitch = kSegPairs | 1;  // odd: a column of 32 rows is free of conflicts
+    // end of the segment of rows that starts at row r
+    static __host__ __device__ constexpr int seg_end(int r)
+    {
+        int e = r;
+        while (e < Dims<NN>::n && (e + 1) * (e + 2) / 2 - r * (r + 1) / 2 <= kSegPairs) ++e;
+        return e;
+    }
     static constexpr size_t smem = in_regs ? 0 : sizeof(double) * 32 * (pitch + Dims<NN>::n);
 };
 
-template <int NN>
-__global__ void __launch_bounds__(PredictDims<NN>::threads)
+template <int NN, bool SEG>
+__global__ void __launch_bounds__(PredictDims<NN, SEG>::threads)
 predict_kernel(NewtonState S, const double *__restrict__ u, NewtonParams np, const int32_t *__restrict__ list,
                const int32_t *__restrict__ count)
 {
-    using D = PredictDims<NN>;
+    using D = PredictDims<NN, SEG>;
     constexpr int n = Dims<NN>::n, npairs = Dims<NN>::npairs;
     extern __shared__ __align__(16) double predict_smem[];  // [32][pitch] factors, [n][32] vectors
     const int cnt = *count;
@@ -142,19 +155,23 @@ predict_kernel(NewtonState S, const double *__restrict__ u, NewtonParams np, con
         const int it = rd * stride + blockIdx.x * blockDim.x + threadIdx.x;
         bool cont = false;
         int cell = it < cnt ? list[it] : -1;
-        if constexpr (!D::in_regs) {
+        // rows [r0, r1) of the warp's factors into shared memory
+        auto stage = [&](int r0, int r1) {
+            const int p0 = tri_idx(r0, 0), len = tri_idx(r1, 0) - p0;
             __syncwarp();
             for (int r = 0; r < 32; ++r) {
                 const int c = __shfl_sync(kFull, cell, r);
                 if (c < 0) break;
-                const double *row = S.L + (size_t)c * npairs;
-                for (int p = threadIdx.x; p < npairs; p += 32) kitrt_async::cp_async8(predict_smem + r * D::pitch + p, row + p);
+                const double *row = S.L + (size_t)c * npairs + p0;
+                for (int p = threadIdx.x; p < len; p += 32) kitrt_async::cp_async8(predict_smem + r * D::pitch + p, row + p);
             }
             kitrt_async::cp_async_wait_all();
             __syncwarp();
-        }
-        if (it < cnt) {
-            const size_t off = (size_t)cell * n;
+        };
+        // with segments every lane of the warp takes part in the staging
+        if (!D::in_regs || it < cnt) {
+            const bool mine = it < cnt;
+            const size_t off = (size_t)(mine ? cell : 0) * n;
             double gn2 = 0.0, un2 = 0.0, au = 0.0, ar2 = 0.0, gd = 0.0;
             auto gradient = [&](int a) {
                 const double ua = u[off + a], al = S.alpha[off + a];
@@ -201,26 +218,46 @@ predict_kernel(NewtonState S, const double *__restrict__ u, NewtonParams np, con
             } else {
                 const double *L = predict_smem + threadIdx.x * D::pitch;
                 double *y = predict_smem + 32 * D::pitch + threadIdx.x;
+                int r0 = 0;
 #pragma unroll 1
-                for (int i = 0; i < n; ++i) {
-                    const double *row = L + tri_idx(i, 0);
-                    double t = -gradient(i);
+                for (int r1 = D::seg_end(0);; r0 = r1, r1 = D::seg_end(r1)) {
+                    stage(r0, r1);
+                    if (mine) {
+#pragma unroll 1
+                        for (int i = r0; i < r1; ++i) {
+                            const double *row = L + tri_idx(i, 0) - tri_idx(r0, 0);
+                            double t = -gradient(i);
 #pragma unroll 4
-                    for (int k = 0; k < i; ++k) t = fma(-row[k], y[k * 32], t);
-                    t *= row[i];
-                    y[i * 32] = t;
-                    gd = fma(-t, t, gd);  // g . d = -|L^-1 g|^2
+                            for (int k = 0; k < i; ++k) t = fma(-row[k], y[k * 32], t);
+                            t *= row[i];
+                            y[i * 32] = t;
+                            gd = fma(-t, t, gd);  // g . d = -|L^-1 g|^2
+                        }
+                    }
+                    if (r1 == n) break;
                 }
+                // backward from the last segment, which is still there
 #pragma unroll 1
-                for (int i = n - 1; i >= 0; --i) {
-                    const double *row = L + tri_idx(i, 0);
-                    const double x = y[i * 32] * row[i];
-                    S.dir[off + i] = x;
+                for (int r1 = n;;) {
+                    if (mine) {
+#pragma unroll 1
+                        for (int i = r1 - 1; i >= r0; --i) {
+                            const double *row = L + tri_idx(i, 0) - tri_idx(r0, 0);
+                            const double x = y[i * 32] * row[i];
+                            S.dir[off + i] = x;
 #pragma unroll 4
-                    for (int k = 0; k < i; ++k) y[k * 32] = fma(-row[k], x, y[k * 32]);
+                            for (int k = 0; k < i; ++k) y[k * 32] = fma(-row[k], x, y[k * 32]);
+                        }
+                    }
+                    if (r0 == 0) break;
+                    r1 = r0;
+                    for (r0 = 0; D::seg_end(r0) < r1;) r0 = D::seg_end(r0);
+                    stage(r0, r1);
                 }
             }
-            if (gn2 <= np.tau * np.tau * un2) {
+            if (!mine) {
+                // a lane without a cell
+            } else if (gn2 <= np.tau * np.tau * un2) {
                 S.phase[cell] = PH_DONE;  // converged; d is the polish step
             } else {
                 if (S.gnorm) S.gnorm[cell] = gn2;
@@ -648,15 +685,18 @@ int grid_for(const kitrt_mn *mn, int C, int per_sm)
     return need < cap ? (need > 0 ? need : 1) : cap;
 }
 
-template <int NN>
+template <int NN, bool SEG = false>
 int predict_launch(kitrt_mn *mn, const NewtonState &S, int C, const double *u, NewtonParams np,
                    const int32_t *list, const int32_t *count, cudaStream_t s)
 {
-    using D = PredictDims<NN>;
-    if (ensure_dyn_smem(predict_kernel<NN>, D::smem)) return KITRT_ECUDA;
+    using D = PredictDims<NN, SEG>;
+    // the factors of more cells than three warps on every SM hold: in segments
+    if constexpr (NN == 5 && !SEG)
+        if (C > mn->nsm * 3 * 32) return predict_launch<NN, true>(mn, S, C, u, np, list, count, s);
+    if (ensure_dyn_smem(predict_kernel<NN, SEG>, D::smem)) return KITRT_ECUDA;
     int tb = (C + D::threads - 1) / D::threads;
     if (tb > mn->nsm * 32) tb = mn->nsm * 32;
-    predict_kernel<NN><<<tb > 0 ? tb : 1, D::threads, D::smem, s>>>(S, u, np, list, count);
+    predict_kernel<NN, SEG><<<tb > 0 ? tb : 1, D::threads, D::smem, s>>>(S, u, np, list, count);
     return KITRT_OK;
 }
 

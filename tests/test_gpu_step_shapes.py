@@ -49,6 +49,21 @@ def case(N, order, k=11, seed=4):
     return m, G, T, u, blk, sa, ss, q, dt
 
 
+@pytest.mark.parametrize("mode,bar", [("fp64", 1e-11), ("mixed_tf32", 1e-6)])
+def test_predictor_in_segments(K, mode, bar):
+    """M_5 on more cells (a ragged last warp) than the predictor takes with whole factors in shared
+    memory: its rows then come in segments."""
+    m, G, T, u0, blk, sa, ss, q, dt = case(5, 12, k=90)
+    assert len(u0) > 152 * 96 and len(u0) % 32
+    u, a = u0.copy(), O.isotropic_alpha(T, u0)
+    nf, _ = O.mn_run(T, G, u, a, sa[blk], ss[blk], q, dt, 3, bc=0)
+    assert nf == 0
+    s = K.MNSolver(K.Mesh(m.xy, m.tri), 5, 12, mode=mode, bc="neumann")
+    ud = dev(u0)
+    s.step(ud, s.isotropic_alpha(ud), dev(sa[blk]), dev(ss[blk]), dev(q), dt=dt, nsteps=3)
+    assert rel_l2(ud.cpu().numpy(), u) <= bar
+
+
 @pytest.mark.parametrize("bc", ["neumann", "vacuum"])
 @pytest.mark.parametrize("mode,bar", [("fp64", 1e-11), ("mixed_tf32", 1e-6)])
 @pytest.mark.parametrize("N,order", SHAPES)
