@@ -37,6 +37,8 @@ constexpr int kThreadBlock = 64;  // block of the thread-per-cell Newton kernels
 // succeeded, so the stored state is exactly the state behind the given alpha; the first case
 // otherwise (the cell's stored <exp> is then poisoned, so that the learned pass cannot mistake
 // it for a previous point).
+// renew: a converged cell is evaluated all the same, so that the sweeps write its ansatz (the closure
+// that left its state wrote none).
 // ---------------------------------------------------------------------------------------------
 
 // Warp-aggregated append of `cell` to a list when pred holds (all active lanes call it).
@@ -56,7 +58,7 @@ __device__ __forceinline__ void push_if(int32_t *list, int32_t *cnt, int cell, b
 template <int NN>
 __global__ void __launch_bounds__(256)
 begin_test_kernel(NewtonState S, const double *__restrict__ u, const double *__restrict__ alpha_in,
-                  int first, NewtonParams np, int C, int learned)
+                  int first, NewtonParams np, int C, int learned, int renew)
 {
     constexpr int n = Dims<NN>::n;
     for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < C; cell += gridDim.x * blockDim.x) {
@@ -103,7 +105,8 @@ begin_test_kernel(NewtonState S, const double *__restrict__ u, const double *__r
                 // is at round-off, where it would move alpha by less than its own rounding)
 #pragma unroll
                 for (int a = 0; a < n; ++a) S.dir[off + a] = 0.0;
-                S.phase[cell] = PH_DONE;
+                S.phase[cell] = renew ? PH_INIT : PH_DONE;
+                to_eval = renew;
             } else {
                 to_predict = true;
             }
@@ -803,14 +806,14 @@ int launch_ansatz(const Tables &T, int C, const double *alpha, double *psi, cuda
 
 int launch_begin(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
                  const double *u, const double *alpha_in, int first, NewtonParams np,
-                 cudaStream_t s, int learned)
+                 cudaStream_t s, int learned, int renew)
 {
     (void)T;
     int blocks = (C + 255) / 256;
     if (blocks > mn->nsm * 8) blocks = mn->nsm * 8;
     {
         LaunchScope ls(mn, PK_BEGIN, s, C);
-        KITRT_DISPATCH_N(mn->N, begin_test_kernel<NN><<<blocks > 0 ? blocks : 1, 256, 0, s>>>(S, u, alpha_in, first, np, C, learned));
+        KITRT_DISPATCH_N(mn->N, begin_test_kernel<NN><<<blocks > 0 ? blocks : 1, 256, 0, s>>>(S, u, alpha_in, first, np, C, learned, renew));
         if (cudaGetLastError() != cudaSuccess) return KITRT_ECUDA;
     }
     if (first == 1 || learned) return KITRT_OK;

@@ -913,7 +913,11 @@ static int run_closure(kitrt_mn *mn, int C, const double *u, const double *alpha
     const bool learned = mn->p.mode == KITRT_LEARNED;
     if (learned && !mn->has_mlp) return KITRT_EINVAL;
     CUDA_OK(cudaMemsetAsync(mn->st.cnt, 0, 16 * sizeof(int32_t), s));
-    int rc = launch_begin(mn, T, mn->st, C, u, alpha_in, first, np, s, learned);
+    // a batch closure writes no ansatz: a step that continues from its state has the converged cells
+    // evaluated once more
+    const bool writes32 = psi32 != nullptr, renew = writes32 && mn->psi32_stale;
+    if (!writes32 && mn->p.mode != KITRT_FP64) mn->psi32_stale = true;
+    int rc = launch_begin(mn, T, mn->st, C, u, alpha_in, first, np, s, learned, renew);
     if (rc) return rc;
     if (learned) {
         rc = launch_mlp_infer(mn, u, mn->st.list[1], mn->st.cnt + 8, C, mn->d_alpha_nn, s);
@@ -970,6 +974,7 @@ static int run_closure(kitrt_mn *mn, int C, const double *u, const double *alpha
         for (int32_t v : stv)
             if (v) return v;
     }
+    if (writes32) mn->psi32_stale = false;
     return KITRT_OK;
 }
 

@@ -159,6 +159,7 @@ struct kitrt_mn {
     void *d_psif = nullptr;    // second order: [C x 3 x Qp] reconstructed face values (FP64/FP32)
     double *d_ustage = nullptr;  // second order: [C x n] the Heun stage u*
     float *d_psi32 = nullptr;  // [C x Qp] FP32 ansatz (mixed modes)
+    bool psi32_stale = false;  // a closure has moved the stored state on without writing d_psi32
     float *d_zero32 = nullptr; // [Qp] zeros: the vacuum ghost's row in the FP32 flux
     // transformed CSD equation (kitrt_mn_set_density): 1 / rho per cell, FP64 and FP32 (NULL:
     // no density, rho = 1)
@@ -244,7 +245,7 @@ inline int resident_ctas(Kern *kernel, int threads, size_t dyn_smem, int cap)
 int launch_isotropic(const Tables &T, int C, const double *u, double *alpha, cudaStream_t s);
 int launch_begin(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C,
                  const double *u, const double *alpha_in, int first, NewtonParams np,
-                 cudaStream_t s, int learned = 0);
+                 cudaStream_t s, int learned = 0, int renew = 0);
 int launch_mlp_infer(kitrt_mn *mn, const double *u, const int32_t *list, const int32_t *cnt, int C,
                      double *alpha, cudaStream_t s);
 int launch_learned_pass(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, const double *u,
