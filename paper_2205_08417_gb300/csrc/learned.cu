@@ -190,7 +190,8 @@ learned_decide_kernel(Tables T, NewtonState S, const double *__restrict__ u, con
                 for (int a = 1; a < n; ++a) S.U[off + a] = c * moment(a);
                 S.fsum[cell] = u0 / T.m0;
                 S.phase[cell] = PH_DONE;
-            } else if (!use_nn && first != 1 && S.lfac && S.lfac[cell]) {
+            } else if (!use_nn && first != 1 && S.lfac && S.lfac[cell] && isfinite(S.fsum[cell])) {
+                // (a cold cell's <exp> is poisoned: its stored moments and factor belong to another alpha)
                 to_predict = true;
             } else {
                 S.phase[cell] = PH_INIT;
