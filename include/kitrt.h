@@ -348,6 +348,8 @@ int32_t kitrt_closure_noalloc(const kitrt_mn *mn, const double *u, double *alpha
  *            isotropic scattering.
  *   dt       time step; dt <= 0 selects cfl * (smallest inradius).
  * Asynchronous on `stream` (nsteps launches, plus one device copy when nsteps is odd).
+ * Calls of one solver may be on different streams: each starts, on its stream, when the one before
+ * has ended. Under stream capture the per-cell coefficients take graph memory (12 C values).
  * KITRT_EINVAL for NULL arguments, nsteps < 0, overlapping buffers, g[0] != 1 or a non-finite
  * g. */
 int32_t kitrt_sn_step(kitrt_mn *mn, void *psi, void *work, int32_t fp32, const double *sigma_a,

@@ -472,6 +472,7 @@ int32_t kitrt_mn_destroy(kitrt_mn *mn)
     if (mn->h_cnt) cudaFreeHost(mn->h_cnt);
     if (mn->h_check) cudaFreeHost(mn->h_check);
     if (mn->d_adj) cudaFree(mn->d_adj);
+    if (mn->sn_done) cudaEventDestroy(mn->sn_done);
     delete mn;
     return KITRT_OK;
 }
@@ -811,6 +812,10 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
         double *cellc = nullptr;
         TRY(dev_alloc(mn, &cellc, C * 12));
         mn->d_sn_cell = cellc;
+        if (cudaEventCreateWithFlags(&mn->sn_done, cudaEventDisableTiming) != cudaSuccess) {
+            kitrt_mn_destroy(mn);
+            return KITRT_ECUDA;
+        }
     }
     if (p.order == 2) {
         TRY(dev_alloc(mn, &mn->d_ustage, C * n));

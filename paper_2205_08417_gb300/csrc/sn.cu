@@ -219,11 +219,10 @@ int dispatch_sn(kitrt_mn *mn, const QuadTab<P> &X, const P *psi, P *out, const P
 }
 
 template <typename P>
-int run_sn(kitrt_mn *mn, const QuadTab<P> &X, P *psi, P *work, const double *sa, const double *ss,
+int run_sn(kitrt_mn *mn, const QuadTab<P> &X, P *psi, P *work, P *cellc, const double *sa, const double *ss,
            const double *q, const SnScat<P> &sc, bool iso, double dt, int nsteps, cudaStream_t s)
 {
     const kitrt_mesh *m = mn->mesh;
-    P *cellc = (P *)mn->d_sn_cell;
     {
         int blocks = (m->C + 255) / 256;
         if (blocks > mn->nsm * 8) blocks = mn->nsm * 8;
@@ -281,16 +280,36 @@ int32_t kitrt_sn_step(kitrt_mn *mn, void *psi, void *work, int32_t fp32, const d
     if (nsteps == 0) return KITRT_OK;
     cudaStream_t s = (cudaStream_t)stream;
     if (dt <= 0.0) dt = mn->p.cfl * mn->mesh->min_inradius;
+    // The per-cell coefficients lie in the solver's workspace, which a call on another stream would
+    // overwrite: every call waits on its stream (not on the host) for the end of the one before. A
+    // captured call cannot wait for work outside its graph, and a replay overlaps anything: its
+    // coefficients lie in memory of the graph's own.
+    cudaStreamCaptureStatus capture;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) return KITRT_ECUDA;
+    const bool captured = capture != cudaStreamCaptureStatusNone;
+    void *cellc = mn->d_sn_cell;
+    if (captured) {
+        if (cudaMallocAsync(&cellc, (fp32 ? 4 : 8) * (size_t)mn->mesh->C * kCellSlots, s) != cudaSuccess)
+            return KITRT_ENOMEM;
+    } else if (mn->sn_pending && cudaStreamWaitEvent(s, mn->sn_done, 0) != cudaSuccess) {
+        return KITRT_ECUDA;
+    }
+    int rc;
     if (fp32) {
         SnScat<float> sc{};
         for (int a = 0; a < KITRT_MAX_NMOM; ++a) sc.ga[a] = (float)ga[a];
-        return run_sn<float>(mn, quad_tab32(mn), (float *)psi, (float *)work, sigma_a, sigma_s, q, sc, iso, dt,
-                             nsteps, s);
+        rc = run_sn<float>(mn, quad_tab32(mn), (float *)psi, (float *)work, (float *)cellc, sigma_a, sigma_s, q, sc,
+                           iso, dt, nsteps, s);
+    } else {
+        SnScat<double> sc{};
+        for (int a = 0; a < KITRT_MAX_NMOM; ++a) sc.ga[a] = ga[a];
+        rc = run_sn<double>(mn, quad_tab64(mn), (double *)psi, (double *)work, (double *)cellc, sigma_a, sigma_s, q,
+                            sc, iso, dt, nsteps, s);
     }
-    SnScat<double> sc{};
-    for (int a = 0; a < KITRT_MAX_NMOM; ++a) sc.ga[a] = ga[a];
-    return run_sn<double>(mn, quad_tab64(mn), (double *)psi, (double *)work, sigma_a, sigma_s, q, sc, iso, dt,
-                          nsteps, s);
+    if (captured) return cudaFreeAsync(cellc, s) != cudaSuccess && !rc ? KITRT_ECUDA : rc;
+    if (cudaEventRecord(mn->sn_done, s) != cudaSuccess) return rc ? rc : KITRT_ECUDA;
+    mn->sn_pending = true;
+    return rc;
 }
 
 }  // extern "C"
