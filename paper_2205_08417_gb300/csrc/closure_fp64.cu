@@ -465,8 +465,8 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
                 if (pb >= 0) *(double2 *)(row + 2 * pb) = make_double2(fx_psi(e[2]), fx_psi(e[3]));
             }
             if (pb < 0) e[2] = e[3] = Exp{0, -100000};
-            fx_accumulate<L2>(e, tr, L2, jq == 0, pb < 0, qd == q_begin, B, [&](int d) {
-                for (int c = 0; c < n2; ++c) mine[c * kSweepThreads] = kitrt_fx::sar(mine[c * kSweepThreads], d);
+            fx_accumulate<L2>(e, tr, L2, jq == 0, qd == q_begin, B, [&](int d) {
+                for (int c = 0; c < n2; ++c) mine[c * kSweepThreads] = kitrt_fx::sar_round(mine[c * kSweepThreads], d);
             });
             if (++jq == T.J) {
                 fx_flush<L2>(T.fx_ringW + (size_t)ring * n2, T.fx_sumshift, B, moment);

@@ -379,9 +379,9 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
                         bad = !fx_slow_quad<NN>(T.Mt, Qp, T.exptab, al, di, lam, pa, pb, e) || bad;
                     }
                     if (pb < 0) e[2] = e[3] = Exp{0, -100000};
-                    fx_accumulate<NN>(e, tr, NN, jq == 0, pb < 0, i == 0 && c == c_begin, B, [&](int d) {
+                    fx_accumulate<NN>(e, tr, NN, jq == 0, i == 0 && c == c_begin, B, [&](int d) {
 #pragma unroll
-                        for (int a = 0; a < n; ++a) U[a] = kitrt_fx::sar(U[a], d);
+                        for (int a = 0; a < n; ++a) U[a] = kitrt_fx::sar_round(U[a], d);
                     });
 #pragma unroll
                     for (int t = 0; t < 4; ++t) f[t] = __uint_as_float(kitrt_fx::fx_float_bits(e[t]));
@@ -460,7 +460,7 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
             const int top = poison ? 0 : max(B.Sx, x1), unit = fx_unit(top, T);
 #pragma unroll
             for (int a = 0; a < n; ++a) {
-                const long long v = poison ? 0 : kitrt_fx::sar(U[a], top - B.Sx) + kitrt_fx::sar(sU[a * kTileM + r], top - x1);
+                const long long v = poison ? 0 : kitrt_fx::sar_round(U[a], top - B.Sx) + kitrt_fx::sar_round(sU[a * kTileM + r], top - x1);
                 row[(size_t)a * vs_c] = poison ? __longlong_as_double(0x7ff8000000000000LL) : kitrt_fx::fx_to_double(v, unit);
             }
         }

@@ -14,9 +14,12 @@
 //   exponential e = y 2^(m - 61), y in [2^61, 2^62]: T_j (1 + p) with the 2048-entry table and
 //   p = exp(r ln2/2048) - 1 on r in [0, 1) by a cubic whose quartic term is folded in (error below
 //   2^-57); |error| of y below 2^-51 relative;
-//   sums in units of 2^(Sx - 61): e is shifted down by Sx - m >= 8, so that it stays below 2^54 and
+//   sums in units of 2^(Sx - 61): e is shifted down by Sx - m >= 7, so that it stays below 2^55 and
 //   32 quads fit; Sx belongs to the row and is raised (and the sums shifted) when a larger
-//   exponential appears.
+//   exponential appears. Shifts round to nearest: an exponential far below the row's largest adds no
+//   more than itself to the error, so that the moments of a peaked density, whose Hessian is badly
+//   conditioned, are as good as FP64 sums (rounding down and adding the mean half unit back put half
+//   a unit per point into them: up to 300 times the FP64 error in the Hessian's own metric).
 // Written as plain C++ so that the host can check the arithmetic bit for bit.
 #pragma once
 
@@ -35,7 +38,7 @@ namespace kitrt_fx {
 
 constexpr int kFracBits = 42;             // fraction bits of the exponent s
 constexpr float kFxMaxZ = 245.0f;         // sum_c |alpha_c| max|m_c| below this: |s| < 2^61.5
-constexpr int kGuard = 8;                 // y (2^62) >> 8 = 2^54
+constexpr int kGuard = 7;                 // y (2^62) >> 7 = 2^55
 
 struct Limb {
     int h, l;
@@ -55,7 +58,12 @@ KITRT_FX uint64_t shr(uint64_t y, int n)
     return n >= 64 ? 0 : y >> n;
 #endif
 }
+KITRT_FX int imax(int a, int b) { return a > b ? a : b; }
+
+// y / 2^n rounded to the nearest integer (halves up), n >= 1
+KITRT_FX uint64_t shr_round(uint64_t y, int n) { return (shr(y, n - 1) + 1) >> 1; }
 KITRT_FX long long sar(long long y, int n) { return y >> (n > 63 ? 63 : n); }
+KITRT_FX long long sar_round(long long y, int n) { return n > 0 ? (sar(y, n - 1) + 1) >> 1 : y; }
 
 // v = h 2^B + l, |l| <= 2^(B - 1), for |v| < 2^(30 + B)
 template <int B>
@@ -79,7 +87,7 @@ struct DotAcc {
     KITRT_FX long long value() const { return (hh << 4) + (hl >> 23) + (lh >> 27); }
 };
 
-// Azimuthal sum of e T_k over up to 32 quads (e below 2^56 in magnitude, 27-bit limbs both), in
+// Azimuthal sum of e T_k over up to 32 quads (e below 2^57 in magnitude, 27-bit limbs both), in
 // units of e.
 struct SumAcc {
     long long hh, m;
@@ -91,15 +99,15 @@ struct SumAcc {
         m += wide(e.l, t.x);
     }
     KITRT_FX long long value() const { return hh + (m >> 27); }
-    KITRT_FX void scale_down(int n) { hh = sar(hh, n), m = sar(m, n); }
+    KITRT_FX void scale_down(int n) { hh = sar_round(hh, n), m = sar_round(m, n); }
 };
 
-// One term B w P of a moment: B an azimuthal sum (below 2^61, split<32>), wP in units of 2^-57 (split<27>),
-// in units of 2^sh of B (0 <= sh <= 4).
+// One term B w P of a moment: B an azimuthal sum (below 2^62, split<32>), wP in units of 2^-57 (split<27>),
+// in units of 2^sh of B (-20 < sh <= 2), rounded once.
 KITRT_FX long long moment_term(Limb b, int2 wp, int sh)
 {
-    return ((wide(b.h, wp.x) << 2) >> sh) + ((wide(b.h, wp.y) + (1LL << (24 + sh))) >> (25 + sh)) +
-           ((wide(b.l, wp.x) + (wide(b.l, wp.y) >> 27) + (1LL << (29 + sh))) >> (30 + sh));
+    const long long t = (wide(b.h, wp.y) << 5) + wide(b.l, wp.x) + (wide(b.l, wp.y) >> 27);  // units 2^-30
+    return (wide(b.h, wp.x) << (2 - sh)) + ((t + (1LL << (29 + sh))) >> (30 + sh));
 }
 
 // A double as an integer in units of 2^-52, rounded (|x| < 2048).
@@ -238,6 +246,147 @@ KITRT_FX int fx_scale_of(double u0)
     b.d = u0;
     const int ex = (int)(b.u >> 52);  // sign makes it large
     return ex == 0 || ex >= 0x7ff ? 100000 : ex - 1023 - 2 + 4 + kGuard;
+}
+
+// ---------------------------------------------------------------------------------------------
+// One row's pass over the rule (sweep.cuh): exponent coefficients of a ring, exponents of a quad, azimuthal
+// sums, moments.
+// ---------------------------------------------------------------------------------------------
+// Index of basis function (l, k), l + |k| even, in the order l ascending, then k ascending.
+KITRT_FX constexpr int cindex(int l, int k) { return l * (l + 1) / 2 + (k + l) / 2; }
+
+// Exponent coefficients of one ring: A0 (k = 0) and A[2(k-1)], A[2(k-1)+1] for cos(k phi),
+// sin(k phi), from the trial alpha's limbs (at(c)).
+template <int NN, typename At>
+KITRT_FX void fx_coeffs(At &&at, const int2 *Pr, long long &A0, Limb (&A)[2 * NN])
+{
+#pragma unroll
+    for (int k = -NN; k <= NN; ++k) {
+        CoefAcc acc;
+        const int ak = k < 0 ? -k : k;
+#pragma unroll
+        for (int l = ak; l <= NN; l += 2) acc.add(at(cindex(l, k)), Pr[cindex(l, k)]);
+        const long long v = acc.value();
+        if (k == 0) A0 = v;
+        else A[2 * (ak - 1) + (k < 0)] = split<31>(v);
+    }
+}
+
+// A row's azimuthal sums of the current ring, degree LB, and the exponent of their unit
+// (units of 2^(Sx - 61)).
+template <int LB>
+struct FxSums {
+    long long b0;
+    SumAcc b[2 * LB];  // cos(k phi), sin(k phi) at 2(k-1), 2(k-1)+1
+    int Sx;
+    KITRT_FX void clear()
+    {
+        b0 = 0;
+#pragma unroll
+        for (int j = 0; j < 2 * LB; ++j) b[j].clear();
+    }
+};
+
+// Moments of the finished ring: V_c += w_r P_c(mu_r) B_k(c), c over the degree-LB basis; the
+// azimuthal sums are cleared for the next ring.
+template <int LB, typename Acc>
+KITRT_FX void fx_flush(const int2 *wPr, int sumshift, FxSums<LB> &B, Acc &&V)
+{
+#pragma unroll
+    for (int k = -LB; k <= LB; ++k) {
+        const int ak = k < 0 ? -k : k;
+        const Limb v = split<32>(k == 0 ? B.b0 : B.b[k == 0 ? 0 : 2 * (ak - 1) + (k < 0)].value());
+#pragma unroll
+        for (int l = ak; l <= LB; l += 2) V(cindex(l, k)) += moment_term(v, wPr[cindex(l, k)], sumshift);
+    }
+    B.clear();
+}
+
+// The exponents of one quad's four points (t: its cosines, k = 1.., then from t + L2 its sines).
+template <int NN>
+KITRT_FX void fx_exponents(long long A0, const Limb (&A)[2 * NN], const int2 *t, int L2, bool axes, long long (&s)[4])
+{
+    long long ce = A0, co = 0, se = 0, so = 0;
+    if (!axes) {
+        DotAcc acc[4];  // C_e, C_o, S_e, S_o
+#pragma unroll
+        for (int k = 1; k <= NN; ++k) {
+            acc[k & 1].add(A[2 * (k - 1)], t[k - 1]);
+            acc[2 + (k & 1)].add(A[2 * (k - 1) + 1], t[L2 + k - 1]);
+        }
+        if (NN >= 2) ce += acc[0].value();
+        co = acc[1].value();
+        if (NN >= 2) se = acc[2].value();
+        so = acc[3].value();
+        const long long p = ce + co, m = ce - co, q = so + se, w = so - se;
+        s[0] = p + q;
+        s[1] = p - q;
+        s[2] = m + w;
+        s[3] = m - w;
+    } else {
+        // phi = 0, pi, pi/2, 3 pi/2: cos(k phi) and sin(k phi) are 0 and +-1
+        long long ce2 = A0;
+#pragma unroll
+        for (int k = 1; k <= NN; ++k) {
+            const long long a = ((long long)A[2 * (k - 1)].h << 31) + A[2 * (k - 1)].l;
+            const long long b = ((long long)A[2 * (k - 1) + 1].h << 31) + A[2 * (k - 1) + 1].l;
+            if (k & 1) {
+                co += a;
+                so += (k & 2) ? -b : b;
+            } else {
+                ce += a;
+                ce2 += (k & 2) ? -a : a;
+            }
+        }
+        s[0] = ce + co;
+        s[1] = ce - co;
+        s[2] = ce2 + so;
+        s[3] = ce2 - so;
+    }
+}
+
+// One quad's exponentials into the azimuthal sums. `first`: the row's first quad of this item
+// (uniform), which lowers a scale that lies far above the row's exponentials. shift_moments(d)
+// shifts the row's moments down by d when the scale rises.
+template <int LB, typename Shift>
+KITRT_FX void fx_accumulate(const Exp (&e)[4], const int2 *t, int L2, bool axes, bool first, FxSums<LB> &B,
+                            Shift &&shift_moments)
+{
+    const int mm = imax(imax(e[0].m, e[1].m), imax(e[2].m, e[3].m));
+    if (first && B.Sx - kGuard - mm > 22) B.Sx = mm + kGuard + 1;
+    if (mm + kGuard > B.Sx) {
+        const int d = mm + kGuard + 1 - B.Sx;
+        B.Sx += d;
+        B.b0 = sar_round(B.b0, d);
+#pragma unroll
+        for (int j = 0; j < 2 * LB; ++j) B.b[j].scale_down(d);
+        shift_moments(d);
+    }
+    long long f[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) f[i] = (long long)shr_round(e[i].y, B.Sx - e[i].m);
+    const long long p = f[0] + f[1], d = f[0] - f[1], p2 = f[2] + f[3], d2 = f[2] - f[3];
+    const long long all = p + p2;
+    B.b0 += all;
+    if (!axes) {
+        const Limb ce = split<27>(all), co = split<27>(p - p2);
+        const Limb so = split<27>(d + d2), se = split<27>(d - d2);
+#pragma unroll
+        for (int k = 1; k <= LB; ++k) {
+            B.b[2 * (k - 1)].add(k & 1 ? co : ce, t[k - 1]);
+            B.b[2 * (k - 1) + 1].add(k & 1 ? so : se, t[L2 + k - 1]);
+        }
+    } else {
+#pragma unroll
+        for (int k = 1; k <= LB; ++k) {
+            if (k & 1) {
+                B.b[2 * (k - 1)].hh += d;
+                B.b[2 * (k - 1) + 1].hh += (k & 2) ? -d2 : d2;
+            } else {
+                B.b[2 * (k - 1)].hh += (k & 2) ? p - p2 : all;
+            }
+        }
+    }
 }
 
 }  // namespace kitrt_fx

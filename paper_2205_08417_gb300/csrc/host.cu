@@ -256,9 +256,7 @@ Tables kitrt_mn::tables() const
     T.nquad = R * J;
     T.Qs = Qs;
     T.fx_wexp = fx_wexp;
-    // Qf exponentials below 2^54 each: their sums stay below 2^63
-    T.fx_sumshift = 0;
-    while ((Qf >> T.fx_sumshift) >= 512) ++T.fx_sumshift;
+    T.fx_sumshift = fx_sumshift;
     T.fx_trig = d_fx_trig;
     T.fx_ringA = d_fx_ringA;
     T.fx_ringW = d_fx_ringW;
@@ -679,6 +677,19 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
                 }
         }
         frexp(wmax, &mn->fx_wexp);  // wmax < 2^fx_wexp
+        // unit of the moments: exponentials below 2^(62 - kGuard) at every point give sums below 2^63
+        double most = 0.0;
+        for (int cc = 0; cc < n2; ++cc) {
+            double sum = 0.0;
+            for (int rg = 0; rg < mn->R; ++rg) sum += 2.0 * mn->P * fabs(r.ring_w[rg] * P[(size_t)rg * n2 + cc]);
+            most = std::max(most, sum);
+        }
+        frexp(ldexp(1.001 * most, -mn->fx_wexp), &mn->fx_sumshift);
+        mn->fx_sumshift -= kitrt_fx::kGuard + 1;
+        if (mn->fx_sumshift > 2) {  // moment_term's limit
+            mn->fx_wexp += mn->fx_sumshift - 2;
+            mn->fx_sumshift = 2;
+        }
         const long double scale = 2048.0L / logl(2.0L);
         std::vector<float> mmax(n, 0.0f);
         for (int rg = 0; rg < mn->R; ++rg)

@@ -145,7 +145,7 @@ struct kitrt_mn {
     int2 *d_fx_trig = nullptr, *d_fx_ringA = nullptr, *d_fx_ringW = nullptr;
     uint64_t *d_fx_exp = nullptr;
     float *d_fx_mmax = nullptr;
-    int fx_wexp = 0;
+    int fx_wexp = 0, fx_sumshift = 0;
     double *d_exptab = nullptr;          // [2048] exp table (Tables::exptab)
     double *d_quad64 = nullptr;          // tables of the quads (quad_lane.cuh), FP64 and FP32
     float *d_quad32 = nullptr;

@@ -109,9 +109,9 @@ learned_sweep_kernel(Tables T, NewtonState S, const double *__restrict__ alpha_n
                 if (pb >= 0) *(float2 *)(row + 2 * pb) = make_float2(f[2], f[3]);
             }
             if (pb < 0) e[2] = e[3] = Exp{0, -100000};
-            fx_accumulate<NN>(e, tr, NN, jq == 0, pb < 0, qd == q_begin, B, [&](int d) {
+            fx_accumulate<NN>(e, tr, NN, jq == 0, qd == q_begin, B, [&](int d) {
 #pragma unroll
-                for (int c = 0; c < n; ++c) U[c] = kitrt_fx::sar(U[c], d);
+                for (int c = 0; c < n; ++c) U[c] = kitrt_fx::sar_round(U[c], d);
             });
             if (++jq == T.J) {
                 fx_flush<NN>(T.fx_ringW + (size_t)ring * Dims<NN>::n2, T.fx_sumshift, B, moment);

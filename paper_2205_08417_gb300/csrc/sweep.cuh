@@ -34,58 +34,14 @@
 
 namespace kitrt_dev {
 
-// Index of basis function (l, k), l + |k| even, in the order l ascending, then k ascending.
-__host__ __device__ constexpr int cindex(int l, int k) { return l * (l + 1) / 2 + (k + l) / 2; }
-
+using kitrt_fx::cindex;
 using kitrt_fx::Exp;
+using kitrt_fx::fx_accumulate;
+using kitrt_fx::fx_coeffs;
+using kitrt_fx::fx_exponents;
+using kitrt_fx::fx_flush;
+using kitrt_fx::FxSums;
 using kitrt_fx::Limb;
-
-// Exponent coefficients of one ring: A0 (k = 0) and A[2(k-1)], A[2(k-1)+1] for cos(k phi),
-// sin(k phi), from the trial alpha's limbs (at(c)).
-template <int NN, typename At>
-__device__ __forceinline__ void fx_coeffs(At &&at, const int2 *Pr, long long &A0, Limb (&A)[2 * NN])
-{
-#pragma unroll
-    for (int k = -NN; k <= NN; ++k) {
-        kitrt_fx::CoefAcc acc;
-        const int ak = k < 0 ? -k : k;
-#pragma unroll
-        for (int l = ak; l <= NN; l += 2) acc.add(at(cindex(l, k)), Pr[cindex(l, k)]);
-        const long long v = acc.value();
-        if (k == 0) A0 = v;
-        else A[2 * (ak - 1) + (k < 0)] = kitrt_fx::split<31>(v);
-    }
-}
-
-// A row's azimuthal sums of the current ring, degree LB, and the exponent of their unit
-// (units of 2^(Sx - 61)).
-template <int LB>
-struct FxSums {
-    long long b0;
-    kitrt_fx::SumAcc b[2 * LB];  // cos(k phi), sin(k phi) at 2(k-1), 2(k-1)+1
-    int Sx;
-    __device__ __forceinline__ void clear()
-    {
-        b0 = 0;
-#pragma unroll
-        for (int j = 0; j < 2 * LB; ++j) b[j].clear();
-    }
-};
-
-// Moments of the finished ring: V_c += w_r P_c(mu_r) B_k(c), c over the degree-LB basis; the
-// azimuthal sums are cleared for the next ring.
-template <int LB, typename Acc>
-__device__ __forceinline__ void fx_flush(const int2 *wPr, int sumshift, FxSums<LB> &B, Acc &&V)
-{
-#pragma unroll
-    for (int k = -LB; k <= LB; ++k) {
-        const int ak = k < 0 ? -k : k;
-        const Limb v = kitrt_fx::split<32>(k == 0 ? B.b0 : B.b[k == 0 ? 0 : 2 * (ak - 1) + (k < 0)].value());
-#pragma unroll
-        for (int l = ak; l <= LB; l += 2) V(cindex(l, k)) += kitrt_fx::moment_term(v, wPr[cindex(l, k)], sumshift);
-    }
-    B.clear();
-}
 
 // The two pairs of points of quad j of a ring (the second is -1 in quad 0 of a ring with an odd
 // number of pairs).
@@ -131,97 +87,6 @@ __device__ __forceinline__ bool fx_slow_quad(const double *__restrict__ Mt, int 
 #pragma unroll
     for (int i = 0; i < 4; ++i) e[i] = t[i];
     return ok;
-}
-
-// The exponents of one quad's four points (t: its cosines, k = 1.., then from t + L2 its sines).
-template <int NN>
-__device__ __forceinline__ void fx_exponents(long long A0, const Limb (&A)[2 * NN], const int2 *__restrict__ t,
-                                             int L2, bool axes, long long (&s)[4])
-{
-    long long ce = A0, co = 0, se = 0, so = 0;
-    if (!axes) {
-        kitrt_fx::DotAcc acc[4];  // C_e, C_o, S_e, S_o
-#pragma unroll
-        for (int k = 1; k <= NN; ++k) {
-            acc[k & 1].add(A[2 * (k - 1)], t[k - 1]);
-            acc[2 + (k & 1)].add(A[2 * (k - 1) + 1], t[L2 + k - 1]);
-        }
-        if (NN >= 2) ce += acc[0].value();
-        co = acc[1].value();
-        if (NN >= 2) se = acc[2].value();
-        so = acc[3].value();
-        const long long p = ce + co, m = ce - co, q = so + se, w = so - se;
-        s[0] = p + q;
-        s[1] = p - q;
-        s[2] = m + w;
-        s[3] = m - w;
-    } else {
-        // phi = 0, pi, pi/2, 3 pi/2: cos(k phi) and sin(k phi) are 0 and +-1
-        long long ce2 = A0;
-#pragma unroll
-        for (int k = 1; k <= NN; ++k) {
-            const long long a = ((long long)A[2 * (k - 1)].h << 31) + A[2 * (k - 1)].l;
-            const long long b = ((long long)A[2 * (k - 1) + 1].h << 31) + A[2 * (k - 1) + 1].l;
-            if (k & 1) {
-                co += a;
-                so += (k & 2) ? -b : b;
-            } else {
-                ce += a;
-                ce2 += (k & 2) ? -a : a;
-            }
-        }
-        s[0] = ce + co;
-        s[1] = ce - co;
-        s[2] = ce2 + so;
-        s[3] = ce2 - so;
-    }
-}
-
-// One quad's exponentials into the azimuthal sums. `first`: the row's first quad of this item
-// (uniform), which lowers a scale that lies far above the row's exponentials. shift_moments(d)
-// shifts the row's moments down by d when the scale rises. `two`: quad 0 of a ring with an odd
-// number of pairs (e[2], e[3] are zero).
-template <int LB, typename Shift>
-__device__ __forceinline__ void fx_accumulate(const Exp (&e)[4], const int2 *__restrict__ t, int L2, bool axes,
-                                              bool two, bool first, FxSums<LB> &B, Shift &&shift_moments)
-{
-    const int mm = max(max(e[0].m, e[1].m), max(e[2].m, e[3].m));
-    if (first && B.Sx - kitrt_fx::kGuard - mm > 22) B.Sx = mm + kitrt_fx::kGuard + 2;
-    if (mm + kitrt_fx::kGuard > B.Sx) {
-        const int d = mm + kitrt_fx::kGuard + 2 - B.Sx;
-        B.Sx += d;
-        B.b0 = kitrt_fx::sar(B.b0, d);
-#pragma unroll
-        for (int j = 0; j < 2 * LB; ++j) B.b[j].scale_down(d);
-        shift_moments(d);
-    }
-    long long f[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) f[i] = (long long)kitrt_fx::shr(e[i].y, B.Sx - e[i].m);
-    const long long p = f[0] + f[1], d = f[0] - f[1], p2 = f[2] + f[3], d2 = f[2] - f[3];
-    // every shift rounds down, by half a unit on average: given back to the sum
-    const long long all = p + p2 + (two ? 1 : 2);
-    B.b0 += all;
-    if (!axes) {
-        const Limb ce = kitrt_fx::split<27>(all), co = kitrt_fx::split<27>(p - p2);
-        const Limb so = kitrt_fx::split<27>(d + d2), se = kitrt_fx::split<27>(d - d2);
-#pragma unroll
-        for (int k = 1; k <= LB; ++k) {
-            B.b[2 * (k - 1)].add(k & 1 ? co : ce, t[k - 1]);
-            B.b[2 * (k - 1) + 1].add(k & 1 ? so : se, t[L2 + k - 1]);
-        }
-    } else {
-        // the two halves of the correction cancel where p2 enters with a minus sign
-#pragma unroll
-        for (int k = 1; k <= LB; ++k) {
-            if (k & 1) {
-                B.b[2 * (k - 1)].hh += d;
-                B.b[2 * (k - 1) + 1].hh += (k & 2) ? -d2 : d2;
-            } else {
-                B.b[2 * (k - 1)].hh += (k & 2) ? p - p2 + (two ? 1 : 0) : all;
-            }
-        }
-    }
 }
 
 // Exponent of the unit of a row's moments (for fx_to_double).
