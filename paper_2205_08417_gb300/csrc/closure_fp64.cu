@@ -349,9 +349,9 @@ constexpr int kSweepThreads = 128;
 constexpr int kUnit64 = 4;
 int units64(int nquad) { return (nquad + kUnit64 - 1) / kUnit64; }
 
-// An exponential of the sweeps as a double: the range test that fx_double leaves out (rows of the
-// FP64 exponentials reach 0 and, when not finite, y = 2^61 with a large m).
-__device__ __forceinline__ double fx_psi(const Exp &e) 
+// An exponential of the sweeps as a double: the range test that fx_double leaves out (scaled rows
+// and those of the FP64 exponentials reach 0 and beyond the double range).
+__device__ __forceinline__ double fx_psi(const Exp &e)
 {
     return e.m < -1022 ? 0.0 : e.m > 1023 ? __longlong_as_double(0x7ff0000000000000LL) : kitrt_fx::fx_double(e);
 }
@@ -414,8 +414,16 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
             myA[a * kSweepThreads] = make_int2(w.h, w.l);
             bound = fmaf(fabsf(d2f_bits(x)), T.fx_mmax[a], bound);
         }
-        // rows outside the fixed-point range (or not finite) take the FP64 exponentials
-        const bool wide = !(bound < kitrt_fx::kFxMaxZ);
+        // rows outside the range are scaled down; beyond that (-1) they take FP64 exponentials
+        const int sh = fx_row_shift(bound);
+        if (sh > 0) {
+#pragma unroll 1
+            for (int a = 0; a < n; ++a) {
+                const double x = lam != 0.0 ? fma(lam, di[a], al[a]) : al[a];
+                const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(x, sh));
+                myA[a * kSweepThreads] = make_int2(w.h, w.l);
+            }
+        }
         bool bad = false;
 #pragma unroll
         for (int c = 0; c < n2; ++c) mine[c * kSweepThreads] = 0;
@@ -440,11 +448,10 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
             const int2 *tr = trig + jq * 2 * L2;
             const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
             Exp e[4];
-            if (!wide) {
-                long long s[4];
-                fx_exponents<NN>(A0, A, tr, L2, jq == 0, s);
-#pragma unroll
-                for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_exp(s[t], tab);
+            if (sh == 0) {
+                fx_quad<NN>(A0, A, tr, L2, jq == 0, tab, e);
+            } else if (sh > 0) {
+                bad = !fx_quad_scaled<NN>(A0, A, tr, L2, jq == 0, sh, tab, e) || bad;
             } else {
                 bad = !fx_slow_quad<NN>(T.Mt, T.Qp, T.exptab, al, di, lam, pa, pb, e) || bad;
             }
@@ -546,7 +553,8 @@ finish_kernel(Tables T, NewtonState S, double *__restrict__ alpha_out, double *_
         }
         sB[tid] = bound;
         sDiff[tid] = differs;
-        __syncthreads();
+        // a row outside the range has a quarter of the components outside a quarter of it
+        const bool any_wide = __syncthreads_or(!(bound < kitrt_fx::kFxMaxZ / kFinishWarps));
         differs = 0;
         bound = 0.0f;
 #pragma unroll
@@ -554,12 +562,22 @@ finish_kernel(Tables T, NewtonState S, double *__restrict__ alpha_out, double *_
             differs |= sDiff[w * 32 + lane];
             bound += sB[w * 32 + lane];
         }
+        const int sh = fx_row_shift(bound);  // outside the range: scaled down; beyond that (-1) in FP64
+        if (any_wide) {
+            if (sh > 0)
+                for (int c = warp; c < n; c += kFinishWarps) {
+                    double a = S.alpha[off + c];
+                    if (add) a += S.dir[off + c];
+                    const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(a, sh));
+                    sA[c * 32 + lane] = make_int2(w.h, w.l);
+                }
+            __syncthreads();
+        }
         const bool store = differs && base + lane < C;
         if (!__any_sync(kFull, store)) continue;
         const int qd0 = warp * T.nquad / kFinishWarps, qd1 = (warp + 1) * T.nquad / kFinishWarps;
         double *row = psi + (size_t)cell * T.Qp;
-        const bool wide = !(bound < kitrt_fx::kFxMaxZ);  // outside the fixed-point range
-        if (store && wide)
+        if (store && sh < 0)
             psi_row_fp64<NN>(T, alpha_out + off, row, warp * T.Qf / kFinishWarps, (warp + 1) * T.Qf / kFinishWarps);
         int ring = qd0 / T.J, jq = qd0 - ring * T.J;
         bool fresh = true;
@@ -577,12 +595,18 @@ finish_kernel(Tables T, NewtonState S, double *__restrict__ alpha_out, double *_
                 fresh = false;
             }
             const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
-            long long s[4];
-            fx_exponents<NN>(A0, A, trig + jq * 2 * NN, NN, jq == 0, s);
+            Exp x[4];
             double e[4];
+            if (sh == 0) {
+                fx_quad<NN>(A0, A, trig + jq * 2 * NN, NN, jq == 0, tab, x);
 #pragma unroll
-            for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_double(kitrt_fx::fx_exp(s[t], tab));
-            if (store && !wide) {
+                for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_double(x[t]);
+            } else {
+                fx_quad_scaled<NN>(A0, A, trig + jq * 2 * NN, NN, jq == 0, max(sh, 1), tab, x);
+#pragma unroll
+                for (int t = 0; t < 4; ++t) e[t] = fx_psi(x[t]);
+            }
+            if (store && sh >= 0) {
                 *(double2 *)(row + 2 * pa) = make_double2(e[0], e[1]);
                 if (pb >= 0) *(double2 *)(row + 2 * pb) = make_double2(e[2], e[3]);
             }

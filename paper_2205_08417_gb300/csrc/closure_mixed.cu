@@ -302,17 +302,27 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
             }
         }
         float bound = 0.0f;
+        auto component = [&](int a) { return !active ? 0.0 : lam != 0.0 ? fma(lam, di[a], al[a]) : al[a]; };
         for (int a = h; a < n; a += 2) {
-            double x = 0.0;
-            if (active) x = lam != 0.0 ? fma(lam, di[a], al[a]) : al[a];
+            const double x = component(a);
             const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(x));
             sA[a * kTileM + r] = make_int2(w.h, w.l);
             bound = fmaf(fabsf(d2f_bits(x)), T.fx_mmax[a], bound);
         }
         sB[tid] = bound;
-        __syncthreads();
-        // rows outside the fixed-point range (or not finite) take the FP64 exponentials
-        const bool wide = !(sB[r] + sB[kTileM + r] < kitrt_fx::kFxMaxZ);
+        // rows outside the fixed-point range (one of their halves is outside half of it) are scaled down;
+        // beyond that (-1) they take FP64 exponentials
+        const bool any_wide = __syncthreads_or(!(bound < 0.5f * kitrt_fx::kFxMaxZ));
+        const int sh = fx_row_shift(sB[r] + sB[kTileM + r]);
+        if (any_wide) {
+            if (sh > 0)
+#pragma unroll 1
+                for (int a = h; a < n; a += 2) {
+                    const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(component(a), sh));
+                    sA[a * kTileM + r] = make_int2(w.h, w.l);
+                }
+            __syncthreads();
+        }
         bool bad = false;
         long long U[n], A0 = 0;
         Limb A[2 * NN];
@@ -370,11 +380,10 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
                     const int2 *tr = trig + jq * 2 * NN;
                     const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
                     Exp e[4];
-                    if (!wide) {
-                        long long s[4];
-                        fx_exponents<NN>(A0, A, tr, NN, jq == 0, s);
-#pragma unroll
-                        for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_exp(s[t], tab);
+                    if (sh == 0) {
+                        fx_quad<NN>(A0, A, tr, NN, jq == 0, tab, e);
+                    } else if (sh > 0) {
+                        bad = !fx_quad_scaled<NN>(A0, A, tr, NN, jq == 0, sh, tab, e) || bad;
                     } else {
                         bad = !fx_slow_quad<NN>(T.Mt, Qp, T.exptab, al, di, lam, pa, pb, e) || bad;
                     }

@@ -8,7 +8,8 @@
 // products the low one is dropped, which costs at most 4 units of the result and has no bias.
 // Formats:
 //   exponent s = (alpha . m) 2048 / ln2 in units of 2^-42 (2^-53.5 of alpha . m), |s| < 2^61.5: rows
-//   with sum_c |alpha_c| max|m_c| >= kFxMaxZ take their exponentials from the FP64 kexp instead;
+//   with sum_c |alpha_c| max|m_c| >= kFxMaxZ are scaled down by a power of two (fx_row_shift), which
+//   leaves them at least 2^8 units per rounding error of an FP64 sum of that size;
 //   azimuthal factors cos(k phi), sin(k phi) in units of 2^-54, the weighted Legendre factors of
 //   the moments in units of 2^-57 of a power of two, the exponent's in units of 2^-45;
 //   exponential e = y 2^(m - 61), y in [2^61, 2^62]: T_j (1 + p) with the 2048-entry table and
@@ -38,6 +39,7 @@ namespace kitrt_fx {
 
 constexpr int kFracBits = 42;             // fraction bits of the exponent s
 constexpr float kFxMaxZ = 245.0f;         // sum_c |alpha_c| max|m_c| below this: |s| < 2^61.5
+constexpr int kMaxShift = 32;             // largest power of two of a scaled row
 constexpr int kGuard = 7;                 // y (2^62) >> 7 = 2^55
 
 struct Limb {
@@ -110,15 +112,15 @@ KITRT_FX long long moment_term(Limb b, int2 wp, int sh)
     return (wide(b.h, wp.x) << (2 - sh)) + ((t + (1LL << (29 + sh))) >> (30 + sh));
 }
 
-// A double as an integer in units of 2^-52, rounded (|x| < 2048).
-KITRT_FX long long fx_from_double(double x)
+// x 2^-sh as an integer in units of 2^-52, rounded (below 2048 in magnitude).
+KITRT_FX long long fx_from_double(double x, int sh = 0)
 {
     union {
         double d;
         uint64_t u;
     } b;
     b.d = x;
-    const int ex = (int)((b.u >> 52) & 0x7ff) - 1023;
+    const int ex = (int)((b.u >> 52) & 0x7ff) - 1023 - sh;
     const uint64_t mant = (b.u & 0xfffffffffffffULL) | (1ULL << 52);
     uint64_t v;
     if (ex >= 0) v = mant << (ex > 10 ? 10 : ex);
@@ -192,6 +194,36 @@ KITRT_FX Exp fx_exp(long long s, const uint64_t *tab)
     Exp e;
     e.y = T + (((uint64_t)Th * ph) << 8) + (((uint64_t)Th * pl + (uint64_t)Tl * ph) >> 24);
     e.m = k >> 11;
+    return e;
+}
+
+// The power of two by which a row is scaled down, from its bound sum_c |alpha_c| max|m_c|: 0 inside the
+// range, the bound below 128 otherwise; -1 for one beyond 2^38 or not finite.
+KITRT_FX int fx_row_shift(float bound)
+{
+    if (bound < kFxMaxZ) return 0;
+    union {
+        float f;
+        uint32_t u;
+    } b;
+    b.f = bound;
+    const int sh = (int)(b.u >> 23) - 127 - 6;
+    return sh <= kMaxShift ? sh : -1;
+}
+
+// 2^(s 2^sh / 2048), s in units of 2^-42, 0 < sh <= kMaxShift; as kexp, 0 at exponents of -707 and below.
+// Beyond the double range m is 1024.
+KITRT_FX Exp fx_exp_scaled(long long s, int sh, const uint64_t *tab)
+{
+    constexpr long long kFraction = (1LL << kFracBits) - 1;
+    const long long k = s >> (kFracBits - sh);
+    Exp e = fx_exp((long long)(((uint64_t)(k & 2047) << kFracBits) | (((uint64_t)s << sh) & kFraction)), tab);
+    const long long m = k >> 11;
+    e.m = m > 1024 ? 1024 : (int)m;
+    if (k <= -2088931) {  // -707 2048 / ln2
+        e.y = 0;
+        e.m = -100000;
+    }
     return e;
 }
 

@@ -67,7 +67,14 @@ learned_sweep_kernel(Tables T, NewtonState S, const double *__restrict__ alpha_n
             myA[a * kSweepThreads] = make_int2(w.h, w.l);
             bound = fmaf(fabsf(d2f_bits(x)), T.fx_mmax[a], bound);
         }
-        const bool wide = !(bound < kitrt_fx::kFxMaxZ);
+        const int sh = fx_row_shift(bound);  // outside the range: scaled down; beyond that (-1) in FP64
+        if (sh > 0) {
+#pragma unroll 1
+            for (int a = 0; a < n; ++a) {
+                const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(a ? al[a] : 0.0, sh));
+                myA[a * kSweepThreads] = make_int2(w.h, w.l);
+            }
+        }
         bool bad = false;
         long long U[n], A0 = 0;
 #pragma unroll
@@ -92,11 +99,10 @@ learned_sweep_kernel(Tables T, NewtonState S, const double *__restrict__ alpha_n
             const int2 *tr = trig + jq * 2 * NN;
             const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
             Exp e[4];
-            if (!wide) {
-                long long s[4];
-                fx_exponents<NN>(A0, A, tr, NN, jq == 0, s);
-#pragma unroll
-                for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_exp(s[t], tab);
+            if (sh == 0) {
+                fx_quad<NN>(A0, A, tr, NN, jq == 0, tab, e);
+            } else if (sh > 0) {
+                bad = !fx_quad_scaled<NN>(A0, A, tr, NN, jq == 0, sh, tab, e) || bad;
             } else {
                 bad = !fx_slow_quad<NN>(T.Mt, T.Qp, T.exptab, al, al, 0.0, pa, pb, e) || bad;
             }

@@ -40,6 +40,7 @@ using kitrt_fx::fx_accumulate;
 using kitrt_fx::fx_coeffs;
 using kitrt_fx::fx_exponents;
 using kitrt_fx::fx_flush;
+using kitrt_fx::fx_row_shift;
 using kitrt_fx::FxSums;
 using kitrt_fx::Limb;
 
@@ -51,8 +52,7 @@ __device__ __forceinline__ int quad_pair1(int ring, int j, int P)
     return j ? ring * P + P - j : (P & 1) ? -1 : ring * P + P / 2;
 }
 
-// A quad's exponentials in FP64, for rows outside the fixed-point range (very large or non-finite
-// alpha): full sums against the basis at the points of pairs pa and pb. False when one of them is
+// A quad's exponentials in FP64, for rows beyond the scaled range too (alpha of 1e11 or not finite): full sums against the basis at the points of pairs pa and pb. False when one of them is
 // not finite.
 template <int NN>
 __device__ __noinline__ bool fx_slow_exps(const double *__restrict__ Mt, int Qp, const double *__restrict__ exptab,
@@ -86,6 +86,35 @@ __device__ __forceinline__ bool fx_slow_quad(const double *__restrict__ Mt, int 
     const bool ok = fx_slow_exps<NN>(Mt, Qp, exptab, alpha, dir, lam, pa, pb, t);
 #pragma unroll
     for (int i = 0; i < 4; ++i) e[i] = t[i];
+    return ok;
+}
+
+// A quad's four exponentials inside the fixed-point range.
+template <int NN>
+__device__ __forceinline__ void fx_quad(long long A0, const Limb (&A)[2 * NN], const int2 *t, int L2, bool axes,
+                                        const uint64_t *tab, Exp (&e)[4])
+{
+    long long s[4];
+    fx_exponents<NN>(A0, A, t, L2, axes, s);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) e[i] = kitrt_fx::fx_exp(s[i], tab);
+}
+
+// The same for rows scaled down by 2^sh: they take what the others take, where FP64 exponents and
+// exponentials (a thread per row, a few rows of a warp) held the FP64 pipe for 12 times the work of a
+// warp per row. False when one of them is beyond the double range.
+template <int NN>
+__device__ __forceinline__ bool fx_quad_scaled(long long A0, const Limb (&A)[2 * NN], const int2 *t, int L2, bool axes,
+                                               int sh, const uint64_t *tab, Exp (&e)[4])
+{
+    long long s[4];
+    fx_exponents<NN>(A0, A, t, L2, axes, s);
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        e[i] = kitrt_fx::fx_exp_scaled(s[i], sh, tab);
+        ok = ok && e[i].m <= 1023;
+    }
     return ok;
 }
 

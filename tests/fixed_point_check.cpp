@@ -1,5 +1,5 @@
 // Host check of the sweeps' fixed-point arithmetic (csrc/fixed.cuh) against long double: prints, per part,
-// the largest error over its bound. usage: fixed_point_check exp | conv | sums N order
+// the largest error over its bound. usage: fixed_point_check exp | scaled | conv | sums N order
 #include "fixed.cuh"
 
 #include <math.h>
@@ -39,6 +39,32 @@ double check_exp()
     return (double)(worst * ldexpl(1, 51));
 }
 
+// 2^(s 2^sh / 2048) of scaled rows: relative error over 2^-51; 0 at -707 and below, m = 1024 beyond a double
+double check_scaled()
+{
+    const auto tab = exp_table();
+    std::mt19937_64 g(3);
+    LD worst = 0;
+    for (int i = 0; i < 2000000; ++i) {
+        const int sh = 1 + (int)(g() % kMaxShift);
+        // z in +-800, or of any size that the row's range has
+        const LD z = ((LD)(long long)g() / 9223372036854775808.0L) * (i % 4 ? 800.0L : ldexpl(128, sh));
+        const long long s = llroundl(ldexpl(z * 2048 / logl(2), kFracBits - sh));
+        const LD x = ldexpl((LD)s, sh - 53);  // log2 of the value
+        const Exp e = fx_exp_scaled(s, sh, tab.data());
+        if (x * logl(2) < -707.001L) worst = std::max(worst, (LD)(e.y == 0 && e.m < -2000 ? 0 : 1e9));
+        else if (x >= 1024) worst = std::max(worst, (LD)(e.m == 1024 ? 0 : 1e9));
+        else if (x * logl(2) > -706.999L) worst = std::max(worst, fabsl(ldexpl((LD)e.y, e.m - 61) / exp2l(x) - 1));
+    }
+    for (float b : {0.0f, 244.99f, 245.0f, 256.0f, 1e4f, 1e11f, 5e11f}) {
+        const int sh = fx_row_shift(b);
+        if (sh < 0 || !(ldexpf(b, -sh) < (sh ? 128.0f : 245.0f))) worst = 1e9;
+    }
+    for (float b : {1e13f, INFINITY, NAN})
+        if (fx_row_shift(b) != -1) worst = 1e9;
+    return (double)(worst * ldexpl(1, 51));
+}
+
 // conversions, exact up to their rounding (half a unit of the result)
 double check_conv()
 {
@@ -47,6 +73,8 @@ double check_conv()
     for (int i = 0; i < 1000000; ++i) {
         const double x = ldexp((double)(long long)g(), -63) * ldexp(1.0, (int)(g() % 80) - 70);
         worst = std::max(worst, fabsl((LD)fx_from_double(x) - ldexpl((LD)x, 52)) * 2);
+        const int down = (int)(g() % 33);
+        worst = std::max(worst, fabsl((LD)fx_from_double(x, down) - ldexpl((LD)x, 52 - down)) * 2);
         const long long v = (long long)g() >> (g() % 64);
         const int sh = (int)(g() % 200) - 100;
         const double d = fx_to_double(v, sh);
@@ -226,6 +254,7 @@ int main(int argc, char **argv)
     const char *what = argc > 1 ? argv[1] : "";
     double r = 1e9;
     if (!strcmp(what, "exp")) r = check_exp();
+    if (!strcmp(what, "scaled")) r = check_scaled();
     if (!strcmp(what, "conv")) r = check_conv();
     if (!strcmp(what, "sums") && argc > 3) {
         const int N = atoi(argv[2]), order = atoi(argv[3]);

@@ -27,6 +27,10 @@ def test_exponential(check):
     assert check("exp") <= 1.0  # 2^-51 relative
 
 
+def test_scaled_exponential(check):
+    assert check("scaled") <= 1.0  # 2^-51 relative
+
+
 def test_conversions(check):
     assert check("conv") <= 1.0  # half a unit
 
