@@ -367,7 +367,8 @@ size_t sweep64_smem(int n, int n2, int N, int J)
 enum class Cells {
     kListed,   // FP64 mode: the listed cells at their trial points
     kHanded,   // mixed modes: the cells handed over to the FP64 Hessian (positions in the list), their
-               // trial points' FP32 ansatz into psi
+               // trial points' FP32 ansatz into psi; the first part goes to the cell's own column, the
+               // others to columns from C on
     kGiven     // every cell at the given alpha (one part), its FP64 ansatz into psi (the adjoint)
 };
 
@@ -483,7 +484,8 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
             }
         }
         if (!fresh) fx_flush<L2>(T.fx_ringW + (size_t)ring * n2, T.fx_sumshift, B, moment);
-        double *col = Vacc + (size_t)part * cnt_in + slot;
+        double *col = Vacc + (!HANDED ? (size_t)part * cnt_in + slot
+                              : part ? (size_t)C + (size_t)(part - 1) * cnt_in + slot : (size_t)pos_in[slot]);
         const int unit = fx_unit(B.Sx, T);
 #pragma unroll 4
         for (int c = 0; c < n2; ++c)
@@ -794,11 +796,11 @@ int launch_post(kitrt_mn *mn, const Tables &T, const NewtonState &S, int C, cons
     if (mixed) {
         KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(post_group_kernel<NN, true>, smem));
         if (rc) return rc;
-        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, true><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, nunits, mn->grid_fp64, mn->target_fp64, nu64, upto)));
+        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, true><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->vs_handed, mn->gaunt_nnz, sweep_grid, target, nunits, mn->grid_fp64, mn->target_fp64, nu64, upto)));
     } else {
         KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(post_group_kernel<NN, false>, smem));
         if (rc) return rc;
-        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, false><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->gaunt_nnz, sweep_grid, target, nunits, mn->grid_fp64, mn->target_fp64, nu64, upto)));
+        KITRT_DISPATCH_N(mn->N, (post_group_kernel<NN, false><<<blocks, kGroupBlock, smem, s>>>(T, S, u, k, np, Vacc, mn->vs, mn->vs_handed, mn->gaunt_nnz, sweep_grid, target, nunits, mn->grid_fp64, mn->target_fp64, nu64, upto)));
     }
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }
@@ -891,7 +893,7 @@ int launch_eval_fp64(kitrt_mn *mn, const Tables &T, const NewtonState &S, const 
 
 // Mixed modes: the cells handed over to the FP64 Hessian in earlier rounds. They are few (often none)
 // and lie side by side in the list, so they are swept from a list of their own, split over as many
-// parts as fill the SMs, into columns of their own (a warp per flagged entry of the list took 0.3 to
+// parts as fill the SMs (a warp per flagged entry of the list took 0.3 to
 // 0.8 ms a round for a handful of M_5 cells, and 1.19 of 2.8 ms of a checkerboard step).
 int launch_eval_handed(kitrt_mn *mn, const Tables &T, const NewtonState &S, const double *u, int k, float *psi32,
                        cudaStream_t s)
@@ -901,7 +903,7 @@ int launch_eval_handed(kitrt_mn *mn, const Tables &T, const NewtonState &S, cons
     int rc = KITRT_OK;
     KITRT_DISPATCH_N(mn->N, rc = ensure_dyn_smem(sweep64_kernel<NN, Cells::kHanded>, smem));
     if (rc) return rc;
-    KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN, Cells::kHanded><<<mn->grid_fp64, kSweepThreads, smem, s>>>(T, S, u, k, mn->d_Vacc + mn->vs / 2, mn->vs, mn->target_fp64, nullptr, psi32, 0)));
+    KITRT_DISPATCH_N(mn->N, (sweep64_kernel<NN, Cells::kHanded><<<mn->grid_fp64, kSweepThreads, smem, s>>>(T, S, u, k, mn->d_Vacc, mn->vs, mn->target_fp64, nullptr, psi32, mn->vs_handed)));
     return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
 }
 

@@ -777,8 +777,10 @@ int32_t kitrt_mn_init(const kitrt_mesh *mesh, const kitrt_mn_params *params, kit
     mn->target_mixed = 4 * mn->grid_mixed;
     mn->grid_fp64 = fp64_sweep_grid(mn);
     mn->target_fp64 = 2 * mn->grid_fp64;
-    mn->vs = (int)C + 128 * std::max(mn->target_mixed, mn->target_fp64) + 128;
-    if (p.mode != KITRT_FP64) mn->vs *= 2;
+    // In the mixed modes the handed-over cells' sweep puts its first part into the cell's own column,
+    // which the tensor-core sweep leaves alone, and the others (at most 128 columns per item) behind.
+    mn->vs_handed = (int)C + 128 * std::max(mn->target_mixed, mn->target_fp64) + 128;
+    mn->vs = mn->vs_handed + (p.mode != KITRT_FP64 ? 128 * mn->target_fp64 : 0);
     TRY(dev_alloc(mn, &mn->d_Vacc, (size_t)mn->vs * n2));
     if (cudaMemset(mn->d_Vacc, 0, sizeof(double) * (size_t)mn->vs * n2) != cudaSuccess) {
         kitrt_mn_destroy(mn);

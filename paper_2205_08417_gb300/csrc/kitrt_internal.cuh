@@ -137,8 +137,8 @@ struct kitrt_mn {
     float *d_wox32 = nullptr, *d_woy32 = nullptr, *d_mbar32 = nullptr;
     double *d_V = nullptr;               // [C x n2] moments scratch (kitrt_hessian)
     double *d_Vacc = nullptr;            // [n2 x vs] sweeps: partial moments per list slot and part; in the
-                                         // mixed modes the second half of the columns is for handed cells
-    int vs = 0;                          // column stride of d_Vacc
+                                         // mixed modes, from vs_handed on, the handed cells' later parts
+    int vs = 0, vs_handed = 0;           // column stride of d_Vacc, first column of those parts
     int target_mixed = 0, target_fp64 = 0;  // work items the sweeps aim at per launch
     int grid_mixed = 0, grid_fp64 = 0;      // persistent grids of the sweeps
     int R = 0, P = 0, J = 0, Qs = 0;     // rings, pairs and quads per ring, points of a sweep (padded)

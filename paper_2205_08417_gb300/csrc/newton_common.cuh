@@ -696,8 +696,8 @@ __host__ __device__ inline size_t group_smem_bytes(int n2, int npairs, int nnz, 
 template <int NN, bool MIXED>
 __global__ void __launch_bounds__(kGroupBlock, MIXED && NN <= 3 ? 3 : 2)
 post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, NewtonParams np,
-                  const double *__restrict__ Vacc, int vs, int nnz, int sweep_grid, int target_items, int nunits, int grid64,
-                  int target64, int nunits64, int upto)
+                  const double *__restrict__ Vacc, int vs, int vs_handed, int nnz, int sweep_grid, int target_items,
+                  int nunits, int grid64, int target64, int nunits64, int upto)
 {
     constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, npairs = Dims<NN>::npairs, SL = (n + 7) / 8;
     extern __shared__ __align__(16) unsigned char group_smem[];
@@ -714,7 +714,7 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
     // uniform: not this kernel's round, or no slot for this block
     if (cnt_in > upto || (int)blockIdx.x * kGroupCells >= cnt_in) return;
     const int parts = sweep_split(cnt_in, sweep_grid, target_items, nunits).parts;
-    // handed cells: columns from vs / 2 on, split on their own
+    // handed cells: split on their own, the parts after the first from column vs_handed on
     const int handed = MIXED ? S.cnt[12 + k % 3] : 0;
     const int parts64 = MIXED ? sweep_split(handed, grid64, target64, nunits64).parts : 1;
     int32_t *cnt_out = &S.cnt[(k + 1) % 3];
@@ -765,7 +765,7 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
         for (int e = tid; e < n2 * kGroupCells; e += kGroupBlock) {
             const int c = e / kGroupCells, j = e % kGroupCells;
             const int f = MIXED ? sh64[j] : 0;  // 1 + place among the handed cells
-            const double *col = Vacc + (size_t)c * vs + (f ? vs / 2 + f - 1 : min(base + j, cnt_in - 1));
+            const double *col = Vacc + (size_t)c * vs + min(base + j, cnt_in - 1);
             if (MIXED && c >= n && !sh64[j]) {
                 float v = d2f_bits(col[0]);
 #pragma unroll 4
@@ -773,9 +773,10 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
                 sVf[c * kGroupPitch + j] = v;
             } else {
                 const int np_ = f ? parts64 : parts, step = f ? handed : cnt_in;
+                const double *more = f ? Vacc + (size_t)c * vs + vs_handed + f - 1 : col + cnt_in;
                 double v = col[0];
 #pragma unroll 4
-                for (int p = 1; p < np_; ++p) v += col[(size_t)p * step];
+                for (int p = 1; p < np_; ++p) v += more[(size_t)(p - 1) * step];
                 sV[c * kGroupPitch + j] = v;
                 if (MIXED) sVf[c * kGroupPitch + j] = d2f_bits(v);
             }
