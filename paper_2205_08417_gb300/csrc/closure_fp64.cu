@@ -349,12 +349,9 @@ constexpr int kSweepThreads = 128;
 constexpr int kUnit64 = 4;
 int units64(int nquad) { return (nquad + kUnit64 - 1) / kUnit64; }
 
-// An exponential of the sweeps as a double: the range test that fx_double leaves out (scaled rows
-// and those of the FP64 exponentials reach 0 and beyond the double range).
-__device__ __forceinline__ double fx_psi(const Exp &e)
-{
-    return e.m < -1022 ? 0.0 : e.m > 1023 ? __longlong_as_double(0x7ff0000000000000LL) : kitrt_fx::fx_double(e);
-}
+// An exponential of the sweeps as a double, with the range test that fx_double leaves out (rows outside the
+// fixed-point range reach 2^-1024).
+__device__ __forceinline__ double fx_psi(const Exp &e) { return e.m < -1022 ? 0.0 : kitrt_fx::fx_double(e); }
 
 // Dynamic shared memory of sweep64_kernel: the exp table, the moments [n2][thread] and the trial
 // alpha's limbs [n][thread], the azimuthal factors.
@@ -417,14 +414,7 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
         }
         // rows outside the range are scaled down; beyond that (-1) they take FP64 exponentials
         const int sh = fx_row_shift(bound);
-        if (sh > 0) {
-#pragma unroll 1
-            for (int a = 0; a < n; ++a) {
-                const double x = lam != 0.0 ? fma(lam, di[a], al[a]) : al[a];
-                const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(x, sh));
-                myA[a * kSweepThreads] = make_int2(w.h, w.l);
-            }
-        }
+        if (sh > 0) fx_scale_limbs(al, di, lam, 0, 1, n, sh, myA, kSweepThreads);
         bool bad = false;
 #pragma unroll
         for (int c = 0; c < n2; ++c) mine[c * kSweepThreads] = 0;
@@ -449,13 +439,13 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
             const int2 *tr = trig + jq * 2 * L2;
             const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
             Exp e[4];
-            if (sh == 0) {
-                fx_quad<NN>(A0, A, tr, L2, jq == 0, tab, e);
-            } else if (sh > 0) {
-                bad = !fx_quad_scaled<NN>(A0, A, tr, L2, jq == 0, sh, tab, e) || bad;
-            } else {
-                bad = !fx_slow_quad<NN>(T.Mt, T.Qp, T.exptab, al, di, lam, pa, pb, e) || bad;
-            }
+            long long s[4];
+            fx_exponents<NN>(A0, A, tr, L2, jq == 0, s);
+            if (sh != 0)
+                bad = !fx_outside_quad<NN>(sh, T, point_of(S, GIVEN ? alpha : nullptr),
+                                           GIVEN ? slot : list_in[HANDED ? pos_in[slot] : slot], pa, pb, s) || bad;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_exp(s[t], tab);
             if (HANDED) {
                 // ansatz of the trial point (the last accepted trial leaves the solution's)
                 if (psi) {
@@ -474,7 +464,7 @@ sweep64_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, dou
             }
             if (pb < 0) e[2] = e[3] = Exp{0, -100000};
             fx_accumulate<L2>(e, tr, L2, jq == 0, qd == q_begin, B, [&](int d) {
-                for (int c = 0; c < n2; ++c) mine[c * kSweepThreads] = kitrt_fx::sar_round(mine[c * kSweepThreads], d);
+                for (int c = 0; c < n2; ++c) mine[c * kSweepThreads] = kitrt_fx::sar(mine[c * kSweepThreads], d);
             });
             if (++jq == T.J) {
                 fx_flush<L2>(T.fx_ringW + (size_t)ring * n2, T.fx_sumshift, B, moment);
@@ -597,16 +587,18 @@ finish_kernel(Tables T, NewtonState S, double *__restrict__ alpha_out, double *_
                 fresh = false;
             }
             const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
-            Exp x[4];
+            long long s[4];
+            fx_exponents<NN>(A0, A, trig + jq * 2 * NN, NN, jq == 0, s);
             double e[4];
             if (sh == 0) {
-                fx_quad<NN>(A0, A, trig + jq * 2 * NN, NN, jq == 0, tab, x);
 #pragma unroll
-                for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_double(x[t]);
+                for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_double(kitrt_fx::fx_exp(s[t], tab));
             } else {
-                fx_quad_scaled<NN>(A0, A, trig + jq * 2 * NN, NN, jq == 0, max(sh, 1), tab, x);
 #pragma unroll
-                for (int t = 0; t < 4; ++t) e[t] = fx_psi(x[t]);
+                for (int t = 0; t < 4; ++t) {
+                    const bool ok = sh < 0 || kitrt_fx::fx_unscale(s[t], sh);
+                    e[t] = ok ? fx_psi(kitrt_fx::fx_exp(s[t], tab)) : __longlong_as_double(0x7ff0000000000000LL);
+                }
             }
             if (store && sh >= 0) {
                 *(double2 *)(row + 2 * pa) = make_double2(e[0], e[1]);

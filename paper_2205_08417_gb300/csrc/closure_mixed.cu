@@ -315,12 +315,7 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
         const bool any_wide = __syncthreads_or(!(bound < 0.5f * kitrt_fx::kFxMaxZ));
         const int sh = fx_row_shift(sB[r] + sB[kTileM + r]);
         if (any_wide) {
-            if (sh > 0)
-#pragma unroll 1
-                for (int a = h; a < n; a += 2) {
-                    const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(component(a), sh));
-                    sA[a * kTileM + r] = make_int2(w.h, w.l);
-                }
+            if (sh > 0) fx_scale_limbs(al, di, lam, h, 2, n, sh, sA + r, kTileM);
             __syncthreads();
         }
         bool bad = false;
@@ -380,17 +375,16 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
                     const int2 *tr = trig + jq * 2 * NN;
                     const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
                     Exp e[4];
-                    if (sh == 0) {
-                        fx_quad<NN>(A0, A, tr, NN, jq == 0, tab, e);
-                    } else if (sh > 0) {
-                        bad = !fx_quad_scaled<NN>(A0, A, tr, NN, jq == 0, sh, tab, e) || bad;
-                    } else {
-                        bad = !fx_slow_quad<NN>(T.Mt, Qp, T.exptab, al, di, lam, pa, pb, e) || bad;
-                    }
+                    long long s[4];
+                    fx_exponents<NN>(A0, A, tr, NN, jq == 0, s);
+                    if (sh != 0)
+                        bad = !fx_outside_quad<NN>(sh, T, point_of(S, MOMENTS_ONLY ? alpha_in : nullptr), cell, pa, pb, s) || bad;
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_exp(s[t], tab);
                     if (pb < 0) e[2] = e[3] = Exp{0, -100000};
                     fx_accumulate<NN>(e, tr, NN, jq == 0, i == 0 && c == c_begin, B, [&](int d) {
 #pragma unroll
-                        for (int a = 0; a < n; ++a) U[a] = kitrt_fx::sar_round(U[a], d);
+                        for (int a = 0; a < n; ++a) U[a] = kitrt_fx::sar(U[a], d);
                     });
 #pragma unroll
                     for (int t = 0; t < 4; ++t) f[t] = __uint_as_float(kitrt_fx::fx_float_bits(e[t]));
@@ -469,7 +463,7 @@ eval_mixed_kernel(Tables T, NewtonState S, int k, const void *__restrict__ Mhi,
             const int top = poison ? 0 : max(B.Sx, x1), unit = fx_unit(top, T);
 #pragma unroll
             for (int a = 0; a < n; ++a) {
-                const long long v = poison ? 0 : kitrt_fx::sar_round(U[a], top - B.Sx) + kitrt_fx::sar_round(sU[a * kTileM + r], top - x1);
+                const long long v = poison ? 0 : kitrt_fx::sar(U[a], top - B.Sx) + kitrt_fx::sar(sU[a * kTileM + r], top - x1);
                 row[(size_t)a * vs_c] = poison ? __longlong_as_double(0x7ff8000000000000LL) : kitrt_fx::fx_to_double(v, unit);
             }
         }

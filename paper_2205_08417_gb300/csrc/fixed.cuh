@@ -17,7 +17,7 @@
 //   2^-57); |error| of y below 2^-51 relative;
 //   sums in units of 2^(Sx - 61): e is shifted down by Sx - m >= 7, so that it stays below 2^55 and
 //   32 quads fit; Sx belongs to the row and is raised (and the sums shifted) when a larger
-//   exponential appears. Shifts round to nearest: an exponential far below the row's largest adds no
+//   exponential appears. Exponentials are rounded to nearest: one far below the row's largest adds no
 //   more than itself to the error, so that the moments of a peaked density, whose Hessian is badly
 //   conditioned, are as good as FP64 sums (rounding down and adding the mean half unit back put half
 //   a unit per point into them: up to 300 times the FP64 error in the Hessian's own metric).
@@ -65,7 +65,6 @@ KITRT_FX int imax(int a, int b) { return a > b ? a : b; }
 // y / 2^n rounded to the nearest integer (halves up), n >= 1
 KITRT_FX uint64_t shr_round(uint64_t y, int n) { return (shr(y, n - 1) + 1) >> 1; }
 KITRT_FX long long sar(long long y, int n) { return y >> (n > 63 ? 63 : n); }
-KITRT_FX long long sar_round(long long y, int n) { return n > 0 ? (sar(y, n - 1) + 1) >> 1 : y; }
 
 // v = h 2^B + l, |l| <= 2^(B - 1), for |v| < 2^(30 + B)
 template <int B>
@@ -101,7 +100,7 @@ struct SumAcc {
         m += wide(e.l, t.x);
     }
     KITRT_FX long long value() const { return hh + (m >> 27); }
-    KITRT_FX void scale_down(int n) { hh = sar_round(hh, n), m = sar_round(m, n); }
+    KITRT_FX void scale_down(int n) { hh = sar(hh, n), m = sar(m, n); }
 };
 
 // One term B w P of a moment: B an azimuthal sum (below 2^62, split<32>), wP in units of 2^-57 (split<27>),
@@ -211,40 +210,23 @@ KITRT_FX int fx_row_shift(float bound)
     return sh <= kMaxShift ? sh : -1;
 }
 
-// 2^(s 2^sh / 2048), s in units of 2^-42, 0 < sh <= kMaxShift; as kexp, 0 at exponents of -707 and below.
-// Beyond the double range m is 1024.
-KITRT_FX Exp fx_exp_scaled(long long s, int sh, const uint64_t *tab)
+// s 2^sh of a scaled row, 0 < sh <= kMaxShift: an s of 64 bits reaches as far as the doubles (-+ 709.78). As in
+// kexp, exponents of -707 and below give no more than 2^-1024, which a double moment or ansatz has as
+// 0. False, and the largest s, beyond the double range.
+KITRT_FX bool fx_unscale(long long &s, int sh)
 {
-    constexpr long long kFraction = (1LL << kFracBits) - 1;
     const long long k = s >> (kFracBits - sh);
-    Exp e = fx_exp((long long)(((uint64_t)(k & 2047) << kFracBits) | (((uint64_t)s << sh) & kFraction)), tab);
-    const long long m = k >> 11;
-    e.m = m > 1024 ? 1024 : (int)m;
-    if (k <= -2088931) {  // -707 2048 / ln2
-        e.y = 0;
-        e.m = -100000;
-    }
-    return e;
+    const bool low = k <= -2088931, high = k > (1 << 21) - 1;  // -707 2048 / ln2; 2^21: 2^1024
+    s = low ? INT64_MIN : high ? INT64_MAX : (long long)((uint64_t)s << sh);
+    return !high;
 }
 
-// A non-negative double (kexp's result) as (y, m); 0 gives (0, very small m). Returns false for
-// an infinity or NaN.
-KITRT_FX bool fx_exp_from_double(double d, Exp &e)
+// The same of an exponent in FP64 (NaN: false).
+KITRT_FX bool fx_exponent_of(double z, long long &s)
 {
-    union {
-        double d;
-        uint64_t u;
-    } b;
-    b.d = d;
-    const int ex = (int)(b.u >> 52);
-    e.y = b.u ? ((b.u & 0xfffffffffffffULL) | (1ULL << 52)) << 9 : 0;
-    e.m = b.u ? ex - 1023 : -100000;
-    if (ex >= 0x7ff) {
-        e.y = 1ULL << 61;
-        e.m = 0;
-        return false;
-    }
-    return true;
+    const bool ok = z < 709.78, live = ok && z > -707.0;
+    s = live ? (long long)(z * (2954.639443740597 * 4398046511104.0)) : ok ? INT64_MIN : INT64_MAX;
+    return ok;
 }
 
 // e as a float's bits, rounded half up; below the smallest normal float 0, beyond the range +inf.
@@ -389,7 +371,7 @@ KITRT_FX void fx_accumulate(const Exp (&e)[4], const int2 *t, int L2, bool axes,
     if (mm + kGuard > B.Sx) {
         const int d = mm + kGuard + 1 - B.Sx;
         B.Sx += d;
-        B.b0 = sar_round(B.b0, d);
+        B.b0 = sar(B.b0, d);
 #pragma unroll
         for (int j = 0; j < 2 * LB; ++j) B.b[j].scale_down(d);
         shift_moments(d);

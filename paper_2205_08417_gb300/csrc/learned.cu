@@ -68,13 +68,7 @@ learned_sweep_kernel(Tables T, NewtonState S, const double *__restrict__ alpha_n
             bound = fmaf(fabsf(d2f_bits(x)), T.fx_mmax[a], bound);
         }
         const int sh = fx_row_shift(bound);  // outside the range: scaled down; beyond that (-1) in FP64
-        if (sh > 0) {
-#pragma unroll 1
-            for (int a = 0; a < n; ++a) {
-                const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(a ? al[a] : 0.0, sh));
-                myA[a * kSweepThreads] = make_int2(w.h, w.l);
-            }
-        }
+        if (sh > 0) fx_scale_limbs(al, al, 0.0, 0, 1, n, sh, myA, kSweepThreads);  // al[0] = 0
         bool bad = false;
         long long U[n], A0 = 0;
 #pragma unroll
@@ -99,13 +93,11 @@ learned_sweep_kernel(Tables T, NewtonState S, const double *__restrict__ alpha_n
             const int2 *tr = trig + jq * 2 * NN;
             const int pa = quad_pair0(ring, jq, T.P), pb = quad_pair1(ring, jq, T.P);
             Exp e[4];
-            if (sh == 0) {
-                fx_quad<NN>(A0, A, tr, NN, jq == 0, tab, e);
-            } else if (sh > 0) {
-                bad = !fx_quad_scaled<NN>(A0, A, tr, NN, jq == 0, sh, tab, e) || bad;
-            } else {
-                bad = !fx_slow_quad<NN>(T.Mt, T.Qp, T.exptab, al, al, 0.0, pa, pb, e) || bad;
-            }
+            long long s[4];
+            fx_exponents<NN>(A0, A, tr, NN, jq == 0, s);
+            if (sh != 0) bad = !fx_outside_quad<NN>(sh, T, point_of(S, alpha_nn), cell, pa, pb, s) || bad;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) e[t] = kitrt_fx::fx_exp(s[t], tab);
             if (psi32) {
                 float *row = psi32 + (size_t)cell * T.Qp;
                 float f[4];
@@ -117,7 +109,7 @@ learned_sweep_kernel(Tables T, NewtonState S, const double *__restrict__ alpha_n
             if (pb < 0) e[2] = e[3] = Exp{0, -100000};
             fx_accumulate<NN>(e, tr, NN, jq == 0, qd == q_begin, B, [&](int d) {
 #pragma unroll
-                for (int c = 0; c < n; ++c) U[c] = kitrt_fx::sar_round(U[c], d);
+                for (int c = 0; c < n; ++c) U[c] = kitrt_fx::sar(U[c], d);
             });
             if (++jq == T.J) {
                 fx_flush<NN>(T.fx_ringW + (size_t)ring * Dims<NN>::n2, T.fx_sumshift, B, moment);

@@ -52,70 +52,69 @@ __device__ __forceinline__ int quad_pair1(int ring, int j, int P)
     return j ? ring * P + P - j : (P & 1) ? -1 : ring * P + P / 2;
 }
 
-// A quad's exponentials in FP64, for rows beyond the scaled range too (alpha of 1e11 or not finite): full sums against the basis at the points of pairs pa and pb. False when one of them is
-// not finite.
+// Where a row's trial point lies: a given alpha (phase NULL), or the Newton state's alpha + lam dir.
+struct NewtonPoint {
+    const double *alpha, *dir, *lam;
+    const int32_t *phase;
+};
+__device__ __forceinline__ NewtonPoint point_of(const NewtonState &S, const double *given)
+{
+    return given ? NewtonPoint{given, given, nullptr, nullptr} : NewtonPoint{S.alpha, S.dir, S.lam, S.phase};
+}
+
+// The exponents s of a quad (points of pairs pa and pb) of a row outside the fixed-point range, in the units of
+// the others: scaled back by 2^sh, or, for alpha of 1e11 or not finite (sh = -1), full FP64 sums against
+// the basis. False when one is beyond the double range. The trial point (given, or that of the Newton
+// state) is read again here, and the function is not inlined, so that the other rows carry none of
+// it. Scaled rows take what the others take; FP64 exponents and exponentials (a thread per row, a few
+// rows of a warp) held the FP64 pipe for 12 times the work of a warp per row.
 template <int NN>
-__device__ __noinline__ bool fx_slow_exps(const double *__restrict__ Mt, int Qp, const double *__restrict__ exptab,
-                                          const double *alpha, const double *dir, double lam, int pa, int pb, Exp *e)
+__device__ __noinline__ bool fx_outside(int sh, const double *__restrict__ Mt, int Qp, const NewtonPoint at, int cell,
+                                        int pa, int pb, long long *s)
 {
     constexpr int n = (NN + 1) * (NN + 2) / 2;
     bool ok = true;
+    if (sh > 0) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) ok = kitrt_fx::fx_unscale(s[t], sh) && ok;
+        return ok;
+    }
+    if (cell < 0) return true;  // a place without a cell
+    const double *alpha = at.alpha + (size_t)cell * n, *dir = at.dir + (size_t)cell * n;
+    const double lam = at.phase && at.phase[cell] == PH_NEWTON ? at.lam[cell] : 0.0;
 #pragma unroll 1
     for (int t = 0; t < 4; ++t) {
         const int q = 2 * (t < 2 ? pa : max(pb, 0)) + (t & 1);
         double z = 0.0;
 #pragma unroll 1
-        for (int c = 0; c < n; ++c) {
-            const double a = lam != 0.0 ? fma(lam, dir[c], alpha[c]) : alpha[c];
-            z = fma(a, __ldg(Mt + (size_t)c * Qp + q), z);
-        }
-        ok = kitrt_fx::fx_exp_from_double(kexp(z, exptab), e[t]) && ok;
+        for (int c = 0; c < n; ++c) z = fma(lam != 0.0 ? fma(lam, dir[c], alpha[c]) : alpha[c], __ldg(Mt + (size_t)c * Qp + q), z);
+        ok = kitrt_fx::fx_exponent_of(z, s[t]) && ok;
     }
     return ok;
 }
 
-// The same into registers: an array whose address goes to a function that is not inlined stays in local
-// memory, for the fixed-point path too, which then stores and loads every exponential through it
-// (1.9 of 7 stalls an issue on local loads; mixed sweep, M_3, 99,458 cells, 12 rounds: 1.70 -> 1.53 ms).
+// The same on registers: an array whose address goes to a function that is not inlined stays in local
+// memory, and the other rows' exponents with it if it were the same one.
 template <int NN>
-__device__ __forceinline__ bool fx_slow_quad(const double *__restrict__ Mt, int Qp, const double *__restrict__ exptab,
-                                             const double *alpha, const double *dir, double lam, int pa, int pb,
-                                             Exp (&e)[4])
+__device__ __forceinline__ bool fx_outside_quad(int sh, const Tables &T, const NewtonPoint &at, int cell, int pa, int pb,
+                                                long long (&s)[4])
 {
-    Exp t[4];
-    const bool ok = fx_slow_exps<NN>(Mt, Qp, exptab, alpha, dir, lam, pa, pb, t);
+    long long t[4] = {s[0], s[1], s[2], s[3]};
+    const bool ok = fx_outside<NN>(sh, T.Mt, T.Qp, at, cell, pa, pb, t);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) e[i] = t[i];
+    for (int i = 0; i < 4; ++i) s[i] = t[i];
     return ok;
 }
 
-// A quad's four exponentials inside the fixed-point range.
-template <int NN>
-__device__ __forceinline__ void fx_quad(long long A0, const Limb (&A)[2 * NN], const int2 *t, int L2, bool axes,
-                                        const uint64_t *tab, Exp (&e)[4])
+// Limbs of a row's trial alpha 2^-sh, components from, from + step, ...
+__device__ __noinline__ static void fx_scale_limbs(const double *alpha, const double *dir, double lam, int from, int step,
+                                                   int n, int sh, int2 *limbs, int pitch)
 {
-    long long s[4];
-    fx_exponents<NN>(A0, A, t, L2, axes, s);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) e[i] = kitrt_fx::fx_exp(s[i], tab);
-}
-
-// The same for rows scaled down by 2^sh: they take what the others take, where FP64 exponents and
-// exponentials (a thread per row, a few rows of a warp) held the FP64 pipe for 12 times the work of a
-// warp per row. False when one of them is beyond the double range.
-template <int NN>
-__device__ __forceinline__ bool fx_quad_scaled(long long A0, const Limb (&A)[2 * NN], const int2 *t, int L2, bool axes,
-                                               int sh, const uint64_t *tab, Exp (&e)[4])
-{
-    long long s[4];
-    fx_exponents<NN>(A0, A, t, L2, axes, s);
-    bool ok = true;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        e[i] = kitrt_fx::fx_exp_scaled(s[i], sh, tab);
-        ok = ok && e[i].m <= 1023;
+#pragma unroll 1
+    for (int c = from; c < n; c += step) {
+        const Limb w = kitrt_fx::split<32>(kitrt_fx::fx_from_double(lam != 0.0 ? fma(lam, dir[c], alpha[c]) : alpha[c], sh));
+        limbs[c * pitch] = make_int2(w.h, w.l);
     }
-    return ok;
 }
 
 // Exponent of the unit of a row's moments (for fx_to_double).

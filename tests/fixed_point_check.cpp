@@ -39,7 +39,7 @@ double check_exp()
     return (double)(worst * ldexpl(1, 51));
 }
 
-// 2^(s 2^sh / 2048) of scaled rows: relative error over 2^-51; 0 at -707 and below, m = 1024 beyond a double
+// 2^(s 2^sh / 2048) of scaled rows: relative error over 2^-51; 2^-1024 at -707 and below, refused beyond a double
 double check_scaled()
 {
     const auto tab = exp_table();
@@ -51,10 +51,24 @@ double check_scaled()
         const LD z = ((LD)(long long)g() / 9223372036854775808.0L) * (i % 4 ? 800.0L : ldexpl(128, sh));
         const long long s = llroundl(ldexpl(z * 2048 / logl(2), kFracBits - sh));
         const LD x = ldexpl((LD)s, sh - 53);  // log2 of the value
-        const Exp e = fx_exp_scaled(s, sh, tab.data());
-        if (x * logl(2) < -707.001L) worst = std::max(worst, (LD)(e.y == 0 && e.m < -2000 ? 0 : 1e9));
-        else if (x >= 1024) worst = std::max(worst, (LD)(e.m == 1024 ? 0 : 1e9));
-        else if (x * logl(2) > -706.999L) worst = std::max(worst, fabsl(ldexpl((LD)e.y, e.m - 61) / exp2l(x) - 1));
+        long long full = s;
+        const bool in = fx_unscale(full, sh);
+        const Exp e = fx_exp(full, tab.data());
+        if (x * logl(2) < -707.001L) worst = std::max(worst, (LD)(in && e.m == -1024 ? 0 : 1e9));
+        else if (x >= 1024) worst = std::max(worst, (LD)(!in && e.m == 1023 ? 0 : 1e9));
+        else if (x * logl(2) > -706.999L) worst = std::max(worst, in ? fabsl(ldexpl((LD)e.y, e.m - 61) / exp2l(x) - 1) : 1e9L);
+    }
+    for (double z : {0.0, -1e-300, -706.99, 1.0, -3.25, 700.0, 709.7}) {
+        long long s;
+        const bool in = fx_exponent_of(z, s);
+        // the exponent rounded twice to 53 bits
+        const LD tol = ldexpl(1, -51) + ldexpl(fabs(z), -51);
+        const Exp e = fx_exp(s, tab.data());
+        worst = std::max(worst, in ? fabsl(ldexpl((LD)e.y, e.m - 61) / expl(z) - 1) / tol * ldexpl(1, -51) : 1e9L);
+    }
+    for (double z : {709.79, (double)INFINITY, (double)NAN, -707.0, -1e300, (double)-INFINITY}) {
+        long long s;
+        if (fx_exponent_of(z, s) != (z < 0) || s != (z < 0 ? INT64_MIN : INT64_MAX)) worst = 1e9;
     }
     for (float b : {0.0f, 244.99f, 245.0f, 256.0f, 1e4f, 1e11f, 5e11f}) {
         const int sh = fx_row_shift(b);
@@ -87,7 +101,7 @@ double check_conv()
 // Moments of one pass over the rule, degree 2N, against the sums of the same (rounded) exponentials and tables.
 // In units of the sums: an exponential e is rounded by at most min(e, 1/2), a quad's dropped low
 // product is at most min(c, 2^26) 2^-28 (c: the quad's combination), each azimuthal sum is rounded by
-// 1/2, each ring's term of a moment by 2^sh / 2; when the scale rises, each sum by 1/2 more. These
+// 1/2, each ring's term of a moment by 2^sh / 2; when the scale rises, each sum loses up to 1. These
 // are independent and without bias, so that the bound is six standard deviations (each at most its
 // largest value over sqrt 3) of their sum: a bias of a fraction of a unit per point fails it.
 template <int N>
@@ -198,7 +212,7 @@ double check_sums(int order)
                     if (pass)
                         fx_accumulate<L2>(q, &trig[(size_t)j * 2 * L2], L2, j == 0, r + j == 0, B, [&](int d) {
                             ++raises;
-                            for (auto &x : V) x = sar_round(x, d);
+                            for (auto &x : V) x = sar(x, d);
                         });
                 }
                 if (pass)
@@ -209,7 +223,7 @@ double check_sums(int order)
         for (int l = 0; l <= L2; ++l)
             for (int k = -l; k <= l; k += 2) {
                 const int c = cindex(l, k), ak = abs(k);
-                LD ref = 0, var = raises * ldexpl(0.25L, 2 * sh);  // 3 x variance
+                LD ref = 0, var = raises * ldexpl(1.0L, 2 * sh);  // 3 x variance
                 for (int r = 0; r < R; ++r) {
                     LD b = 0, vb = k ? 0.25L : 0;
                     for (int j = 0; j < J; ++j) {
@@ -241,7 +255,7 @@ double check_sums(int order)
                     }
                     const LD wp = value(rW[(size_t)r * n2 + c], 57);
                     ref += b * wp;
-                    var += (vb + 0.25L * raises) * wp * wp + ldexpl(0.25L, 2 * sh);
+                    var += (vb + 1.0L * raises) * wp * wp + ldexpl(0.25L, 2 * sh);
                 }
                 worst = std::max(worst, fabsl(ldexpl((LD)V[c], sh) - ref) / (6 * sqrtl(var / 3)));
             }
