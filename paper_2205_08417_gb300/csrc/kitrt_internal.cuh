@@ -178,7 +178,8 @@ struct kitrt_mn {
     size_t adj_bytes = 0;
     void *d_sn_cell = nullptr;     // [C x 12] per-cell coefficients of the S_N step (FP32 or FP64)
     cudaEvent_t sn_done = nullptr; // end of the last S_N call, which the next waits for on its stream
-    bool sn_pending = false;       // sn_done has been recorded
+    bool sn_pending = false;       // sn_done has been recorded, on the stream of this id
+    unsigned long long sn_stream = 0;
     std::vector<void *> allocs;
     // tracing
     bool prof_on = false;

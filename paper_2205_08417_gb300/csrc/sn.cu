@@ -291,8 +291,12 @@ int32_t kitrt_sn_step(kitrt_mn *mn, void *psi, void *work, int32_t fp32, const d
     if (captured) {
         if (cudaMallocAsync(&cellc, (fp32 ? 4 : 8) * (size_t)mn->mesh->C * kCellSlots, s) != cudaSuccess)
             return KITRT_ENOMEM;
-    } else if (mn->sn_pending && cudaStreamWaitEvent(s, mn->sn_done, 0) != cudaSuccess) {
-        return KITRT_ECUDA;
+    }
+    unsigned long long id = 0;  // of the stream, unlike its handle never used again
+    if (!captured) {
+        if (cudaStreamGetId(s, &id) != cudaSuccess) return KITRT_ECUDA;
+        if (mn->sn_pending && id != mn->sn_stream && cudaStreamWaitEvent(s, mn->sn_done, 0) != cudaSuccess)
+            return KITRT_ECUDA;
     }
     int rc;
     if (fp32) {
@@ -309,6 +313,7 @@ int32_t kitrt_sn_step(kitrt_mn *mn, void *psi, void *work, int32_t fp32, const d
     if (captured) return cudaFreeAsync(cellc, s) != cudaSuccess && !rc ? KITRT_ECUDA : rc;
     if (cudaEventRecord(mn->sn_done, s) != cudaSuccess) return rc ? rc : KITRT_ECUDA;
     mn->sn_pending = true;
+    mn->sn_stream = id;
     return rc;
 }
 
