@@ -38,9 +38,10 @@ struct QuadLane {
     int ci, j;
     int oA1, oA2, oB1, oB2;
     F sA, cA, sB, cB;
-    __device__ __forceinline__ QuadLane(const QuadTab<F> &X, int lane)
+    // lane: this thread's place among the `width` threads that share cells
+    __device__ __forceinline__ QuadLane(const QuadTab<F> &X, int lane, int width = 32)
     {
-        const int cpw = 32 / X.J, P = X.P;
+        const int cpw = width / X.J, P = X.P;
         live = lane < cpw * X.J;
         ci = live ? lane / X.J : cpw - 1;
         j = live ? lane - ci * X.J : 0;

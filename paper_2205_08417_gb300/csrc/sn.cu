@@ -63,21 +63,55 @@ __global__ void sn_cell_prep_kernel(const double *__restrict__ nrm, const double
 }
 
 // Dynamic shared memory: the ring tables (w P, and P when anisotropic; sin theta), the azimuthal
-// factors (anisotropic), and per warp [nm x 32] sums and [32 / J x nm] scattered moments.
+// factors (anisotropic), and per warp [nm x 32] sums and [32 / J x nm] scattered moments; with a block per
+// group of cells [nm x 256] sums, then [cells x nm] and [split x cells x nm], at most 256 nm / J each.
 inline size_t sn_smem(size_t size, int R, int J, int n, bool iso)
 {
     const int nm = iso ? 1 : n;
-    return size * ((size_t)R * nm * (iso ? 1 : 2) + R + (iso ? 0 : (size_t)J * n) + (size_t)kWarps * nm * 64);
+    return size * ((size_t)R * nm * (iso ? 1 : 2) + R + (iso ? 0 : (size_t)J * n) + (size_t)nm * std::max(kWarps * 64, 256 + 512 / J));
 }
 
-template <typename P, int NN, bool ISO>
+// How the step's work is laid out. A warp with 32 / J cells of its own walks their rings, twice, without a
+// block barrier: best where there are cells for every warp. On a small mesh that is one chain of R
+// rings in a few blocks, and for J > 10 it leaves up to 15 lanes idle: there a block takes
+// 256 / (split J) cells together and its threads divide the rings into `split` parts. Eight warps of
+// an SM keep its FP64 pipe busy, so that the time goes with the blocks of the fullest SM, each of its
+// rings and two more for coefficients and sums (three with the block's barriers); the layout with the
+// least of that is taken. In FP32 a warp with its own cells is taken throughout (its sums keep their order).
+// FP64, 10 moments, ms a step, warp -> block: 338 cells, order 20 0.061 -> 0.020; 722 cells, order 15
+// 0.053 -> 0.022; 3,362 cells, order 34 0.36 -> 0.18; 10,082 cells, order 22 0.31 -> 0.26, order 34
+// 0.82 -> 0.47. 20,000 cells, order 15 (J = 8) keep the warp: 0.231.
+struct SnLayout {
+    int split;   // 0: a warp per group of cells
+    int blocks;
+};
+inline SnLayout sn_layout(int C, int R, int J, int nsm, bool fp64)
+{
+    const int most = nsm * (fp64 ? 2 : 3), per_block = kWarps * (32 / J), need = (C + per_block - 1) / per_block;
+    SnLayout best{0, std::min(need, most)};
+    if (!fp64) return best;
+    long cost = (long)((need + nsm - 1) / nsm) * (R + 2);
+    for (int split = 1; split <= 8 && split <= R && 32 * kWarps / split >= J; split *= 2) {
+        const int cells = 32 * kWarps / split / J, blocks = (C + cells - 1) / cells;
+        const long c = (long)((blocks + nsm - 1) / nsm) * ((R + split - 1) / split + 3);
+        if (c < cost) {
+            cost = c;
+            best = SnLayout{split, std::min(blocks, most)};
+        }
+    }
+    return best;
+}
+
+template <typename P, int NN, bool ISO, bool BLOCK>
 __global__ void __launch_bounds__(kWarps * 32, sizeof(P) == 4 ? 3 : 2)
 sn_quad_kernel(QuadTab<P> X, int Qf, const int4 *__restrict__ nbr, const P *__restrict__ cellc,
-               const P *__restrict__ psi, P *__restrict__ out, SnScat<P> sc, P dts, int bc, int C)
+               const P *__restrict__ psi, P *__restrict__ out, SnScat<P> sc, P dts, int bc, int C, int split)
 {
     constexpr int n = (NN + 1) * (NN + 2) / 2, nm = ISO ? 1 : n;
     extern __shared__ __align__(16) unsigned char sn_smem_raw[];
-    const int J = X.J, cpw = 32 / J;
+    // threads that share cells and their number of cells; the first ring of this thread and their distance
+    const int J = X.J, width = BLOCK ? 32 * kWarps / split : 32, cpw = width / J;
+    const int part = BLOCK ? threadIdx.x / width : 0, step = BLOCK ? split : 1;
     P *sW = reinterpret_cast<P *>(sn_smem_raw);  // [R][nm] w P
     P *sS = sW + X.R * nm;                       // [R] sin theta
     P *sP = sS + X.R;                            // [R][n] P (anisotropic)
@@ -91,9 +125,11 @@ sn_quad_kernel(QuadTab<P> X, int Qf, const int4 *__restrict__ nbr, const P *__re
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    P *red = sRed + wib * nm * 64, *mom = red + nm * 32;
-    const QuadLane<P> Q(X, lane);
-    for (int base = (blockIdx.x * kWarps + wib) * cpw; base < C; base += gridDim.x * kWarps * cpw) {
+    const int pitch = BLOCK ? 32 * kWarps : 32, at0 = BLOCK ? threadIdx.x : lane;  // of the sums
+    P *red = BLOCK ? sRed : sRed + wib * nm * 64, *mom = red + nm * pitch, *sums = mom + cpw * nm;
+    const QuadLane<P> Q(X, BLOCK ? threadIdx.x - part * width : lane, width);
+    const int groups = BLOCK ? gridDim.x : gridDim.x * kWarps;
+    for (int base = (BLOCK ? blockIdx.x : blockIdx.x * kWarps + wib) * cpw; base < C; base += groups * cpw) {
         const int i = min(base + Q.ci, C - 1);
         const bool store = Q.live && base + Q.ci < C;
         const P *own = psi + (size_t)i * Qf;
@@ -124,7 +160,7 @@ sn_quad_kernel(QuadTab<P> X, int Qf, const int4 *__restrict__ nbr, const P *__re
 #pragma unroll
         for (int a = 0; a < nm; ++a) G[a] = P(0);
 #pragma unroll 2
-        for (int r = 0; r < X.R; ++r) {
+        for (int r = part; r < X.R; r += step) {
             const P *p = own + r * 2 * X.P;
             P a1, a2, b1, b2;
             quad_load(Q, p, a1, a2, b1, b2);
@@ -135,16 +171,31 @@ sn_quad_kernel(QuadTab<P> X, int Qf, const int4 *__restrict__ nbr, const P *__re
                 quad_project<NN, P>(Q.axes, a1 + a2, a1 - a2, b1 + b2, b1 - b2, sW + r * n, G);
         }
         const P dtA = cf[6], keep = cf[7], src = cf[8], sig_s = cf[9];
-        __syncwarp();
+        auto barrier = [] {
+            if constexpr (BLOCK) __syncthreads();
+            else __syncwarp();
+        };
+        // (a block's sums of the former cells were read before its last two barriers)
+        if constexpr (!BLOCK) __syncwarp();
 #pragma unroll
-        for (int a = 0; a < nm; ++a) red[a * 32 + lane] = ISO ? G[a] : G[a] * sT[ISO ? 0 : Q.j * n + a];
-        __syncwarp();
-        P b[nm], iso = P(0);  // scattered moments times the lane's azimuthal factors
-        if constexpr (ISO) {
-            for (int t = 0; t < J; ++t) iso += red[Q.ci * J + t];
-            // dt (O Sigma M psi + q): sigma_s m_0 (sum_q w_q m_0 psi_q), the ring table holds w m_0
-            iso = q_fma(dts * sig_s * X.ringP[0], iso, src);
-        } else {
+        for (int a = 0; a < nm; ++a) red[a * pitch + at0] = ISO ? G[a] : G[a] * sT[ISO ? 0 : Q.j * n + a];
+        barrier();
+        if constexpr (BLOCK) {
+            // the J sums of each part, then the parts
+            for (int e = threadIdx.x; e < split * cpw * nm; e += 32 * kWarps) {
+                const int sp = e / (cpw * nm), cc = (e - sp * cpw * nm) / nm, a = e % nm;
+                P v = P(0);
+                for (int t = 0; t < J; ++t) v += red[a * pitch + sp * width + cc * J + t];
+                sums[e] = v;
+            }
+            __syncthreads();
+            for (int e = threadIdx.x; e < cpw * nm; e += 32 * kWarps) {
+                P v = P(0);
+                for (int sp = 0; sp < split; ++sp) v += sums[sp * cpw * nm + e];
+                mom[e] = ISO ? v : sc.ga[e % nm] * v;
+            }
+            __syncthreads();
+        } else if constexpr (!ISO) {
             for (int e = lane; e < cpw * n; e += 32) {
                 const int cc = e / n, a = e - cc * n;
                 P v = P(0);
@@ -152,13 +203,22 @@ sn_quad_kernel(QuadTab<P> X, int Qf, const int4 *__restrict__ nbr, const P *__re
                 mom[cc * n + a] = sc.ga[a] * v;
             }
             __syncwarp();
+        }
+        P b[nm], iso = P(0);  // scattered moments times the lane's azimuthal factors
+        if constexpr (ISO) {
+            if constexpr (BLOCK) iso = mom[Q.ci];
+            else
+                for (int t = 0; t < J; ++t) iso += red[Q.ci * J + t];
+            // dt (O Sigma M psi + q): sigma_s m_0 (sum_q w_q m_0 psi_q), the ring table holds w m_0
+            iso = q_fma(dts * sig_s * X.ringP[0], iso, src);
+        } else {
 #pragma unroll
             for (int a = 0; a < nm; ++a) b[a] = mom[Q.ci * n + a] * (dts * sig_s) * sT[Q.j * n + a];
         }
         // update
         P *o = out + (size_t)i * Qf;
 #pragma unroll(sizeof(P) == 4 ? 2 : 1)
-        for (int r = 0; r < X.R; ++r) {
+        for (int r = part; r < X.R; r += step) {
             const int at = r * 2 * X.P;
             P a1, a2, b1, b2;
             quad_load(Q, own + at, a1, a2, b1, b2);
@@ -188,20 +248,27 @@ sn_quad_kernel(QuadTab<P> X, int Qf, const int4 *__restrict__ nbr, const P *__re
     }
 }
 
+template <typename P, int NN, bool ISO, bool BLOCK>
+int launch_sn_as(kitrt_mn *mn, const QuadTab<P> &X, const P *psi, P *out, const P *cellc, const SnScat<P> &sc, double dt,
+                 const SnLayout &lay, cudaStream_t s)
+{
+    const kitrt_mesh *m = mn->mesh;
+    const size_t smem = sn_smem(sizeof(P), mn->R, mn->J, mn->n, ISO);
+    if (ensure_dyn_smem(sn_quad_kernel<P, NN, ISO, BLOCK>, smem)) return KITRT_ECUDA;
+    LaunchScope ls(mn, PK_SN, s, m->C);
+    sn_quad_kernel<P, NN, ISO, BLOCK><<<lay.blocks, kWarps * 32, smem, s>>>(X, mn->Qf, m->d_nbr, cellc, psi, out, sc,
+                                                                            (P)dt, mn->p.bc, m->C, lay.split);
+    return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
+}
+
 template <typename P, int NN, bool ISO>
 int launch_sn(kitrt_mn *mn, const QuadTab<P> &X, const P *psi, P *out, const P *cellc, const SnScat<P> &sc,
               double dt, cudaStream_t s)
 {
-    const kitrt_mesh *m = mn->mesh;
-    const int C = m->C;
-    const size_t smem = sn_smem(sizeof(P), mn->R, mn->J, mn->n, ISO);
-    if (ensure_dyn_smem(sn_quad_kernel<P, NN, ISO>, smem)) return KITRT_ECUDA;
-    const int per_block = kWarps * (32 / mn->J), need = (C + per_block - 1) / per_block;
-    const int most = mn->nsm * (sizeof(P) == 4 ? 3 : 2);  // persistent: the blocks resident at once
-    LaunchScope ls(mn, PK_SN, s, C);
-    sn_quad_kernel<P, NN, ISO><<<need < most ? need : most, kWarps * 32, smem, s>>>(
-        X, mn->Qf, m->d_nbr, cellc, psi, out, sc, (P)dt, mn->p.bc, C);
-    return cudaGetLastError() == cudaSuccess ? KITRT_OK : KITRT_ECUDA;
+    const SnLayout lay = sn_layout(mn->mesh->C, mn->R, mn->J, mn->nsm, sizeof(P) == 8);
+    if constexpr (sizeof(P) == 8)
+        if (lay.split) return launch_sn_as<P, NN, ISO, true>(mn, X, psi, out, cellc, sc, dt, lay, s);
+    return launch_sn_as<P, NN, ISO, false>(mn, X, psi, out, cellc, sc, dt, lay, s);
 }
 
 template <typename P, bool ISO>

@@ -19,3 +19,13 @@ def test_sn_shapes(K, N, order, aniso, fp32):  # noqa: F811
     # FP64 as the other S_N tests; FP32: the start, three steps of about twenty operations, and a sum
     # over Q' ordinates per step, each at 6e-8
     assert np.abs(got - ref).max() <= (5e-6 if fp32 else 1e-12) * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("aniso", [False, True])
+@pytest.mark.parametrize("N,order,k", [(1, 2, 7), (1, 3, 75), (4, 5, 75), (3, 9, 75), (5, 15, 40), (2, 22, 30), (1, 34, 24)])
+def test_sn_layouts(K, N, order, k, aniso):  # noqa: F811
+    """FP64 on meshes of both sides of the rule between a warp and a block per group of cells, and of one to
+    eight parts of the rings."""
+    g = [0.7 ** l for l in range(N + 1)] if aniso else None
+    got, ref, _ = _run_pair(K, k, N, order, "vacuum", g, 2, fp32=False, seed=order)
+    assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
