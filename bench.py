@@ -195,13 +195,14 @@ def multiplier_peak(torch, sm_mhz):
 def sweep_multiplies(W, fp64):
     """32 x 32-bit multiplications of one cell evaluation in the 64-bit fixed-point sweep. A quad of
     azimuths (J of them in each of the R rings) takes 3 per product of its 2N exponent terms and its
-    2L moment sums (two limbs each way, without the low product), and 7 per exponential; a ring
-    takes 3 per exponent coefficient and 4 per moment. L = N in the mixed modes, 2N in FP64 mode."""
+    2L moment sums (two limbs each way, without the low product; none for the quad on the axes), and
+    7 per exponential; a ring takes 4 per exponent coefficient and 4 per moment. L = N in the mixed
+    modes, 2N in FP64 mode."""
     N, R = W["N"], (W["order"] + 1) // 2
     J = (W["order"] + 1) // 2
     L = 2 * N if fp64 else N
     nout = (L + 1) * (L + 2) // 2
-    return R * J * (3 * 2 * N + 4 * 7 + 3 * 2 * L) + R * (3 * W["n"] + 4 * nout)
+    return R * ((J - 1) * (3 * 2 * N + 3 * 2 * L) + J * 4 * 7) + R * (4 * W["n"] + 4 * nout)
 
 
 def train_network(K, torch, W, samples, seed=4):
@@ -652,7 +653,6 @@ def main():
                                     "/ the sweep's CUDA-event time",
                      "multiplies_per_cell_eval": ops,
                      "fp64_flops_per_cell_eval": fl,
-                     "fp64_tflops_achieved": pe["units"] * fl / sweep_s / 1e12,
                      "exps_per_cell_eval": work["exps"],
                      "sweep_grid": work["sweep_grid"], "sweep_items": work["sweep_items"],
                      "tensor_flops_per_cell_eval": work["tensor_flops"],

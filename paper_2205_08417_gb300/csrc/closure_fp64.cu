@@ -1,16 +1,20 @@
 // FP64 entropy closure: Newton's method on the dual of the minimum-entropy problem
 // [Sec. 3.1, Eq. entropyOCP; Maxwell-Boltzmann entropy], with Armijo backtracking.
 //
-// One warp owns one cell. The quadrature sums run lane-strided over the folded points:
-//   z_q = alpha . m_q,  e_q = w_q exp(z_q),  V_c = sum_q e_q m~_c(q)   (c over the degree-2N
-// basis), so that U = V[0:n] are the ansatz moments, <exp(alpha.m)> = V_0 / m_0 and the Hessian
-// H_ab = sum_c G_abc V_c (Gaunt coefficients) comes without per-point pair products. The Cholesky
-// factorisation and the triangular solves are spread over the warp (lane = matrix row).
+// A round evaluates every listed cell at its trial point and takes its Newton step, in two kernels:
+//  - the sweep (a thread per cell and part of the quadrature) forms the degree-2N moments
+//      V_c = sum_q w_q exp(alpha.m_q) m~_c(q)
+//    in the sum-factorised fixed-point form of sweep.cuh, so that U = V[0:n] are the ansatz moments,
+//    <exp(alpha.m)> = V_0 / m_0 and the Hessian H_ab = sum_c G_abc V_c (Gaunt coefficients) comes
+//    without per-point pair products;
+//  - the Newton kernel (newton_common.cuh: 8 lanes or a thread per cell) adds the parts, decides the line
+//    search, factorises the Hessian and finds the next direction.
+// Here are also the start of a closure (continuation test, predictor), its end (alpha, FP64 ansatz) and the
+// allocation-free closure's kernel, a warp per cell in FP64.
 //
-// Cells that still iterate are kept in a compacted list; every launch advances each listed cell
-// by one evaluation (one trial point of the line search) and writes the cells that continue into
-// the next list. Counters rotate over three slots so that no launch has to clear the slot it
-// fills.
+// Cells that still iterate are kept in a compacted list; every round advances each listed cell by one
+// evaluation (one trial point of the line search) and writes the cells that continue into the next
+// list. Counters rotate over three slots so that no launch has to clear the slot it fills.
 #include <math.h>
 
 #include "async_copy.cuh"
@@ -124,9 +128,9 @@ begin_test_kernel(NewtonState S, const double *__restrict__ u, const double *__r
 // too. M_5, 996,872 cells: a warp per cell took 8.2 ms a step, strided reads 7.0, whole factors in
 // shared memory (3 warps on an SM) 3.4, with the test that precedes it. SEG (M_5, more cells than those 3
 // warps on every SM take at once) stages the rows in segments of at most kSegPairs entries, each but
-// the last once more for the backward solve, so that 8 warps fit: 2.2 ms. With one wave the segments'
-// round trips only add latency: M_4, 20,000 cells, 6 warps on an SM, two steps 0.094 ms whole, 0.114 in
-// segments.
+// the last once more for the backward solve, so that 8 warps fit: 2.2 ms. For M_4 whole factors leave
+// room for 6 warps, and segments gain nothing: the test and two predictors on 20,000, 178,802 and
+// 498,002 cells take 0.092, 0.511 and 1.320 ms whole, 0.093, 0.537 and 1.326 in segments.
 template <int NN, bool SEG>
 struct PredictDims {
     static constexpr bool in_regs = NN <= 3;
@@ -331,7 +335,7 @@ eval_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, Newton
         for (int c = 0; c < n2; ++c)
             if (lane == (c & 31)) Vs[c] = V[c];
         __syncwarp();
-        newton_post<NN>(T, S, np, cell, ph, lam, at, ua, Vs, H, list_out, cnt_out, lane, false);
+        newton_post<NN>(T, S, np, cell, ph, lam, at, ua, Vs, H, list_out, cnt_out, lane);
         __syncwarp();
     }
 }
@@ -741,8 +745,9 @@ int launch_isotropic(const Tables &T, int C, const double *u, double *alpha, cud
 }
 
 // Cells up to which a round of the FP64 mode goes to the 8-lane kernel (N <= 3): there a warp's FP64
-// instructions serve 4 cells instead of 32, which is slower once the thread-per-cell kernel fills
-// the SMs. M_3: 8 lanes take about 8 us per 2,500 cells, a thread per cell 45 us up to 39,000.
+// instructions serve 4 cells instead of 32, which is slower once the thread-per-cell kernel has warps for
+// the SMs. M_3, whole passes with the line at 8,192 and at 14,000 cells: 20,001 closures of 24 rounds
+// 2.385 and 2.416 ms, adjoint of 59,168 cells 41.65 and 41.78 ms.
 constexpr int kGroupUpTo = 8192;
 
 // Newton step of the listed cells.

@@ -105,13 +105,12 @@ __device__ double warp_chol_solve(const double *sH, double b, int lane)
 
 // Newton logic of one cell after an evaluation of the dual at the trial point `at` (lane a holds
 // component a). Vs holds the n2 degree-2N moments sum_q w_q e_q m~_c(q) (warp-visible), whose
-// first n entries are the ansatz moments U. One warp per cell; every branch is warp-uniform.
-//   mixed: the moments Vs[n..n2) came from tensor cores; a Cholesky breakdown or a stalled
-//          residual sends the cell to the FP64 Hessian (S.h64) instead of failing it.
+// first n entries are the ansatz moments U. One warp per cell; every branch is warp-uniform. Used by the
+// allocation-free closure, in FP64 throughout.
 template <int NN>
 __device__ void newton_post(const Tables &T, const NewtonState &S, const NewtonParams &np,
                             int cell, int ph, double lam, double at, double ua, const double *Vs,
-                            double *H, int32_t *list_out, int32_t *cnt_out, int lane, bool mixed)
+                            double *H, int32_t *list_out, int32_t *cnt_out, int lane)
 {
     constexpr int n = Dims<NN>::n, n2 = Dims<NN>::n2, npairs = Dims<NN>::npairs;
     const size_t off = (size_t)cell * n;
@@ -141,15 +140,7 @@ __device__ void newton_post(const Tables &T, const NewtonState &S, const NewtonP
     }
     if (!accept) {
         const int h = S.halv[cell] + 1;
-        if (h > np.max_halvings && mixed && !S.h64[cell]) {
-            // as in post_group_kernel: restart from the accepted point with the FP64 Hessian
-            if (lane == 0) {
-                hand_over(S, cell);
-                S.halv[cell] = 0;
-                S.phase[cell] = PH_INIT;
-            }
-            push(list_out, cnt_out, cell, lane);
-        } else if (h > np.max_halvings) {
+        if (h > np.max_halvings) {
             fail(S, cell, KITRT_ELINESEARCH, lane);
         } else {
             if (lane == 0) {
@@ -174,13 +165,7 @@ __device__ void newton_post(const Tables &T, const NewtonState &S, const NewtonP
     __syncwarp();
     if (!warp_cholesky<n>(H, lane)) {
         __syncwarp();
-        if (mixed) {
-            // tensor-core rounding broke positive definiteness: redo this point in FP64
-            if (lane == 0) hand_over(S, cell);
-            push(list_out, cnt_out, cell, lane);
-        } else {
-            fail(S, cell, KITRT_ECHOL, lane);
-        }
+        fail(S, cell, KITRT_ECHOL, lane);
         return;
     }
     // accepted: store the point, its moments and the factor of H
@@ -195,7 +180,6 @@ __device__ void newton_post(const Tables &T, const NewtonState &S, const NewtonP
     }
     for (int a = lane; a < n; a += 32)
         for (int b = 0; b <= a; ++b) S.L[(size_t)cell * npairs + tri_idx(a, b)] = H[a * n + b];
-    if (lane == 0 && S.lfac) S.lfac[cell] = 1;
     const double g = lane < n ? fma(lane >= np.reg0 ? np.gamma : 0.0, at, Ua - ua) : 0.0;
     const double d = warp_chol_solve<n>(H, -g, lane);
     __syncwarp();
@@ -213,8 +197,6 @@ __device__ void newton_post(const Tables &T, const NewtonState &S, const NewtonP
         return;
     }
     if (lane == 0) {
-        if (mixed && ph == PH_NEWTON && gn2 > kStallRatio * kStallRatio * S.gnorm[cell]) hand_over(S, cell);
-        if (S.gnorm) S.gnorm[cell] = gn2;
         S.gd[cell] = gd;
         S.lam[cell] = 1.0;
         S.halv[cell] = 0;

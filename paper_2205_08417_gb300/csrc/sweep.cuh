@@ -16,7 +16,7 @@
 // pi/2, 3 pi/2 (only the first two when the number of pairs per ring is odd) need no products.
 // The arithmetic is 64-bit fixed point (fixed.cuh): the FP64 pipe (16 cycles per warp instruction)
 // bound the FP64 form of this pass. Measured on 99,458 cells, M_3, order 20 (400 folded points):
-// tensor-core sweep 4.86 -> 1.71 ms for 350,160 cell evaluations, FP64-mode sweep 3.83 -> 0.89 ms
+// tensor-core sweep 4.86 -> 1.53 ms for 350,160 cell evaluations, FP64-mode sweep 3.83 -> 0.86 ms
 // for 219,742. Now bound by integer issue: about 25 32x32->64-bit products per point, each 4 cycles
 // of the multiply pipe of a scheduler, and twice as many other instructions.
 //
