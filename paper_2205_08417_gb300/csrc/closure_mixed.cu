@@ -16,7 +16,7 @@
 //
 // What bounds it (M_3, a round of 99,458 cells): issue 56% of active cycles, the multipliers' pipe
 // 51% of elapsed, the ALU 50%; the rest is fixed latency with 16 warps on an SM (8 for N >= 4, where
-// a row's state takes 216 registers; 16 warps there, with the moments in shared memory, took 42.4 ms
+// a row's state takes 220 registers; 16 warps there, with the moments in shared memory, took 42.4 ms
 // against 39.9 for M_5: more instructions and barrier waits than the latency it hid).
 //
 // One CTA (256 threads) owns a tile of 128 listed cells (the MMA's M = 128 rows, row = cell). The
