@@ -672,7 +672,7 @@ __device__ __forceinline__ bool group_factor_solve_shared(const Tables &T, const
 __host__ __device__ inline size_t group_smem_bytes(int n2, int npairs, int nnz, bool mixed)
 {
     return (size_t)n2 * kGroupPitch * (mixed ? 12 : 8) + (size_t)kGroupCells * npairs * 8 + (size_t)nnz * (mixed ? 4 : 8) +
-           (size_t)((nnz + 3) / 4 * 4) + (size_t)(npairs + 1) * 4 + 2 * kGroupCells * 4;
+           (size_t)((nnz + 3) / 4 * 4) + (size_t)(npairs + 1) * 4 + 2 * kGroupCells * 4 + 2 * kGroupCells * 8;
 }
 
 template <int NN, bool MIXED>
@@ -685,7 +685,8 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
     extern __shared__ __align__(16) unsigned char group_smem[];
     double *sV = reinterpret_cast<double *>(group_smem);                           // [n2][pitch]
     double *sH = sV + n2 * kGroupPitch;                                            // [cell][npairs]
-    unsigned char *coef = reinterpret_cast<unsigned char *>(sH + kGroupCells * npairs);
+    double *sAu = sH + kGroupCells * npairs;                                       // [2][cell]
+    unsigned char *coef = reinterpret_cast<unsigned char *>(sAu + 2 * kGroupCells);
     float *sVf = reinterpret_cast<float *>(coef + (size_t)nnz * (MIXED ? 4 : 8));  // [n2][pitch]
     int32_t *gstart = reinterpret_cast<int32_t *>(sVf + (MIXED ? n2 * kGroupPitch : 0));
     int32_t *scell = gstart + npairs + 1, *sh64 = scell + kGroupCells;
@@ -723,7 +724,6 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
         const int ph = valid ? S.phase[cell] : PH_DONE;
         const double lam = ph == PH_NEWTON ? S.lam[cell] : 0.0;
         double at[SL], ua[SL], gr[SL];
-        double au = 0.0, ar2 = 0.0;
 #pragma unroll
         for (int s = 0; s < SL; ++s) {
             const int c = g + 8 * s;
@@ -731,8 +731,11 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
             const double al = in ? S.alpha[off + c] : 0.0;
             at[s] = in && ph == PH_NEWTON ? fma(lam, S.dir[off + c], al) : al;
             ua[s] = in ? u[off + c] : 0.0;
-            au = fma(at[s], ua[s], au);
-            if (reg && c >= np.reg0) ar2 = fma(at[s], at[s], ar2);
+            // for alpha.u below: component c of the pass's cells, rotated so that neither side conflicts
+            if (c < n) {
+                sH[c * kGroupCells + (slot ^ ((c & 7) << 2))] = at[s];
+                sH[(n + c) * kGroupCells + (slot ^ ((c & 7) << 2))] = ua[s];
+            }
         }
         double fs0 = 0.0, f0 = 0.0, gd0 = 0.0, gnorm0 = 0.0;  // of the accepted point (gnorm: squared)
         if (ph == PH_NEWTON) {
@@ -764,6 +767,22 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
             }
         }
         __syncthreads();
+        // alpha.u in the order of the components, as in the predictor and the thread-per-cell kernel: the
+        // line search compares sums of terms far larger than themselves where alpha is large, and
+        // summed over the lanes in a tree twice as many badly conditioned closures stalled in it. A
+        // thread per cell, so that an FP64 instruction serves the block's 32 (in every group, by
+        // shuffles, the M_3 mixed pass took 2.5% longer).
+        if (tid < kGroupCells) {
+            double sum = 0.0, sq = 0.0;
+#pragma unroll
+            for (int c = 0; c < n; ++c) {
+                const double x = sH[c * kGroupCells + (tid ^ ((c & 7) << 2))];
+                sum = fma(x, sH[(n + c) * kGroupCells + (tid ^ ((c & 7) << 2))], sum);
+                if (reg && c >= np.reg0) sq = fma(x, x, sq);
+            }
+            sAu[tid] = sum;
+            if (reg) sAu[kGroupCells + tid] = sq;
+        }
         const double *V = sV + slot;
         const float *Vf = sVf + slot;
         bool fin = true;
@@ -771,8 +790,8 @@ post_group_kernel(Tables T, NewtonState S, const double *__restrict__ u, int k, 
             fin = fin && (c < n || !h32 ? finite_bits(V[c * kGroupPitch])
                                         : (__float_as_uint(Vf[c * kGroupPitch]) & 0x7f800000u) != 0x7f800000u);
         const bool finite = ((~__ballot_sync(kFull, fin) >> (lane & 24)) & 0xffu) == 0;
-        au = group_sum(au);
-        if (reg) ar2 = group_sum(ar2);
+        __syncthreads();
+        const double au = sAu[slot], ar2 = reg ? sAu[kGroupCells + slot] : 0.0;
         const double fs = V[0] * T.rm0;
         const double ft = reg ? fma(0.5 * np.gamma, ar2, fs - au) : fs - au;
         bool accept = valid && finite;
