@@ -1,5 +1,7 @@
 """Device memory of a solver: what it keeps per cell is its state, one column of moments, the ansatz
 and the coefficients of the S_N step, in every mode."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -25,6 +27,7 @@ def test_bytes_per_cell(mode):
     if mode == "learned":
         doubles += n
         ints += 1
+    gc.collect()  # no solver of another test is freed between the readings
     used, cells, keep = [], [], []
     for k in (60, 480):  # the first one also loads the kernels
         m = synth.jittered_mesh(k, 0.0, 1.0, seed=1)
